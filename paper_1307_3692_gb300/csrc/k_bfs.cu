@@ -40,7 +40,8 @@
 // over the frontier list (every level-r vertex is on it) and one more grid
 // barrier.  The first bottom-up round of a run examines every
 // vertex the BFS owns; each round lists the vertices still above level r + 1,
-// and the next bottom-up round examines only those.
+// and the next bottom-up round examines only those.  Large bottom-up rounds
+// stop at a pivot instead of the floor and have a second pass (pull_rest).
 //
 // Rounds with an empty frontier jump straight to the next non-empty start
 // bucket; the loop stops as soon as every vertex with an arc is settled.
@@ -67,10 +68,27 @@ constexpr int kWinBatch = 3;   // window items per thread in flight
 // three)
 constexpr int pull_width(int per_sm) { return per_sm >= 2 ? 2 : 3; }
 constexpr int kPullLong = 32;  // longer adjacency lists are scanned by the whole warp
+// Bottom-up rounds of at least kDeferMin candidates stop their scans at a
+// pivot rank and have a second, edge-balanced pass (pull_rest); smaller rounds
+// save its grid barrier.
+constexpr u32 kDeferMin = 1u << 16;
+// A warp with at least kDeferLanes scans still going after kPullShort
+// neighbours puts them all off to that pass, any other warp those with at
+// least kDeferLong neighbours left.
+constexpr int kPullShort = 8;
+constexpr u32 kDeferLanes = 32;
+constexpr int kDeferLong = 2048;
+constexpr int kRestBatch = 8;   // the second pass: neighbours per lane in flight
+constexpr u32 kPushFlag = 1u << 31;  // on its list: a frontier vertex that pushes
+constexpr int kRestSide = 2;    // the side of the frontier arrays that holds the list
+// the pivot is the kPivotSkip-th smallest (from 0) of kPivotSamples sampled ranks
+constexpr u32 kPivotSamples = 128;
+constexpr u32 kPivotSkip = 2;
 constexpr int kPullCoop = 4;   // neighbours per lane per step of a warp-wide scan
-// Unions of at most this many members keep their per-member floors in shared
-// memory (two tables after Smem); larger unions use the global table directly.
-constexpr u32 kSmemMembers = 4096;
+// Unions of at most this many members keep their per-member floors and pivots
+// in shared memory (after Smem: 16 bytes per member, 32 KB, so that two CTAs
+// per SM still fit); larger unions use the global tables directly.
+constexpr u32 kSmemMembers = 2048;
 constexpr int kLdBatch = 8;    // low-degree rounds: arcs per frontier vertex and step
 constexpr int kLdItems = 1;    // low-degree rounds: items per thread in flight
 
@@ -84,12 +102,14 @@ struct Smem {
   // the next round's frontier counter, bottom-up floor and unsettled-list
   // length, read by thread 0 as the barrier releases
   u64 next_c;
+  u64 next_rest;         // a large bottom-up round's list for its second pass
   u32 next_minrank;
   u32 next_ucnt;
   int next_lo, next_hi;  // the next round's start bucket (lvl + 1) bounds
   u32 next_ovf;          // the next round's overflow-list length (windows)
   u32 lcnt[3];           // windows: local-queue lengths, rotating (read, fill, clear)
   u32 nstart;            // a scan's result, shared by the CTA
+  u32 pivot;             // the round's pivot rank
 };
 // Windows of levels keep two local queues whose entries carry a vertex, the
 // key it was pushed with and its adjacency range (20 bytes, as four arrays).
@@ -176,6 +196,7 @@ __device__ __forceinline__ void grid_barrier(Control* ctl, u32& gen, u32 nblocks
       s.next_minrank = ld_cg_u32(&ctl->minrank[post]);
       s.next_ucnt = ld_cg_u32(&ctl->ucnt[post]);
       s.next_ovf = ld_cg_u32(&ctl->ovf[post]);
+      s.next_rest = ld_cg_u64(&ctl->rest[post]);
       s.next_lo = s.next_hi = 0;
       if (blevel >= 0) {  // bounds of start bucket blevel, for the round after the barrier
         s.next_lo = __ldg(bptr + blevel);
@@ -224,6 +245,12 @@ __device__ __forceinline__ u64 warp_min64(u64 x) {
   return x;
 }
 
+__device__ __forceinline__ u64 warp_max64(u64 x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = max(x, (u64)__shfl_xor_sync(kFull, x, o));
+  return x;
+}
+
 // Records a successful next-level key (vertex v, rank) for the bottom-up
 // floor of the next round: the thread's running minimum, folded into the
 // CTA's and the grid's at the barrier.  Unions track nothing here: their floor
@@ -243,50 +270,79 @@ __device__ __forceinline__ void note_rank(const BfsArgs& a, u32 slot, bool valid
 
 // Unions: the per-member floors of level-L keys (the smallest rank among each
 // member's keys of the frontier's level) from the frontier list qv of Q
-// vertices, into slot `slot` of a.mrank (all ~0 on entry).  A warp whose
-// vertices share one member makes one update; small unions gather the minima
-// per CTA in shared memory (s_acc) and flush them.  The caller then waits at a
-// grid barrier before the floors are read.
+// vertices, into slot `slot` of a.mrank (all ~0 on entry), and with kPivot
+// every member's frontier vertex of the largest degree into a.mpivot (as
+// (degree << 32) | vertex, all zero on entry; see pull_rest).  A warp whose
+// vertices share one member makes one update; small unions gather both per CTA
+// in shared memory (s_acc, s_piv) and flush them.  The caller then waits at a
+// grid barrier before they are read.
+template <bool kPivot>
 __device__ __forceinline__ void member_floors(const BfsArgs& a, const u32* qv, u32 Q, u32 slot,
-                                              u32* s_acc) {
+                                              u32* s_acc, u64* s_piv) {
   const u32 lane = threadIdx.x & 31;
   const u32 stride = gridDim.x * blockDim.x;
   for (u32 base = warp_first_item(1); base < Q; base += stride) {
     const u32 i = base + lane;
     const bool valid = i < Q;
     u32 v = 0, m = 0xffffffffu, r = 0xffffffffu;
+    u64 pv = 0;
     if (valid) {
       v = ld_cg_u32(qv + i);
       m = __ldg(a.wmem + (v >> 5));
       r = (u32)ld_cg_u64(a.key + v);
+      if (kPivot) pv = (u64)(u32)(__ldg(a.row_ptr + v + 1) - __ldg(a.row_ptr + v)) << 32 | v;
     }
     const u32 act = __ballot_sync(kFull, valid);
     const u32 m0 = __shfl_sync(kFull, m, __ffs(act) - 1);
     const bool one = __all_sync(kFull, !valid || m == m0);
     const u32 rr = one ? warp_min(r) : r;
+    const u64 pp = kPivot && one ? warp_max64(pv) : pv;
     if ((one && lane == 0) || (!one && valid)) {
       const u32 mm = one ? m0 : m;
       if (s_acc) {
         if (rr < s_acc[mm]) atomicMin(s_acc + mm, rr);
+        if (kPivot && pp > s_piv[mm]) atomicMax(s_piv + mm, pp);
       } else {
         u32* p = a.mrank + (size_t)slot * a.kmem + mm;
         if (rr < ld_cg_u32(p)) atomicMin(p, rr);
+        u64* q = a.mpivot + (size_t)slot * a.kmem + mm;
+        if (kPivot && pp > ld_cg_u64(q)) atomicMax(q, pp);
       }
     }
   }
 }
 
-// Union: the CTA's per-member minima into slot `slot` of a.mrank, and the
-// shared table reset.  Called by the whole CTA between __syncthreads.
-__device__ __forceinline__ void flush_members(const BfsArgs& a, u32 slot, u32* s_acc) {
+// Union: the CTA's per-member minima into slot `slot` of a.mrank (and the
+// pivots into a.mpivot), and the shared tables reset.  Called by the whole CTA
+// between __syncthreads.
+template <bool kPivot>
+__device__ __forceinline__ void flush_members(const BfsArgs& a, u32 slot, u32* s_acc,
+                                              u64* s_piv) {
   for (u32 m = threadIdx.x; m < a.kmem; m += blockDim.x) {
     const u32 r = s_acc[m];
     if (r != 0xffffffffu) {
       u32* p = a.mrank + (size_t)slot * a.kmem + m;
       if (r < ld_cg_u32(p)) atomicMin(p, r);
       s_acc[m] = 0xffffffffu;
+      if (kPivot) {
+        u64* q = a.mpivot + (size_t)slot * a.kmem + m;
+        if (s_piv[m] > ld_cg_u64(q)) atomicMax(q, s_piv[m]);
+        s_piv[m] = 0;
+      }
     }
   }
+}
+
+// Union: what a bottom-up scan of w may stop at, the smallest rank of its
+// member's level-L keys or (pivot) the rank of the member's pivot; ~0 when the
+// member has no level-L key.  s_floor: the CTA's copy, already the one of the two.
+__device__ __forceinline__ u32 member_floor(const BfsArgs& a, u32 w, u32 slot, const u32* s_floor,
+                                            bool pivot) {
+  const u32 m = __ldg(a.wmem + (w >> 5));
+  if (s_floor) return s_floor[m];
+  if (!pivot) return ld_cg_u32(a.mrank + (size_t)slot * a.kmem + m);
+  const u64 pv = ld_cg_u64(a.mpivot + (size_t)slot * a.kmem + m);
+  return pv ? (u32)ld_cg_u64(a.key + (u32)pv) : 0xffffffffu;
 }
 
 // Appends to the frontier every vertex v[i] whose bit i is set in `mask`, for
@@ -957,6 +1013,237 @@ __device__ __forceinline__ void pull_append(u32 mask, u32 keep, const u32 (&v)[K
     if (keep >> i & 1u) list[kbase++] = v[i];
 }
 
+// Puts vertices w[i] (bits of mask; with kPushFlag: see pull_rest) with the
+// arcs [e[i], re[i]) on the list that pull_rest works off, in the frontier's
+// own format (vertex, first arc, exclusive arc offset, first slot of every base
+// chunk) on side kRestSide of the frontier arrays.
+template <int K>
+__device__ __forceinline__ void defer_append(u32 mask, const u32 (&w)[K], const int (&e)[K],
+                                             const int (&re)[K], const BfsArgs& a, u64* ctr) {
+  if (!__any_sync(kFull, mask != 0u)) return;
+  const u32 lane = threadIdx.x & 31;
+  u64 mine = 0;
+#pragma unroll
+  for (int i = 0; i < K; ++i)
+    if (mask >> i & 1u) mine += kLevelOne | (u32)(re[i] - e[i]);
+  u64 incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const u64 y = __shfl_up_sync(kFull, incl, o);
+    if (lane >= (u32)o) incl += y;
+  }
+  u64 base = 0;
+  if (lane == 31) base = atomicAdd(ctr, incl);
+  base = __shfl_sync(kFull, base, 31) + (incl - mine);
+  u32 slot = (u32)(base >> 32), off = (u32)base;
+#pragma unroll
+  for (int i = 0; i < K; ++i)
+    if (mask >> i & 1u) {
+      a.qv[kRestSide][slot] = w[i];
+      a.qrow[kRestSide][slot] = e[i];
+      a.qoff[kRestSide][slot] = off;
+      const u32 end = off + (u32)(re[i] - e[i]);
+      for (u32 c = (off + kBfsBase - 1) / kBfsBase; c * kBfsBase < end; ++c)
+        a.cf[kRestSide][c] = slot;
+      ++slot;
+      off = end;
+    }
+}
+
+// A bottom-up round's pivot rank (single graphs): kPivotSamples evenly spaced
+// samples of the frontier's E arcs, each with the rank of its vertex's key; the
+// kPivotSkip-th smallest.  Every CTA takes the same samples of a list that no
+// longer changes, so all get the same pivot without a barrier.
+__device__ __forceinline__ u32 pivot_rank(const BfsArgs& a, Smem& s, int cur, u32 Q, u32 E) {
+  const u32 nb = (E + kBfsBase - 1) / kBfsBase;
+  u32* smp = reinterpret_cast<u32*>(s.owner);
+  u32 r = 0;
+  __syncthreads();
+  if (threadIdx.x < kPivotSamples) {
+    const u32 slot = ld_cg_u32(a.cf[cur] + (u32)((u64)threadIdx.x * nb / kPivotSamples));
+    r = (u32)ld_cg_u64(a.key + ld_cg_u32(a.qv[cur] + min(slot, Q - 1)));
+    smp[threadIdx.x] = r;
+  }
+  __syncthreads();
+  if (threadIdx.x < kPivotSamples) {
+    u32 less = 0, same = 0;
+#pragma unroll 8
+    for (u32 i = 0; i < kPivotSamples; ++i) {
+      const u32 x = smp[i];
+      less += x < r ? 1u : 0u;
+      same += x == r ? 1u : 0u;
+    }
+    if (less <= kPivotSkip && kPivotSkip < less + same) s.pivot = r;  // one value
+  }
+  __syncthreads();
+  return s.pivot;
+}
+
+// The frontier vertices whose rank lies below the pivot (their member's pivot)
+// go on pull_rest's list, to push.
+template <bool U>
+__device__ __forceinline__ void list_pushes(const BfsArgs& a, int cur, u32 Q, u32 pivot,
+                                            u32 mslot, int qi, const u32* s_floor) {
+  const u32 lane = threadIdx.x & 31;
+  const u32 stride = gridDim.x * blockDim.x;
+  for (u32 base = warp_first_item(1); base < Q; base += stride) {
+    const u32 i = base + lane;
+    u32 v[1] = {0};
+    int rs[1] = {0}, re[1] = {0};
+    bool push = false;
+    if (i < Q) {
+      v[0] = ld_cg_u32(a.qv[cur] + i);
+      const u32 r = (u32)ld_cg_u64(a.key + v[0]);
+      push = r < (U ? member_floor(a, v[0], mslot, s_floor, true) : pivot);
+      if (push) {
+        rs[0] = __ldg(a.row_ptr + v[0]);
+        re[0] = __ldg(a.row_ptr + v[0] + 1);
+        v[0] |= kPushFlag;
+      }
+    }
+    defer_append<1>(push && rs[0] < re[0] ? 1u : 0u, v, rs, re, a, &a.ctl->rest[qi]);
+  }
+}
+
+// Second pass of a large bottom-up round.  The first pass stops a scan at the
+// first key of level L whose rank is at most the pivot, a rank that most of
+// the frontier's arcs carry (the floor itself may belong to a center that
+// hardly any candidate can reach; scans that wait for it read every arc).
+// What can beat such a key comes from the few frontier vertices of smaller
+// rank, which push instead.  The list (Q entries, E arcs) holds these, marked
+// with kPushFlag, and the scans that the first pass put off.
+//
+// Arcs are dealt out in equal shares whatever the rows' lengths: a lane takes
+// 8 k consecutive ones (a warp 256 k), k up to 4 once every warp has work, and
+// finds their first row by a search between the slots of the chunk's ends.  It
+// reads kRestBatch neighbours at a time.  A scan keeps its smallest offer and
+// sends one atomicMin per row and lane (one per warp when all lanes end in the
+// same row), and is passed over once its key cannot be beaten; a push sends
+// one atomicMin per neighbour it improves.
+//
+// What bounded such rounds was the number of arcs scanned (up to 123 of R-MAT
+// 22's 128 M) and the chain of one warp alone on a 160,000-arc row; now it is
+// the latency of the first pass.  R-MAT 22's round loop, 24 shift seeds at
+// beta 0.02 / 0.1 / 0.5: mean 189 / 205 / 605 -> 183 / 183 / 197 us, worst
+// 289 / 385 / 4794 -> 279 / 281 / 301 us.  Putting scans off without the pivot
+// left the mean at 339 us at beta 0.5; a grid barrier inside the round instead
+// of a second one only when something is listed cost 20 us per decomposition.
+// The pivot needs a frontier of fewer vertices than there are candidates (else
+// listing the pushes costs more than the scans: 8 -> 42 us in R-MAT 22's second
+// bottom-up round) and at least kDeferMin candidates.
+template <bool U>
+__device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lvl, u32 pivot,
+                                          u32 mslot, int qi, int qb, u32& myrank, u32* s_acc,
+                                          const u32* s_floor) {
+  constexpr u32 kNone = 0xffffffffu;
+  const u32 lane = threadIdx.x & 31;
+  const u32 L = (u32)lvl;
+  const u64 lvl_key = (u64)(L + 1) << 32;
+  const u32 nchunk = (E + kBfsBase - 1) / kBfsBase;
+  const u32 W = gridDim.x * (blockDim.x >> 5);
+  const u32 k = max(1u, min(nchunk / W, 4u));
+  const u32 nunit = (nchunk + k - 1) / k;
+  const u32* qv = a.qv[kRestSide];
+  const int* qrow = a.qrow[kRestSide];
+  const u32* qoff = a.qoff[kRestSide];
+  const u32* cf = a.cf[kRestSide];
+  u32 scanned = 0, pushed = 0;
+  for (u32 unit = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; unit < nunit; unit += W) {
+    const u32 c0 = unit * k, c1 = min(c0 + k, nchunk);
+    u32 lo = ld_cg_u32(cf + c0);
+    u32 hi = c1 < nchunk ? ld_cg_u32(cf + c1) : Q - 1;
+    u32 p = c0 * kBfsBase + lane * (k * (kBfsBase / 32));
+    const u32 p1 = min(min(p + k * (kBfsBase / 32), c1 * kBfsBase), E);
+    if (lo >= Q || hi >= Q) {  // chunk table broken: cannot happen
+      atomicOr(&a.ctl->err, kErrInternal);
+      return;
+    }
+    if (p < p1)
+      while (lo < hi) {  // the last slot whose first arc is at most p
+        const u32 mid = (lo + hi + 1) >> 1;
+        if (ld_cg_u32(qoff + mid) <= p) lo = mid;
+        else hi = mid - 1;
+      }
+    u32 slot = lo, w = kNone, end = p;  // end == p: the row at p is not open yet
+    int rowd = 0;
+    u64 kw = 0, fl = 0, best = ~0ull;
+    bool fresh = true, push = false;
+    while (__any_sync(kFull, p < p1)) {
+      if (p < p1 && p == end) {  // open the row of slot: its range, key and floor
+        if (!fresh) ++slot;
+        fresh = false;
+        w = ld_cg_u32(qv + slot);
+        push = (w & kPushFlag) != 0;
+        w &= ~kPushFlag;
+        const u32 off = ld_cg_u32(qoff + slot);
+        rowd = ld_cg_i32(qrow + slot) - (int)off;
+        end = slot + 1 < Q ? ld_cg_u32(qoff + slot + 1) : E;
+        kw = ld_cg_u64(a.key + w);
+        fl = lvl_key | (U ? member_floor(a, w, mslot, s_floor, true) : pivot);
+        best = ~0ull;
+      }
+      const u32 stop = min(end, p1);
+      if (!push && p < stop && min(kw, best) <= fl) p = stop;  // nothing can beat it
+      u32 vv[kRestBatch];
+#pragma unroll
+      for (int q = 0; q < kRestBatch; ++q)
+        vv[q] = p + q < stop ? (u32)__ldg(a.col + (rowd + (int)(p + q))) : kNone;
+      u64 kv[kRestBatch];
+#pragma unroll
+      for (int q = 0; q < kRestBatch; ++q) kv[q] = vv[q] < a.n ? ld_cg_u64(a.key + vv[q]) : ~0ull;
+      u32 got = p < stop ? min(stop - p, (u32)kRestBatch) : 0u;
+      u32 join = 0;
+      if (push) {
+        const u64 cand = kw + kLevelOne;
+        pushed += got;
+#pragma unroll
+        for (int q = 0; q < kRestBatch; ++q)
+          if (vv[q] < a.n && cand < kv[q]) {
+            const u64 old = atomicMin(a.key + vv[q], cand);
+            if (old > cand) note_rank<U>(a, (u32)qi, true, vv[q], (u32)cand, myrank, s_acc);
+            if ((u32)(old >> 32) > L + 1) join |= 1u << q;
+          }
+      } else {
+        scanned += got;
+#pragma unroll
+        for (int q = 0; q < kRestBatch; ++q)
+          if ((u32)(kv[q] >> 32) == L) best = min(best, kv[q] + kLevelOne);
+      }
+      warp_append<kRestBatch, false>(join, vv, a, qi, qb);
+      p += got;
+      // the end of a scan, or of this lane's share of it: offer what was found
+      const bool offer = !push && w != kNone && p == stop && best < kw;
+      const u32 om = __ballot_sync(kFull, offer);
+      if (om) {
+        const int first = __ffs(om) - 1;
+        const u32 w0 = __shfl_sync(kFull, w, first);
+        bool mine = offer;
+        if (__all_sync(kFull, !offer || w == w0)) {
+          const u64 b = warp_min64(offer ? best : ~0ull);
+          if (offer) best = b;
+          mine = (int)lane == first;
+        }
+        u32 won = 0;
+        if (mine) {
+          const u64 old = atomicMin(a.key + w, best);
+          if (old > best) note_rank<U>(a, (u32)qi, true, w, (u32)best, myrank, s_acc);
+          if ((u32)(old >> 32) > L + 1) won = 1;
+        }
+        const u32 ww[1] = {w};
+        warp_append<1, false>(won, ww, a, qi, qb);
+        if (offer) kw = best;  // not offered again
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    scanned += __shfl_xor_sync(kFull, scanned, o);
+    pushed += __shfl_xor_sync(kFull, pushed, o);
+  }
+  if (lane == 0 && scanned) atomicAdd(&a.ctl->pull_arcs, (u64)scanned);
+  if (lane == 0 && pushed) atomicAdd(&a.ctl->push_arcs, (u64)pushed);
+}
+
 // Bottom-up round from level lvl (see the file comment).  Candidates are every
 // vertex not in excl (from_list = false; a.active lists them when it is set)
 // or the list `cand` of ncand vertices.
@@ -970,7 +1257,8 @@ template <bool U, bool LD, int kPullV>
 __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minrank, u32 mslot,
                                            int qi, int qb, bool from_list, const u32* cand,
                                            u32 ncand, u32* ulist_out, u32* ucnt_out,
-                                           u32& myrank, u32* s_acc, const u32* s_floor) {
+                                           u32& myrank, u32* s_acc, const u32* s_floor,
+                                           bool defer) {
   constexpr u32 kNone = 0xffffffffu;
   u32 scanned = 0, examined = 0;
   const u32 lane = threadIdx.x & 31;
@@ -1056,10 +1344,7 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
 #pragma unroll
     for (int j = 0; j < kPullV; ++j) {
       fr[j] = minrank;
-      if (U && w[j] != kNone) {
-        const u32 m = __ldg(a.wmem + (w[j] >> 5));
-        fr[j] = s_floor ? s_floor[m] : ld_cg_u32(a.mrank + (size_t)mslot * a.kmem + m);
-      }
+      if (U && w[j] != kNone) fr[j] = member_floor(a, w[j], mslot, s_floor, !LD && defer);
     }
     const u64 lvl_key = (u64)(L + 1) << 32;
 #pragma unroll
@@ -1071,7 +1356,15 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
     }
     // one neighbour of every still-scanning candidate per step, for at most
     // kPullLong steps: most scans stop at their first neighbours
+    bool all_off = false;
     for (int step = 0; step < kPullLong; ++step) {
+      if (!LD && defer && step == kPullShort) {
+        u32 going = 0;
+#pragma unroll
+        for (int j = 0; j < kPullV; ++j) going += e[j] < re[j] ? 1u : 0u;
+        all_off = __reduce_add_sync(kFull, going) >= kDeferLanes;
+        if (all_off) break;
+      }
       bool any = false;
       u32 vv[kPullV];
 #pragma unroll
@@ -1084,7 +1377,7 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
           any = true;
         }
       }
-      if (!any) break;
+      if (!LD && defer ? !__any_sync(kFull, any) : !any) break;  // with defer: the warp together
       u64 kv[kPullV];
 #pragma unroll
       for (int j = 0; j < kPullV; ++j) kv[j] = (vv[j] < a.n) ? ld_cg_u64(a.key + vv[j]) : ~0ull;
@@ -1094,9 +1387,19 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
         if (best[j] <= (lvl_key | fr[j])) re[j] = e[j];  // nothing can beat (L + 1, fr)
       }
     }
-    // scans still going after kPullLong neighbours (hubs with no early exit):
-    // the warp takes them one at a time, 32 x kPullCoop coalesced neighbours
-    // per step, with the same early exit per step
+    // scans still going (no early exit): put off to pull_rest, or the warp
+    // takes them one at a time, 32 x kPullCoop coalesced neighbours per step,
+    // with the same early exit per step
+    if (!LD && defer) {
+      u32 dm = 0;
+#pragma unroll
+      for (int j = 0; j < kPullV; ++j)
+        if (e[j] < re[j] && (all_off || re[j] - e[j] >= kDeferLong)) dm |= 1u << j;
+      defer_append<kPullV>(dm, w, e, re, a, &a.ctl->rest[qi]);
+#pragma unroll
+      for (int j = 0; j < kPullV; ++j)
+        if (dm >> j & 1u) e[j] = re[j];
+    }
 #pragma unroll
     for (int j = 0; j < kPullV; ++j) {
       u32 lm = __ballot_sync(kFull, e[j] < re[j]);
@@ -1190,8 +1493,12 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
                    ? reinterpret_cast<u32*>(smem_raw + sizeof(Smem) + (LD ? lq_extra(kPerSm) : 0))
                    : nullptr;
   u32* s_floor = s_acc ? s_acc + kSmemMembers : nullptr;
+  u64* s_piv = s_acc ? reinterpret_cast<u64*>(s_acc + 2 * kSmemMembers) : nullptr;
   if (s_acc)
-    for (u32 m = threadIdx.x; m < a.kmem; m += blockDim.x) s_acc[m] = 0xffffffffu;
+    for (u32 m = threadIdx.x; m < a.kmem; m += blockDim.x) {
+      s_acc[m] = 0xffffffffu;
+      s_piv[m] = 0;
+    }
   Control* ctl = a.ctl;
   if (threadIdx.x == 0) {
     s.minrank = 0xffffffffu;
@@ -1264,12 +1571,17 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
       ctl->ovf[(phase + 2) % 3] = 0;
       ctl->nstart[(phase + 2) % 3] = 0;
       ctl->pull_ctr[(phase + 2) % 3] = 0;
+      ctl->rest[(phase + 2) % 3] = 0;
     }
     if (U)  // the members' floors of the slot that the next round fills
-      for (u32 m = blockIdx.x * blockDim.x + threadIdx.x; m < a.kmem; m += G * blockDim.x)
+      for (u32 m = blockIdx.x * blockDim.x + threadIdx.x; m < a.kmem; m += G * blockDim.x) {
         a.mrank[(size_t)((phase + 2) % 3) * a.kmem + m] = 0xffffffffu;
+        if (!LD) a.mpivot[(size_t)((phase + 2) % 3) * a.kmem + m] = 0;
+      }
     const int qi = (int)((phase + 1) % 3), qb = (int)((phase + 1) & 1);
     int nlvl;
+    bool defer = false;  // a bottom-up round with a second pass ...
+    u32 stop_rank = 0;   // ... and the rank its scans stop at
     // a window of levels: low-degree rounds whose frontier is thin enough, and
     // always while overflow entries of the last window wait
     bool window = false;
@@ -1312,23 +1624,34 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
       else if (pulling && (u64)Q * a.pull_beta < a.n_active)
         pulling = false;
       if (pulling) {
-        if (U) {  // this level's per-member floors, from the frontier list
-          member_floors(a, a.qv[phase & 1], Q, phase % 3, s_acc);
+        // large rounds stop at a pivot rank and have a second pass
+        defer = !LD && max(Q, kDeferMin) <= (was_pulling ? ncand : a.n_active);
+        stop_rank = minrank;
+        if (U) {  // this level's per-member floors and pivots, from the frontier list
+          member_floors<!LD>(a, a.qv[phase & 1], Q, phase % 3, s_acc, s_piv);
           if (s_acc) {
             __syncthreads();
-            flush_members(a, phase % 3, s_acc);
+            flush_members<!LD>(a, phase % 3, s_acc, s_piv);
           }
           grid_barrier(ctl, gen, G, a.bar_phantom, a.spin_limit, kNoPost, a.bptr, -1, s);
           if (s.stop) break;
           if (s_floor) {  // read once per CTA
-            for (u32 m = threadIdx.x; m < a.kmem; m += blockDim.x)
-              s_floor[m] = ld_cg_u32(a.mrank + (size_t)(phase % 3) * a.kmem + m);
+            for (u32 m = threadIdx.x; m < a.kmem; m += blockDim.x) {
+              u32 f = ld_cg_u32(a.mrank + (size_t)(phase % 3) * a.kmem + m);
+              if (defer && f != 0xffffffffu)
+                f = (u32)ld_cg_u64(a.key + (u32)ld_cg_u64(a.mpivot + (size_t)(phase % 3) * a.kmem + m));
+              s_floor[m] = f;
+            }
             __syncthreads();
           }
+        } else if (defer) {
+          stop_rank = pivot_rank(a, s, (int)(phase & 1), Q, E);
         }
-        pull_round<U, LD, pull_width(kPerSm)>(a, lvl, minrank, phase % 3, qi, qb, was_pulling,
+        if (!LD && defer && (U || stop_rank > minrank))
+          list_pushes<U>(a, (int)(phase & 1), Q, stop_rank, phase % 3, qi, s_floor);
+        pull_round<U, LD, pull_width(kPerSm)>(a, lvl, stop_rank, phase % 3, qi, qb, was_pulling,
                                               a.ulist[phase & 1], ncand, a.ulist[(phase + 1) & 1],
-                                              &ctl->ucnt[qi], myrank, s_acc, s_floor);
+                                              &ctl->ucnt[qi], myrank, s_acc, s_floor, defer);
         ++pulls;
         if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
         if (lvl + 1 <= A) {
@@ -1384,6 +1707,13 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
     post_cta_min(s, myrank);
     grid_barrier(ctl, gen, G, a.bar_phantom, a.spin_limit, (u32)qi, a.bptr,
                  nlvl + 1 <= A ? nlvl + 1 : -1, s);
+    if (!LD && defer && !s.stop && (u32)s.next_rest) {  // pushes and put-off scans are listed
+      pull_rest<U>(a, (u32)(s.next_rest >> 32), (u32)s.next_rest, lvl, stop_rank, phase % 3, qi,
+                   qb, myrank, s_acc, s_floor);
+      post_cta_min(s, myrank);
+      grid_barrier(ctl, gen, G, a.bar_phantom, a.spin_limit, (u32)qi, a.bptr,
+                   nlvl + 1 <= A ? nlvl + 1 : -1, s);
+    }
     ++phase;
     lvl = nlvl;
     if (profiler && phase < (u32)kRoundProfile) {
@@ -1402,7 +1732,7 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->pull_rounds = pulls;
-    if (!LD) ctl->push_arcs = push_arcs;
+    if (!LD) atomicAdd(&ctl->push_arcs, push_arcs);
     ctl->rounds = phase;
     ctl->last_level = lvl;
     atomicAdd(&ctl->items, windowed ? items : settled);
@@ -1418,7 +1748,7 @@ size_t bfs_smem_bytes() { return sizeof(Smem); }
 
 namespace {
 size_t bfs_smem(bool u, int per_sm, bool ld) {
-  return sizeof(Smem) + (ld ? lq_extra(per_sm) : 0) + (u ? 2 * kSmemMembers * sizeof(u32) : 0);
+  return sizeof(Smem) + (ld ? lq_extra(per_sm) : 0) + (u ? kSmemMembers * (2 * sizeof(u32) + sizeof(u64)) : 0);
 }
 
 const void* bfs_kernel(bool u, int per_sm, bool ld) {

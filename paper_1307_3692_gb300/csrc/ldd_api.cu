@@ -138,6 +138,7 @@ int free_graph_memory(ldd_graph* g) {
     cudaFree(g->uni->d_wmem);
     cudaFree(g->uni->d_amax);
     cudaFree(g->uni->d_mrank);
+    cudaFree(g->uni->d_mpivot);
     delete g->uni;
     g->uni = nullptr;
   }
@@ -184,6 +185,8 @@ int alloc_scratch(ldd_graph* g) {
       {(void**)&g->d_qv[0], 4 * n},       {(void**)&g->d_qv[1], 4 * n},
       {(void**)&g->d_qrow[0], 4 * n},     {(void**)&g->d_qrow[1], 4 * n},
       {(void**)&g->d_qoff[0], 4 * n},     {(void**)&g->d_qoff[1], 4 * n},
+      {(void**)&g->d_qv[2], 4 * n},       {(void**)&g->d_qrow[2], 4 * n},
+      {(void**)&g->d_qoff[2], 4 * n},     {(void**)&g->d_cf[2], 4 * ncf},
       {(void**)&g->d_cf[0], 4 * ncf},     {(void**)&g->d_cf[1], 4 * ncf},
       {(void**)&g->d_ulist[0], 4 * n},    {(void**)&g->d_ulist[1], 4 * n},
       {(void**)&g->d_slots, n ? fraction_slot_bytes((u32)n) : 0},
@@ -390,12 +393,12 @@ BfsArgs bfs_args(ldd_graph* g) {
   a.bptr = g->d_bptr;
   a.rk[0] = a.rk[1] = reinterpret_cast<const u32*>(g->d_k[0]);  // start rounds, 32-bit
   a.rv[0] = a.rv[1] = g->d_v[0];                                 // start-bucket vertices
-  for (int b = 0; b < 2; ++b) {
+  for (int b = 0; b < 3; ++b) {
     a.qv[b] = g->d_qv[b];
     a.qrow[b] = g->d_qrow[b];
     a.qoff[b] = g->d_qoff[b];
     a.cf[b] = g->d_cf[b];
-    a.ulist[b] = g->d_ulist[b];
+    if (b < 2) a.ulist[b] = g->d_ulist[b];
   }
   a.excl = g->d_excl;
   a.active = g->d_active;
@@ -417,6 +420,7 @@ BfsArgs bfs_args(ldd_graph* g) {
   a.span = g->bfs_span;
   a.wmem = g->uni ? g->uni->d_wmem : nullptr;
   a.mrank = g->uni ? g->uni->d_mrank : nullptr;
+  a.mpivot = g->uni ? g->uni->d_mpivot : nullptr;
   a.kmem = g->uni ? g->uni->k : 0;
   return a;
 }
@@ -431,6 +435,8 @@ int run_bfs_finalize(ldd_graph* g, int* center, int* dist, int* status) {
     cudaError_t e = cudaMemsetAsync((char*)g->d_ctl + kCtlMinrankOffset, 0xff, 3 * sizeof(u32), s);
     if (e == cudaSuccess && g->uni)
       e = cudaMemsetAsync(g->uni->d_mrank, 0xff, 3 * (size_t)g->uni->k * sizeof(u32), s);
+    if (e == cudaSuccess && g->uni)
+      e = cudaMemsetAsync(g->uni->d_mpivot, 0, 3 * (size_t)g->uni->k * sizeof(u64), s);
     if (e != cudaSuccess) {
       *status = fail(LDD_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
       return -1;
@@ -951,10 +957,10 @@ u64 union_bytes(const UnionCaps& c) {
   const u64 N = c.N, words = std::max<u64>(N / 32, 1);
   u64 b = 4 * (N + 1) + 4 * c.E + 4 * c.M + 20 * c.G + 8 * (c.M / 32 + 1) + 8 * words +
           8 * c.C + 8 * c.T + 4 * N + 4 * words;
-  b += 16 * c.total + 8 * c.total + 32ull * (c.k + 1) + 8ull * c.k + sizeof(UnionMember) * c.k;
+  b += 16 * c.total + 8 * c.total + 32ull * (c.k + 1) + 44ull * c.k + sizeof(UnionMember) * c.k;
   const u64 nk = std::max<u64>(N, 64);
   b += 8 * N + 4 * N + 16 * nk + 8 * N + ((N + kSortTile - 1) / kSortTile + 1) * 2048 + 4 * N +
-       8 * N + 24 * N + 8 * (c.E / kBfsBase + 2) + 8 * N + (N ? fraction_slot_bytes((u32)N) : 0) +
+       8 * N + 36 * N + 12 * (c.E / kBfsBase + 2) + 8 * N + (N ? fraction_slot_bytes((u32)N) : 0) +
        8 * N + sizeof(Control);
   b += 12 * (N + 2);
   return b;
@@ -1003,7 +1009,8 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
       cudaMalloc(&U.d_cut, K * 8) != cudaSuccess ||
       cudaMalloc(&U.d_wmem, words * 4) != cudaSuccess ||
       cudaMalloc(&U.d_amax, 2 * K * 4) != cudaSuccess ||
-      cudaMalloc(&U.d_mrank, 3 * K * 4) != cudaSuccess) {
+      cudaMalloc(&U.d_mrank, 3 * K * 4) != cudaSuccess ||
+      cudaMalloc(&U.d_mpivot, 3 * K * 8) != cudaSuccess) {
     cudaGetLastError();
     return bail(fail(LDD_ERR_OOM, "device allocation of a union (%llu vertices, %llu arcs) "
                      "failed", (unsigned long long)N, (unsigned long long)c.E));

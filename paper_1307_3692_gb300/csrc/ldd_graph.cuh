@@ -105,10 +105,10 @@ struct ldd_graph {
   u64* d_status = nullptr;
   u32* d_order = nullptr;
   u64* d_key = nullptr;
-  u32* d_qv[2] = {nullptr, nullptr};
-  int* d_qrow[2] = {nullptr, nullptr};
-  u32* d_qoff[2] = {nullptr, nullptr};
-  u32* d_cf[2] = {nullptr, nullptr};
+  u32* d_qv[3] = {};
+  int* d_qrow[3] = {};
+  u32* d_qoff[3] = {};
+  u32* d_cf[3] = {};
   u32* d_ulist[2] = {nullptr, nullptr};
   void* d_slots = nullptr;
   int* d_center = nullptr;
@@ -172,6 +172,7 @@ struct ldd_graph {
     u32* d_wmem = nullptr;         // [N / 32] member of every 32-vertex word
     int* d_amax = nullptr;         // [k] largest floor of each member, then [k] its lift
     u32* d_mrank = nullptr;        // [3][k] the round loop's per-member bottom-up floors
+    u64* d_mpivot = nullptr;       // [3][k] ... and pivots
   };
   Union* uni = nullptr;
   // block decomposition (ldd_block_decompose, ldd_blocks.cu): residual graphs,

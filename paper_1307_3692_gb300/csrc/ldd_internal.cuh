@@ -100,6 +100,8 @@ struct Control {
   // bottom-up rounds: the next unit of candidates a warp takes once the
   // units dealt out in advance are done (rotating like qctr)
   u32 pull_ctr[3];
+  // ... and their list for the second pass: (entries << 32) | arcs (rotating)
+  u64 rest[3];
 };
 constexpr size_t kCtlHeaderBytes = 40;       // err .. cut
 constexpr size_t kCtlBfsStateOffset = 40;    // bar_count .. pull_rounds
@@ -113,11 +115,11 @@ struct BfsArgs {
   const int* bptr;   // [A + 2] start-bucket offsets into the round-sorted list
   const u32* rk[2];  // round-sorted keys (start rounds), ping-pong pair
   const u32* rv[2];  // round-sorted vertices, ping-pong pair
-  u32* qv[2];        // frontier queues: vertex
-  int* qrow[2];      //                  row_ptr[vertex]
-  u32* qoff[2];      //                  exclusive edge offset in the frontier
+  u32* qv[3];        // frontier queues: vertex (side 2: put-off work of bottom-up rounds)
+  int* qrow[3];      //                  row_ptr[vertex]
+  u32* qoff[3];      //                  exclusive edge offset in the frontier
                      // (low-degree rounds use qv alone)
-  u32* cf[2];        // first queue slot of every base chunk of edges
+  u32* cf[3];        // first queue slot of every base chunk of edges
   u32* ulist[2];     // vertices still unsettled after a bottom-up round (ping-pong)
   const u32* excl;   // bit v: v is not handled by the BFS
   const u32* active; // the vertices the BFS handles, ascending (n_active), or null
@@ -141,6 +143,8 @@ struct BfsArgs {
   u32 span;          // edge-balanced rounds: arcs per CTA step at most (kBfsBase .. kBfsMaxSpan)
   const u32* wmem;   // unions: member of every 32-vertex word; else null
   u32* mrank;        // unions: [3][kmem] smallest rank per level slot and member (~0 on entry)
+  u64* mpivot;       // unions: [3][kmem] (degree << 32) | vertex of every member's frontier vertex
+                     // of the largest degree per level slot (zero on entry)
   u32 kmem;          // unions: members
 };
 
