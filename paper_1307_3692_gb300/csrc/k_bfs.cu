@@ -1,13 +1,23 @@
 // Round-synchronous, delayed-start multi-source BFS (Algorithm 1 step 3;
 // Section 4 of Miller, Peng, Xu 2013), as one persistent cooperative kernel.
 //
-// State: key[v] = (level << 32) | rank, initialised to v's own start label
-// (level R_v = floor(delta_max) - floor(delta_v)).  Round r expands the
-// frontier F_r = {v : final level of v is r}: every arc (v, w) offers
-// key[v] + 2^32 to w with a 64-bit atomicMin.  Because key[v] is final once
-// round r - 1 has finished, and an offer made in round r carries level r + 1,
-// the minimum over all offers is the exact label the paper's super-source
-// shortest path assigns (Section 4), including the fraction tie-break.
+// State: key[v] = level and tie-break (KeyFmt, ldd_internal.cuh), initialised to
+// v's own start label.  Levels run from that of the largest floor the loop
+// handles.  Round r expands the frontier F_r = {v : final level of v is r}:
+// every arc (v, w) offers key[v], one level further out, to w with a 64-bit
+// atomicMin.  Because key[v] is final once round r - 1 has finished, and an
+// offer made in round r carries level r + 1, the minimum over all offers is the
+// exact label the paper's super-source shortest path assigns (Section 4),
+// including the fraction tie-break.  Wherever two direct keys that differ only
+// in their ids meet -- at a vertex, or in the minimum that a bottom-up round
+// stops at -- the meeting is listed (note_tie) and finalize compares the exact
+// fractions, so a decomposition that ends without an error bit is exact.
+//
+// Start buckets.  With direct keys the loop itself fills the buckets, some
+// levels ahead at a time (build_buckets): it passes over the blocks of vertices
+// whose largest floor is too small and drops the vertices that somebody has
+// claimed, so the buckets hold about as many vertices as pieces, not all of
+// them.
 //
 // F_{r+1} is built during round r from two disjoint sources:
 //   * pushes: the one atomicMin that lowers w's level from > r + 1 to r + 1
@@ -28,7 +38,7 @@
 // frontier's arcs outweigh the arcs of the still-unsettled vertices, a round
 // runs bottom-up instead: every unsettled vertex w scans its neighbours for
 // keys of level r and keeps the smallest key + 2^32.  The scan can stop once it
-// holds (r + 1, minrank_r), where minrank_r is the smallest rank among level-r
+// holds (r + 1, minrank_r), where minrank_r is the smallest tie-break among level-r
 // keys: nothing can beat it.  minrank_r is tracked exactly during round r - 1
 // as the minimum over every successful key update and every appended start
 // (each final level-r key is one of these, and each of these is >= the final
@@ -78,6 +88,11 @@ constexpr u32 kDeferMin = 1u << 16;
 constexpr int kPullShort = 8;
 constexpr u32 kDeferLanes = 32;
 constexpr int kDeferLong = 2048;
+// Start buckets are filled kBuildMin vertices at a time at least, at first a
+// 2^-kBuildShift share of the handled ones, then eight times as many: most
+// loops end long before the buckets that hold most vertices.
+constexpr u32 kBuildShift = 10;
+constexpr u32 kBuildMin = 1024;
 constexpr int kRestBatch = 8;   // the second pass: neighbours per lane in flight
 constexpr u32 kPushFlag = 1u << 31;  // on its list: a frontier vertex that pushes
 constexpr int kRestSide = 2;    // the side of the frontier arrays that holds the list
@@ -86,30 +101,35 @@ constexpr u32 kPivotSamples = 128;
 constexpr u32 kPivotSkip = 2;
 constexpr int kPullCoop = 4;   // neighbours per lane per step of a warp-wide scan
 // Unions of at most this many members keep their per-member floors and pivots
-// in shared memory (after Smem: 16 bytes per member, 32 KB, so that two CTAs
+// in shared memory (after Smem: 24 bytes per member, 30 KB, so that two CTAs
 // per SM still fit); larger unions use the global tables directly.
-constexpr u32 kSmemMembers = 2048;
+constexpr u32 kSmemMembers = 1280;
 constexpr int kLdBatch = 8;    // low-degree rounds: arcs per frontier vertex and step
 constexpr int kLdItems = 1;    // low-degree rounds: items per thread in flight
+
+__device__ __forceinline__ void note_tie(const BfsArgs& a, u32 w, u64 x, u64 y) {
+  note_tie(a.ctl, a.f, w, x, y);
+}
 
 struct Smem {
   int owner[kBfsMaxSpan];
   int rowd[kBfsMaxSpan + 1];
   u64 cand[kBfsMaxSpan + 1];
   int wtot[kBfsThreads / 32];
-  u32 minrank;  // this CTA's smallest successful next-level rank in the round
+  u64 minlow[kBfsThreads / 32];  // each warp's smallest successful next-level tie-break
   u32 stop;     // thread 0 saw an error bit: the whole CTA leaves the loop
   // the next round's frontier counter, bottom-up floor and unsettled-list
   // length, read by thread 0 as the barrier releases
   u64 next_c;
   u64 next_rest;         // a large bottom-up round's list for its second pass
-  u32 next_minrank;
+  u64 next_minlow;
   u32 next_ucnt;
   int next_lo, next_hi;  // the next round's start bucket (lvl + 1) bounds
   u32 next_ovf;          // the next round's overflow-list length (windows)
   u32 lcnt[3];           // windows: local-queue lengths, rotating (read, fill, clear)
   u32 nstart;            // a scan's result, shared by the CTA
-  u32 pivot;             // the round's pivot rank
+  u64 pivot;             // the round's pivot
+  int built;             // build_buckets: the last level filled
 };
 // Windows of levels keep two local queues whose entries carry a vertex, the
 // key it was pushed with and its adjacency range (20 bytes, as four arrays).
@@ -150,32 +170,48 @@ __device__ __forceinline__ LocalQueue lq_buf(Smem& s, int b) {
   return q;
 }
 
+// 64-bit minimum and maximum over the warp: of the high words, then of the low
+// words of the lanes that have it.
+__device__ __forceinline__ u64 warp_min64(u64 x) {
+  const u32 hi = (u32)(x >> 32), h = __reduce_min_sync(kFull, hi);
+  return (u64)h << 32 | __reduce_min_sync(kFull, hi == h ? (u32)x : 0xffffffffu);
+}
+__device__ __forceinline__ u64 warp_max64(u64 x) { return ~warp_min64(~x); }
+
 // Grid-wide barrier on a monotonic arrival counter: the k-th barrier of a
 // launch completes when the counter reaches k * nblocks (+ phantom), so
 // arrival is one fire-and-forget add and nobody has to reset anything.
-// Before arriving, thread 0 publishes this CTA's smallest next-level rank to
-// ctl->minrank[post] (and resets the CTA value).  The poll is an acquire
+// Before arriving, thread 0 publishes this CTA's smallest next-level tie-break to
+// ctl->minlow[post] (and resets the CTA value).  The poll is an acquire
 // load, so once it sees every arrival the round's writes of all CTAs are
-// visible.  The wait is bounded: after `limit` polls (or once any CTA has
-// recorded an error) it sets kErrTimeout and returns.  Thread 0 then reads,
+// visible.  The wait is bounded: it ends after a.spin_limit polls, with
+// kErrTimeout, or once any CTA has recorded an error.  Thread 0 then reads,
 // in one round trip, the error word and the next round's state (slot `post`
 // of the frontier counter, bottom-up floor and unsettled-list length, and the
-// bounds of start bucket blevel unless it is negative) into shared memory, so that every thread of the CTA sees the same values and
+// bounds of start bucket blevel, of levels from lv0 on, unless it is negative) into shared memory, so that every thread of the CTA sees the same values and
 // takes the same branch after the barrier (a thread that left the loop alone
-// would leave the others at a CTA barrier).  phantom > 0 waits for CTAs that
+// would leave the others at a CTA barrier).  a.bar_phantom > 0 waits for CTAs that
 // do not exist: the barrier can then only end by running out of polls, which
 // is how the timeout path is tested.
 constexpr u32 kNoPost = 0xffffffffu;  // grid_barrier: a barrier inside a round
 
-__device__ __forceinline__ void grid_barrier(Control* ctl, u32& gen, u32 nblocks, u32 phantom,
-                                             u32 limit, u32 post, const int* bptr, int blevel,
-                                             Smem& s) {
+template <bool kTrack>
+__device__ __forceinline__ void grid_barrier(const BfsArgs& a, u32& gen, u32 post, int lv0,
+                                             int blevel, Smem& s) {
+  Control* ctl = a.ctl;
   __syncthreads();
+  u64 mine = ~0ull;  // this CTA's smallest next-level tie-break
+  if (kTrack && post != kNoPost && threadIdx.x < 32) {
+    const u64 x = threadIdx.x < kBfsThreads / 32 ? s.minlow[threadIdx.x] : ~0ull;
+    mine = warp_min64(x);
+    if (x != ~0ull) note_tie(a, 0, x, mine);
+  }
   if (threadIdx.x == 0) {
-    if (post != kNoPost && s.minrank != 0xffffffffu) atomicMin(&ctl->minrank[post], s.minrank);
-    if (post != kNoPost) s.minrank = 0xffffffffu;
+    if (mine != ~0ull)
+      asm volatile("red.relaxed.gpu.global.min.u64 [%0], %1;" ::"l"(&ctl->minlow[post]), "l"(mine)
+                   : "memory");
     ++gen;
-    const u64 target = (u64)gen * nblocks + phantom;
+    const u64 target = (u64)gen * gridDim.x + a.bar_phantom;
     __threadfence();
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(&ctl->bar), "l"(1ull) : "memory");
     u32 spins = 0;
@@ -183,7 +219,8 @@ __device__ __forceinline__ void grid_barrier(Control* ctl, u32& gen, u32 nblocks
       u64 seen;
       asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(&ctl->bar) : "memory");
       if (seen >= target) break;
-      if (++spins > limit || ld_acquire_u32(&ctl->err) != 0u) {
+      if (ld_acquire_u32(&ctl->err) != 0u) break;  // another CTA has left the loop
+      if (++spins > a.spin_limit) {
         atomicOr(&ctl->err, kErrTimeout);
         __threadfence();
         break;
@@ -193,22 +230,21 @@ __device__ __forceinline__ void grid_barrier(Control* ctl, u32& gen, u32 nblocks
     const u32 err = ld_cg_u32(&ctl->err);
     if (post != kNoPost) {
       s.next_c = ld_cg_u64(&ctl->qctr[post]);
-      s.next_minrank = ld_cg_u32(&ctl->minrank[post]);
+      s.next_minlow = ld_cg_u64(&ctl->minlow[post]);
+      if (mine != ~0ull) note_tie(a, 0, mine, s.next_minlow);
       s.next_ucnt = ld_cg_u32(&ctl->ucnt[post]);
       s.next_ovf = ld_cg_u32(&ctl->ovf[post]);
       s.next_rest = ld_cg_u64(&ctl->rest[post]);
       s.next_lo = s.next_hi = 0;
       if (blevel >= 0) {  // bounds of start bucket blevel, for the round after the barrier
-        s.next_lo = __ldg(bptr + blevel);
-        s.next_hi = __ldg(bptr + blevel + 1);
+        s.next_lo = __ldg(a.bptr + (blevel - lv0));
+        s.next_hi = (int)ld_cg_u32(a.rcur + (blevel - lv0));
       }
     }
     s.stop = err != 0u ? 1u : 0u;
   }
   __syncthreads();
 }
-
-__device__ __forceinline__ u32 warp_min(u32 x) { return __reduce_min_sync(kFull, x); }
 
 // Exclusive prefix over the warp of small counts x < 2^kBits (and, in *tot,
 // their sum), by one ballot per bit instead of a chain of shuffles.
@@ -239,38 +275,26 @@ __device__ __forceinline__ u32 warp_first_item(u32 k, bool rev = false) {
   return ((threadIdx.x >> 5) * gridDim.x + b) * 32u * k;
 }
 
-__device__ __forceinline__ u64 warp_min64(u64 x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = min(x, (u64)__shfl_xor_sync(kFull, x, o));
-  return x;
+// Records a successful next-level key k for the bottom-up floor of the next
+// round: the thread's smallest tie-break, folded into the CTA's and the grid's
+// at the barrier.  Unions and low-degree rounds track nothing here: they go
+// bottom-up rarely, and their floors are then computed from the frontier list
+// (member_floors, list_floor).  In a union the floor is per member (another
+// member's smaller tie-break can never reach v), and keeping up to kmem minima
+// per CTA in every round cost more than the rare bottom-up rounds of a batch
+// gain from it; in the thin rounds of a low-degree graph the bookkeeping cost
+// 2 % of the loop.
+template <bool kTrack>
+__device__ __forceinline__ void note_low(const BfsArgs& a, bool valid, u64 k, u64& mylow) {
+  if (!kTrack || !valid) return;
+  const u64 low = key_low(a.f, k);
+  note_tie(a, 0, low, mylow);
+  mylow = min(mylow, low);
 }
 
-__device__ __forceinline__ u64 warp_max64(u64 x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = max(x, (u64)__shfl_xor_sync(kFull, x, o));
-  return x;
-}
-
-// Records a successful next-level key (vertex v, rank) for the bottom-up
-// floor of the next round: the thread's running minimum, folded into the
-// CTA's and the grid's at the barrier.  Unions track nothing here: their floor
-// is per member (another member's smaller rank can never reach v), and it is
-// computed from the frontier list only when a round goes bottom-up
-// (member_floors), since keeping up to kmem minima per CTA in every round
-// cost more than the rare bottom-up rounds of a batch gain from it.
-template <bool U>
-__device__ __forceinline__ void note_rank(const BfsArgs& a, u32 slot, bool valid, u32 v, u32 rank,
-                                          u32& myrank, u32* s_acc) {
-  (void)a;
-  (void)slot;
-  (void)v;
-  (void)s_acc;
-  if (!U && valid) myrank = min(myrank, rank);
-}
-
-// Unions: the per-member floors of level-L keys (the smallest rank among each
-// member's keys of the frontier's level) from the frontier list qv of Q
-// vertices, into slot `slot` of a.mrank (all ~0 on entry), and with kPivot
+// Unions: the per-member floors of level-L keys (the smallest tie-break among
+// each member's keys of the frontier's level) from the frontier list qv of Q
+// vertices, into slot `slot` of a.mlow (all ~0 on entry), and with kPivot
 // every member's frontier vertex of the largest degree into a.mpivot (as
 // (degree << 32) | vertex, all zero on entry; see pull_rest).  A warp whose
 // vertices share one member makes one update; small unions gather both per CTA
@@ -278,52 +302,57 @@ __device__ __forceinline__ void note_rank(const BfsArgs& a, u32 slot, bool valid
 // grid barrier before they are read.
 template <bool kPivot>
 __device__ __forceinline__ void member_floors(const BfsArgs& a, const u32* qv, u32 Q, u32 slot,
-                                              u32* s_acc, u64* s_piv) {
+                                              u64* s_acc, u64* s_piv) {
   const u32 lane = threadIdx.x & 31;
   const u32 stride = gridDim.x * blockDim.x;
   for (u32 base = warp_first_item(1); base < Q; base += stride) {
     const u32 i = base + lane;
     const bool valid = i < Q;
-    u32 v = 0, m = 0xffffffffu, r = 0xffffffffu;
-    u64 pv = 0;
+    u32 v = 0, m = 0xffffffffu;
+    u64 r = ~0ull, pv = 0;
     if (valid) {
       v = ld_cg_u32(qv + i);
       m = __ldg(a.wmem + (v >> 5));
-      r = (u32)ld_cg_u64(a.key + v);
+      r = key_low(a.f, ld_cg_u64(a.key + v));
       if (kPivot) pv = (u64)(u32)(__ldg(a.row_ptr + v + 1) - __ldg(a.row_ptr + v)) << 32 | v;
     }
     const u32 act = __ballot_sync(kFull, valid);
     const u32 m0 = __shfl_sync(kFull, m, __ffs(act) - 1);
     const bool one = __all_sync(kFull, !valid || m == m0);
-    const u32 rr = one ? warp_min(r) : r;
+    u64 rr = r;
+    if (one) {
+      rr = warp_min64(r);
+      if (valid) note_tie(a, v, r, rr);
+    }
     const u64 pp = kPivot && one ? warp_max64(pv) : pv;
-    if ((one && lane == 0) || (!one && valid)) {
+    if ((one && lane == (u32)(__ffs(act) - 1)) || (!one && valid)) {
       const u32 mm = one ? m0 : m;
-      if (s_acc) {
-        if (rr < s_acc[mm]) atomicMin(s_acc + mm, rr);
-        if (kPivot && pp > s_piv[mm]) atomicMax(s_piv + mm, pp);
-      } else {
-        u32* p = a.mrank + (size_t)slot * a.kmem + mm;
-        if (rr < ld_cg_u32(p)) atomicMin(p, rr);
-        u64* q = a.mpivot + (size_t)slot * a.kmem + mm;
-        if (kPivot && pp > ld_cg_u64(q)) atomicMax(q, pp);
+      u64* p = s_acc ? s_acc + mm : a.mlow + (size_t)slot * a.kmem + mm;
+      const u64 seen = s_acc ? *(volatile u64*)p : ld_cg_u64(p);
+      if (rr < seen) note_tie(a, v, rr, atomicMin(p, rr));
+      else note_tie(a, v, rr, seen);
+      if (kPivot) {
+        u64* q = s_acc ? s_piv + mm : a.mpivot + (size_t)slot * a.kmem + mm;
+        if (pp > (s_acc ? *(volatile u64*)q : ld_cg_u64(q))) atomicMax(q, pp);
       }
     }
   }
 }
 
-// Union: the CTA's per-member minima into slot `slot` of a.mrank (and the
+// Union: the CTA's per-member minima into slot `slot` of a.mlow (and the
 // pivots into a.mpivot), and the shared tables reset.  Called by the whole CTA
 // between __syncthreads.
 template <bool kPivot>
-__device__ __forceinline__ void flush_members(const BfsArgs& a, u32 slot, u32* s_acc,
+__device__ __forceinline__ void flush_members(const BfsArgs& a, u32 slot, u64* s_acc,
                                               u64* s_piv) {
   for (u32 m = threadIdx.x; m < a.kmem; m += blockDim.x) {
-    const u32 r = s_acc[m];
-    if (r != 0xffffffffu) {
-      u32* p = a.mrank + (size_t)slot * a.kmem + m;
-      if (r < ld_cg_u32(p)) atomicMin(p, r);
-      s_acc[m] = 0xffffffffu;
+    const u64 r = s_acc[m];
+    if (r != ~0ull) {
+      u64* p = a.mlow + (size_t)slot * a.kmem + m;
+      const u64 seen = ld_cg_u64(p);
+      const u64 met = r < seen ? atomicMin(p, r) : seen;
+      if (met != ~0ull) note_tie(a, __ldg(a.voff + m), met, r);
+      s_acc[m] = ~0ull;
       if (kPivot) {
         u64* q = a.mpivot + (size_t)slot * a.kmem + m;
         if (s_piv[m] > ld_cg_u64(q)) atomicMax(q, s_piv[m]);
@@ -333,16 +362,16 @@ __device__ __forceinline__ void flush_members(const BfsArgs& a, u32 slot, u32* s
   }
 }
 
-// Union: what a bottom-up scan of w may stop at, the smallest rank of its
-// member's level-L keys or (pivot) the rank of the member's pivot; ~0 when the
+// Union: what a bottom-up scan of w may stop at, the smallest tie-break of its
+// member's level-L keys or (pivot) that of the member's pivot; ~0 when the
 // member has no level-L key.  s_floor: the CTA's copy, already the one of the two.
-__device__ __forceinline__ u32 member_floor(const BfsArgs& a, u32 w, u32 slot, const u32* s_floor,
+__device__ __forceinline__ u64 member_floor(const BfsArgs& a, u32 w, u32 slot, const u64* s_floor,
                                             bool pivot) {
   const u32 m = __ldg(a.wmem + (w >> 5));
   if (s_floor) return s_floor[m];
-  if (!pivot) return ld_cg_u32(a.mrank + (size_t)slot * a.kmem + m);
+  if (!pivot) return ld_cg_u64(a.mlow + (size_t)slot * a.kmem + m);
   const u64 pv = ld_cg_u64(a.mpivot + (size_t)slot * a.kmem + m);
-  return pv ? (u32)ld_cg_u64(a.key + (u32)pv) : 0xffffffffu;
+  return pv ? key_low(a.f, ld_cg_u64(a.key + (u32)pv)) : ~0ull;
 }
 
 // Appends to the frontier every vertex v[i] whose bit i is set in `mask`, for
@@ -421,15 +450,11 @@ __device__ __forceinline__ void warp_append(u32 mask, const u32 (&v)[K], const B
     }
 }
 
-// Unclaimed vertices of start bucket rr join the frontier of level rr.
+// Unclaimed vertices of start bucket rr (entries lo .. hi of rv) join the
+// frontier of level rr.
 template <bool U>
-__device__ __forceinline__ void append_bucket(const BfsArgs& a, int rr, const u32* rv, int qi,
-                                              int qb, u32& myrank, u32* s_acc, int lo = -1,
-                                              int hi = -1) {
-  if (lo < 0) {  // bounds not known yet
-    lo = __ldg(a.bptr + rr);
-    hi = __ldg(a.bptr + rr + 1);
-  }
+__device__ __forceinline__ void append_bucket(const BfsArgs& a, int rr, int lo, int hi, int qi,
+                                              int qb, u64& mylow) {
   const u32 cnt = (u32)(hi - lo);
   const u32 lane = threadIdx.x & 31;
   const u32 stride = gridDim.x * blockDim.x;
@@ -440,18 +465,84 @@ __device__ __forceinline__ void append_bucket(const BfsArgs& a, int rr, const u3
     bool want = false;
     u64 k = 0;
     if (i < cnt) {
-      u[0] = __ldg(rv + lo + i);
+      u[0] = ld_cg_u32(a.rv + lo + i);
       k = ld_cg_u64(a.key + u[0]);
-      want = (u32)(k >> 32) == (u32)rr;
+      want = key_level(a.f, k) == (u32)rr;
     }
-    note_rank<U>(a, (u32)qi, want, u[0], (u32)k, myrank, s_acc);
+    note_low<!U>(a, want, k, mylow);
     warp_append<1, false>(want ? 1u : 0u, u, a, qi, qb);
   }
 }
 
+// Direct keys: fills the start buckets of levels from .. to, to the last level
+// (at least from) that keeps their vertices, claimed ones included, within
+// `most`; returns it, the same in every CTA.  The buckets' room follows from
+// the counts of all floors (bptr); an entry is a vertex whose key still names
+// itself.  The caller waits at a grid barrier before they are read.  first: from
+// is the loop's first level, lv0; its vertices start the frontier (slot 0) at
+// once, without a pass over their bucket and its barrier.
+template <bool U, bool LD>
+__device__ __forceinline__ int build_buckets(const BfsArgs& a, Smem& s, int lv0, int from, int A,
+                                             u32 most, bool first, u64& mylow) {
+  // the last of blockDim.x evenly spaced levels within `most`
+  const int step = (A - from) / (int)blockDim.x + 1;
+  __syncthreads();
+  if (threadIdx.x == 0) s.built = from;
+  __syncthreads();
+  {
+    const int r = min(from + (int)threadIdx.x * step, A);
+    const int room = __ldg(a.bptr + (r + 1 - lv0)) - __ldg(a.bptr + (from - lv0));
+    if ((u32)room <= most) atomicMax(&s.built, r);
+  }
+  __syncthreads();
+  const int to = s.built;
+  const u32 lane = threadIdx.x & 31;
+  const u32 least = a.f.cap - (u32)to + 1;  // a block's entry in bmax: its largest floor plus one
+  const u32 nblk = (a.n + kMaxBlock - 1) / kMaxBlock;
+  // block after block to different warps, 32 of a warp's own looked up at once
+  const u32 W = gridDim.x * (blockDim.x >> 5);
+  for (u32 b0 = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; b0 < nblk; b0 += 32 * W) {
+    const u32 b = b0 + lane * W;
+    u32 have = __ballot_sync(kFull, b < nblk && __ldg(a.bmax + b) >= least);
+    while (have) {
+      const u32 v0 = (b0 + (u32)(__ffs(have) - 1) * W) * kMaxBlock + lane;
+      have &= have - 1;
+      u64 k[kMaxBlock / 32];
+#pragma unroll
+      for (int q = 0; q < (int)kMaxBlock / 32; ++q)
+        k[q] = v0 + (u32)q * 32 < a.n ? ld_cg_u64(a.key + v0 + (u32)q * 32) : ~0ull;
+#pragma unroll
+      for (int q = 0; q < (int)kMaxBlock / 32; ++q) {
+        const u32 v = v0 + (u32)q * 32;
+        const int lev = (int)key_level(a.f, k[q]);
+        bool take = v < a.n && lev >= from && lev <= to;
+        if (take && ((__ldg(a.excl + (v >> 5)) >> lane) & 1u)) take = false;
+        if (take)  // unclaimed: the key names its own vertex
+          take = key_id(a.f, k[q]) == (U ? v - __ldg(a.voff + __ldg(a.wmem + (v >> 5))) : v);
+        if (!__any_sync(kFull, take)) continue;
+        if (first) {
+          const u32 vv[1] = {v};
+          const bool start = take && lev == from;
+          note_low<!U && !LD>(a, start, k[q], mylow);
+          warp_append<1, LD>(start ? 1u : 0u, vv, a, 0, 0);
+          take = take && !start;
+        }
+        // one reservation per level and warp
+        const u32 peers = __match_any_sync(kFull, take ? lev : -1);
+        const int leader = __ffs(peers) - 1;
+        u32 at = 0;
+        if (take && (int)lane == leader) at = atomicAdd(a.rcur + (lev - lv0), (u32)__popc(peers));
+        at = __shfl_sync(kFull, at, leader);
+        if (take) a.rv[at + (u32)__popc(peers & lanemask_lt())] = v;
+      }
+    }
+  }
+  return to;
+}
+
 template <bool U>
 __device__ __forceinline__ void expand(const BfsArgs& a, Smem& s, int cur, u32 Q, u32 E, int lvl,
-                                       int qi, int qb, u32& myrank, u32* s_acc) {
+                                       int qi, int qb, u64& mylow) {
   const u32 nb = (E + kBfsBase - 1) / kBfsBase;
   u32 k = (nb + gridDim.x - 1) / gridDim.x;
   k = max(1u, min(k, a.span / kBfsBase));
@@ -498,7 +589,7 @@ __device__ __forceinline__ void expand(const BfsArgs& a, Smem& s, int cur, u32 Q
         if (off[i] < e1) {
           const int j = j0 + i * kBfsThreads + (int)threadIdx.x;
           s.rowd[j] = row[i] - (int)off[i];
-          s.cand[j] = kv[i] + kLevelOne;
+          s.cand[j] = key_up(a.f, kv[i]);
           atomicMax(&s.owner[off[i] > e0 ? off[i] - e0 : 0u], j);
         }
     }
@@ -528,13 +619,20 @@ __device__ __forceinline__ void expand(const BfsArgs& a, Smem& s, int cur, u32 Q
 #pragma unroll
       for (int i = 0; i < kEdgeBatch; ++i)
         if (cand[i] < cur[i]) {
-          const u64 old = atomicMin(a.key + w[i], cand[i]);
-          if (old > cand[i]) won |= 1u << i;
-          if ((u32)(old >> 32) > lvl_next) mask |= 1u << i;
+          cur[i] = atomicMin(a.key + w[i], cand[i]);
+          if (cur[i] > cand[i]) won |= 1u << i;
+          if (key_level(a.f, cur[i]) > lvl_next) mask |= 1u << i;
         }
+      bool tie = false;  // one branch for the batch: meetings are rare
 #pragma unroll
-      for (int i = 0; i < kEdgeBatch; ++i)
-        note_rank<U>(a, (u32)qi, (won >> i) & 1u, w[i], (u32)cand[i], myrank, s_acc);
+      for (int i = 0; i < kEdgeBatch; ++i) tie |= w[i] < a.n && key_near(cand[i], cur[i]);
+      if (tie) {
+#pragma unroll
+        for (int i = 0; i < kEdgeBatch; ++i)
+          if (w[i] < a.n) note_tie(a, w[i], cand[i], cur[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < kEdgeBatch; ++i) note_low<!U>(a, (won >> i) & 1u, cand[i], mylow);
       warp_append<kEdgeBatch, false>(mask, w, a, qi, qb);
     }
     __syncthreads();
@@ -558,8 +656,8 @@ __device__ __forceinline__ void expand(const BfsArgs& a, Smem& s, int cur, u32 Q
 // such chain.  `pushed` adds the arcs offered.
 template <bool U>
 __device__ __forceinline__ void expand_ld(const BfsArgs& a, const u32* qv_cur, u32 Q, u32 lvl_next,
-                                          const u32* rv, int lo, u32 cnt, u32 rb, bool probe,
-                                          int qi, int qb, u32& myrank, u32* s_acc, u64& pushed) {
+                                          int lo, u32 cnt, u32 rb, bool probe, int qi, int qb,
+                                          u64& pushed) {
   constexpr u32 kNone = 0xffffffffu;
   constexpr int KI = kLdItems;
   constexpr int KA = kLdItems * kLdBatch;
@@ -576,7 +674,7 @@ __device__ __forceinline__ void expand_ld(const BfsArgs& a, const u32* qv_cur, u
       buck[t] = !front[t] && i < total;
       v[t] = 0;
       if (front[t]) v[t] = ld_cg_u32(qv_cur + i);
-      else if (buck[t]) v[t] = __ldg(rv + lo + (int)(i - Q));
+      else if (buck[t]) v[t] = ld_cg_u32(a.rv + lo + (int)(i - Q));
     }
     u64 kv[KI];
     int rs[KI], re[KI];
@@ -594,9 +692,7 @@ __device__ __forceinline__ void expand_ld(const BfsArgs& a, const u32* qv_cur, u
     u32 smask = 0;
 #pragma unroll
     for (int t = 0; t < KI; ++t) {
-      const bool start = buck[t] && (u32)(kv[t] >> 32) == rb;
-      if (start) smask |= 1u << t;
-      note_rank<U>(a, (u32)qi, start, v[t], (u32)kv[t], myrank, s_acc);
+      if (buck[t] && key_level(a.f, kv[t]) == rb) smask |= 1u << t;
     }
     warp_append<KI, true>(smask, v, a, qi, qb);
     int nch = 0;
@@ -619,20 +715,24 @@ __device__ __forceinline__ void expand_ld(const BfsArgs& a, const u32* qv_cur, u
 #pragma unroll
       for (int x = 0; x < KA; ++x)
         cur[x] = (w[x] < a.n) ? (probe ? ld_cg_u64(a.key + w[x]) : ~0ull) : 0ull;
-      u32 mask = 0, won = 0;
+      u32 mask = 0;
 #pragma unroll
       for (int x = 0; x < KA; ++x) {
-        const u64 cand = kv[x / kLdBatch] + kLevelOne;
+        const u64 cand = key_up(a.f, kv[x / kLdBatch]);
         if (cand < cur[x]) {
-          const u64 old = atomicMin(a.key + w[x], cand);
-          if (old > cand) won |= 1u << x;
-          if ((u32)(old >> 32) > lvl_next) mask |= 1u << x;
+          cur[x] = atomicMin(a.key + w[x], cand);
+          if (key_level(a.f, cur[x]) > lvl_next) mask |= 1u << x;
         }
       }
+      bool tie = false;  // one branch for the batch: meetings are rare
 #pragma unroll
       for (int x = 0; x < KA; ++x)
-        note_rank<U>(a, (u32)qi, (won >> x) & 1u, w[x], (u32)(kv[x / kLdBatch] + kLevelOne),
-                     myrank, s_acc);
+        tie |= w[x] < a.n && key_near(key_up(a.f, kv[x / kLdBatch]), cur[x]);
+      if (tie) {
+#pragma unroll
+        for (int x = 0; x < KA; ++x)
+          if (w[x] < a.n) note_tie(a, w[x], key_up(a.f, kv[x / kLdBatch]), cur[x]);
+      }
       warp_append<KA, true>(mask, w, a, qi, qb);
     }
   }
@@ -714,7 +814,7 @@ __device__ __forceinline__ void window_push(u32 mask, const u32 (&w)[K], const u
     if (spill >> i & 1u) {
       if (sbase < a.n) {
         reinterpret_cast<u32*>(a.qrow[qb])[sbase] = w[i];
-        a.qoff[qb][sbase] = (u32)(k[i] >> 32);
+        a.qoff[qb][sbase] = key_level(a.f, k[i]);
       } else {
         atomicOr(&a.ctl->err, kErrInternal);  // more pushes than vertices: cannot happen
       }
@@ -733,15 +833,13 @@ __device__ __forceinline__ void window_push(u32 mask, const u32 (&w)[K], const u
 template <bool U, int kCap>
 __device__ __forceinline__ void window_expand(const BfsArgs& a, Smem& s, bool valid, u64 kv,
                                               int rs, int re, u32 H, int nb, int nc, int qi,
-                                              int qb,
-                                              u32& myrank, u32* s_acc, u64& pushed,
-                                              u64& expanded) {
+                                              int qb, u64& pushed, u64& expanded) {
   constexpr u32 kNone = 0xffffffffu;
   if (!valid) re = rs;
   else ++expanded;
   pushed += (u64)(re - rs);
-  const u64 cand = kv + kLevelOne;
-  const u32 cl = (u32)(cand >> 32);
+  const u64 cand = key_up(a.f, kv);
+  const u32 cl = key_level(a.f, cand);
   const int nch = (int)__reduce_max_sync(kFull, (u32)((re - rs + kLdBatch - 1) / kLdBatch));
   for (int ch = 0; ch < nch; ++ch) {
     const int e0 = rs + ch * kLdBatch;
@@ -750,10 +848,12 @@ __device__ __forceinline__ void window_expand(const BfsArgs& a, Smem& s, bool va
     for (int q = 0; q < kLdBatch; ++q) w[q] = (e0 + q < re) ? (u32)__ldg(a.col + e0 + q) : kNone;
     u64 kk[kLdBatch];
     int wrs[kLdBatch], wre[kLdBatch];
-    u32 local = 0, glob = 0, won = 0;
+    u64 met[kLdBatch];
+    u32 local = 0, glob = 0;
 #pragma unroll
     for (int q = 0; q < kLdBatch; ++q) {
       kk[q] = cand;
+      met[q] = cand;
       wrs[q] = 0;
       wre[q] = 0;
       if (w[q] < a.n) {
@@ -761,17 +861,20 @@ __device__ __forceinline__ void window_expand(const BfsArgs& a, Smem& s, bool va
           wrs[q] = __ldg(a.row_ptr + w[q]);
           wre[q] = __ldg(a.row_ptr + w[q] + 1);
         }
-        const u64 old = atomicMin(a.key + w[q], cand);
-        if (old > cand) {
-          won |= 1u << q;
+        met[q] = atomicMin(a.key + w[q], cand);
+        if (met[q] > cand) {
           if (cl < H) local |= 1u << q;
-          else if ((u32)(old >> 32) > H) glob |= 1u << q;
+          else if (key_level(a.f, met[q]) > H) glob |= 1u << q;
         }
       }
     }
+    bool tie = false;  // one branch for the batch: meetings are rare
 #pragma unroll
-    for (int q = 0; q < kLdBatch; ++q)  // the next round's bottom-up floor: level-H keys
-      note_rank<U>(a, (u32)qi, ((won >> q) & 1u) && cl == H, w[q], (u32)cand, myrank, s_acc);
+    for (int q = 0; q < kLdBatch; ++q) tie |= key_near(cand, met[q]);
+    if (tie) {
+#pragma unroll
+      for (int q = 0; q < kLdBatch; ++q) note_tie(a, w[q], cand, met[q]);
+    }
     window_push<kLdBatch, kCap>(local, w, kk, wrs, wre, a, s, nb, nc, qi, qb);
     warp_append<kLdBatch, true>(glob, w, a, qi, qb);
   }
@@ -784,9 +887,12 @@ __device__ __forceinline__ void window_expand(const BfsArgs& a, Smem& s, bool va
 // Only pushes that find the local queue full wait for the next round (on the
 // overflow list).  `expanded` counts expansions.
 template <bool U, int kCap>
-__device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, const u32* rv, int A,
+__device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, int lv0, int A,
                                           u32 Q, u32 nov, int qcur, u32 L, u32 H, int qi, int qb,
-                                          u32& myrank, u32* s_acc, u64& pushed, u64& expanded) {
+                                          u64& pushed, u64& expanded) {
+  const int* bp = a.bptr - lv0;    // start buckets by level
+  const u32* rc = a.rcur - lv0;
+  const u32* rv = a.rv;
   const u32 lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     s.lcnt[0] = 0;
@@ -806,15 +912,15 @@ __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, const u32* 
   auto bucket_ok = [&](u32 r) { return (int)r <= A && r <= H; };
   int b1lo = 0, b1hi = 0, b2lo = 0, b2hi = 0;  // buckets lv + 1 and lv + 2
   if (bucket_ok(L + 1)) {
-    b1lo = __ldg(a.bptr + L + 1);
-    b1hi = __ldg(a.bptr + L + 2);
+    b1lo = __ldg(bp + L + 1);
+    b1hi = (int)ld_cg_u32(rc + L + 1);
   }
   if (bucket_ok(L + 2)) {
-    b2lo = __ldg(a.bptr + L + 2);
-    b2hi = __ldg(a.bptr + L + 3);
+    b2lo = __ldg(bp + L + 2);
+    b2hi = (int)ld_cg_u32(rc + L + 2);
   }
   u32 pu = kNoItem;  // this thread's first entry of bucket lv + 1
-  if (i0 < (u32)(b1hi - b1lo)) pu = __ldg(rv + b1lo + (int)i0);
+  if (i0 < (u32)(b1hi - b1lo)) pu = ld_cg_u32(rv + b1lo + (int)i0);
   int lb = 0;  // the local queue being read (level lv); the other one is filled
   int cr = 0;  // the counter of the queue being read; (cr + 1) % 3 counts the filled one
   for (u32 lv = L;; ++lv) {
@@ -836,11 +942,11 @@ __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, const u32* 
       pr1 = __ldg(a.row_ptr + pu + 1);
     }
     u32 pu2 = kNoItem;
-    if (i0 < (u32)(b2hi - b2lo)) pu2 = __ldg(rv + b2lo + (int)i0);
+    if (i0 < (u32)(b2hi - b2lo)) pu2 = ld_cg_u32(rv + b2lo + (int)i0);
     int b3lo = 0, b3hi = 0;
     if (bucket_ok(lv + 3)) {
-      b3lo = __ldg(a.bptr + lv + 3);
-      b3hi = __ldg(a.bptr + lv + 4);
+      b3lo = __ldg(bp + lv + 3);
+      b3hi = (int)ld_cg_u32(rc + lv + 3);
     }
     // (1) the window's first level: the global frontier and the overflow list,
     // whose keys and ranges are loaded here
@@ -862,10 +968,9 @@ __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, const u32* 
           kv = ld_cg_u64(a.key + v);
           rs = __ldg(a.row_ptr + v);
           re = __ldg(a.row_ptr + v + 1);
-          ok = (u32)(kv >> 32) >= lev;  // lowered since: its lowerer pushed it again
+          ok = key_level(a.f, kv) >= lev;  // lowered since: its lowerer pushed it again
         }
-        window_expand<U, kCap>(a, s, ok, kv, rs, re, H, nb, nc, qi, qb, myrank, s_acc, pushed,
-                               expanded);
+        window_expand<U, kCap>(a, s, ok, kv, rs, re, H, nb, nc, qi, qb, pushed, expanded);
       }
     }
     // (2) this CTA's local queue of level lv: keys and ranges come with the entries
@@ -875,8 +980,7 @@ __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, const u32* 
         const u32 i = base + lane;
         const bool ok = i < nloc;
         window_expand<U, kCap>(a, s, ok, ok ? lq.key[i] : 0ull, ok ? (int)lq.rs[i] : 0,
-                               ok ? (int)lq.re[i] : 0, H, nb, nc, qi, qb, myrank, s_acc, pushed,
-                               expanded);
+                               ok ? (int)lq.re[i] : 0, H, nb, nc, qi, qb, pushed, expanded);
       }
     }
     // (3) start bucket lv + 1: a vertex whose key still has its start level joins level lv + 1
@@ -895,17 +999,16 @@ __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, const u32* 
             urs[0] = pr0;
             ure[0] = pr1;
           } else {
-            u[0] = __ldg(rv + b1lo + (int)i);
+            u[0] = ld_cg_u32(rv + b1lo + (int)i);
             k[0] = ld_cg_u64(a.key + u[0]);
             urs[0] = __ldg(a.row_ptr + u[0]);
             ure[0] = __ldg(a.row_ptr + u[0] + 1);
           }
-          start = (u32)(k[0] >> 32) == lv + 1;
+          start = key_level(a.f, k[0]) == lv + 1;
         }
         if (lv + 1 < H) {
           window_push<1, kCap>(start ? 1u : 0u, u, k, urs, ure, a, s, nb, nc, qi, qb);
         } else {
-          note_rank<U>(a, (u32)qi, start, u[0], (u32)k[0], myrank, s_acc);
           warp_append<1, true>(start ? 1u : 0u, u, a, qi, qb);
         }
       }
@@ -921,30 +1024,40 @@ __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, const u32* 
   }
 }
 
-// The smallest start level >= from among start-bucket entries whose key still
-// has their start level (a vertex nobody has claimed), into ctl->nstart[slot]
-// as ~level by atomicMax (0 if none); the caller waits at a grid barrier.
-__device__ __forceinline__ void scan_unclaimed(const BfsArgs& a, const u32* rk, const u32* rv,
-                                               int from, int A, u32 slot) {
-  if (from > A) return;
-  const int lo = __ldg(a.bptr + from), hi = __ldg(a.bptr + A + 1);
+// The smallest start level in from .. to among start-bucket entries whose key
+// still has their start level (a vertex nobody has claimed), into
+// ctl->nstart[slot] as ~level by atomicMax (0 if none); the caller waits at a
+// grid barrier.  A thread takes one place of the buckets' room at a time and
+// finds its bucket by a search in bptr.
+__device__ __forceinline__ void scan_unclaimed(const BfsArgs& a, int lv0, int from, int to,
+                                               u32 slot) {
+  const int* bp = a.bptr - lv0;
+  const int lo = __ldg(bp + from), hi = __ldg(bp + to + 1);
   u32 best = 0;
-  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; (int)i < hi - lo;
-       i += gridDim.x * blockDim.x) {
-    const u32 r = __ldg(rk + lo + (int)i);
-    const u64 k = ld_cg_u64(a.key + __ldg(rv + lo + (int)i));
-    if ((u32)(k >> 32) == r) best = max(best, ~r);
+  for (int i = lo + (int)(blockIdx.x * blockDim.x + threadIdx.x); i < hi;
+       i += (int)(gridDim.x * blockDim.x)) {
+    int r = from, r1 = to;  // the last bucket that starts at or before i
+    while (r < r1) {
+      const int mid = (r + r1 + 1) >> 1;
+      if (__ldg(bp + mid) <= i) r = mid;
+      else r1 = mid - 1;
+    }
+    if (i >= (int)ld_cg_u32(a.rcur + (r - lv0))) continue;  // room not used
+    if (key_level(a.f, ld_cg_u64(a.key + ld_cg_u32(a.rv + i))) == (u32)r)
+      best = max(best, ~(u32)r);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kFull, best, o));
+  best = __reduce_max_sync(kFull, best);
   if ((threadIdx.x & 31) == 0 && best) atomicMax(&a.ctl->nstart[slot], best);
 }
 
-// Folds a thread's smallest rank into the CTA's (lane 0 of each warp) and resets it.
-__device__ __forceinline__ void post_cta_min(Smem& s, u32& myrank) {
-  const u32 wm = warp_min(myrank);
-  if ((threadIdx.x & 31) == 0 && wm != 0xffffffffu) atomicMin(&s.minrank, wm);
-  myrank = 0xffffffffu;
+// Leaves the warp's smallest tie-break for the barrier and resets the thread's.
+template <bool kTrack>
+__device__ __forceinline__ void post_cta_min(const BfsArgs& a, Smem& s, u64& mylow) {
+  if (!kTrack) return;
+  const u64 wm = warp_min64(mylow);
+  if (mylow != ~0ull) note_tie(a, 0, mylow, wm);
+  if ((threadIdx.x & 31) == 0) s.minlow[threadIdx.x >> 5] = wm;
+  mylow = ~0ull;
 }
 
 // The two appends of a bottom-up step in one pass.  The vertices of `mask`
@@ -1013,6 +1126,18 @@ __device__ __forceinline__ void pull_append(u32 mask, u32 keep, const u32 (&v)[K
     if (keep >> i & 1u) list[kbase++] = v[i];
 }
 
+// Low-degree rounds of a single graph: the floor of a bottom-up round, from its
+// frontier list, with a grid barrier.
+__device__ __forceinline__ u64 list_floor(const BfsArgs& a, Smem& s, const u32* qv, u32 Q, u32 slot,
+                                          u32& gen, int lv0) {
+  u64 low = ~0ull;
+  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x)
+    note_low<true>(a, true, ld_cg_u64(a.key + ld_cg_u32(qv + i)), low);
+  post_cta_min<true>(a, s, low);
+  grid_barrier<true>(a, gen, slot, lv0, -1, s);
+  return s.next_minlow;
+}
+
 // Puts vertices w[i] (bits of mask; with kPushFlag: see pull_rest) with the
 // arcs [e[i], re[i]) on the list that pull_rest works off, in the frontier's
 // own format (vertex, first arc, exclusive arc offset, first slot of every base
@@ -1050,18 +1175,18 @@ __device__ __forceinline__ void defer_append(u32 mask, const u32 (&w)[K], const 
     }
 }
 
-// A bottom-up round's pivot rank (single graphs): kPivotSamples evenly spaced
-// samples of the frontier's E arcs, each with the rank of its vertex's key; the
+// A bottom-up round's pivot (single graphs): kPivotSamples evenly spaced
+// samples of the frontier's E arcs, each with its vertex's tie-break; the
 // kPivotSkip-th smallest.  Every CTA takes the same samples of a list that no
 // longer changes, so all get the same pivot without a barrier.
-__device__ __forceinline__ u32 pivot_rank(const BfsArgs& a, Smem& s, int cur, u32 Q, u32 E) {
+__device__ __forceinline__ u64 pivot_low(const BfsArgs& a, Smem& s, int cur, u32 Q, u32 E) {
   const u32 nb = (E + kBfsBase - 1) / kBfsBase;
-  u32* smp = reinterpret_cast<u32*>(s.owner);
-  u32 r = 0;
+  u64* smp = s.cand;
+  u64 r = 0;
   __syncthreads();
   if (threadIdx.x < kPivotSamples) {
     const u32 slot = ld_cg_u32(a.cf[cur] + (u32)((u64)threadIdx.x * nb / kPivotSamples));
-    r = (u32)ld_cg_u64(a.key + ld_cg_u32(a.qv[cur] + min(slot, Q - 1)));
+    r = key_low(a.f, ld_cg_u64(a.key + ld_cg_u32(a.qv[cur] + min(slot, Q - 1))));
     smp[threadIdx.x] = r;
   }
   __syncthreads();
@@ -1069,7 +1194,7 @@ __device__ __forceinline__ u32 pivot_rank(const BfsArgs& a, Smem& s, int cur, u3
     u32 less = 0, same = 0;
 #pragma unroll 8
     for (u32 i = 0; i < kPivotSamples; ++i) {
-      const u32 x = smp[i];
+      const u64 x = smp[i];
       less += x < r ? 1u : 0u;
       same += x == r ? 1u : 0u;
     }
@@ -1079,11 +1204,11 @@ __device__ __forceinline__ u32 pivot_rank(const BfsArgs& a, Smem& s, int cur, u3
   return s.pivot;
 }
 
-// The frontier vertices whose rank lies below the pivot (their member's pivot)
-// go on pull_rest's list, to push.
+// The frontier vertices whose tie-break lies below the pivot (their member's
+// pivot), or differs from it only in the id, go on pull_rest's list, to push.
 template <bool U>
-__device__ __forceinline__ void list_pushes(const BfsArgs& a, int cur, u32 Q, u32 pivot,
-                                            u32 mslot, int qi, const u32* s_floor) {
+__device__ __forceinline__ void list_pushes(const BfsArgs& a, int cur, u32 Q, u64 pivot,
+                                            u32 mslot, int qi, const u64* s_floor) {
   const u32 lane = threadIdx.x & 31;
   const u32 stride = gridDim.x * blockDim.x;
   for (u32 base = warp_first_item(1); base < Q; base += stride) {
@@ -1093,8 +1218,9 @@ __device__ __forceinline__ void list_pushes(const BfsArgs& a, int cur, u32 Q, u3
     bool push = false;
     if (i < Q) {
       v[0] = ld_cg_u32(a.qv[cur] + i);
-      const u32 r = (u32)ld_cg_u64(a.key + v[0]);
-      push = r < (U ? member_floor(a, v[0], mslot, s_floor, true) : pivot);
+      const u64 r = key_low(a.f, ld_cg_u64(a.key + v[0]));
+      const u64 pv = U ? member_floor(a, v[0], mslot, s_floor, true) : pivot;
+      push = r < pv || key_tie(a.f, r, pv);
       if (push) {
         rs[0] = __ldg(a.row_ptr + v[0]);
         re[0] = __ldg(a.row_ptr + v[0] + 1);
@@ -1132,13 +1258,13 @@ __device__ __forceinline__ void list_pushes(const BfsArgs& a, int cur, u32 Q, u3
 // listing the pushes costs more than the scans: 8 -> 42 us in R-MAT 22's second
 // bottom-up round) and at least kDeferMin candidates.
 template <bool U>
-__device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lvl, u32 pivot,
-                                          u32 mslot, int qi, int qb, u32& myrank, u32* s_acc,
-                                          const u32* s_floor) {
+__device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lvl, u64 pivot,
+                                          u32 mslot, int qi, int qb, u64& mylow,
+                                          const u64* s_floor) {
   constexpr u32 kNone = 0xffffffffu;
   const u32 lane = threadIdx.x & 31;
   const u32 L = (u32)lvl;
-  const u64 lvl_key = (u64)(L + 1) << 32;
+  const u64 lvl_key = level_key(a.f, L + 1);
   const u32 nchunk = (E + kBfsBase - 1) / kBfsBase;
   const u32 W = gridDim.x * (blockDim.x >> 5);
   const u32 k = max(1u, min(nchunk / W, 4u));
@@ -1194,25 +1320,40 @@ __device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lv
       u32 got = p < stop ? min(stop - p, (u32)kRestBatch) : 0u;
       u32 join = 0;
       if (push) {
-        const u64 cand = kw + kLevelOne;
+        const u64 cand = key_up(a.f, kw);
+        bool won = false, tie = false;
         pushed += got;
 #pragma unroll
         for (int q = 0; q < kRestBatch; ++q)
-          if (vv[q] < a.n && cand < kv[q]) {
-            const u64 old = atomicMin(a.key + vv[q], cand);
-            if (old > cand) note_rank<U>(a, (u32)qi, true, vv[q], (u32)cand, myrank, s_acc);
-            if ((u32)(old >> 32) > L + 1) join |= 1u << q;
+          if (vv[q] < a.n) {
+            if (cand < kv[q]) {
+              kv[q] = atomicMin(a.key + vv[q], cand);
+              won |= kv[q] > cand;
+              if (key_level(a.f, kv[q]) > L + 1) join |= 1u << q;
+            }
+            tie |= key_near(cand, kv[q]);
           }
+        note_low<!U>(a, won, cand, mylow);
+        if (tie) {
+#pragma unroll
+          for (int q = 0; q < kRestBatch; ++q)
+            if (vv[q] < a.n) note_tie(a, vv[q], cand, kv[q]);
+        }
       } else {
         scanned += got;
 #pragma unroll
         for (int q = 0; q < kRestBatch; ++q)
-          if ((u32)(kv[q] >> 32) == L) best = min(best, kv[q] + kLevelOne);
+          if (vv[q] < a.n && key_level(a.f, kv[q]) == L) {
+            const u64 cand = key_up(a.f, kv[q]);
+            note_tie(a, w, cand, best);
+            best = min(best, cand);
+          }
       }
       warp_append<kRestBatch, false>(join, vv, a, qi, qb);
       p += got;
       // the end of a scan, or of this lane's share of it: offer what was found
       const bool offer = !push && w != kNone && p == stop && best < kw;
+      if (!push && w != kNone && p == stop && best > kw) note_tie(a, w, best, kw);
       const u32 om = __ballot_sync(kFull, offer);
       if (om) {
         const int first = __ffs(om) - 1;
@@ -1220,14 +1361,18 @@ __device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lv
         bool mine = offer;
         if (__all_sync(kFull, !offer || w == w0)) {
           const u64 b = warp_min64(offer ? best : ~0ull);
-          if (offer) best = b;
+          if (offer) {
+            note_tie(a, w, best, b);
+            best = b;
+          }
           mine = (int)lane == first;
         }
         u32 won = 0;
         if (mine) {
           const u64 old = atomicMin(a.key + w, best);
-          if (old > best) note_rank<U>(a, (u32)qi, true, w, (u32)best, myrank, s_acc);
-          if ((u32)(old >> 32) > L + 1) won = 1;
+          note_tie(a, w, best, old);
+          note_low<!U>(a, old > best, best, mylow);
+          if (key_level(a.f, old) > L + 1) won = 1;
         }
         const u32 ww[1] = {w};
         warp_append<1, false>(won, ww, a, qi, qb);
@@ -1254,11 +1399,10 @@ __device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lv
 // loaded beside its key, so it needs no col round trip.  Adds the arcs it
 // scans and the vertices it examines to the statistics.
 template <bool U, bool LD, int kPullV>
-__device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minrank, u32 mslot,
+__device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u64 stop_low, u32 mslot,
                                            int qi, int qb, bool from_list, const u32* cand,
                                            u32 ncand, u32* ulist_out, u32* ucnt_out,
-                                           u32& myrank, u32* s_acc, const u32* s_floor,
-                                           bool defer) {
+                                           u64& mylow, const u64* s_floor, bool defer) {
   constexpr u32 kNone = 0xffffffffu;
   u32 scanned = 0, examined = 0;
   const u32 lane = threadIdx.x & 31;
@@ -1340,19 +1484,19 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
       re0[j] = re[j];
     }
     u64 best[kPullV];
-    u32 fr[kPullV];  // floor rank: nothing beats (L + 1, fr); union: w's own member's
+    u64 fr[kPullV];  // nothing beats (L + 1, fr); union: w's own member's
 #pragma unroll
     for (int j = 0; j < kPullV; ++j) {
-      fr[j] = minrank;
+      fr[j] = stop_low;
       if (U && w[j] != kNone) fr[j] = member_floor(a, w[j], mslot, s_floor, !LD && defer);
     }
-    const u64 lvl_key = (u64)(L + 1) << 32;
+    const u64 lvl_key = level_key(a.f, L + 1);
 #pragma unroll
     for (int j = 0; j < kPullV; ++j) {
       best[j] = kw[j];
       if (w[j] != kNone) ++examined;
-      if (!((u32)(kw[j] >> 32) > L && kw[j] > (lvl_key | fr[j]))) re[j] = e[j];  // settled or unbeatable
-      if (U && fr[j] == 0xffffffffu) re[j] = e[j];  // w's member has no level-L key
+      if (!(key_level(a.f, kw[j]) > L && kw[j] > (lvl_key | fr[j]))) re[j] = e[j];  // settled or unbeatable
+      if (U && fr[j] == ~0ull) re[j] = e[j];  // w's member has no level-L key
     }
     // one neighbour of every still-scanning candidate per step, for at most
     // kPullLong steps: most scans stop at their first neighbours
@@ -1383,7 +1527,11 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
       for (int j = 0; j < kPullV; ++j) kv[j] = (vv[j] < a.n) ? ld_cg_u64(a.key + vv[j]) : ~0ull;
 #pragma unroll
       for (int j = 0; j < kPullV; ++j) {
-        if ((u32)(kv[j] >> 32) == L) best[j] = min(best[j], kv[j] + kLevelOne);
+        if (vv[j] < a.n && key_level(a.f, kv[j]) == L) {
+          const u64 cand = key_up(a.f, kv[j]);
+          note_tie(a, w[j], cand, best[j]);
+          best[j] = min(best[j], cand);
+        }
         if (best[j] <= (lvl_key | fr[j])) re[j] = e[j];  // nothing can beat (L + 1, fr)
       }
     }
@@ -1409,6 +1557,7 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
         const int eb = __shfl_sync(kFull, e[j], src), ee = __shfl_sync(kFull, re[j], src);
         const u64 fj = lvl_key | __shfl_sync(kFull, fr[j], src);
         u64 b = __shfl_sync(kFull, best[j], src);
+        const u32 ws = __shfl_sync(kFull, w[j], src);
         int pos = eb;
         while (pos < ee) {
           u32 vq[kPullCoop];
@@ -1421,9 +1570,16 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
 #pragma unroll
           for (int q = 0; q < kPullCoop; ++q) {
             const u64 kq = vq[q] < a.n ? ld_cg_u64(a.key + vq[q]) : ~0ull;
-            if ((u32)(kq >> 32) == L) lb = min(lb, kq + kLevelOne);
+            if (vq[q] < a.n && key_level(a.f, kq) == L) {
+              const u64 cand = key_up(a.f, kq);
+              note_tie(a, ws, cand, lb);
+              note_tie(a, ws, cand, b);
+              lb = min(lb, cand);
+            }
           }
-          b = min(b, warp_min64(lb));
+          const u64 wb = warp_min64(lb);
+          if (lb != ~0ull) note_tie(a, ws, lb, wb);
+          b = min(b, wb);
           pos += 32 * kPullCoop;
           if (b <= fj) break;  // warp-uniform: nothing can beat (L + 1, minrank)
         }
@@ -1440,18 +1596,18 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u32 minran
     u32 mask = 0, keep = 0, won = 0;
 #pragma unroll
     for (int j = 0; j < kPullV; ++j) {
-      const bool pending = w[j] != kNone && (u32)(kw[j] >> 32) > L;
+      const bool pending = w[j] != kNone && key_level(a.f, kw[j]) > L;
       if (pending && best[j] < kw[j]) {
         a.key[w[j]] = best[j];  // only this thread writes key[w] in a bottom-up round
         won |= 1u << j;
-        if ((u32)(kw[j] >> 32) > L + 1) mask |= 1u << j;
+        if (key_level(a.f, kw[j]) > L + 1) mask |= 1u << j;
       }
       // still above level L + 1: examined again by a following bottom-up round
-      if (pending && (u32)(min(best[j], kw[j]) >> 32) > L + 1) keep |= 1u << j;
+      if (pending && key_level(a.f, min(best[j], kw[j])) > L + 1) keep |= 1u << j;
     }
 #pragma unroll
     for (int j = 0; j < kPullV; ++j)
-      note_rank<U>(a, (u32)qi, (won >> j) & 1u, w[j], (u32)best[j], myrank, s_acc);
+      note_low<!U && !LD>(a, (won >> j) & 1u, best[j], mylow);
     pull_append<kPullV, LD>(mask, keep, w, rs0, re0, a, qi, qb, ulist_out, ucnt_out);
 #pragma unroll
     for (int j = 0; j < kPullV; ++j) {
@@ -1489,41 +1645,44 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
   Smem& s = *reinterpret_cast<Smem*>(smem_raw);
   // union with few enough members: per-member next-level minima and
   // current-level floors in shared memory, after Smem
-  u32* s_acc = (U && a.kmem <= kSmemMembers)
-                   ? reinterpret_cast<u32*>(smem_raw + sizeof(Smem) + (LD ? lq_extra(kPerSm) : 0))
+  u64* s_acc = (U && a.kmem <= kSmemMembers)
+                   ? reinterpret_cast<u64*>(smem_raw + sizeof(Smem) + (LD ? lq_extra(kPerSm) : 0))
                    : nullptr;
-  u32* s_floor = s_acc ? s_acc + kSmemMembers : nullptr;
-  u64* s_piv = s_acc ? reinterpret_cast<u64*>(s_acc + 2 * kSmemMembers) : nullptr;
+  u64* s_floor = s_acc ? s_acc + kSmemMembers : nullptr;
+  u64* s_piv = s_acc ? s_acc + 2 * kSmemMembers : nullptr;
   if (s_acc)
     for (u32 m = threadIdx.x; m < a.kmem; m += blockDim.x) {
-      s_acc[m] = 0xffffffffu;
+      s_acc[m] = ~0ull;
       s_piv[m] = 0;
     }
   Control* ctl = a.ctl;
   if (threadIdx.x == 0) {
-    s.minrank = 0xffffffffu;
     s.stop = ld_acquire_u32(&ctl->err) != 0u ? 1u : 0u;  // validation failed upstream
   }
   __syncthreads();
   if (s.stop) return;  // CTA-uniform: read once by thread 0
-  const int A = ctl->A;
-  const u32 par_r = __popc(ctl->mask_r) & 1u;
-  const u32* rk = a.rk[par_r];
-  const u32* rv = a.rv[par_r];
-  const u32 G = gridDim.x;
+  // levels lv0 .. A: with direct keys those of the handled vertices' floors
+  const int lv0 = a.f.cap ? (int)a.f.cap - ctl->Ab : 0;
+  const int A = a.f.cap ? (int)a.f.cap : ctl->A;
+  constexpr bool kTrack = !U && !LD;
   u32 gen = 0;
-  u32 myrank = 0xffffffffu;  // this thread's smallest successful next-level rank
-
+  u64 mylow = ~0ull;  // this thread's smallest successful next-level tie-break
+  // start buckets filled so far, and the room for the next ones
+  int built = a.f.cap ? lv0 - 1 : A;
+  u32 room = max(a.n_active >> kBuildShift, kBuildMin);
   u64 pushed = 0;  // low-degree mode: arcs offered by this thread
-  // Level 0: the vertices with the largest integer shift part start.
-  if (LD) {
-    const int lo = __ldg(a.bptr), hi = __ldg(a.bptr + 1);
-    expand_ld<U>(a, nullptr, 0, 0, rv, lo, (u32)(hi - lo), 0, false, 0, 0, myrank, s_acc, pushed);
+  // Level lv0: the vertices with the largest integer shift part start.
+  if (a.f.cap) {
+    built = build_buckets<U, LD>(a, s, lv0, lv0, A, room, true, mylow);
   } else {
-    append_bucket<U>(a, 0, rv, 0, 0, myrank, s_acc);
+    const int lo = __ldg(a.bptr), hi = (int)ld_cg_u32(a.rcur);
+    if (LD)
+      expand_ld<U>(a, nullptr, 0, 0, lo, (u32)(hi - lo), (u32)lv0, false, 0, 0, pushed);
+    else
+      append_bucket<U>(a, lv0, lo, hi, 0, 0, mylow);
   }
-  post_cta_min(s, myrank);
-  grid_barrier(ctl, gen, G, a.bar_phantom, a.spin_limit, 0, a.bptr, A >= 1 ? 1 : -1, s);
+  post_cta_min<kTrack>(a, s, mylow);
+  grid_barrier<kTrack>(a, gen, 0, lv0, A > lv0 && built > lv0 ? lv0 + 1 : -1, s);
   const bool profiler = blockIdx.x == 0 && threadIdx.x == 0;
   if (profiler) {
     const long long t = clock64();
@@ -1537,13 +1696,13 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
   u32 phase = 0, pulls = 0, nwin = 0, overflowed = 0;
   u32 wdepth = a.window_levels;  // levels of the next window
   u64 push_arcs = 0;
-  int lvl = 0;
+  int lvl = lv0;
   bool pulling = false;
   bool windowed = false;  // a window has run: settled vertices are no longer counted exactly
   // No correct run needs more rounds than this (each round settles a level or
   // jumps to a start bucket); a loop that would is stopped with an error
   // instead of holding the GPU.
-  const u64 max_rounds = 2ull * ((u64)a.n_active + (u64)A) + 1024;
+  const u64 max_rounds = 2ull * ((u64)a.n_active + (u64)(A - lv0)) + 1024;
   for (;;) {
     if (s.stop) break;  // set by the last barrier, the same for every thread of the CTA
     if (phase > max_rounds) {  // the same for every thread of every CTA
@@ -1551,7 +1710,7 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
       break;
     }
     const u64 c = s.next_c;  // slot phase % 3, read as the last barrier released
-    const int nb_lo = s.next_lo, nb_hi = s.next_hi;  // start bucket lvl + 1 (if lvl + 1 <= A)
+    int nb_lo = s.next_lo, nb_hi = s.next_hi;  // start bucket lvl + 1 (if lvl + 1 <= A)
     const u32 Q = (u32)(c >> 32);
     // overflow entries of the last window (more than n cannot have been written:
     // that sets kErrInternal, and the loop stops at the barrier)
@@ -1562,11 +1721,11 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
                      : (u32)c;
     settled += Q;
     if (!windowed && settled >= a.n_active) break;  // every vertex the BFS owns has its final key
-    const u32 minrank = s.next_minrank;
+    const u64 minlow = s.next_minlow;
     const u32 ncand = s.next_ucnt;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       ctl->qctr[(phase + 2) % 3] = 0;
-      ctl->minrank[(phase + 2) % 3] = 0xffffffffu;
+      ctl->minlow[(phase + 2) % 3] = ~0ull;
       ctl->ucnt[(phase + 2) % 3] = 0;
       ctl->ovf[(phase + 2) % 3] = 0;
       ctl->nstart[(phase + 2) % 3] = 0;
@@ -1574,14 +1733,22 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
       ctl->rest[(phase + 2) % 3] = 0;
     }
     if (U)  // the members' floors of the slot that the next round fills
-      for (u32 m = blockIdx.x * blockDim.x + threadIdx.x; m < a.kmem; m += G * blockDim.x) {
-        a.mrank[(size_t)((phase + 2) % 3) * a.kmem + m] = 0xffffffffu;
+      for (u32 m = blockIdx.x * blockDim.x + threadIdx.x; m < a.kmem; m += gridDim.x * blockDim.x) {
+        a.mlow[(size_t)((phase + 2) % 3) * a.kmem + m] = ~0ull;
         if (!LD) a.mpivot[(size_t)((phase + 2) % 3) * a.kmem + m] = 0;
       }
     const int qi = (int)((phase + 1) % 3), qb = (int)((phase + 1) & 1);
     int nlvl;
     bool defer = false;  // a bottom-up round with a second pass ...
-    u32 stop_rank = 0;   // ... and the rank its scans stop at
+    u64 stop_low = 0;    // ... and the tie-break its scans stop at
+    if (lvl + 1 <= A && lvl + 1 > built) {  // the next start buckets; each time more at once
+      room = room >= (a.n >> 3) ? a.n : room << 3;
+      built = build_buckets<U, LD>(a, s, lv0, lvl + 1, A, room, false, mylow);
+      grid_barrier<kTrack>(a, gen, kNoPost, lv0, -1, s);
+      if (s.stop) break;
+      nb_lo = __ldg(a.bptr + (lvl + 1 - lv0));
+      nb_hi = (int)ld_cg_u32(a.rcur + (lvl + 1 - lv0));
+    }
     // a window of levels: low-degree rounds whose frontier is thin enough, and
     // always while overflow entries of the last window wait
     bool window = false;
@@ -1595,10 +1762,12 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
       // overflow.  The same for every thread: nov, Q and bptr are.
       if (nov > (Q >> 2)) wdepth = max(wdepth >> 1, 1u);
       else if (nov == 0) wdepth = min(wdepth << 1, a.window_levels);
+      // Buckets lvl + 1 .. H must be filled.
+      const u32 dmax = built < A ? min(wdepth, (u32)(built - lvl)) : wdepth;
       u32 d = 1;
-      for (; d < wdepth; ++d) {
-        const int r = lvl + (int)d;
-        if (r <= A && (u32)(__ldg(a.bptr + r + 1) - __ldg(a.bptr + r)) > a.window_max_q) break;
+      for (; d < dmax; ++d) {
+        const int r = lvl + (int)d - lv0;
+        if (r <= A - lv0 && (u32)(__ldg(a.bptr + r + 1) - __ldg(a.bptr + r)) > a.window_max_q) break;
       }
       window = d > 1 || nov > 0;
       H = (u32)lvl + d;
@@ -1606,8 +1775,8 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
     if (window) {
       edges += E;
       pulling = false;
-      window_ld<U, lq_cap(kPerSm)>(a, s, rv, A, Q, nov, (int)(phase & 1), (u32)lvl, H, qi, qb, myrank, s_acc,
-                   pushed, expanded);
+      window_ld<U, lq_cap(kPerSm)>(a, s, lv0, A, Q, nov, (int)(phase & 1), (u32)lvl, H, qi, qb,
+                                   pushed, expanded);
       if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
       windowed = true;
       ++nwin;
@@ -1626,93 +1795,91 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
       if (pulling) {
         // large rounds stop at a pivot rank and have a second pass
         defer = !LD && max(Q, kDeferMin) <= (was_pulling ? ncand : a.n_active);
-        stop_rank = minrank;
+        stop_low = minlow;
         if (U) {  // this level's per-member floors and pivots, from the frontier list
           member_floors<!LD>(a, a.qv[phase & 1], Q, phase % 3, s_acc, s_piv);
           if (s_acc) {
             __syncthreads();
             flush_members<!LD>(a, phase % 3, s_acc, s_piv);
           }
-          grid_barrier(ctl, gen, G, a.bar_phantom, a.spin_limit, kNoPost, a.bptr, -1, s);
+          grid_barrier<kTrack>(a, gen, kNoPost, lv0, -1, s);
           if (s.stop) break;
           if (s_floor) {  // read once per CTA
             for (u32 m = threadIdx.x; m < a.kmem; m += blockDim.x) {
-              u32 f = ld_cg_u32(a.mrank + (size_t)(phase % 3) * a.kmem + m);
-              if (defer && f != 0xffffffffu)
-                f = (u32)ld_cg_u64(a.key + (u32)ld_cg_u64(a.mpivot + (size_t)(phase % 3) * a.kmem + m));
+              u64 f = ld_cg_u64(a.mlow + (size_t)(phase % 3) * a.kmem + m);
+              if (defer && f != ~0ull) {
+                const u64 pv = ld_cg_u64(a.mpivot + (size_t)(phase % 3) * a.kmem + m);
+                f = key_low(a.f, ld_cg_u64(a.key + (u32)pv));
+              }
               s_floor[m] = f;
             }
             __syncthreads();
           }
+        } else if (LD) {
+          stop_low = list_floor(a, s, a.qv[phase & 1], Q, phase % 3, gen, lv0);
+          if (s.stop) break;
         } else if (defer) {
-          stop_rank = pivot_rank(a, s, (int)(phase & 1), Q, E);
+          stop_low = pivot_low(a, s, (int)(phase & 1), Q, E);
         }
-        if (!LD && defer && (U || stop_rank > minrank))
-          list_pushes<U>(a, (int)(phase & 1), Q, stop_rank, phase % 3, qi, s_floor);
-        pull_round<U, LD, pull_width(kPerSm)>(a, lvl, stop_rank, phase % 3, qi, qb, was_pulling,
+        if (!LD && defer && (U || stop_low > minlow))
+          list_pushes<U>(a, (int)(phase & 1), Q, stop_low, phase % 3, qi, s_floor);
+        pull_round<U, LD, pull_width(kPerSm)>(a, lvl, stop_low, phase % 3, qi, qb, was_pulling,
                                               a.ulist[phase & 1], ncand, a.ulist[(phase + 1) & 1],
-                                              &ctl->ucnt[qi], myrank, s_acc, s_floor, defer);
+                                              &ctl->ucnt[qi], mylow, s_floor, defer);
         ++pulls;
         if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
         if (lvl + 1 <= A) {
           if (LD) {
-            expand_ld<U>(a, nullptr, 0, 0, rv, nb_lo, (u32)(nb_hi - nb_lo), (u32)lvl + 1, false,
-                         qi, qb, myrank, s_acc, pushed);
+            expand_ld<U>(a, nullptr, 0, 0, nb_lo, (u32)(nb_hi - nb_lo), (u32)lvl + 1, false, qi, qb,
+                         pushed);
           } else {
-            append_bucket<U>(a, lvl + 1, rv, qi, qb, myrank, s_acc, nb_lo, nb_hi);
+            append_bucket<U>(a, lvl + 1, nb_lo, nb_hi, qi, qb, mylow);
           }
         }
       } else if (LD) {  // expansion and start bucket lvl + 1 in one pass
-        expand_ld<U>(a, a.qv[phase & 1], Q, (u32)lvl + 1, rv, nb_lo, (u32)(nb_hi - nb_lo),
-                     (u32)lvl + 1, E >= a.probe_min_arcs, qi, qb, myrank, s_acc, pushed);
+        expand_ld<U>(a, a.qv[phase & 1], Q, (u32)lvl + 1, nb_lo, (u32)(nb_hi - nb_lo),
+                     (u32)lvl + 1, E >= a.probe_min_arcs, qi, qb, pushed);
         if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
       } else {
-        expand<U>(a, s, (int)(phase & 1), Q, E, lvl, qi, qb, myrank, s_acc);
+        expand<U>(a, s, (int)(phase & 1), Q, E, lvl, qi, qb, mylow);
         push_arcs += E;
         if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
-        if (lvl + 1 <= A) append_bucket<U>(a, lvl + 1, rv, qi, qb, myrank, s_acc, nb_lo, nb_hi);
+        if (lvl + 1 <= A) append_bucket<U>(a, lvl + 1, nb_lo, nb_hi, qi, qb, mylow);
       }
       nlvl = lvl + 1;
     } else {
       if (lvl + 1 > A) break;
-      int rr;
-      if (windowed) {  // the next start level that still holds an unclaimed vertex
-        scan_unclaimed(a, rk, rv, lvl + 1, A, phase % 3);
-        grid_barrier(ctl, gen, G, a.bar_phantom, a.spin_limit, kNoPost, a.bptr, -1, s);
-        if (s.stop) break;
-        if (threadIdx.x == 0) s.nstart = ld_cg_u32(&ctl->nstart[phase % 3]);
-        __syncthreads();
-        if (s.nstart == 0u) break;  // none: every vertex the BFS owns is settled
-        rr = (int)~s.nstart;
-      } else {
-        const int start = __ldg(a.bptr + lvl + 1);
-        if ((u32)start >= a.n) break;
-        rr = (int)__ldg(rk + start);  // next non-empty start bucket
-        if (rr > A) break;            // only vertices the BFS does not handle remain
+      // the next start level that still holds an unclaimed vertex
+      scan_unclaimed(a, lv0, lvl + 1, built, phase % 3);
+      grid_barrier<kTrack>(a, gen, kNoPost, lv0, -1, s);
+      if (s.stop) break;
+      if (threadIdx.x == 0) s.nstart = ld_cg_u32(&ctl->nstart[phase % 3]);
+      __syncthreads();
+      if (s.nstart == 0u) {  // none in the buckets filled so far
+        if (built >= A) break;  // every vertex the BFS owns is settled
+        lvl = built;
+        continue;
       }
+      const int rr = (int)~s.nstart;
       if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
-      if (LD) {
-        const int lo = __ldg(a.bptr + rr), hi = __ldg(a.bptr + rr + 1);
-        expand_ld<U>(a, nullptr, 0, 0, rv, lo, (u32)(hi - lo), (u32)rr, false, qi, qb, myrank,
-                     s_acc, pushed);
-      } else {
-        append_bucket<U>(a, rr, rv, qi, qb, myrank, s_acc);
-      }
+      const int lo = __ldg(a.bptr + (rr - lv0)), hi = (int)ld_cg_u32(a.rcur + (rr - lv0));
+      if (LD)
+        expand_ld<U>(a, nullptr, 0, 0, lo, (u32)(hi - lo), (u32)rr, false, qi, qb, pushed);
+      else
+        append_bucket<U>(a, rr, lo, hi, qi, qb, mylow);
       // this round left no unsettled list: a bottom-up round after it starts
       // from every vertex the loop owns
       pulling = false;
       nlvl = rr;
     }
     if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][1] = clock64();
-    post_cta_min(s, myrank);
-    grid_barrier(ctl, gen, G, a.bar_phantom, a.spin_limit, (u32)qi, a.bptr,
-                 nlvl + 1 <= A ? nlvl + 1 : -1, s);
+    post_cta_min<kTrack>(a, s, mylow);
+    grid_barrier<kTrack>(a, gen, (u32)qi, lv0, nlvl + 1 <= A ? nlvl + 1 : -1, s);
     if (!LD && defer && !s.stop && (u32)s.next_rest) {  // pushes and put-off scans are listed
-      pull_rest<U>(a, (u32)(s.next_rest >> 32), (u32)s.next_rest, lvl, stop_rank, phase % 3, qi,
-                   qb, myrank, s_acc, s_floor);
-      post_cta_min(s, myrank);
-      grid_barrier(ctl, gen, G, a.bar_phantom, a.spin_limit, (u32)qi, a.bptr,
-                   nlvl + 1 <= A ? nlvl + 1 : -1, s);
+      pull_rest<U>(a, (u32)(s.next_rest >> 32), (u32)s.next_rest, lvl, stop_low, phase % 3, qi, qb,
+                   mylow, s_floor);
+      post_cta_min<kTrack>(a, s, mylow);
+      grid_barrier<kTrack>(a, gen, (u32)qi, lv0, nlvl + 1 <= A ? nlvl + 1 : -1, s);
     }
     ++phase;
     lvl = nlvl;
@@ -1734,7 +1901,7 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
     ctl->pull_rounds = pulls;
     if (!LD) atomicAdd(&ctl->push_arcs, push_arcs);
     ctl->rounds = phase;
-    ctl->last_level = lvl;
+    ctl->last_level = lvl - lv0;
     atomicAdd(&ctl->items, windowed ? items : settled);
     ctl->edges = edges;
     ctl->windows = nwin;
@@ -1748,7 +1915,7 @@ size_t bfs_smem_bytes() { return sizeof(Smem); }
 
 namespace {
 size_t bfs_smem(bool u, int per_sm, bool ld) {
-  return sizeof(Smem) + (ld ? lq_extra(per_sm) : 0) + (u ? kSmemMembers * (2 * sizeof(u32) + sizeof(u64)) : 0);
+  return sizeof(Smem) + (ld ? lq_extra(per_sm) : 0) + (u ? 3 * kSmemMembers * sizeof(u64) : 0);
 }
 
 const void* bfs_kernel(bool u, int per_sm, bool ld) {
@@ -1793,10 +1960,10 @@ int bfs_grid_size(int num_sms, int* blocks_per_sm) {
 int launch_bfs(const BfsArgs& a, int grid, int per_sm, cudaStream_t s, cudaError_t* err) {
   BfsArgs copy = a;
   void* args[] = {&copy};
-  *err = cudaLaunchCooperativeKernel(bfs_kernel(a.mrank != nullptr, per_sm, a.low_degree != 0),
+  *err = cudaLaunchCooperativeKernel(bfs_kernel(a.mlow != nullptr, per_sm, a.low_degree != 0),
                                      dim3(grid),
                                      dim3(kBfsThreads), args,
-                                     bfs_smem(a.mrank != nullptr, per_sm, a.low_degree != 0), s);
+                                     bfs_smem(a.mlow != nullptr, per_sm, a.low_degree != 0), s);
   return *err == cudaSuccess ? 1 : -1;
 }
 

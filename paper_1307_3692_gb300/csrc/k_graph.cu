@@ -1,9 +1,9 @@
 // Per-graph tables, assignment and verification kernels (Miller, Peng, Xu 2013).
 //
-// finalize (Algorithm 1 step 4, Algorithm 2 step 2): a settled key
-// (level << 32) | rank names the center order[rank]; the hop distance is the
-// key's level minus the center's own start level, which is the level of the
-// center's key (a center is its own center, so its key is its start key).
+// finalize (Algorithm 1 step 4, Algorithm 2 step 2): a settled key names its
+// center (by id, or as order[rank]); the hop distance is the key's level minus
+// the center's own start level, which is the level of the center's key (a
+// center is its own center, so its key is its start key).
 //
 // cut (Definition 1.1, second condition; Section 4 notes the check costs
 // O(m) work): edges {v, w} whose endpoints have different centers, each
@@ -39,12 +39,16 @@ constexpr u32 kFull = 0xffffffffu;
 // are in flight together.
 constexpr int kFinIpt = 4;
 
-__global__ void __launch_bounds__(256) k_finalize(const u64* __restrict__ key,
-                                                  const u32* __restrict__ order,
-                                                  const u32* __restrict__ solo, u32 n,
-                                                  int* __restrict__ center, int* __restrict__ dist,
-                                                  const u32* err) {
-  if (*(volatile const u32*)err != 0u) return;  // outputs are not written after a failure
+template <bool kDirect>
+__global__ void __launch_bounds__(256) k_finalize(BfsArgs a, const u32* __restrict__ order,
+                                                  const u32* __restrict__ solo,
+                                                  int* __restrict__ center,
+                                                  int* __restrict__ dist) {
+  if (*(volatile const u32*)&a.ctl->err != 0u) return;  // outputs are not written after a failure
+  const u64* __restrict__ key = a.key;
+  const KeyFmt f = a.f;
+  const u32 n = a.n;
+  if (kDirect && blockIdx.x == 0) tie_check(a.shift, nullptr, nullptr, a.ctl, threadIdx.x);
   const u32 stride = gridDim.x * blockDim.x;
   for (u32 v0 = blockIdx.x * blockDim.x + threadIdx.x; v0 < n; v0 += stride * kFinIpt) {
     u32 v[kFinIpt], c[kFinIpt];
@@ -54,13 +58,16 @@ __global__ void __launch_bounds__(256) k_finalize(const u64* __restrict__ key,
     for (int q = 0; q < kFinIpt; ++q) {
       v[q] = v0 + (u32)q * stride;
       live[q] = v[q] < n;
-      // alone in its component: the key is unused, the vertex is its own center
-      alone[q] = live[q] && ((__ldg(solo + (v[q] >> 5)) >> (v[q] & 31)) & 1u);
+      // ranked: alone in its component, the key is unused, the vertex is its own center
+      alone[q] = !kDirect && live[q] && ((__ldg(solo + (v[q] >> 5)) >> (v[q] & 31)) & 1u);
       k[q] = (live[q] && !alone[q]) ? key[v[q]] : 0ull;
     }
 #pragma unroll
-    for (int q = 0; q < kFinIpt; ++q)
-      c[q] = (live[q] && !alone[q]) ? order[min((u32)k[q], n - 1)] : v[q];
+    for (int q = 0; q < kFinIpt; ++q) {
+      c[q] = v[q];
+      if (live[q] && !alone[q])
+        c[q] = kDirect ? min(key_id(f, k[q]), n - 1) : order[min((u32)k[q], n - 1)];
+    }
 #pragma unroll
     for (int q = 0; q < kFinIpt; ++q)
       kc[q] = (live[q] && !alone[q]) ? key[c[q]] : k[q];
@@ -68,7 +75,7 @@ __global__ void __launch_bounds__(256) k_finalize(const u64* __restrict__ key,
     for (int q = 0; q < kFinIpt; ++q)
       if (live[q]) {
         center[v[q]] = (int)c[q];
-        dist[v[q]] = alone[q] ? 0 : (int)((u32)(k[q] >> 32) - (u32)(kc[q] >> 32));
+        dist[v[q]] = alone[q] ? 0 : (int)(key_level(f, k[q]) - key_level(f, kc[q]));
       }
   }
 }
@@ -480,9 +487,8 @@ __global__ void k_small_adj(const int* __restrict__ row_ptr, const int* __restri
 __global__ void __launch_bounds__(256) k_small_comp(const u32* __restrict__ comp_off,
                                                     const u32* __restrict__ comp_len, u32 ncomp,
                                                     const u32* __restrict__ comp_v,
-                                                    const u32* __restrict__ adj, u64* key,
-                                                    const u32* err) {
-  if (*(volatile const u32*)err != 0u) return;
+                                                    const u32* __restrict__ adj, BfsArgs a) {
+  if (*(volatile const u32*)&a.ctl->err != 0u) return;
   const u32 lane = threadIdx.x & 31;
   const u32 warps = gridDim.x * (blockDim.x / 32);
   for (u32 c = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); c < ncomp; c += warps) {
@@ -492,19 +498,23 @@ __global__ void __launch_bounds__(256) k_small_comp(const u32* __restrict__ comp
     if (lane < sz) {
       v = comp_v[off + lane];
       m = adj[off + lane];
-      k = key[v];
+      k = a.key[v];
     }
     for (u32 it = 0; it < sz; ++it) {
       u64 best = k;
       for (u32 t = 0; t < sz; ++t) {
         const u64 kt = __shfl_sync(kFull, k, t);
-        if (m >> t & 1u) best = min(best, kt + kLevelOne);
+        if (m >> t & 1u) {
+          const u64 cand = key_up(a.f, kt);
+          note_tie(a.ctl, a.f, v, cand, best);
+          best = min(best, cand);
+        }
       }
       const bool changed = best != k;
       k = best;
       if (!__any_sync(kFull, changed)) break;
     }
-    if (lane < sz) key[v] = k;
+    if (lane < sz) a.key[v] = k;
   }
 }
 
@@ -832,10 +842,13 @@ u32 grid_for(u32 n, int num_sms) {
 
 }  // namespace
 
-int launch_finalize(const u64* key, const u32* order, const u32* solo, u32 n, int* center,
-                    int* dist, const u32* err, int num_sms, cudaStream_t s) {
-  k_finalize<<<grid_for((n + kFinIpt - 1) / kFinIpt, num_sms), 256, 0, s>>>(key, order, solo, n,
-                                                                         center, dist, err);
+int launch_finalize(const BfsArgs& a, const u32* order, const u32* solo, int* center, int* dist,
+                    int num_sms, cudaStream_t s) {
+  const u32 g = grid_for((a.n + kFinIpt - 1) / kFinIpt, num_sms);
+  if (a.f.cap)
+    k_finalize<true><<<g, 256, 0, s>>>(a, order, solo, center, dist);
+  else
+    k_finalize<false><<<g, 256, 0, s>>>(a, order, solo, center, dist);
   return 1;
 }
 
@@ -914,11 +927,10 @@ int launch_max_dist(const int* dist, u32 n, u32* out, int num_sms, cudaStream_t 
   return 1;
 }
 
-int launch_small_comp(const SmallComps& sc, u64* key, const u32* err, int num_sms, cudaStream_t s) {
+int launch_small_comp(const SmallComps& sc, const BfsArgs& a, int num_sms, cudaStream_t s) {
   if (sc.ncomp == 0) return 0;
   const u32 blocks = (u32)min((long long)(sc.ncomp + 7) / 8, (long long)num_sms * 8);
-  k_small_comp<<<blocks, 256, 0, s>>>(sc.comp_off, sc.comp_len, sc.ncomp, sc.comp_v, sc.adj, key,
-                                      err);
+  k_small_comp<<<blocks, 256, 0, s>>>(sc.comp_off, sc.comp_len, sc.ncomp, sc.comp_v, sc.adj, a);
   return 1;
 }
 

@@ -2,39 +2,31 @@
 //
 //  1. split (Algorithm 1 step 2, Section 4): a_u = floor(delta_u),
 //     f_u = delta_u - a_u (exact in FP64), A = max a_u = floor(delta_max).
-//  2. fraction rank (Section 4: the fractional parts are tie-breakers within
-//     an integer level and can be replaced by a permutation): rank_u = the
-//     position of u in the order (f_u descending, u ascending), order[rank] = u.
-//  3. keys: key_u = ((A - a_u) << 32) | rank_u, i.e. u's own start label at
-//     round R_u = A - a_u.
+//  2. tie-break inside a level (Section 4): larger f_u first, then smaller u.
+//  3. keys (KeyFmt in ldd_internal.cuh): u's own start label.
 //  4. start buckets (Section 4: the super-source edge of length L is looked at
 //     when the frontier reaches distance L): the vertices the BFS handles,
-//     grouped by R_u (any order inside a group); bptr[r] = start of group r,
-//     r = 0 .. A + 1.
+//     grouped by start round R_u = A - a_u (any order inside a group).
 //
-// Fraction rank, fast path (most-significant-digit bucketing): the bucket of u
-// is the top B bits of ~floor(f_u * 2^32), which is monotone in f_u, with
-// 2^B about n / 16 so that buckets hold ~16 vertices.  One pass over the
-// shifts drops a 16-byte record (bits of f_u, a_u, u) into a free slot of its
-// bucket (kSlotCap slots each); an exclusive scan of the bucket counts gives
-// every bucket's first rank; tiles of buckets staged in shared memory then
-// rank every member exactly by (f descending, u ascending) with the full FP64
-// fractions, one thread per record, and write order[] and the keys directly.
-// Vertices alone in their component are not ranked (their center is
-// themselves).  A full bucket (crafted shifts, e.g. all fractions equal)
-// makes the host redo the rank with the exact path: a stable LSD radix sort
-// of the order-preserving bits of f (8 "onesweep" passes of 8 bits) over all
-// vertices.
+// Direct keys (the usual path, k_direct): level, the leading bits of f_u and u
+// in one word, from one pass over the shifts that also counts the floors; an
+// exclusive scan of the counts gives the buckets' offsets (bptr).  The round
+// loop fills the buckets as it reaches them, with the vertices nobody has
+// claimed by then, which are few: bmax, the largest floor of every kMaxBlock
+// vertices, lets it pass over the others.
+//
+// Ranked keys (shifts whose codes tie too often, or levels and ids too wide for
+// a code): a stable LSD radix sort of the order-preserving bits of f (8
+// "onesweep" passes of 8 bits) over all vertices gives the rank; the start
+// buckets are a counting sort by R_u (histogram while the keys are built, an
+// exclusive scan that is bptr, and a scatter in which each CTA reserves its
+// range of every group with one atomic).
 //
 // Batches (disjoint unions of member graphs, k_union.cu): every member's
 // floors are lifted by one integer, lift_s = max_t A_t - A_s, so that each
 // member's own largest shift starts at round 0 and the members' rounds run in
 // step.  A constant added to every level of one member changes no comparison
 // inside that member, and members never compete.
-//
-// Start buckets: a counting sort by R_u (histogram while the keys are built,
-// an exclusive scan that is bptr, and a scatter in which each CTA reserves its
-// range of every group with one atomic).
 #include <algorithm>
 
 #include "ldd_internal.cuh"
@@ -44,7 +36,6 @@ namespace ldd {
 namespace {
 
 constexpr u32 kFull = 0xffffffffu;
-constexpr u32 kSlotCap = 64;                  // record slots per fraction bucket (mean <= 16)
 constexpr int kScanThreads = 256;
 constexpr int kScanIpt = 16;
 constexpr int kScanTile = kScanThreads * kScanIpt;
@@ -68,38 +59,6 @@ __device__ __forceinline__ void hist_add(u32* sh, u32 digit, bool valid, u32 lan
   }
 }
 
-// Splits a shift d into a = floor(d) and the IEEE-754 bits of its fraction
-// f = d - a (exact), with integer operations on d's bits only: FP64
-// arithmetic is slow on this part and the split runs once per vertex.  The
-// bits of a non-negative double order like its value, so fb orders the
-// fractions.  d = -0 counts as +0.  NaN or d < 0 sets kErrShiftArg, d >= 2^31
-// (or +inf) kErrShiftRange; a = 0 and fb = 0 then.
-__device__ __forceinline__ void split_bits(double d, u32& err, int& a, u64& fb) {
-  constexpr u64 kMan = (1ull << 52) - 1;
-  const u64 b = (u64)__double_as_longlong(d);
-  const u32 ex = (u32)(b >> 52) & 0x7ffu;
-  a = 0;
-  fb = 0;
-  if (ex == 0x7ffu && (b & kMan) != 0) {  // NaN, either sign
-    err |= kErrShiftArg;
-  } else if (b >> 63) {                   // negative; -0 is +0
-    if (b << 1) err |= kErrShiftArg;
-  } else if (ex >= 1023u + 31u) {         // >= 2^31 or +inf
-    err |= kErrShiftRange;
-  } else if (ex < 1023u) {                // d < 1: a = 0, f = d
-    fb = b;
-  } else {
-    const u32 E = ex - 1023u;             // d = M * 2^(E - 52), 0 <= E <= 30
-    const u64 M = (b & kMan) | (1ull << 52);
-    a = (int)(M >> (52 - E));
-    const u64 fr = M & ((1ull << (52 - E)) - 1);  // f = fr * 2^(E - 52)
-    if (fr) {
-      const int p = 63 - __clzll((long long)fr);  // leading bit of fr: f in [2^(p+E-52), 2^(p+E-51))
-      fb = ((u64)(p + (int)E - 52 + 1023) << 52) | ((fr << (52 - p)) & kMan);
-    }
-  }
-}
-
 __device__ __forceinline__ void finish_split(u32 err, int amax, Control* ctl) {
   __shared__ int s_amax;
   __shared__ u32 s_err;
@@ -117,33 +76,7 @@ __device__ __forceinline__ void finish_split(u32 err, int amax, Control* ctl) {
   }
 }
 
-// ---------------------------------------------------------------- fast path
-// Top B bits of ~floor(f * 2^32) for the fraction with bits fb: larger
-// fractions get smaller buckets.  f = M * 2^(Ef - 52) with Ef <= -1, so
-// floor(f * 2^32) = M >> (20 - Ef) < 2^32.
-__device__ __forceinline__ u32 bucket_of(u64 fb, int B) {
-  const u32 ef = (u32)(fb >> 52);
-  const u64 M = (fb & ((1ull << 52) - 1)) | (ef ? (1ull << 52) : 0ull);
-  const int Ef = ef ? (int)ef - 1023 : -1022;
-  const int sh = 20 - Ef;
-  const u32 code = sh >= 64 ? 0u : (u32)(M >> sh);
-  return (~code) >> (32 - B);
-}
-
-// Pass 1, the only read of the shifts (vertices u0 .. n-1 per launch; one
-// launch per chunk while the shifts are still arriving): split and validate
-// every shift, and
-// drop a record into the next free slot of u's bucket unless u is alone in
-// its component.  Record: x = bits of f_u; y = (a_u << 32) | u, with bit 31
-// set when the BFS does not handle u (u < 2^30).  Vertices the BFS handles are
-// also counted by their floor a_u into acnt (the start-round histogram in
-// reverse order; acnt is all zero on entry).  Each thread takes kPlaceIpt
-// vertices per step so that their loads and slot atomics overlap: two below
-// 2^24 vertices, four above (the single graphs gain from more resident warps,
-// the larger unions from more loads in flight).  A full bucket sends the host
-// to the exact path.
-constexpr u32 kPlaceWideFrom = 1u << 24;
-
+// ---------------------------------------------------------------- direct keys
 // Adds one to the count of floor value a for every lane with take set, one
 // atomic per distinct a in the warp; floors below kRBins go to the CTA's
 // shared histogram.  A floor beyond the table (a + 2 > cap) sets kErrBucketCap.
@@ -160,256 +93,119 @@ __device__ __forceinline__ void count_floor(int a, bool take, u32* sh, u32* acnt
   }
 }
 
-template <int kPlaceIpt>
-__global__ void __launch_bounds__(256) k_bplace(const double* __restrict__ delta,
-                                                const u32* __restrict__ solo,
+// floor(d), and the complement of the leading cb bits of the fraction
+// (floor(f * 2^cb), cb <= kMaxCodeBits, so larger fractions get smaller codes),
+// from the bits of d.  A bad shift gets floor 0 and an error bit (split_bits).
+__device__ __forceinline__ u64 split_code(double d, u32 cb, u32& err, int& a) {
+  constexpr u64 kMan = (1ull << 52) - 1;
+  const u64 b = (u64)__double_as_longlong(d);
+  const u32 ex = (u32)(b >> 52);  // with the sign bit
+  const u64 M = (b & kMan) | (1ull << 52);
+  u64 top = 0;  // floor(f * 2^cb)
+  a = 0;
+  if (ex - 1023u < 31u) {  // 1 <= d < 2^31: d = M * 2^(E - 52)
+    const u32 E = ex - 1023u;
+    a = (int)(M >> (52 - E));
+    top = (M << (12 + E)) >> (64 - cb);  // the 52 - E fraction bits, left-aligned
+  } else if (ex < 1023u) {  // d < 1: f = d (a subnormal's code is 0)
+    const u32 sh = 1023u + 52u - cb - ex;
+    top = sh >= 64 ? 0ull : M >> sh;
+  } else if (ex == 0x7ffu && (b & kMan)) {
+    err |= kErrShiftArg;  // NaN
+  } else if (ex >= 0x800u) {
+    if (b << 1) err |= kErrShiftArg;  // negative or NaN; -0 is +0
+  } else {
+    err |= kErrShiftRange;  // >= 2^31 or +inf
+  }
+  return ~top & ((1ull << cb) - 1);
+}
+
+// The only pass over the shifts (vertices u0 .. n-1 per launch; one launch per
+// chunk while the shifts are still arriving, u0 a multiple of kMaxBlock): every
+// vertex's direct key, the counts of the floors among the vertices the BFS
+// handles (acnt; the start-round histogram in reverse order, all zero on
+// entry), and bmax.  A warp takes kMaxBlock consecutive vertices per step, four
+// per lane with all loads first.  In a union the shifts are in the caller's
+// layout (a 32-vertex word belongs to one member) and the id is the vertex's
+// place in its member; pads get no key.  Errors: bad shifts, a floor beyond the
+// level field (kErrLevelCap) or beyond the count table.
+//
+// Bound by memory: 8 bytes read and 8 written per vertex.  Ranks by a bucket
+// sort of the fractions (16-byte records scattered by bucket, ranked in shared
+// memory, keys and full start buckets scattered again) were bound by their
+// sectors.  Keys and buckets, before and now: 256^3 grid 1236 -> 149 us, R-MAT
+// 22 145-168 -> 32-42 us, 64 copies of R-MAT 20 as a union 3700 -> 410 us (and
+// its lifts 1300 -> 200), 1000^2 grid 81 -> 32 us.
+constexpr int kDirectIpt = kMaxBlock / 32;
+
+template <bool U>
+__global__ void __launch_bounds__(256) k_direct(const double* __restrict__ delta,
                                                 const u32* __restrict__ excl, u32 u0, u32 n,
-                                                int B, u32* __restrict__ cnt,
-                                                ulonglong2* __restrict__ slots,
-                                                u32* acnt, u32 cap,
+                                                KeyFmt f, u64* __restrict__ key, u32* acnt,
+                                                u32 cap, u32* __restrict__ bmax,
                                                 const u32* __restrict__ wmem,
+                                                const u32* __restrict__ voff,
+                                                const u32* __restrict__ ooff,
                                                 const int* __restrict__ lift, Control* ctl) {
   __shared__ u32 sh[kRBins];
+  __shared__ int s_ab;
   const u32 tid = threadIdx.x, lane = tid & 31;
   for (u32 i = tid; i < kRBins; i += blockDim.x) sh[i] = 0;
+  if (tid == 0) s_ab = 0;
   __syncthreads();
   int amax = 0;
-  u32 err = 0;
-  const u32 stride = gridDim.x * blockDim.x;
-  // warp-uniform trip count: the histogram adds are warp collectives
-  for (u32 wb = u0 + blockIdx.x * blockDim.x + (tid & ~31u); wb < n; wb += stride * kPlaceIpt) {
-    double d[kPlaceIpt];
+  u32 err = 0, ab = 0;  // ab: largest handled floor of this warp's blocks, plus one
+  const u32 stride = gridDim.x * (blockDim.x / 32) * kMaxBlock;
+  for (u32 wb = u0 + (blockIdx.x * (blockDim.x / 32) + (tid >> 5)) * kMaxBlock; wb < n;
+       wb += stride) {
+    double d[kDirectIpt];
+    u32 id[kDirectIpt], ex[kDirectIpt];
+    int lf[kDirectIpt];
+    bool live[kDirectIpt];
 #pragma unroll
-    for (int k = 0; k < kPlaceIpt; ++k) {
-      const u32 u = wb + lane + (u32)k * stride;
-      d[k] = (u < n) ? __ldcs(delta + u) : 0.0;
-    }
-    u32 bkt[kPlaceIpt], pos[kPlaceIpt];
-    int fl[kPlaceIpt];
-    bool own[kPlaceIpt];
-    ulonglong2 rec[kPlaceIpt];
-#pragma unroll
-    for (int k = 0; k < kPlaceIpt; ++k) {
-      const u32 u = wb + lane + (u32)k * stride;
-      bkt[k] = 0xffffffffu;
-      fl[k] = 0;
-      own[k] = false;
-      if (u < n) {
-        u64 fb;
-        split_bits(d[k], err, fl[k], fb);
-        if (lift) fl[k] += __ldg(lift + __ldg(wmem + (u >> 5)));
-        amax = max(amax, fl[k]);
-        if (!((__ldg(solo + (u >> 5)) >> (u & 31)) & 1u)) {
-          const u32 out = (__ldg(excl + (u >> 5)) >> (u & 31)) & 1u;
-          own[k] = out == 0u;
-          bkt[k] = bucket_of(fb, B);
-          rec[k] = make_ulonglong2(fb, ((u64)(u32)fl[k] << 32) | u | (out << 31));
-        }
+    for (int k = 0; k < kDirectIpt; ++k) {
+      const u32 u = wb + (u32)k * 32 + lane;
+      live[k] = u < n;
+      ex[k] = live[k] ? __ldg(excl + (u >> 5)) : 0xffffffffu;
+      id[k] = u;
+      lf[k] = 0;
+      u32 at = u;
+      if (U && live[k]) {
+        const u32 m = __ldg(wmem + (u >> 5)), o = __ldg(ooff + m);
+        id[k] = u - __ldg(voff + m);
+        at = o + id[k];
+        live[k] = at < __ldg(ooff + m + 1);  // else a pad
+        lf[k] = __ldg(lift + m);
       }
+      d[k] = live[k] ? __ldcs(delta + at) : 0.0;
     }
+    u32 top = 0;
 #pragma unroll
-    for (int k = 0; k < kPlaceIpt; ++k) pos[k] = bkt[k] != 0xffffffffu ? atomicAdd(cnt + bkt[k], 1u) : 0u;
-#pragma unroll
-    for (int k = 0; k < kPlaceIpt; ++k) count_floor(fl[k], own[k], sh, acnt, cap, err);
-#pragma unroll
-    for (int k = 0; k < kPlaceIpt; ++k) {
-      if (bkt[k] == 0xffffffffu) continue;
-      if (pos[k] < kSlotCap) slots[(size_t)bkt[k] * kSlotCap + pos[k]] = rec[k];
-      else err |= kErrRankRetry;
+    for (int k = 0; k < kDirectIpt; ++k) {
+      int a;
+      const u64 code = split_code(d[k], f.cb, err, a);
+      a += lf[k];
+      const bool own = live[k] && !((ex[k] >> lane) & 1u);
+      if (live[k]) {
+        amax = max(amax, a);
+        if ((u32)a > f.cap) err |= kErrLevelCap;
+        key[wb + (u32)k * 32 + lane] =
+            level_key(f, f.cap - (u32)a) | (code << f.ib) | id[k];
+      }
+      if (own) top = max(top, (u32)a + 1u);
+      count_floor(a, own, sh, acnt, cap, err);
     }
+    top = __reduce_max_sync(kFull, top);
+    ab = max(ab, top);
+    if (lane == 0) bmax[wb / kMaxBlock] = top;
   }
+  if (lane == 0 && ab) atomicMax(&s_ab, (int)ab - 1);
   __syncthreads();
   for (u32 i = tid; i < kRBins; i += blockDim.x)
     if (sh[i] && (u64)i + 2 <= cap) atomicAdd(acnt + i, sh[i]);
     else if (sh[i]) err |= kErrBucketCap;
+  if (tid == 0 && s_ab) atomicMax(&ctl->Ab, s_ab);
   finish_split(err, amax, ctl);
-}
-
-// True if record o comes before record me in (f descending, id ascending).
-__device__ __forceinline__ bool rec_before(const ulonglong2 o, const ulonglong2 me) {
-  const u32 uo = (u32)o.y & 0x7fffffffu, um = (u32)me.y & 0x7fffffffu;
-  return o.x > me.x || (o.x == me.x && uo < um);
-}
-
-// Writes what rank p of record rec gives: order[p] = u and u's start key
-// ((A - a_u) << 32) | p.  Returns true if u goes into a start bucket (the BFS
-// handles u).
-__device__ __forceinline__ bool emit_key(bool valid, const ulonglong2 rec, u32 p, u32 n, int A,
-                                         u32* __restrict__ order, u64* __restrict__ key) {
-  const u32 u = (u32)rec.y & 0x7fffffffu;
-  if (!(valid && p < n && u < n)) return false;
-  const u32 R = (u32)(A - (int)(u32)(rec.y >> 32));
-  order[p] = u;
-  key[u] = ((u64)R << 32) | p;
-  return !((u32)rec.y >> 31);
-}
-
-// Places u into start bucket R (bv[pos] = u, rk[pos] = R, pos from the
-// bucket's global cursor), one atomic per distinct R in the warp.  Called by
-// the whole warp.
-__device__ __forceinline__ void place_start_warp(bool take, u32 u, u32 R, u32 n, u32* rcur,
-                                                 u32* __restrict__ bv, u32* __restrict__ rk) {
-  const u32 lane = threadIdx.x & 31;
-  const u32 act = __ballot_sync(kFull, take);
-  if (!act) return;
-  const u32 peers = __match_any_sync(kFull, take ? R : 0xffffffffu) & act;
-  const int leader = take ? __ffs(peers) - 1 : (int)lane;
-  u32 base = 0;
-  if (take && (int)lane == leader) base = atomicAdd(rcur + R, (u32)__popc(peers));
-  base = __shfl_sync(kFull, base, leader);
-  if (take) {
-    const u32 pos = base + (u32)__popc(peers & lanemask_lt());
-    if (pos < n) {
-      bv[pos] = u;
-      rk[pos] = R;
-    }
-  }
-}
-
-// Pass 2: CTAs take tiles of kTileBuckets consecutive buckets, in ticket
-// order.  The tile's records (bucket b's len = start[b + 1] - start[b] records
-// sit in slots [b * kSlotCap, b * kSlotCap + len)) are staged densely in
-// shared memory in bucket order: first every position learns its bucket and
-// the bucket's span of positions (one warp per bucket, shared memory only),
-// then one thread per position copies its record.  Every thread then ranks
-// one record against the members of its own bucket: rank = start[b] + the
-// number of members before it in (f descending, id ascending), comparing the
-// fraction bits alone unless another member has the same bits; and writes
-// order[] and the key.  The tile's vertices then go into their start buckets:
-// counted per start round in shared memory, one global reservation per round
-// and tile, then written.  A tile with more than kTileRecs records (crowded
-// fractions just short of a slot overflow) is ranked from global memory
-// instead, and with more than kSortRBins start rounds the reservations are
-// per warp.
-constexpr u32 kTileBuckets = 64;   // <= threads per CTA (one capacity check each); < 256
-constexpr u32 kTileRecs = 1280;    // < 2^16: spans are two 16-bit positions
-constexpr u32 kSortRBins = 2048;
-constexpr int kBsortPerSm = 5;     // resident CTAs per SM: 5 x 39 KB shared, <= 51 registers
-
-struct BsortSmem {
-  u64 fx[kTileRecs];         // fraction bits of the tile's records, bucket order
-  u64 fy[kTileRecs];         // (a_u << 32) | u | (not handled by the BFS) << 31
-  u32 span[kTileRecs];       // (first << 16) | end: the record's bucket as tile positions
-  u32 loc[kTileRecs];        // record's offset within its start round's share of the tile
-  u32 rc[kSortRBins];        // the tile's count per start round, then its base in the round
-  u32 st[kTileBuckets + 1];  // global first rank of every bucket of the tile, and the end
-  unsigned char bi[kTileRecs];  // record's bucket within the tile
-  u32 tile;
-};
-
-__global__ void __launch_bounds__(256, kBsortPerSm)
-    k_bsort(const u32* __restrict__ start, u32 nbkt, const ulonglong2* __restrict__ slots, u32 n,
-            u32* __restrict__ order, u64* __restrict__ key, u32* rcur, u32* __restrict__ bv,
-            u32* __restrict__ rk, u32* ticket, Control* ctl) {
-  extern __shared__ __align__(16) unsigned char bsort_raw[];
-  BsortSmem& sm = *reinterpret_cast<BsortSmem*>(bsort_raw);
-  if (failed(ctl)) return;
-  const int A = ctl->A;
-  const bool small = (u32)A < kSortRBins;
-  const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
-  if (small)
-    for (u32 i = tid; i <= (u32)A; i += blockDim.x) sm.rc[i] = 0;
-  const u32 ntiles = (nbkt + kTileBuckets - 1) / kTileBuckets;
-  for (;;) {
-    __syncthreads();  // previous tile done with sm
-    if (tid == 0) sm.tile = atomicAdd(ticket, 1u);
-    __syncthreads();
-    const u32 t = sm.tile;
-    if (t >= ntiles) break;
-    const u32 b0 = t * kTileBuckets;
-    const u32 nb = min(kTileBuckets, nbkt - b0);
-    for (u32 i = tid; i <= nb; i += blockDim.x) sm.st[i] = start[b0 + i];
-    __syncthreads();
-    // a bucket beyond kSlotCap cannot reach here (k_bplace flags it); checked anyway
-    const bool full = tid < nb && sm.st[tid + 1] - sm.st[tid] > kSlotCap;
-    const bool overfull = __syncthreads_or(full) != 0;
-    const u32 total = sm.st[nb] - sm.st[0];
-    if (!overfull && total <= kTileRecs) {
-      for (u32 i = warp; i < nb; i += nwarp) {
-        const u32 s0 = sm.st[i] - sm.st[0], e = sm.st[i + 1] - sm.st[0];
-        for (u32 q = s0 + lane; q < e; q += 32) {
-          sm.span[q] = (s0 << 16) | e;
-          sm.bi[q] = (unsigned char)i;
-        }
-      }
-      __syncthreads();
-#pragma unroll 4
-      for (u32 q = tid; q < total; q += blockDim.x) {
-        const u32 i = sm.bi[q];
-        const ulonglong2 rec = slots[(size_t)(b0 + i) * kSlotCap + (q - (sm.span[q] >> 16))];
-        sm.fx[q] = rec.x;
-        sm.fy[q] = rec.y;
-      }
-      __syncthreads();
-      for (u32 q0 = 0; q0 < total; q0 += blockDim.x) {
-        const u32 q = q0 + tid;
-        const bool valid = q < total;
-        ulonglong2 me = make_ulonglong2(0ull, 0ull);
-        u32 p = 0;
-        if (valid) {
-          me = make_ulonglong2(sm.fx[q], sm.fy[q]);
-          const u32 sp = sm.span[q], lo = sp >> 16, hi = sp & 0xffffu;
-          u32 r = 0, eq = 0;
-          for (u32 j = lo; j < hi; ++j) {
-            const u64 x = sm.fx[j];
-            r += x > me.x ? 1u : 0u;
-            eq += x == me.x ? 1u : 0u;
-          }
-          if (eq > 1) {  // another member with the same fraction: the smaller id goes first
-            const u32 um = (u32)me.y & 0x7fffffffu;
-            for (u32 j = lo; j < hi; ++j)
-              r += (sm.fx[j] == me.x && ((u32)sm.fy[j] & 0x7fffffffu) < um) ? 1u : 0u;
-          }
-          p = sm.st[0] + lo + r;
-        }
-        const bool take = emit_key(valid, me, p, n, A, order, key);
-        const u32 R = (u32)(A - (int)(u32)(me.y >> 32));
-        if (small) {
-          if (take) sm.loc[q] = atomicAdd(&sm.rc[R], 1u);
-        } else {
-          place_start_warp(take, (u32)me.y & 0x7fffffffu, R, n, rcur, bv, rk);
-        }
-      }
-      if (small) {
-        __syncthreads();
-        for (u32 i = tid; i <= (u32)A; i += blockDim.x) {
-          const u32 c = sm.rc[i];
-          sm.rc[i] = c ? atomicAdd(rcur + i, c) : 0u;  // this tile's base in round i
-        }
-        __syncthreads();
-        for (u32 q = tid; q < total; q += blockDim.x) {
-          const u64 y = sm.fy[q];
-          const u32 u = (u32)y & 0x7fffffffu;
-          if (((u32)y >> 31) || u >= n) continue;
-          const u32 R = (u32)(A - (int)(u32)(y >> 32));
-          const u32 pos = sm.rc[R] + sm.loc[q];
-          if (pos < n) {
-            bv[pos] = u;
-            rk[pos] = R;
-          }
-        }
-        __syncthreads();
-        for (u32 i = tid; i <= (u32)A; i += blockDim.x) sm.rc[i] = 0;
-      }
-    } else {
-      // one warp per bucket, records read from global memory
-      for (u32 i = warp; i < nb; i += nwarp) {
-        const u32 s0 = sm.st[i], len = sm.st[i + 1] - sm.st[i];
-        if (len > kSlotCap) continue;  // cannot happen: k_bplace flags a full bucket
-        const ulonglong2* bs = slots + (size_t)(b0 + i) * kSlotCap;
-        for (u32 i0 = 0; i0 < len; i0 += 32) {
-          const u32 q = i0 + lane;
-          const bool valid = q < len;
-          const ulonglong2 me = valid ? bs[q] : make_ulonglong2(0ull, 0ull);
-          u32 r = 0;
-          for (u32 j = 0; j < len; ++j) r += rec_before(bs[j], me) ? 1u : 0u;
-          const bool take = emit_key(valid, me, s0 + r, n, A, order, key);
-          place_start_warp(take, (u32)me.y & 0x7fffffffu, (u32)(A - (int)(u32)(me.y >> 32)), n,
-                           rcur, bv, rk);
-        }
-      }
-    }
-  }
 }
 
 // ---------------------------------------------------------------- exact path
@@ -644,8 +440,9 @@ __global__ void __launch_bounds__(256) k_rank_scatter(const u32* __restrict__ v0
 // ---------------------------------------------------------------- device scan
 // In-place exclusive scan of data[0 .. len), single pass with decoupled
 // look-back over 4096-element tiles.  len = A + 2 when len_from_A (the
-// start-round histogram), else len_host.  With rev_src (fast path), the input
-// is the floor histogram read in reverse, data[r] = rev_src[A - r] for
+// start-round histogram), else len_host.  With rev_src (direct keys), A is the
+// largest floor among the vertices the BFS handles, the input is the floor
+// histogram read in reverse, data[r] = rev_src[A - r] for
 // r = 0 .. A and 0 for r = A + 1, and rev_src is cleared on the way (all zero
 // for the next decomposition); a table of fewer than A + 2 entries (cap) sets
 // kErrBucketCap.  Optionally copies the result to copy[] and records the
@@ -666,13 +463,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_excl(u32* data, u32* copy
     // an upstream error skips the scan; the floor counts are still cleared, so
     // a decomposition queued behind this one starts from zero counts
     if (rev_src) {
-      const u32 end = (u32)min((u64)(u32)ctl->A + 1, (u64)cap);
+      const u32 end = (u32)min((u64)(u32)ctl->Ab + 1, (u64)cap);
       for (u32 r = blockIdx.x * blockDim.x + threadIdx.x; r < end; r += gridDim.x * blockDim.x)
         rev_src[r] = 0;
     }
     return;
   }
   const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (rev_src && blockIdx.x == 0 && tid < 3) ctl->minlow[tid] = ~0ull;  // for the round loop
   if (tid == 0) {
     s_tile = atomicAdd(tile_ctr, 1u);
     s_bad = 0;
@@ -680,7 +478,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_excl(u32* data, u32* copy
   }
   __syncthreads();
   const u32 tile = s_tile;
-  const int A = ctl->A;
+  const int A = rev_src ? ctl->Ab : ctl->A;
   if (rev_src && (u64)A + 2 > cap) {
     if (tile == 0 && tid == 0) atomicOr(&ctl->err, kErrBucketCap);
     for (u32 r = tile * kScanTile + tid; r < min(cap, (tile + 1) * kScanTile); r += blockDim.x)
@@ -839,14 +637,12 @@ __global__ void __launch_bounds__(256) k_keys(const int* __restrict__ a,
       if (sh[i]) atomicAdd(rcnt + i, sh[i]);
 }
 
-// Start-bucket scatter: bv[pos] = u, rk[pos] = R_u for every vertex the BFS
-// handles.  With few rounds, each CTA counts its chunk in shared memory and
+// Start-bucket scatter: bv[pos] = u for every vertex the BFS handles.  With few rounds, each CTA counts its chunk in shared memory and
 // reserves its range of every group with one atomic; otherwise one atomic per
 // warp and round.
 __global__ void __launch_bounds__(256) k_rscatter(const int* __restrict__ a,
                                                   const u32* __restrict__ excl, Control* ctl,
-                                                  u32 n, u32* cursor, u32* __restrict__ bv,
-                                                  u32* __restrict__ rk) {
+                                                  u32 n, u32* cursor, u32* __restrict__ bv) {
   __shared__ u32 s_cnt[kRBins];
   if (failed(ctl)) return;
   const int A = ctl->A;
@@ -895,10 +691,7 @@ __global__ void __launch_bounds__(256) k_rscatter(const int* __restrict__ a,
       const u32 u = c0 + (u32)k * blockDim.x + tid;
       if (R[k] != 0xffffffffu) {
         const u32 pos = (small ? s_cnt[R[k]] : 0u) + local[k];
-        if (pos < n) {
-          bv[pos] = u;
-          rk[pos] = R[k];
-        }
+        if (pos < n) bv[pos] = u;
       }
     }
     if (small) __syncthreads();
@@ -937,29 +730,20 @@ u32 grid_stride_blocks(u32 n, int num_sms) {
   return (u32)max(1ll, min((long long)(n + 255) / 256, (long long)num_sms * 8));
 }
 
-void allow_bsort_smem() {
-  static bool done[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
-  if (!done[dev]) {
-    cudaFuncSetAttribute(k_bsort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(BsortSmem));
-    done[dev] = true;
-  }
-}
-
-// CTAs of a k_bplace instance resident on one SM: its grid is one full wave.
-int bplace_blocks_per_sm(bool wide) {
+// CTAs of a k_direct instance resident on one SM: its grid is one full wave.
+int direct_blocks_per_sm(bool u) {
   static int per_sm[2][64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 4;
-  int& b = per_sm[wide ? 1 : 0][dev];
+  int& b = per_sm[u ? 1 : 0][dev];
   if (b <= 0) {
-    const void* fn = wide ? (const void*)k_bplace<4> : (const void*)k_bplace<2>;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, 256, 0) != cudaSuccess || b < 1) {
+    const void* fn = u ? (const void*)k_direct<true> : (const void*)k_direct<false>;
+    int got = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, fn, 256, 0) != cudaSuccess || got < 1) {
       cudaGetLastError();
-      b = 4;
+      got = 4;
     }
+    b = got;
   }
   return b;
 }
@@ -977,20 +761,8 @@ void allow_sort_smem() {
 
 }  // namespace
 
-u32 fraction_bucket_bits(u32 n) {
-  u32 b = 1;
-  while (b < 26 && (1ull << (b + 4)) < n) ++b;  // about 16 vertices per bucket
-  return b;
-}
-
-size_t rank_status_words(u32 n, u32 bptr_cap) {
-  const u32 nbkt = 1u << fraction_bucket_bits(n);
-  return std::max<size_t>((nbkt + 1 + kScanTile - 1) / kScanTile,
-                          ((size_t)bptr_cap + kScanTile - 1) / kScanTile);
-}
-
-size_t fraction_slot_bytes(u32 n) {
-  return ((size_t)1 << fraction_bucket_bits(n)) * kSlotCap * sizeof(ulonglong2);
+size_t scan_status_words(u32 bptr_cap) {
+  return ((size_t)bptr_cap + kScanTile - 1) / kScanTile;
 }
 
 int launch_rank_and_buckets(const RankBufs& r, bool exact64, cudaStream_t s,
@@ -1002,50 +774,37 @@ int launch_rank_and_buckets(const RankBufs& r, bool exact64, cudaStream_t s,
   const u32 rtiles = (r.bptr_cap + kScanTile - 1) / kScanTile;
   u32* rcnt = reinterpret_cast<u32*>(r.bptr);
   if (!exact64) {
-    // split + records + floor counts; bucket starts; round counts (the scan
-    // below makes them bptr); ranks, keys and the start buckets in one pass
-    const u32 B = fraction_bucket_bits(n), nbkt = 1u << B;
-    u32* cnt = reinterpret_cast<u32*>(r.k1);  // [nbkt + 1] counts, then first ranks
-    ulonglong2* slots = reinterpret_cast<ulonglong2*>(r.slots);
+    // keys and floor counts, then the start buckets' offsets
     if (r.acnt_dirty) cudaMemsetAsync(r.acnt, 0, (size_t)r.bptr_cap * 4, s);
-    cudaMemsetAsync(cnt, 0, (size_t)(nbkt + 1) * 4, s);
     const int nchunk = chunks ? chunks->n : 0;
+    const bool u = r.wmem != nullptr;
     u32 lo = 0;
     for (int c = 0; c <= nchunk; ++c) {
       // chunk c is vertices [lo, hi), complete once its event has fired
       const u32 hi = c < nchunk ? std::min(chunks->end[c], n) : n;
       if (c < nchunk) cudaStreamWaitEvent(s, chunks->ev[c], 0);
       if (hi <= lo) continue;
-      const u32 m = hi - lo;
-      const bool wide = n >= kPlaceWideFrom;
-      const int ipt = wide ? 4 : 2;
-      const u32 place_grid =
-          (u32)min((long long)(m + 256 * ipt - 1) / (256 * ipt),
-                   (long long)r.num_sms * bplace_blocks_per_sm(wide));
-      if (wide)
-        k_bplace<4><<<max(place_grid, 1u), 256, 0, s>>>(r.shift, r.solo, r.excl, lo, hi, (int)B,
-                                                        cnt, slots, r.acnt, r.bptr_cap, r.wmem,
-                                                        r.lift, ctl);
+      const u32 per_cta = 8 * kMaxBlock;
+      const u32 grid = (u32)min(((long long)(hi - lo) + per_cta - 1) / per_cta,
+                                (long long)r.num_sms * direct_blocks_per_sm(u));
+      if (u)
+        k_direct<true><<<grid, 256, 0, s>>>(r.shift, r.excl, lo, hi, r.f, r.key, r.acnt,
+                                            r.bptr_cap, r.bmax, r.wmem, r.voff, r.ooff, r.lift,
+                                            ctl);
       else
-        k_bplace<2><<<max(place_grid, 1u), 256, 0, s>>>(r.shift, r.solo, r.excl, lo, hi, (int)B,
-                                                        cnt, slots, r.acnt, r.bptr_cap, r.wmem,
-                                                        r.lift, ctl);
+        k_direct<false><<<grid, 256, 0, s>>>(r.shift, r.excl, lo, hi, r.f, r.key, r.acnt,
+                                             r.bptr_cap, r.bmax, nullptr, nullptr, nullptr,
+                                             nullptr, ctl);
       ++launches;
       lo = hi;
     }
-    k_scan_excl<<<(nbkt + 1 + kScanTile - 1) / kScanTile, kScanThreads, 0, s>>>(
-        cnt, nullptr, nbkt + 1, 0, r.status, ++(*r.epoch), &ctl->tile_ctr[0], nullptr, nullptr, 0,
-        ctl, r.lookback_limit, r.stall_lookback);
-    k_scan_excl<<<rtiles, kScanThreads, 0, s>>>(rcnt, r.rcur, 0, 1, r.status, ++(*r.epoch),
-                                                 &ctl->tile_ctr[1], nullptr, r.acnt, r.bptr_cap,
-                                                 ctl, r.lookback_limit, r.stall_lookback);
-    allow_bsort_smem();
-    const u32 ntiles = (nbkt + kTileBuckets - 1) / kTileBuckets;
-    const u32 sort_grid = (u32)min((long long)ntiles, (long long)r.num_sms * kBsortPerSm);
-    k_bsort<<<sort_grid, 256, sizeof(BsortSmem), s>>>(
-        cnt, nbkt, slots, n, r.order, r.key, r.rcur, r.v0, reinterpret_cast<u32*>(r.k0),
-        &ctl->tile_ctr[kFracDigits + kRoundDigits - 1], ctl);
-    return launches + 3;
+    // no floor exceeds f.cap, so neither do the rounds
+    const u32 tiles = (u32)((std::min<u64>(r.bptr_cap, (u64)r.f.cap + 2) + kScanTile - 1) /
+                            kScanTile);
+    k_scan_excl<<<tiles, kScanThreads, 0, s>>>(rcnt, r.rcur, 0, 1, r.status, ++(*r.epoch),
+                                               &ctl->tile_ctr[1], nullptr, r.acnt, r.bptr_cap,
+                                               ctl, r.lookback_limit, r.stall_lookback);
+    return launches + 1;
   }
   // exact path: stable LSD radix sort of all fractions, then keys and the
   // start-round counting sort (groups in any order inside)
@@ -1073,7 +832,7 @@ int launch_rank_and_buckets(const RankBufs& r, bool exact64, cudaStream_t s,
                                                r.lookback_limit, r.stall_lookback);
   k_rscatter<<<(u32)min((long long)(n + 256 * kRChunk - 1) / (256 * kRChunk),
                         (long long)r.num_sms * 8),
-               256, 0, s>>>(r.a, r.excl, ctl, n, r.rcur, r.v0, reinterpret_cast<u32*>(r.k0));
+               256, 0, s>>>(r.a, r.excl, ctl, n, r.rcur, r.v0);
   return launches + 5;
 }
 
@@ -1104,7 +863,7 @@ int launch_ranked_and_buckets(const RankBufs& r, const int* levels, const int* p
                                                r.lookback_limit, r.stall_lookback);
   k_rscatter<<<(u32)min((long long)(n + 256 * kRChunk - 1) / (256 * kRChunk),
                         (long long)r.num_sms * 8),
-               256, 0, s>>>(r.a, r.excl, ctl, n, r.rcur, r.v0, reinterpret_cast<u32*>(r.k0));
+               256, 0, s>>>(r.a, r.excl, ctl, n, r.rcur, r.v0);
   return 5;
 }
 

@@ -159,23 +159,18 @@ __device__ __forceinline__ int floor_of(double d) {
   return (int)(M >> (52 - (ex - 1023u)));
 }
 
-// Concatenated input shifts (caller layout) to the union layout (pads get 0),
-// and into amax[s] (zero on entry) the largest floor among member s's vertices
-// that the round loop handles (excl bit clear): isolated vertices and small
-// components never enter the rounds, so they must not set the alignment.  A
-// warp's 32 consecutive union vertices belong to one member (members start on
-// 32-vertex boundaries) and share one excl word, so each warp step ends in
-// one atomicMax.
+// Into amax[s] (zero on entry) the largest floor among member s's vertices that
+// the round loop handles (excl bit clear): isolated vertices and small
+// components never enter the rounds, so they must not set the alignment.
 // Members are padded to multiples of 32 vertices, so every 32-vertex chunk
-// of the union belongs to one member.  A warp takes kSpreadIpt consecutive
-// chunks at a time, finds the member of the first once and walks forward for
-// the others, and issues all their loads before any store.
-constexpr int kSpreadIpt = 4;
+// of the union belongs to one member and has one excl word.  A warp takes
+// kSpreadIpt consecutive chunks at a time, all their loads first, and sends one
+// atomicMax per member it saw.
+constexpr int kSpreadIpt = 8;
 
-__global__ void __launch_bounds__(256) k_union_spread(const double* __restrict__ in,
-                                                      UnionOffsets off, u32 k,
-                                                      const u32* __restrict__ excl,
-                                                      double* __restrict__ out, int* amax) {
+__global__ void __launch_bounds__(256) k_union_amax(const double* __restrict__ in,
+                                                    UnionOffsets off, u32 k,
+                                                    const u32* __restrict__ excl, int* amax) {
   const u32 N = off.v[k];
   const u32 lane = threadIdx.x & 31;
   const u32 span = 32u * kSpreadIpt;
@@ -193,25 +188,45 @@ __global__ void __launch_bounds__(256) k_union_spread(const double* __restrict__
       sm[q] = m;
       const u32 v = wb + lane - off.v[m];
       const u32 n = off.o[m + 1] - off.o[m];
-      d[q] = (wb < N && v < n) ? __ldcs(in + off.o[m] + v) : 0.0;
+      d[q] = (wb < N && v < n && !((__ldg(excl + (wb >> 5)) >> lane) & 1u))
+                 ? __ldcg(in + off.o[m] + v) : 0.0;
     }
+    u32 best = 0;
 #pragma unroll
     for (int q = 0; q < kSpreadIpt; ++q) {
-      const u32 wb = wb0 + (u32)q * 32;
-      if (wb >= N) break;  // warp-uniform
-      out[wb + lane] = d[q];
-      int a = ((__ldg(excl + (wb >> 5)) >> lane) & 1u) ? 0 : floor_of(d[q]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
-      if (lane == 0 && a > 0) atomicMax(amax + sm[q], a);
+      best = max(best, (u32)floor_of(d[q]));
+      if (q + 1 == kSpreadIpt || sm[q + 1] != sm[q]) {  // warp-uniform
+        best = __reduce_max_sync(0xffffffffu, best);
+        if (lane == 0 && best > 0) atomicMax(amax + sm[q], (int)best);
+        best = 0;
+      }
     }
+  }
+}
+
+// Caller-layout shifts to the union layout (pads get 0), for the ranked keys.
+__global__ void __launch_bounds__(256) k_union_spread(const double* __restrict__ in,
+                                                      UnionOffsets off, u32 k,
+                                                      double* __restrict__ out) {
+  const u32 N = off.v[k];
+  for (u32 u = blockIdx.x * blockDim.x + threadIdx.x; u < N; u += gridDim.x * blockDim.x) {
+    const u32 m = member_of(off.v, k, u);
+    const u32 v = u - off.v[m];
+    out[u] = v < off.o[m + 1] - off.o[m] ? in[off.o[m] + v] : 0.0;
   }
 }
 
 // lift[s] = max_t amax[t] - amax[s]: every member's largest shift then starts
 // the round loop at round 0.  One CTA.
+// The round loop's per-member tables (three slots each) start as it expects them.
 __global__ void __launch_bounds__(1024) k_union_lift(const int* __restrict__ amax, u32 k,
-                                                     int* __restrict__ lift) {
+                                                     int* __restrict__ lift,
+                                                     u64* __restrict__ mlow,
+                                                     u64* __restrict__ mpivot) {
+  for (u32 s = threadIdx.x; s < 3 * k; s += blockDim.x) {
+    mlow[s] = ~0ull;
+    mpivot[s] = 0;
+  }
   __shared__ int wmax[32];
   __shared__ int gmax;
   int m = 0;
@@ -230,23 +245,25 @@ __global__ void __launch_bounds__(1024) k_union_lift(const int* __restrict__ ama
 }
 
 // Algorithm 1 step 4 in the caller's layout: output i is vertex v of member
-// s, union vertex u = voff_s + v.  Its settled key names the center
-// order[rank] (a union id of the same member); the member-local center id is
-// that minus voff_s, and the hop distance is the key's level minus the
-// center's own level.
+// s, union vertex u = voff_s + v.  Its settled key names the center, by its
+// member-local id or as order[rank] (a union id of the same member), and the
+// hop distance is the key's level minus the center's own level.
 // A warp takes 32 x kUFinIpt consecutive caller-layout entries at a time,
 // finds the member of the first once and walks forward from it per entry;
 // the loads of a lane's entries go out level by level (own keys, centers,
 // centers' keys), so that their dependent gathers overlap.
 constexpr int kUFinIpt = 4;
 
-__global__ void __launch_bounds__(256) k_union_finalize(const u64* __restrict__ key,
-                                                        const u32* __restrict__ order,
+template <bool kDirect>
+__global__ void __launch_bounds__(256) k_union_finalize(BfsArgs a, const u32* __restrict__ order,
                                                         const u32* __restrict__ solo,
                                                         UnionOffsets off, u32 k,
                                                         int* __restrict__ center,
-                                                        int* __restrict__ dist, const u32* err) {
-  if (*(volatile const u32*)err != 0u) return;
+                                                        int* __restrict__ dist) {
+  if (*(volatile const u32*)&a.ctl->err != 0u) return;
+  const u64* __restrict__ key = a.key;
+  const KeyFmt f = a.f;
+  if (kDirect && blockIdx.x == 0) tie_check(a.shift, a.wmem, a.ooff, a.ctl, threadIdx.x);
   const u32 total = off.o[k], N = off.v[k];
   const u32 lane = threadIdx.x & 31;
   const u32 span = 32u * kUFinIpt;
@@ -254,7 +271,7 @@ __global__ void __launch_bounds__(256) k_union_finalize(const u64* __restrict__ 
   for (u32 wbase = (blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5)) * span; wbase < total;
        wbase += nwarps * span) {
     const u32 s0 = member_of(off.o, k, wbase);
-    u32 idx[kUFinIpt], sm[kUFinIpt], u[kUFinIpt], c[kUFinIpt];
+    u32 idx[kUFinIpt], vb[kUFinIpt], u[kUFinIpt], c[kUFinIpt];
     bool live[kUFinIpt], alone[kUFinIpt];
     u64 kv[kUFinIpt], kc[kUFinIpt];
 #pragma unroll
@@ -264,22 +281,25 @@ __global__ void __launch_bounds__(256) k_union_finalize(const u64* __restrict__ 
       u32 m = s0;
       if (live[q])
         while (__ldg(off.o + m + 1) <= idx[q]) ++m;
-      sm[q] = m;
-      u[q] = live[q] ? off.v[m] + (idx[q] - off.o[m]) : 0u;
-      alone[q] = live[q] && ((__ldg(solo + (u[q] >> 5)) >> (u[q] & 31)) & 1u);
+      vb[q] = off.v[m];
+      u[q] = live[q] ? vb[q] + (idx[q] - off.o[m]) : 0u;
+      alone[q] = !kDirect && live[q] && ((__ldg(solo + (u[q] >> 5)) >> (u[q] & 31)) & 1u);
       kv[q] = (live[q] && !alone[q]) ? key[u[q]] : 0ull;
     }
 #pragma unroll
-    for (int q = 0; q < kUFinIpt; ++q)
-      c[q] = (live[q] && !alone[q]) ? order[min((u32)kv[q], N - 1)] : u[q];
+    for (int q = 0; q < kUFinIpt; ++q) {
+      c[q] = u[q];
+      if (live[q] && !alone[q])
+        c[q] = kDirect ? min(vb[q] + key_id(f, kv[q]), N - 1) : order[min((u32)kv[q], N - 1)];
+    }
 #pragma unroll
     for (int q = 0; q < kUFinIpt; ++q)
       kc[q] = (live[q] && !alone[q]) ? key[c[q]] : kv[q];
 #pragma unroll
     for (int q = 0; q < kUFinIpt; ++q)
       if (live[q]) {
-        center[idx[q]] = (int)(c[q] - off.v[sm[q]]);
-        dist[idx[q]] = alone[q] ? 0 : (int)((u32)(kv[q] >> 32) - (u32)(kc[q] >> 32));
+        center[idx[q]] = (int)(c[q] - vb[q]);
+        dist[idx[q]] = alone[q] ? 0 : (int)(key_level(f, kv[q]) - key_level(f, kc[q]));
       }
   }
 }
@@ -299,21 +319,29 @@ int launch_union_concat(const UnionMember* mem, const UnionOffsets& off, u32 k,
   return 2;
 }
 
-int launch_union_spread(const double* in, const UnionOffsets& off, u32 k, u32 N,
-                        const u32* excl, double* out, int* amax, int* lift, int num_sms,
-                        cudaStream_t s) {
+int launch_union_lift(const double* in, const UnionOffsets& off, u32 k, u32 N, const u32* excl,
+                      int* amax, int* lift, u64* mlow, u64* mpivot, int num_sms, cudaStream_t s) {
   cudaMemsetAsync(amax, 0, (size_t)k * sizeof(int), s);
-  k_union_spread<<<blocks_for((N + kSpreadIpt - 1) / kSpreadIpt, num_sms), 256, 0, s>>>(
-      in, off, k, excl, out, amax);
-  k_union_lift<<<1, 1024, 0, s>>>(amax, k, lift);
+  k_union_amax<<<blocks_for((N + kSpreadIpt - 1) / kSpreadIpt, num_sms), 256, 0, s>>>(in, off, k,
+                                                                                    excl, amax);
+  k_union_lift<<<1, 1024, 0, s>>>(amax, k, lift, mlow, mpivot);
   return 2;
 }
 
-int launch_union_finalize(const u64* key, const u32* order, const u32* solo,
+int launch_union_spread(const double* in, const UnionOffsets& off, u32 k, u32 N, double* out,
+                        int num_sms, cudaStream_t s) {
+  k_union_spread<<<blocks_for(N, num_sms), 256, 0, s>>>(in, off, k, out);
+  return 1;
+}
+
+int launch_union_finalize(const BfsArgs& a, const u32* order, const u32* solo,
                           const UnionOffsets& off, u32 k, u32 total, int* center, int* dist,
-                          const u32* err, int num_sms, cudaStream_t s) {
-  k_union_finalize<<<blocks_for((total + kUFinIpt - 1) / kUFinIpt, num_sms), 256, 0, s>>>(
-      key, order, solo, off, k, center, dist, err);
+                          int num_sms, cudaStream_t s) {
+  const u32 g = blocks_for((total + kUFinIpt - 1) / kUFinIpt, num_sms);
+  if (a.f.cap)
+    k_union_finalize<true><<<g, 256, 0, s>>>(a, order, solo, off, k, center, dist);
+  else
+    k_union_finalize<false><<<g, 256, 0, s>>>(a, order, solo, off, k, center, dist);
   return 1;
 }
 

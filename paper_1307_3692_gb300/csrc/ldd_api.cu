@@ -2,8 +2,8 @@
 // checks, host/device pointer handling, scratch memory and the order of the
 // kernels of one decomposition (Miller, Peng, Xu 2013, Algorithm 1):
 //   step 1 (shifts)      : given by the caller, copied to the device if needed
-//   step 2 (delta_max)   : the split of k_bplace / k_split64   (k_rank.cu)
-//   Section 4 tie-break  : fraction rank, keys, start buckets  (k_rank.cu)
+//   step 2 (delta_max)   : the split of k_direct / k_split64   (k_rank.cu)
+//   Section 4 tie-break  : keys and start buckets              (k_rank.cu)
 //   step 3 (BFS)         : persistent cooperative k_bfs        (k_bfs.cu)
 //                          and k_small_comp for components of <= 32 vertices
 //   step 4 (assignment)  : k_finalize                          (k_graph.cu)
@@ -35,7 +35,7 @@ static_assert(offsetof(Control, bar) == kCtlBfsStateOffset, "control layout");
 static_assert(offsetof(Control, mask_f) == kCtlBfsStateOffset + kCtlBfsStateBytes,
               "control layout");
 static_assert(offsetof(Control, cut) + sizeof(u64) == kCtlHeaderBytes, "control layout");
-static_assert(offsetof(Control, minrank) == kCtlMinrankOffset, "control layout");
+static_assert(offsetof(Control, minlow) == kCtlMinlowOffset, "control layout");
 
 namespace ldd {
 
@@ -137,7 +137,7 @@ int free_graph_memory(ldd_graph* g) {
     cudaFree(g->uni->d_cut);
     cudaFree(g->uni->d_wmem);
     cudaFree(g->uni->d_amax);
-    cudaFree(g->uni->d_mrank);
+    cudaFree(g->uni->d_mlow);
     cudaFree(g->uni->d_mpivot);
     delete g->uni;
     g->uni = nullptr;
@@ -189,7 +189,7 @@ int alloc_scratch(ldd_graph* g) {
       {(void**)&g->d_qoff[2], 4 * n},     {(void**)&g->d_cf[2], 4 * ncf},
       {(void**)&g->d_cf[0], 4 * ncf},     {(void**)&g->d_cf[1], 4 * ncf},
       {(void**)&g->d_ulist[0], 4 * n},    {(void**)&g->d_ulist[1], 4 * n},
-      {(void**)&g->d_slots, n ? fraction_slot_bytes((u32)n) : 0},
+      {(void**)&g->d_bmax, 4 * (n / kMaxBlock + 1)},
       {(void**)&g->d_center, 4 * n},      {(void**)&g->d_dist, 4 * n},
       {(void**)&g->d_ctl, sizeof(Control)},
   };
@@ -385,14 +385,19 @@ float elapsed(ldd_graph* g, int a, int b) {
   return ms;
 }
 
-BfsArgs bfs_args(ldd_graph* g) {
+BfsArgs bfs_args(ldd_graph* g, KeyFmt f, const double* shift) {
   BfsArgs a;
   a.row_ptr = g->d_row;
   a.col = g->d_col;
   a.key = g->d_key;
   a.bptr = g->d_bptr;
-  a.rk[0] = a.rk[1] = reinterpret_cast<const u32*>(g->d_k[0]);  // start rounds, 32-bit
-  a.rv[0] = a.rv[1] = g->d_v[0];                                 // start-bucket vertices
+  a.rcur = g->d_rcur;
+  a.rv = g->d_v[0];
+  a.bmax = g->d_bmax;
+  a.f = f;
+  a.shift = shift;
+  a.voff = g->uni ? g->uni->off.v : nullptr;
+  a.ooff = g->uni ? g->uni->off.o : nullptr;
   for (int b = 0; b < 3; ++b) {
     a.qv[b] = g->d_qv[b];
     a.qrow[b] = g->d_qrow[b];
@@ -409,34 +414,39 @@ BfsArgs bfs_args(ldd_graph* g) {
   a.nnz_active = g->nnz_active;
   a.spin_limit = g->spin_limit;
   a.bar_phantom = g->stall_barrier ? 1u : 0u;
-  a.pull_alpha = g->pull_alpha;
+  a.pull_alpha = g->low_pull() ? 0 : g->pull_alpha;
   a.pull_beta = g->pull_beta;
   a.pull_gamma = g->pull_gamma;
   a.probe_min_arcs = g->probe_min_arcs;
-  a.low_degree = (g->low_degree_rounds && g->max_degree <= (u32)kLdMaxDegree) ? 1u : 0u;
+  a.low_degree = g->low_degree() ? 1u : 0u;
   a.window_levels = g->window_levels;
   a.window_max_q = g->window_max_q;
   a.window_queue = g->window_queue;
   a.span = g->bfs_span;
   a.wmem = g->uni ? g->uni->d_wmem : nullptr;
-  a.mrank = g->uni ? g->uni->d_mrank : nullptr;
+  a.mlow = g->uni ? g->uni->d_mlow : nullptr;
   a.mpivot = g->uni ? g->uni->d_mpivot : nullptr;
   a.kmem = g->uni ? g->uni->k : 0;
   return a;
 }
 
-// Small components, BFS and finalize into (center, dist) device buffers.
-// Returns launches or < 0.
-int run_bfs_finalize(ldd_graph* g, int* center, int* dist, int* status) {
+// Small components, BFS and finalize into (center, dist) device buffers, with
+// keys of layout f (direct: of these shifts).  Returns launches or < 0.
+int run_bfs_finalize(ldd_graph* g, KeyFmt f, const double* shift, int* center, int* dist,
+                     int* status) {
   int launches = 0;
   cudaStream_t s = g->stream;
-  launches += launch_small_comp(g->sc, g->d_key, &g->d_ctl->err, g->num_sms, s);
+  const BfsArgs args = bfs_args(g, f, shift);
+  launches += launch_small_comp(g->sc, args, g->num_sms, s);
   if (g->n_active > 0) {
-    cudaError_t e = cudaMemsetAsync((char*)g->d_ctl + kCtlMinrankOffset, 0xff, 3 * sizeof(u32), s);
-    if (e == cudaSuccess && g->uni)
-      e = cudaMemsetAsync(g->uni->d_mrank, 0xff, 3 * (size_t)g->uni->k * sizeof(u32), s);
-    if (e == cudaSuccess && g->uni)
-      e = cudaMemsetAsync(g->uni->d_mpivot, 0, 3 * (size_t)g->uni->k * sizeof(u64), s);
+    cudaError_t e = cudaSuccess;
+    if (!f.cap) {  // direct keys: set by the scan and the lift
+      e = cudaMemsetAsync((char*)g->d_ctl + kCtlMinlowOffset, 0xff, 3 * sizeof(u64), s);
+      if (e == cudaSuccess && g->uni)
+        e = cudaMemsetAsync(g->uni->d_mlow, 0xff, 3 * (size_t)g->uni->k * sizeof(u64), s);
+      if (e == cudaSuccess && g->uni)
+        e = cudaMemsetAsync(g->uni->d_mpivot, 0, 3 * (size_t)g->uni->k * sizeof(u64), s);
+    }
     if (e != cudaSuccess) {
       *status = fail(LDD_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
       return -1;
@@ -450,7 +460,7 @@ int run_bfs_finalize(ldd_graph* g, int* center, int* dist, int* status) {
         return -1;
       }
     }
-    if (launch_bfs(bfs_args(g), g->bfs_grid, g->bfs_per_sm, s, &e) < 0) {
+    if (launch_bfs(args, g->bfs_grid, g->bfs_per_sm, s, &e) < 0) {
       *status = fail(LDD_ERR_CUDA, "cooperative launch of the BFS kernel (%d x %d) failed: %s",
                      g->bfs_grid, kBfsThreads, cudaGetErrorString(e));
       return -1;
@@ -466,11 +476,10 @@ int run_bfs_finalize(ldd_graph* g, int* center, int* dist, int* status) {
   }
   record(g, 3);
   if (g->uni)  // caller layout, member-local ids
-    launches += launch_union_finalize(g->d_key, g->d_order, g->d_solo, g->uni->off, g->uni->k,
-                                      g->uni->total, center, dist, &g->d_ctl->err, g->num_sms, s);
+    launches += launch_union_finalize(args, g->d_order, g->d_solo, g->uni->off, g->uni->k,
+                                      g->uni->total, center, dist, g->num_sms, s);
   else
-    launches += launch_finalize(g->d_key, g->d_order, g->d_solo, (u32)g->n, center, dist,
-                                &g->d_ctl->err, g->num_sms, s);
+    launches += launch_finalize(args, g->d_order, g->d_solo, center, dist, g->num_sms, s);
   return launches;
 }
 
@@ -496,15 +505,20 @@ int finish_setup(ldd_graph* g) {
   if (bfs_grid_size(g->num_sms, &max_per_sm) <= 0)
     return fail(LDD_ERR_CUDA, "BFS kernel occupancy query failed");
   // one CTA per SM for a single graph (thin frontiers, cheapest barrier), two
-  // for a union (its wide bottom-up rounds of many members want the warps);
-  // ldd_autotune and ldd_set_tuning choose per workload
+  // for a union (its wide bottom-up rounds of many members want the warps), but
+  // one if it runs low-degree rounds (64 random geometric graphs 5.55 -> 5.09
+  // ms); ldd_autotune and ldd_set_tuning choose per workload
   g->bfs_per_sm = std::min(max_per_sm, g->uni ? 2 : 1);
   const u32 per_sm = env_u32("LDD_BFS_BLOCKS_PER_SM", 0);
-  if (per_sm > 0 && (int)per_sm <= max_per_sm) g->bfs_per_sm = (int)per_sm;
+  if (per_sm > 0 && (int)per_sm <= max_per_sm) {
+    g->bfs_per_sm = (int)per_sm;
+    g->per_sm_set = true;
+  }
   g->bfs_grid = g->bfs_per_sm * g->num_sms;
   g->spin_limit = env_u32("LDD_SPIN_LIMIT", kDefaultBarrierPolls);
   g->lookback_limit = kDefaultLookbackPolls;
   g->pull_alpha = env_u32("LDD_PULL_ALPHA", 14);
+  g->pull_set = getenv("LDD_PULL_ALPHA") != nullptr;
   g->pull_beta = env_u32("LDD_PULL_BETA", 24);
   g->pull_gamma = env_u32("LDD_PULL_GAMMA", 8);
   g->probe_min_arcs = env_u32("LDD_PROBE_MIN_ARCS", 1u << 16);
@@ -522,6 +536,39 @@ int finish_setup(ldd_graph* g) {
   return LDD_OK;
 }
 
+int bits_of(u64 x) {  // bits of x's binary form
+  int b = 0;
+  for (; x; x >>= 1) ++b;
+  return b;
+}
+
+// The direct key layout for floors up to `floors` (cap 0: too few bits would be
+// left for the code, the ranked layout is needed).
+KeyFmt direct_fmt(const ldd_graph* g, u64 floors) {
+  KeyFmt f;
+  const u32 ids = g->uni ? g->uni->max_n : (u32)g->n;
+  const int ib = std::max(bits_of(ids > 0 ? ids - 1 : 0), 1);
+  const int lb = bits_of(floors + 1);  // floors + 2 <= 2^lb
+  int cb = 64 - ib - lb;
+  if (lb > 30 || cb < (int)kMinCodeBits) return f;
+  cb = std::min(cb, (int)kMaxCodeBits);
+  f.ib = (u32)ib;
+  f.cb = (u32)cb;
+  f.s2 = (u32)(ib + cb - 32);
+  f.cap = (1u << (64 - ib - cb)) - 2u;
+  return f;
+}
+
+// The largest floor to expect of shifts drawn with Exp(beta): -ln(U) / beta with
+// a 53-bit U is below 36.8 / beta.  Only a hint for the key layout: larger floors
+// make the call widen the level field and run again.  In a union a vertex that
+// the round loop does not handle may be lifted beyond it.
+u64 floors_for(const ldd_graph* g, double beta) {
+  if (!(beta > 0.0)) return 65534;
+  const double x = std::min(36.8 / beta + 2.0, 1073741824.0);
+  return (u64)x * (g->uni ? 2 : 1);
+}
+
 struct Header {  // the control block up to and including the BFS runtime state
   u32 err;
   int A;
@@ -532,8 +579,9 @@ struct Header {  // the control block up to and including the BFS runtime state
   u64 cut;
   u64 bar;
   u64 qctr[3];
-  u32 minrank[3];
+  u64 minlow[3];
   u32 pull_rounds;
+  u32 pad_p;
   u64 push_arcs;
   u64 pull_arcs;
   u64 pull_verts;
@@ -544,9 +592,10 @@ struct Header {  // the control block up to and including the BFS runtime state
 };
 static_assert(sizeof(Header) == kCtlHeaderBytes + kCtlBfsStateBytes, "header layout");
 
-RankBufs rank_bufs(ldd_graph* g, const double* d_shift) {
+RankBufs rank_bufs(ldd_graph* g, const double* d_shift, KeyFmt f) {
   RankBufs rb;
   rb.shift = d_shift;
+  rb.f = f;
   rb.n = (u32)g->n;
   rb.num_sms = g->num_sms;
   rb.a = g->d_a;
@@ -554,14 +603,15 @@ RankBufs rank_bufs(ldd_graph* g, const double* d_shift) {
   rb.k1 = g->d_k[1];
   rb.v0 = g->d_v[0];
   rb.v1 = g->d_v[1];
-  rb.slots = g->d_slots;
+  rb.bmax = g->d_bmax;
   rb.status = g->d_status;
   rb.epoch = &g->epoch;
   rb.order = g->d_order;
   rb.key = g->d_key;
   rb.excl = g->d_excl;
-  rb.solo = g->d_solo;
   rb.wmem = g->uni ? g->uni->d_wmem : nullptr;
+  rb.voff = g->uni ? g->uni->off.v : nullptr;
+  rb.ooff = g->uni ? g->uni->off.o : nullptr;
   rb.lift = g->uni ? g->uni->d_amax + g->uni->k : nullptr;
   rb.ctl = g->d_ctl;
   rb.lookback_limit = g->lookback_limit;
@@ -607,37 +657,47 @@ void drop_replay(ldd_graph* g) {
     }
 }
 
-// One decomposition with the shifts already on the device and device
-// outputs, on the graph's stream (events 1 .. 4 when timing): rank and start
-// buckets, the round loop, finalize, with the retries of the fast rank path.
+// The errors that a decomposition is redone for: another key layout, or a
+// larger start-bucket table.
+constexpr u32 kErrRetry = kErrRankRetry | kErrLevelCap | kErrBucketCap;
+
+// One decomposition with the shifts already on the device (a union's in the
+// caller's layout, its lifts computed) and device outputs, on the graph's
+// stream (events 1 .. 4 when timing): keys and start buckets, the round loop,
+// finalize, with the retries of the direct keys.
 // Fills the device-side statistics of g->stats.
-int decompose_on_device(ldd_graph* g, const double* d_shift, int* center, int* dist,
+int decompose_on_device(ldd_graph* g, double beta, const double* d_shift, int* center, int* dist,
                         int* launches_out, const int* d_levels, const int* d_perm) {
   cudaStream_t s = g->stream;
   int launches = 0;
-  RankBufs rb = rank_bufs(g, d_shift);
   Header h;
   int status = LDD_OK;
-  bool exact64 = false;
+  KeyFmt f = direct_fmt(g, floors_for(g, beta));
+  bool exact64 = f.cap == 0;
+  if (d_levels) f = KeyFmt();
   if (g->epoch > 0xfffff000u) {  // status tags would wrap: clear and restart
     CUDA_TRY(cudaMemsetAsync(g->d_status, 0, g->status_bytes, s));
     g->epoch = 0;
   }
   CUDA_TRY(cudaMemsetAsync(g->d_ctl, 0, sizeof(Control), s));
   record(g, 1);
-  for (int attempt = 0; attempt < 4; ++attempt) {
+  for (int attempt = 0; attempt < 5; ++attempt) {
     if (attempt) CUDA_TRY(cudaMemsetAsync(g->d_ctl, 0, sizeof(Control), s));
-    rb = rank_bufs(g, d_shift);
-    rb.bptr = g->d_bptr;
-    rb.rcur = g->d_rcur;
-    rb.acnt = g->d_acnt;
-    rb.acnt_dirty = g->acnt_dirty;
-    rb.bptr_cap = g->bptr_cap;
+    const double* ranked_shift = d_shift;
+    if (exact64 && !d_levels) {
+      f = KeyFmt();
+      if (g->uni) {
+        launches += launch_union_spread(d_shift, g->uni->off, g->uni->k, (u32)g->n, g->d_shift,
+                                        g->num_sms, s);
+        ranked_shift = g->d_shift;
+      }
+    }
+    RankBufs rb = rank_bufs(g, exact64 ? ranked_shift : d_shift, f);
     if (!exact64 && !d_levels) g->acnt_dirty = true;  // until this attempt has consumed the counts
     launches += d_levels ? launch_ranked_and_buckets(rb, d_levels, d_perm, s)
                          : launch_rank_and_buckets(rb, exact64, s);
     record(g, 2);
-    const int l = run_bfs_finalize(g, center, dist, &status);
+    const int l = run_bfs_finalize(g, f, d_shift, center, dist, &status);
     if (l < 0) return status;
     launches += l;
     record(g, 4);
@@ -646,11 +706,14 @@ int decompose_on_device(ldd_graph* g, const double* d_shift, int* center, int* d
     CUDA_TRY(cudaStreamSynchronize(s));
     memcpy(&h, g->h_hdr, sizeof(h));
     if (!exact64 && !d_levels && h.err == 0) g->acnt_dirty = false;  // the scan cleared them
-    const u32 retry = kErrRankRetry | kErrBucketCap;
-    if (h.err == 0 || (h.err & ~retry) != 0) break;
-    // A fraction bucket too full to rank in place (crafted shifts): every
-    // kernel after the split was skipped; redo with the exact path.
+    if (h.err == 0 || (h.err & ~kErrRetry) != 0) break;
+    // Equal codes that the ids order wrongly, or many of them: ranked keys.
+    // Floors beyond the level field: a wider one, if that leaves code bits.
     if (h.err & kErrRankRetry) exact64 = true;
+    if (h.err & kErrLevelCap) {
+      f = direct_fmt(g, (u64)h.A);
+      if (f.cap == 0) exact64 = true;
+    }
     if (h.err & kErrBucketCap) {
       // floor(delta_max) + 2 exceeds the start-bucket table: grow it, redo.
       const size_t need = (size_t)h.A + 2;
@@ -668,7 +731,7 @@ int decompose_on_device(ldd_graph* g, const double* d_shift, int* center, int* d
         return fail(LDD_ERR_OOM, "start-bucket table of %zu entries", need);
       }
       g->bptr_cap = (u32)need;
-      g->acnt_dirty = true;  // cleared by the next fast-path attempt
+      g->acnt_dirty = true;  // cleared by the next attempt with direct keys
       drop_replay(g);        // a captured replay holds the old table
     }
   }
@@ -690,27 +753,27 @@ int* replay_dist(ldd_graph* g) { return g->uni ? g->uni->d_out_d : g->d_dist; }
 
 // Queues one fast-path decomposition on g->stream with no host synchronisation,
 // as it is captured: control block and look-back status cleared, [a union's
-// shifts spread from the caller layout,] rank with the fixed epochs 1 and 2,
-// BFS, finalize into the library's outputs, [the union's cut counts,] and the
+// lifts,] direct keys with the fixed scan epoch 1, BFS, finalize into the library's outputs, [the union's cut counts,] and the
 // header copied to the pinned host block.  Returns kernels queued, or -1.
-int enqueue_fast(ldd_graph* g, bool want_cut) {
+int enqueue_fast(ldd_graph* g, KeyFmt f, bool want_cut) {
   cudaStream_t s = g->stream;
   int launches = 0;
   if (cudaMemsetAsync(g->d_ctl, 0, sizeof(Control), s) != cudaSuccess) return -1;
-  const size_t words = rank_status_words((u32)g->n, g->bptr_cap);
+  const size_t words = scan_status_words(g->bptr_cap);
   if (cudaMemsetAsync(g->d_status, 0, words * sizeof(u64), s) != cudaSuccess) return -1;
   if (g->uni) {
     ldd_graph::Union& U = *g->uni;
-    launches += launch_union_spread(U.d_shift_in, U.off, U.k, (u32)g->n, g->d_excl, g->d_shift,
-                                    U.d_amax, U.d_amax + U.k, g->num_sms, s);
+    launches += launch_union_lift(U.d_shift_in, U.off, U.k, (u32)g->n, g->d_excl, U.d_amax,
+                                  U.d_amax + U.k, U.d_mlow, U.d_mpivot, g->num_sms, s);
   }
-  u32 epoch = 0;  // the two scans run with epochs 1 and 2 on cleared status words
-  RankBufs rb = rank_bufs(g, g->d_shift);
+  u32 epoch = 0;  // the scan runs with epoch 1 on cleared status words
+  const double* shift = g->uni ? g->uni->d_shift_in : g->d_shift;
+  RankBufs rb = rank_bufs(g, shift, f);
   rb.epoch = &epoch;
   rb.acnt_dirty = false;  // cleared before every launch of the replay
   launches += launch_rank_and_buckets(rb, false, s);
   int status = LDD_OK;
-  const int l = run_bfs_finalize(g, replay_center(g), replay_dist(g), &status);
+  const int l = run_bfs_finalize(g, f, shift, replay_center(g), replay_dist(g), &status);
   if (l < 0) return -1;
   launches += l;
   if (g->uni && want_cut) {
@@ -730,7 +793,7 @@ int enqueue_fast(ldd_graph* g, bool want_cut) {
 // Captures enqueue_fast into an executable graph (slot: with union cut
 // counts).  A capture that fails marks the graph replay_broken; the regular
 // path then runs.
-void capture_fast(ldd_graph* g, bool want_cut) {
+void capture_fast(ldd_graph* g, KeyFmt f, bool want_cut) {
   const int slot = want_cut ? 1 : 0;
   if (!g->cap_stream &&
       cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
@@ -751,7 +814,7 @@ void capture_fast(ldd_graph* g, bool want_cut) {
   cudaGraph_t graph = nullptr;
   int launches = -1;
   if (cudaStreamBeginCapture(g->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-    launches = enqueue_fast(g, want_cut);
+    launches = enqueue_fast(g, f, want_cut);
     if (cudaStreamEndCapture(g->cap_stream, &graph) != cudaSuccess) launches = -1;
   }
   g->stream = saved;
@@ -772,16 +835,24 @@ constexpr int kRunRegular = 1;  // replay_fast: take the regular path instead
 // One decomposition by graph replay, the shifts already in the library's
 // input buffer (d_shift, or a union's caller-layout d_shift_in).  Returns
 // LDD_OK, an error, or kRunRegular (no capture yet, capture failed, or the
-// fast rank path asked for a retry).
-int replay_fast(ldd_graph* g, bool want_cut, int* launches_out) {
+// direct keys asked for a retry).
+int replay_fast(ldd_graph* g, double beta, bool want_cut, int* launches_out) {
   if (!g->replay || g->replay_broken || g->regular_runs == 0) return kRunRegular;
+  // a captured key layout serves every smaller range of floors
+  const u64 floors = floors_for(g, beta);
+  if (floors > g->replay_floors) {
+    drop_replay(g);
+    g->replay_floors = floors;
+  }
+  const KeyFmt f = direct_fmt(g, g->replay_floors);
+  if (f.cap == 0) return kRunRegular;
   const int slot = want_cut ? 1 : 0;
   cudaStream_t s = g->stream;
   if (g->acnt_dirty) {
     CUDA_TRY(cudaMemsetAsync(g->d_acnt, 0, (size_t)g->bptr_cap * 4, s));
     g->acnt_dirty = false;
   }
-  if (!g->gexec[slot]) capture_fast(g, want_cut);
+  if (!g->gexec[slot]) capture_fast(g, f, want_cut);
   if (!g->gexec[slot]) return kRunRegular;
   record(g, 1);
   CUDA_TRY(cudaGraphLaunch(g->gexec[slot], s));
@@ -789,7 +860,7 @@ int replay_fast(ldd_graph* g, bool want_cut, int* launches_out) {
   CUDA_TRY(cudaStreamSynchronize(s));
   Header h;
   memcpy(&h, g->h_hdr, sizeof(h));
-  if (h.err & (kErrRankRetry | kErrBucketCap)) {
+  if (h.err & kErrRetry) {
     g->acnt_dirty = true;  // the counts may be half consumed
     return kRunRegular;
   }
@@ -829,7 +900,7 @@ int cut_on_device(ldd_graph* g, const int* d_center, int64_t* out_cut) {
 // it has run.  A fast rank path that asks for the exact path leaves the floor
 // counts cleared and skips the rest, so the decompositions queued behind it
 // run as usual.
-int enqueue_rank(ldd_graph* g, const double* d_shift, int* launches,
+int enqueue_rank(ldd_graph* g, KeyFmt f, const double* d_shift, int* launches,
                  const ShiftChunks* chunks = nullptr) {
   cudaStream_t s = g->stream;
   if (g->epoch > 0xfffff000u) {  // status tags would wrap: clear and restart
@@ -841,15 +912,16 @@ int enqueue_rank(ldd_graph* g, const double* d_shift, int* launches,
     CUDA_TRY(cudaMemsetAsync(g->d_acnt, 0, (size_t)g->bptr_cap * 4, s));
     g->acnt_dirty = false;
   }
-  RankBufs rb = rank_bufs(g, d_shift);
+  RankBufs rb = rank_bufs(g, d_shift, f);
   rb.acnt_dirty = false;
-  *launches += launch_rank_and_buckets(rb, false, s, chunks);
+  *launches += launch_rank_and_buckets(rb, f.cap == 0, s, chunks);
   return LDD_OK;
 }
 
-int enqueue_bfs_finalize(ldd_graph* g, int* center, int* dist, int* launches) {
+int enqueue_bfs_finalize(ldd_graph* g, KeyFmt f, const double* d_shift, int* center, int* dist,
+                         int* launches) {
   int status = LDD_OK;
-  const int lb = run_bfs_finalize(g, center, dist, &status);
+  const int lb = run_bfs_finalize(g, f, d_shift, center, dist, &status);
   if (lb < 0) {
     g->acnt_dirty = true;
     return status;
@@ -957,11 +1029,11 @@ u64 union_bytes(const UnionCaps& c) {
   const u64 N = c.N, words = std::max<u64>(N / 32, 1);
   u64 b = 4 * (N + 1) + 4 * c.E + 4 * c.M + 20 * c.G + 8 * (c.M / 32 + 1) + 8 * words +
           8 * c.C + 8 * c.T + 4 * N + 4 * words;
-  b += 16 * c.total + 8 * c.total + 32ull * (c.k + 1) + 44ull * c.k + sizeof(UnionMember) * c.k;
+  b += 16 * c.total + 8 * c.total + 32ull * (c.k + 1) + 56ull * c.k + sizeof(UnionMember) * c.k;
   const u64 nk = std::max<u64>(N, 64);
   b += 8 * N + 4 * N + 16 * nk + 8 * N + ((N + kSortTile - 1) / kSortTile + 1) * 2048 + 4 * N +
-       8 * N + 36 * N + 12 * (c.E / kBfsBase + 2) + 8 * N + (N ? fraction_slot_bytes((u32)N) : 0) +
-       8 * N + sizeof(Control);
+       8 * N + 36 * N + 12 * (c.E / kBfsBase + 2) + 8 * N + 4 * (N / kMaxBlock + 1) + 8 * N +
+       sizeof(Control);
   b += 12 * (N + 2);
   return b;
 }
@@ -1009,7 +1081,7 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
       cudaMalloc(&U.d_cut, K * 8) != cudaSuccess ||
       cudaMalloc(&U.d_wmem, words * 4) != cudaSuccess ||
       cudaMalloc(&U.d_amax, 2 * K * 4) != cudaSuccess ||
-      cudaMalloc(&U.d_mrank, 3 * K * 4) != cudaSuccess ||
+      cudaMalloc(&U.d_mlow, 3 * K * 8) != cudaSuccess ||
       cudaMalloc(&U.d_mpivot, 3 * K * 8) != cudaSuccess) {
     cudaGetLastError();
     return bail(fail(LDD_ERR_OOM, "device allocation of a union (%llu vertices, %llu arcs) "
@@ -1065,8 +1137,17 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
   g->n_active = (u32)n_active;
   g->nnz_active = nnz_active;
   g->max_degree = max_deg;
+  if (!g->per_sm_set) {  // two CTAs per SM are for wide bottom-up rounds (see finish_setup)
+    int most = 1;
+    bfs_grid_size(g->num_sms, &most);
+    g->bfs_per_sm = g->low_degree() ? 1 : std::min(most, 2);
+    g->bfs_grid = g->bfs_per_sm * g->num_sms;
+    g->stats.bfs_grid = g->bfs_grid;
+  }
   g->d_active = (all_active && n_active > 0) ? U.d_active_buf : nullptr;
   U.k = (u32)k;
+  U.max_n = 0;
+  for (int i = 0; i < k; ++i) U.max_n = std::max(U.max_n, (u32)members[i]->n);
   U.total = (u32)need.total;
   g->cut.m = (u32)need.M;
   g->cut.ngrp = (u32)need.G;
@@ -1110,14 +1191,14 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
   return LDD_OK;
 }
 
-int union_run(ldd_graph* u, const double* d_in, int* center, int* dist, bool want_cut,
+int union_run(ldd_graph* u, double beta, const double* d_in, int* center, int* dist, bool want_cut,
               int* launches_out, int* cut_launches_out) {
   ldd_graph::Union& U = *u->uni;
   cudaStream_t s = u->stream;
-  int launches = launch_union_spread(d_in, U.off, U.k, (u32)u->n, u->d_excl, u->d_shift, U.d_amax,
-                                     U.d_amax + U.k, u->num_sms, s);
+  int launches = launch_union_lift(d_in, U.off, U.k, (u32)u->n, u->d_excl, U.d_amax,
+                                   U.d_amax + U.k, U.d_mlow, U.d_mpivot, u->num_sms, s);
   int l = 0, rc;
-  if ((rc = decompose_on_device(u, u->d_shift, center, dist, &l)) != LDD_OK) return rc;
+  if ((rc = decompose_on_device(u, beta, d_in, center, dist, &l)) != LDD_OK) return rc;
   launches += l;
   int cl = 0;
   if (want_cut) {
@@ -1342,7 +1423,7 @@ int ldd_decompose(ldd_graph* g, double beta, const double* shifts, int32_t* out_
     CUDA_TRY(cudaMemcpyAsync(g->d_shift, shifts, n * 8,
                              dev_in ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
     d_shift = g->d_shift;
-    rc = replay_fast(g, false, &launches);
+    rc = replay_fast(g, beta, false, &launches);
     if (rc != LDD_OK && rc != kRunRegular) return rc;
     if (rc == LDD_OK) {
       center = g->d_center;
@@ -1355,7 +1436,8 @@ int ldd_decompose(ldd_graph* g, double beta, const double* shifts, int32_t* out_
     CUDA_TRY(cudaMemcpyAsync(g->d_shift, shifts, n * 8, cudaMemcpyHostToDevice, s));
     d_shift = g->d_shift;
   }
-  if (rc == kRunRegular && (rc = decompose_on_device(g, d_shift, center, dist, &launches)) != LDD_OK)
+  if (rc == kRunRegular &&
+      (rc = decompose_on_device(g, beta, d_shift, center, dist, &launches)) != LDD_OK)
     return rc;
   if (!dev_c) CUDA_TRY(cudaMemcpyAsync(out_center, center, n * 4, cudaMemcpyDeviceToHost, s));
   if (!dev_d) CUDA_TRY(cudaMemcpyAsync(out_dist, dist, n * 4, cudaMemcpyDeviceToHost, s));
@@ -1397,7 +1479,7 @@ int ldd_decompose_ranked(ldd_graph* g, const int32_t* levels, const int32_t* per
     d_perm = reinterpret_cast<const int*>(g->d_k[1]);
   }
   int launches = 0;
-  const int rc = decompose_on_device(g, nullptr, center, dist, &launches, d_levels, d_perm);
+  const int rc = decompose_on_device(g, 0.0, nullptr, center, dist, &launches, d_levels, d_perm);
   if (rc != LDD_OK) return rc;
   if (!dev_c) CUDA_TRY(cudaMemcpyAsync(out_center, center, n * 4, cudaMemcpyDeviceToHost, s));
   if (!dev_d) CUDA_TRY(cudaMemcpyAsync(out_dist, dist, n * 4, cudaMemcpyDeviceToHost, s));
@@ -1448,7 +1530,7 @@ int ldd_decompose_retry(ldd_graph* g, double beta, int k, const double* const* s
       d_shift = g->d_shift;
     }
     int l = 0, rc;
-    if ((rc = decompose_on_device(g, d_shift, center, dist, &l)) != LDD_OK) return rc;
+    if ((rc = decompose_on_device(g, beta, d_shift, center, dist, &l)) != LDD_OK) return rc;
     launches += l;
     if ((rc = cut_on_device(g, center, &cut)) != LDD_OK) return rc;
     launches += g->stats.cut_launches;
@@ -1509,7 +1591,7 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
   const bool chunk_first = !is_device_ptr(shifts[0]) && n >= ((size_t)1 << 20);
   if (chunk_first) {
     for (int c = 0; c < kC; ++c)
-      chunk_end[c] = c + 1 < kC ? (u32)(((n * (c + 1) / kC) + 31) & ~(size_t)31) : (u32)n;
+      chunk_end[c] = c + 1 < kC ? (u32)((n * (c + 1) / kC + kMaxBlock - 1) / kMaxBlock * kMaxBlock) : (u32)n;
     first.n = kC;
     first.end = chunk_end;
     first.ev = g->ev_chunk;
@@ -1578,11 +1660,13 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
     if (!dev_c || !dev_d) CUDA_TRY(cudaStreamWaitEvent(s, g->ev_out[j], 0));
     int* center = dev_c ? out_center[i] : d_c[j];
     int* dist = dev_d ? out_dist[i] : d_d[j];
-    if ((rc = enqueue_rank(g, dev_in ? shifts[i] : d_in[j], &launches,
+    const KeyFmt f = direct_fmt(g, floors_for(g, betas[i]));
+    const double* in = dev_in ? shifts[i] : d_in[j];
+    if ((rc = enqueue_rank(g, f, in, &launches,
                            pieces ? &first : nullptr)) != LDD_OK)
       return drain(rc);
     if (cuts && last_cut >= 0) CUDA_TRY(cudaStreamWaitEvent(s, g->ev_cut[last_cut], 0));
-    if ((rc = enqueue_bfs_finalize(g, center, dist, &launches)) != LDD_OK) return drain(rc);
+    if ((rc = enqueue_bfs_finalize(g, f, in, center, dist, &launches)) != LDD_OK) return drain(rc);
     CUDA_TRY(cudaMemcpyAsync(g->h_bhdr + (size_t)i * sizeof(Header), g->d_ctl, sizeof(Header),
                              cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaEventRecord(g->ev_used[j], s));
@@ -1618,16 +1702,15 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
   CUDA_TRY(cudaStreamSynchronize(g->cut_stream));
   CUDA_TRY(cudaStreamSynchronize(g->copy_out));
   CUDA_TRY(cudaStreamSynchronize(s));
-  // headers in order: the first hard error is the call's status; a fast rank
-  // path that asked for the exact path (or a larger start-bucket table) is
-  // redone alone on the regular path, which handles both
+  // headers in order: the first hard error is the call's status; one that
+  // asked for another key layout (or a larger start-bucket table) is redone
+  // alone on the regular path, which handles both
   for (int i = 0; i < k; ++i) {
     Header h;
     memcpy(&h, g->h_bhdr + (size_t)i * sizeof(Header), sizeof(h));
-    const u32 retry = kErrRankRetry | kErrBucketCap;
-    if (h.err & ~retry) return header_error(h.err);
+    if (h.err & ~kErrRetry) return header_error(h.err);
     if (h.err == 0) {
-      header_stats(g, h, false);
+      header_stats(g, h, direct_fmt(g, floors_for(g, betas[i])).cap == 0);
       if (out_cut) out_cut[i] = (int64_t)g->h_bcut[i];
       continue;
     }
@@ -1638,7 +1721,8 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
     int* center = dev_c ? out_center[i] : d_c[0];
     int* dist = dev_d ? out_dist[i] : d_d[0];
     int l = 0;
-    if ((rc = decompose_on_device(g, dev_in ? shifts[i] : d_in[0], center, dist, &l)) != LDD_OK)
+    if ((rc = decompose_on_device(g, betas[i], dev_in ? shifts[i] : d_in[0], center, dist, &l)) !=
+        LDD_OK)
       return drain(rc);
     launches += l;
     if (out_cut && (rc = cut_on_device(g, center, &out_cut[i])) != LDD_OK) return drain(rc);
@@ -1726,6 +1810,7 @@ int ldd_union_decompose(ldd_graph* u, const double* betas, const double* shifts,
   if (out_cut)
     for (u32 i = 0; i < U.k; ++i) out_cut[i] = 0;
   if (U.total == 0) return LDD_OK;
+  const double beta = *std::min_element(betas, betas + U.k);
   if (!shifts || !out_center || !out_dist) return fail(LDD_ERR_ARG, "NULL shifts or output");
   DeviceGuard dg(u->device);
   if (!dg.ok) return fail(LDD_ERR_CUDA, "cannot select device %d", u->device);
@@ -1743,7 +1828,7 @@ int ldd_union_decompose(ldd_graph* u, const double* betas, const double* shifts,
     CUDA_TRY(cudaMemcpyAsync(U.d_shift_in, shifts, total * 8,
                              dev_in ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
     in = U.d_shift_in;
-    rc = replay_fast(u, out_cut != nullptr, &launches);
+    rc = replay_fast(u, beta, out_cut != nullptr, &launches);
     if (rc != LDD_OK && rc != kRunRegular) return rc;
     if (rc == LDD_OK) {
       center = U.d_out_c;
@@ -1759,7 +1844,7 @@ int ldd_union_decompose(ldd_graph* u, const double* betas, const double* shifts,
     in = U.d_shift_in;
   }
   if (rc == kRunRegular) {
-    if ((rc = union_run(u, in, center, dist, out_cut != nullptr, &launches, &cut_launches)) !=
+    if ((rc = union_run(u, beta, in, center, dist, out_cut != nullptr, &launches, &cut_launches)) !=
         LDD_OK)
       return rc;
     if (out_cut)
@@ -1805,6 +1890,8 @@ int ldd_set_tuning(ldd_graph* g, const ldd_tuning* t) {
       t->window_levels > 4096 || t->window_max_frontier < 0 || t->window_queue < 0 ||
       t->bfs_span < kBfsBase || t->bfs_span > kBfsMaxSpan || t->bfs_span % kBfsBase != 0)
     return fail(LDD_ERR_ARG, "tuning out of range (blocks per SM 1 .. %d)", max_per_sm);
+  g->per_sm_set = g->per_sm_set || g->bfs_per_sm != t->bfs_blocks_per_sm;
+  g->pull_set = g->pull_set || g->pull_alpha != (u32)t->pull_alpha;
   g->bfs_per_sm = t->bfs_blocks_per_sm;
   g->bfs_grid = g->bfs_per_sm * g->num_sms;
   g->pull_alpha = (u32)t->pull_alpha;
@@ -1850,9 +1937,9 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out) 
       int l = 0, cl = 0, rc;
       CUDA_TRY(cudaEventRecord(e0, s));
       if (g->uni)
-        rc = union_run(g, d_in, g->uni->d_out_c, g->uni->d_out_d, false, &l, &cl);
+        rc = union_run(g, 0.0, d_in, g->uni->d_out_c, g->uni->d_out_d, false, &l, &cl);
       else
-        rc = decompose_on_device(g, d_in, g->d_center, g->d_dist, &l);
+        rc = decompose_on_device(g, 0.0, d_in, g->d_center, g->d_dist, &l);
       if (rc != LDD_OK) return rc;
       CUDA_TRY(cudaEventRecord(e1, s));
       CUDA_TRY(cudaEventSynchronize(e1));

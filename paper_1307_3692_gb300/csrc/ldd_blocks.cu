@@ -171,6 +171,7 @@ void sync_params(ldd_graph* g, ldd_graph* r) {
   r->stall_barrier = g->stall_barrier;
   r->stall_lookback = g->stall_lookback;
   r->pull_alpha = g->pull_alpha;
+  r->pull_set = g->pull_set;
   r->pull_beta = g->pull_beta;
   r->pull_gamma = g->pull_gamma;
   r->probe_min_arcs = g->probe_min_arcs;
@@ -250,7 +251,7 @@ extern "C" int ldd_block_decompose(ldd_graph* g, int k, const double* betas,
     int* dist = dev_d ? out_dist[i] : g->d_dist;
     int* cur_center = cur == g ? center : r->d_center;  // in G_i's ids
     int launches = 0;
-    if ((rc = decompose_on_device(cur, d_shift, cur_center, cur == g ? dist : r->d_dist,
+    if ((rc = decompose_on_device(cur, betas[i], d_shift, cur_center, cur == g ? dist : r->d_dist,
                                   &launches)) != LDD_OK) {
       cudaStreamSynchronize(s);
       *out_blocks = blocks;

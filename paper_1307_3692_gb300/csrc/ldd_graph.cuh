@@ -110,7 +110,7 @@ struct ldd_graph {
   u32* d_qoff[3] = {};
   u32* d_cf[3] = {};
   u32* d_ulist[2] = {nullptr, nullptr};
-  void* d_slots = nullptr;
+  u32* d_bmax = nullptr;       // largest handled floor plus one per kMaxBlock vertices
   int* d_center = nullptr;
   int* d_dist = nullptr;
   Control* d_ctl = nullptr;
@@ -137,6 +137,13 @@ struct ldd_graph {
   u32 probe_min_arcs = 1u << 16;
   u32 max_degree = 0;          // largest row of the CSR (unions: of any member)
   bool low_degree_rounds = true;  // tuning: low-degree rounds when max_degree allows
+  bool low_degree() const { return low_degree_rounds && max_degree <= (u32)kLdMaxDegree; }
+  // Set by the user (else bfs_per_sm and pull_alpha follow the graph).
+  bool per_sm_set = false, pull_set = false;
+  // Low-degree rounds stay top-down unless the tuning says otherwise: a scan of
+  // a few arcs has next to none to save, and it reads every unsettled vertex (64
+  // random geometric graphs: 5.09 -> 4.60 ms).
+  bool low_pull() const { return low_degree() && !pull_set; }
   u32 window_levels = 0;          // tuning: levels per window in low-degree rounds (0: none)
   u32 window_max_q = 1u << 18;    // tuning: windows only for frontiers up to this size
   u32 window_queue = 0;           // tuning: local-queue entries per CTA and level (0: all that fit)
@@ -158,6 +165,7 @@ struct ldd_graph {
   struct Union {
     UnionCaps cap;                 // capacities the tables were allocated for
     u32 k = 0;
+    u32 max_n = 0;                 // the largest member's vertices
     u32 total = 0;                 // n_0 + ... + n_{k-1}: caller-layout length
     std::vector<u32> h_ooff;       // caller-layout offsets, k + 1
     std::vector<u32> h_voff;       // union-vertex offsets, k + 1
@@ -171,7 +179,7 @@ struct ldd_graph {
     u64* d_cut = nullptr;          // [k]
     u32* d_wmem = nullptr;         // [N / 32] member of every 32-vertex word
     int* d_amax = nullptr;         // [k] largest floor of each member, then [k] its lift
-    u32* d_mrank = nullptr;        // [3][k] the round loop's per-member bottom-up floors
+    u64* d_mlow = nullptr;         // [3][k] the round loop's per-member bottom-up floors
     u64* d_mpivot = nullptr;       // [3][k] ... and pivots
   };
   Union* uni = nullptr;
@@ -181,6 +189,7 @@ struct ldd_graph {
   // captured CUDA graph of one fast-path decomposition (ldd_set_graph_replay)
   bool replay = false;
   bool replay_broken = false;        // capture failed once: regular path only
+  u64 replay_floors = 0;             // range of floors the captured key layout holds
   int regular_runs = 0;              // regular decompositions so far (capture waits for one)
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec[2] = {};     // [with union cut counts]
@@ -200,11 +209,12 @@ int finish_setup(ldd_graph* g);
 void free_blocks(ldd_graph* g);
 void record(ldd_graph* g, int i);
 float elapsed(ldd_graph* g, int a, int b);
-// One decomposition on g's stream from device shifts into device outputs
-// (union: caller layout), with the fast rank path's retries; synchronises.
+// One decomposition on g's stream from device shifts (union: caller layout, its
+// lifts computed) into device outputs, with the direct keys' retries;
+// synchronises.  beta sizes the keys' level field (0: unknown).
 // d_levels, d_perm: the ranked variant (integer levels and a tie-break
 // permutation in place of FP64 shifts); else null.
-int decompose_on_device(ldd_graph* g, const double* d_shift, int* center, int* dist,
+int decompose_on_device(ldd_graph* g, double beta, const double* d_shift, int* center, int* dist,
                         int* launches_out, const int* d_levels = nullptr,
                         const int* d_perm = nullptr);
 
@@ -217,9 +227,9 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& caps);
 // Fills u from members on stream s (members' tables are read by kernels on
 // s: keep them alive until s has finished); sync: wait for s.
 int union_fill(ldd_graph* u, int k, ldd_graph* const* members, cudaStream_t s, bool sync);
-// Shifts (caller layout, device) spread, decomposition, and optionally the
-// members' cut counts into u's d_cut; outputs in the caller layout (device).
-int union_run(ldd_graph* u, const double* d_in, int* center, int* dist, bool want_cut,
+// Decomposition of shifts and outputs in the caller layout (device), and
+// optionally the members' cut counts into u's d_cut; beta: the smallest.
+int union_run(ldd_graph* u, double beta, const double* d_in, int* center, int* dist, bool want_cut,
               int* launches_out, int* cut_launches_out);
 
 // Cut counts (Definition 1.1) of K = 1 .. 4 labelings centers[0 .. K) of one

@@ -1,14 +1,23 @@
 // Internal declarations shared by the CUDA translation units of libldd.so.
 //
-// Key layout (Section 4 of Miller, Peng, Xu 2013): the shifted distance
-// dist(u, v) - delta_u is compared as the pair
-//     level = (floor(delta_max) - floor(delta_u)) + dist(u, v)   (integer part)
-//     rank  = position of u in the order (frac(delta_u) descending, u ascending)
-// packed into one 64-bit word key = (level << 32) | rank, so that the
-// unsigned minimum of two keys is the lexicographic minimum the paper asks
-// for: smaller integer part first, larger fraction on a tie (Section 4: the
-// fractional parts are tie-breakers within an integer level and can be
-// replaced by a permutation), smaller id on an exact tie (Algorithm 2).
+// Keys.  The shifted distance dist(u, v) - delta_u (Section 4 of Miller, Peng,
+// Xu 2013) is compared as the pair
+//     level = (integer part): a constant - floor(delta_u) + dist(u, v)
+//     tie-break: larger fraction frac(delta_u) first, smaller u on an exact tie
+// packed into one 64-bit word whose unsigned minimum is the lexicographic
+// minimum the paper asks for.  Two layouts (KeyFmt):
+//   direct  level | code | id: the code is the complement of the fraction's
+//           leading bits and the id names u (in a union, inside its member), so
+//           a key is one pass over the shifts, needs no rank, and names its
+//           center.  Two centers whose codes are equal are compared by id.  The
+//           kernels list the meetings of such keys (note_tie) and finalize
+//           compares their exact fractions: if the id order is not theirs, or
+//           meetings are many, the host redoes the decomposition in the other
+//           layout.
+//   ranked  level (32 bits) | rank (32 bits): rank is u's position in the order
+//           (fraction descending, id ascending), order[rank] = u.  The exact
+//           radix sort of all fractions gives it, or the caller's permutation
+//           (ldd_decompose_ranked).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -19,7 +28,24 @@ namespace ldd {
 typedef unsigned long long u64;
 typedef unsigned int u32;
 
-constexpr u64 kLevelOne = 1ull << 32;
+constexpr u64 kLevelOne = 1ull << 32;  // one queue entry in an (entries << 32) | arcs counter
+
+// Key layout: level in the bits from 32 + s2 on, the id in the low ib bits
+// (ranked: ib = 0).  Direct keys: a vertex of floor a starts at level cap - a.
+struct KeyFmt {
+  u32 s2 = 0;
+  u32 ib = 0;
+  u32 cap = 0;  // 0: ranked
+  u32 cb = 0;   // code bits
+};
+constexpr u32 kMinCodeBits = 20;  // fewer: ranked from the start
+constexpr u32 kMaxCodeBits = 32;
+// Direct keys: meetings of equal codes that are compared exactly; with more the
+// host takes the ranked layout.
+constexpr u32 kMaxTies = 64;
+// Vertices per entry of bmax, the largest floor (plus one) among those the
+// round loop handles.
+constexpr u32 kMaxBlock = 128;
 
 // Bits of Control::err.
 enum : u32 {
@@ -28,8 +54,9 @@ enum : u32 {
   kErrTimeout = 1u << 2,     // a bounded device-side wait ran out
   kErrBucketCap = 1u << 3,   // start-bucket table smaller than A + 2 (host grows it, reruns)
   kErrInternal = 1u << 4,    // a capacity invariant failed
-  kErrRankRetry = 1u << 5,   // a long run of equal 32-bit fraction codes: redo the rank exactly
+  kErrRankRetry = 1u << 5,   // direct keys: equal codes decide wrongly or often; redo with ranks
   kErrPermArg = 1u << 6,     // ranked variant: a negative level or perm not a permutation
+  kErrLevelCap = 1u << 7,    // direct keys: a floor beyond the level field (host widens it, reruns)
 };
 
 // Radix sort: 8-bit digits, 256-thread CTAs, 16 keys per thread.
@@ -68,8 +95,9 @@ struct Control {
   // BFS runtime state
   u64 bar;         // grid-barrier arrivals (monotonic within one launch)
   u64 qctr[3];     // frontier counters: (items << 32) | edges
-  u32 minrank[3];  // smallest rank among the keys of each frontier level (reset to ~0)
+  u64 minlow[3];   // smallest tie-break among the keys of each frontier level (reset to ~0)
   u32 pull_rounds; // rounds run bottom-up
+  u32 pad_p;
   u64 push_arcs;   // arcs expanded top-down
   u64 pull_arcs;   // arcs scanned bottom-up
   u64 pull_verts;  // vertices examined bottom-up
@@ -80,7 +108,6 @@ struct Control {
   // sort state
   u32 mask_f;     // bit d: fraction digit pass d is needed (exact path)
   u32 mask_r;     // unused (start buckets are a counting sort)
-  u32 maxbucket;  // largest fraction bucket (fast path)
   u32 tile_ctr[kFracDigits + kRoundDigits];
   u32 hist_f[kFracDigits][256];
   u32 off_f[kFracDigits][256];
@@ -102,19 +129,27 @@ struct Control {
   u32 pull_ctr[3];
   // ... and their list for the second pass: (entries << 32) | arcs (rotating)
   u64 rest[3];
+  int Ab;    // largest floor among the vertices the round loop handles (direct keys)
+  u32 ties;  // meetings of equal codes, and the first ones: a vertex of the member, two ids
+  u32 tie[kMaxTies][3];
 };
 constexpr size_t kCtlHeaderBytes = 40;       // err .. cut
 constexpr size_t kCtlBfsStateOffset = 40;    // bar_count .. pull_rounds
-constexpr size_t kCtlBfsStateBytes = 96;
-constexpr size_t kCtlMinrankOffset = 72;
+constexpr size_t kCtlBfsStateBytes = 112;
+constexpr size_t kCtlMinlowOffset = 72;
 
 struct BfsArgs {
   const int* row_ptr;
   const int* col;
   u64* key;
-  const int* bptr;   // [A + 2] start-bucket offsets into the round-sorted list
-  const u32* rk[2];  // round-sorted keys (start rounds), ping-pong pair
-  const u32* rv[2];  // round-sorted vertices, ping-pong pair
+  const int* bptr;   // [A + 2] start-bucket offsets into rv
+  u32* rcur;         // [A + 2] their ends so far (direct keys: the loop fills the buckets)
+  u32* rv;           // start-bucket vertices
+  const u32* bmax;   // direct keys: largest floor plus one per kMaxBlock vertices
+  KeyFmt f;
+  const double* shift;  // direct keys: the shifts (unions: caller layout), for exact ties
+  const u32* voff;      // unions: first union vertex of every member
+  const u32* ooff;      // unions: first caller-layout entry of every member
   u32* qv[3];        // frontier queues: vertex (side 2: put-off work of bottom-up rounds)
   int* qrow[3];      //                  row_ptr[vertex]
   u32* qoff[3];      //                  exclusive edge offset in the frontier
@@ -142,7 +177,7 @@ struct BfsArgs {
   u32 window_queue;  // ... local-queue entries per CTA and level at most (0: as many as fit)
   u32 span;          // edge-balanced rounds: arcs per CTA step at most (kBfsBase .. kBfsMaxSpan)
   const u32* wmem;   // unions: member of every 32-vertex word; else null
-  u32* mrank;        // unions: [3][kmem] smallest rank per level slot and member (~0 on entry)
+  u64* mlow;         // unions: [3][kmem] smallest tie-break per level slot and member (~0 on entry)
   u64* mpivot;       // unions: [3][kmem] (degree << 32) | vertex of every member's frontier vertex
                      // of the largest degree per level slot (zero on entry)
   u32 kmem;          // unions: members
@@ -173,10 +208,10 @@ struct CompScratch {
 };
 
 // ---------------------------------------------------------------- launchers
-// Fraction rank and start buckets (k_rank.cu).  Returns kernels launched.
-// Buffers of the fraction rank and the start buckets (k_rank.cu).
+// Buffers of the keys and the start buckets (k_rank.cu).
 struct RankBufs {
-  const double* shift;  // [n] shifts on the device
+  const double* shift;  // shifts on the device: [n], direct keys of a union in the caller layout
+  KeyFmt f;             // direct keys' layout
   u32 n;
   int num_sms;
   int* a;               // [n] floor(shift)
@@ -184,7 +219,7 @@ struct RankBufs {
   u64* k1;
   u32* v0;              // [n] values / scratch; ends as the start-bucket vertices
   u32* v1;
-  void* slots;          // fraction_slot_bytes(n): bucket record slots (fast path)
+  u32* bmax;            // [n / kMaxBlock + 1] (direct keys)
   u64* status;          // look-back status words (epoch-tagged)
   u32* epoch;
   u32* order;           // [n] rank -> vertex
@@ -195,18 +230,18 @@ struct RankBufs {
   bool acnt_dirty;      // acnt may hold counts of an unfinished call: clear it first
   u32 bptr_cap;
   const u32* excl;      // bit v: v is not handled by the BFS (no start bucket)
-  const u32* solo;      // bit v: v is alone in its component (no rank needed)
   const u32* wmem;      // unions: member of every 32-vertex word; else null
+  const u32* voff;      // unions: first union vertex, and first caller-layout entry, of a member
+  const u32* ooff;
   const int* lift;      // unions: floor lift of every member (a_u += lift); else null
   Control* ctl;
   u32 lookback_limit = 1u << 24;  // polls of a look-back wait before kErrTimeout
   u32 stall_lookback = 0;         // 1: the scans' first tile waits on a status word that nothing
                                   // writes, so every look-back runs out (timeout-path tests)
 };
-// exact64 = false: fraction buckets + in-bucket exact ranks of the vertices
-// not alone in their component (may set kErrRankRetry); true: exact 64-bit
-// LSD radix sort of all vertices.  The start buckets end in v0 (vertices) and
-// k0 viewed as 32-bit words (their rounds).
+// exact64 = false: direct keys in one pass over the shifts, and the start
+// buckets' offsets (bptr, rcur; the round loop fills the buckets).  true: ranked
+// keys by an exact 64-bit LSD radix sort, and full start buckets in v0.
 // chunks (optional): the shifts are still arriving; chunk c is complete once
 // ev[c] has fired and covers the vertices up to end[c] (ascending).
 struct ShiftChunks {
@@ -221,11 +256,9 @@ int launch_rank_and_buckets(const RankBufs& r, bool exact64, cudaStream_t s,
 // buckets and keys as the exact path.
 int launch_ranked_and_buckets(const RankBufs& r, const int* levels, const int* perm,
                               cudaStream_t s);
-u32 fraction_bucket_bits(u32 n);
-// Look-back status words the fast path's two scans use (status[0 ..)); a
-// captured replay clears them and runs with the fixed epochs 1 and 2.
-size_t rank_status_words(u32 n, u32 bptr_cap);
-size_t fraction_slot_bytes(u32 n);
+// Look-back status words the direct path's scan uses (status[0 ..)); a
+// captured replay clears them and runs with the fixed epoch 1.
+size_t scan_status_words(u32 bptr_cap);
 // Persistent BFS (k_bfs.cu).  Returns kernels launched, or -1 with the CUDA
 // error left in *err.
 // The most CTAs per SM (1 or 2) the round loop can use; returns that times num_sms.
@@ -234,8 +267,9 @@ int bfs_grid_size(int num_sms, int* blocks_per_sm);
 int launch_bfs(const BfsArgs& a, int grid, int per_sm, cudaStream_t s, cudaError_t* err);
 size_t bfs_smem_bytes();
 // Finalize, cut and per-graph component tables (k_graph.cu).
-int launch_finalize(const u64* key, const u32* order, const u32* solo, u32 n, int* center,
-                    int* dist, const u32* err, int num_sms, cudaStream_t s);
+// a.f.cap != 0: direct keys, which name their centers (order and solo unused).
+int launch_finalize(const BfsArgs& a, const u32* order, const u32* solo, int* center, int* dist,
+                    int num_sms, cudaStream_t s);
 // Cut list of Definition 1.1's count.  Every undirected edge {v, w} (repeated
 // edges repeated) is stored once, oriented from its cold endpoint (smaller
 // degree; ties: larger id) to its hot one, and grouped by the cold endpoint:
@@ -265,7 +299,7 @@ struct CutList {
 };
 int launch_cut(const CutList& cl, const int* center, const u32* hot, u32 n_hot, int* hot_center,
                u64* out, int num_sms, cudaStream_t s);
-int launch_small_comp(const SmallComps& sc, u64* key, const u32* err, int num_sms, cudaStream_t s);
+int launch_small_comp(const SmallComps& sc, const BfsArgs& a, int num_sms, cudaStream_t s);
 // The radius of a decomposition: max over v of dist[v], into *out.
 int launch_max_dist(const int* dist, u32 n, u32* out, int num_sms, cudaStream_t s);
 // Labels components and fills t.comp_* and excl (bit v: kept out of the BFS);
@@ -381,13 +415,16 @@ struct UnionTables {
 // largest = the longest table (elements), for the grid size.
 int launch_union_concat(const UnionMember* mem, const UnionOffsets& off, u32 k,
                         const UnionTables& t, u64 largest, int num_sms, cudaStream_t s);
-// Shifts to the union layout, and every member's floor lift (amax, lift: k ints).
-int launch_union_spread(const double* in, const UnionOffsets& off, u32 k, u32 N,
-                        const u32* excl, double* out, int* amax, int* lift, int num_sms,
-                        cudaStream_t s);
-int launch_union_finalize(const u64* key, const u32* order, const u32* solo,
+// Every member's floor lift (amax, lift: k ints) from the caller-layout shifts;
+// also sets the round loop's per-member tables (BfsArgs) to their start values.
+int launch_union_lift(const double* in, const UnionOffsets& off, u32 k, u32 N, const u32* excl,
+                      int* amax, int* lift, u64* mlow, u64* mpivot, int num_sms, cudaStream_t s);
+// Caller-layout shifts to the union layout (ranked keys).
+int launch_union_spread(const double* in, const UnionOffsets& off, u32 k, u32 N, double* out,
+                        int num_sms, cudaStream_t s);
+int launch_union_finalize(const BfsArgs& a, const u32* order, const u32* solo,
                           const UnionOffsets& off, u32 k, u32 total, int* center, int* dist,
-                          const u32* err, int num_sms, cudaStream_t s);
+                          int num_sms, cudaStream_t s);
 // Every member's cut count (cut[s], zero on entry) over the union's cut list
 // (hot ids resolved, no hot table); labels in the caller layout.
 int launch_union_cut(const CutList& cl, const UnionOffsets& off, const u32* wmem,
@@ -400,6 +437,93 @@ __device__ __forceinline__ u32 lanemask_lt() {
   u32 m;
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
   return m;
+}
+
+// ---- keys (KeyFmt)
+__device__ __forceinline__ u32 key_level(const KeyFmt& f, u64 k) { return (u32)(k >> 32) >> f.s2; }
+__device__ __forceinline__ u64 key_up(const KeyFmt& f, u64 k) {  // one level further out
+  return k + ((u64)(1u << f.s2) << 32);
+}
+__device__ __forceinline__ u64 level_key(const KeyFmt& f, u32 level) {
+  return (u64)(level << f.s2) << 32;
+}
+__device__ __forceinline__ u64 key_low(const KeyFmt& f, u64 k) {
+  return k & (((u64)((1u << f.s2) - 1u) << 32) | 0xffffffffull);
+}
+__device__ __forceinline__ u32 key_id(const KeyFmt& f, u64 k) { return (u32)k & ((1u << f.ib) - 1u); }
+// x and y agree but for the id (never for ranked keys, which have none).
+__device__ __forceinline__ bool key_tie(const KeyFmt& f, u64 x, u64 y) {
+  const u64 d = x ^ y;
+  return ((u32)(d >> 32) | ((u32)d >> f.ib)) == 0u && (u32)d != 0u;
+}
+
+// Splits a shift d into a = floor(d) and the IEEE-754 bits of its fraction
+// f = d - a (exact), with integer operations on d's bits only: FP64
+// arithmetic is slow on this part.  The bits of a non-negative double order
+// like its value, so fb orders the fractions.  d = -0 counts as +0.  NaN or
+// d < 0 sets kErrShiftArg, d >= 2^31 (or +inf) kErrShiftRange; a = 0 and
+// fb = 0 then.
+__device__ __forceinline__ void split_bits(double d, u32& err, int& a, u64& fb) {
+  constexpr u64 kMan = (1ull << 52) - 1;
+  const u64 b = (u64)__double_as_longlong(d);
+  const u32 ex = (u32)(b >> 52) & 0x7ffu;
+  a = 0;
+  fb = 0;
+  if (ex == 0x7ffu && (b & kMan) != 0) {  // NaN, either sign
+    err |= kErrShiftArg;
+  } else if (b >> 63) {                   // negative; -0 is +0
+    if (b << 1) err |= kErrShiftArg;
+  } else if (ex >= 1023u + 31u) {         // >= 2^31 or +inf
+    err |= kErrShiftRange;
+  } else if (ex < 1023u) {                // d < 1: a = 0, f = d
+    fb = b;
+  } else {
+    const u32 E = ex - 1023u;             // d = M * 2^(E - 52), 0 <= E <= 30
+    const u64 M = (b & kMan) | (1ull << 52);
+    a = (int)(M >> (52 - E));
+    const u64 fr = M & ((1ull << (52 - E)) - 1);  // f = fr * 2^(E - 52)
+    if (fr) {
+      const int p = 63 - __clzll((long long)fr);  // leading bit of fr: f in [2^(p+E-52), 2^(p+E-51))
+      fb = ((u64)(p + (int)E - 52 + 1023) << 52) | ((fr << (52 - p)) & kMan);
+    }
+  }
+}
+
+// Cheap and nearly as sharp, for the branch around a batch's note_tie calls: the
+// high words (level and the code's leading bits) agree, the low words do not.
+__device__ __forceinline__ bool key_near(u64 x, u64 y) {
+  return (u32)(x >> 32) == (u32)(y >> 32) && (u32)x != (u32)y;
+}
+
+// Two keys of vertex w's member met, x and y.  If only their ids differ, the
+// meeting is listed for finalize (tie_check).
+__device__ __forceinline__ void note_tie(Control* ctl, const KeyFmt& f, u32 w, u64 x, u64 y) {
+  if (key_tie(f, x, y)) {
+    const u32 at = atomicAdd(&ctl->ties, 1u);
+    if (at < kMaxTies) {
+      ctl->tie[at][0] = w;
+      ctl->tie[at][1] = key_id(f, x);
+      ctl->tie[at][2] = key_id(f, y);
+    }
+  }
+}
+
+// Thread t of one CTA checks listed meeting t: the ids are ordered as the exact
+// fractions are (larger first), or the attempt fails, as it does when meetings
+// were too many.
+__device__ __forceinline__ void tie_check(const double* shift, const u32* wmem, const u32* ooff,
+                                          Control* ctl, u32 t) {
+  const u32 ties = ctl->ties;
+  if (t == 0 && ties > kMaxTies) atomicOr(&ctl->err, kErrRankRetry);
+  if (t >= min(ties, kMaxTies)) return;
+  const double* own = shift + (wmem ? ooff[wmem[ctl->tie[t][0] >> 5]] : 0u);
+  const u32 x = ctl->tie[t][1], y = ctl->tie[t][2];
+  u32 err = 0;
+  int a;
+  u64 fx, fy;
+  split_bits(own[min(x, y)], err, a, fx);
+  split_bits(own[max(x, y)], err, a, fy);
+  if (fy > fx) atomicOr(&ctl->err, kErrRankRetry);
 }
 
 __device__ __forceinline__ u64 ld_cg_u64(const u64* p) { return __ldcg(p); }

@@ -170,7 +170,9 @@ int run_batch(ldd_server* S, int slot, const std::vector<Request*>& batch) {
   const double t1 = S->now_us();
   int launches = 0, cut_launches = 0;
   const double t2 = S->now_us();
-  rc = union_run(u, U.d_shift_in, U.d_out_c, U.d_out_d, want_cut, &launches, &cut_launches);
+  double beta = batch[0]->beta;
+  for (const Request* r : batch) beta = std::min(beta, r->beta);
+  rc = union_run(u, beta, U.d_shift_in, U.d_out_c, U.d_out_d, want_cut, &launches, &cut_launches);
   if (rc != LDD_OK) return rc;
   if (want_cut)
     CUDA_TRY(cudaMemcpyAsync(S->h_cut[(size_t)slot], U.d_cut, (size_t)k * 8,
