@@ -137,10 +137,11 @@ __global__ void __launch_bounds__(kCutThreads, 1) k_cut(CutList cl, const int* _
   int* s_hot = reinterpret_cast<int*>(cut_smem);
   __shared__ unsigned long long wsum[kCutThreads / 32];
   const u32 tid = threadIdx.x, lane = tid & 31;
+  const int nsm = (int)min(n_hot, kHotSlots);  // the rest of the table stays in global memory
   if (!U) {
     const int4* hc4 = reinterpret_cast<const int4*>(hot_center);  // cudaMalloc'd: aligned
-    for (u32 i = tid; i < n_hot / 4; i += blockDim.x) cut_smem[i] = __ldg(hc4 + i);
-    for (u32 i = (n_hot & ~3u) + tid; i < n_hot; i += blockDim.x) s_hot[i] = hot_center[i];
+    for (int i = (int)tid; i < nsm / 4; i += blockDim.x) cut_smem[i] = __ldg(hc4 + i);
+    for (int i = (nsm & ~3) + (int)tid; i < nsm; i += blockDim.x) s_hot[i] = hot_center[i];
     __syncthreads();
   }
   const int4* hot4 = reinterpret_cast<const int4*>(cl.hot);  // cudaMalloc'd: aligned
@@ -187,7 +188,10 @@ __global__ void __launch_bounds__(kCutThreads, 1) k_cut(CutList cl, const int* _
         hl[q] = valid ? center[hv[q]] : 0;
       } else {
         cl_lab[q] = valid ? __ldg(cl.grp_lab + g[q]) : 0;
-        hl[q] = valid ? (hv[q] < 0 ? s_hot[hv[q] & 0x7fffffff] : center[hv[q]]) : 0;
+        const int slot = hv[q] & 0x7fffffff;  // hv[q] itself outside the hot table
+        hl[q] = 0;
+        if (valid)
+          hl[q] = hv[q] >= 0 ? center[hv[q]] : slot < nsm ? s_hot[slot] : __ldg(hot_center + slot);
       }
     }
     if (U) {
@@ -836,6 +840,319 @@ __global__ void __launch_bounds__(kCutThreads, 1) k_cut4(CutList cl, const int4*
   }
 }
 
+// ---------------------------------------------------------------- cut counts by piece codes
+// Member s of off[0 .. k]: the last s with off[s] <= x (x < off[k]).
+__device__ __forceinline__ u32 segment_of(const u32* __restrict__ off, u32 k, u32 x) {
+  u32 lo = 0, hi = k;
+  while (hi - lo > 1) {
+    const u32 mid = (lo + hi) >> 1;
+    if (__ldg(off + mid) <= x) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// The first kCodePieces distinct pieces among the kPickFrom highest-degree
+// vertices: one warp per labeling (union: per member).
+constexpr u32 kPickFrom = 256;
+
+template <bool U>
+__global__ void __launch_bounds__(32) k_picks(CutCodes cc, Labels4 L, UnionOffsets off) {
+  const u32 lane = threadIdx.x, b = blockIdx.x;
+  const u32 h0 = U ? off.h[b] : 0u;
+  const u32 nh = U ? off.h[b + 1] - h0 : cc.nhot;
+  const int* center = U ? L.c[0] : L.c[b];
+  u32 lab[kPickFrom / 32];
+#pragma unroll
+  for (u32 i = 0; i < kPickFrom / 32; ++i) {
+    const u32 h = i * 32 + lane;
+    const u32 v = h < nh ? __ldg(cc.hotv + h0 + h) : 0xffffffffu;  // a union's padding: ~0
+    lab[i] = v != 0xffffffffu ? (u32)__ldg(center + v) : 0xffffffffu;
+  }
+  u32 mine = 0xffffffffu;  // lane p: piece p
+  u32 found = 0;
+#pragma unroll
+  for (u32 i = 0; i < kPickFrom / 32; ++i) {
+    bool open = lab[i] != 0xffffffffu;
+    for (u32 p = 0; p < found; ++p) open = open && lab[i] != __shfl_sync(kFull, mine, p);
+    u32 m;
+    while (found < kCodePieces && (m = __ballot_sync(kFull, open)) != 0u) {
+      const u32 x = __shfl_sync(kFull, lab[i], __ffs(m) - 1);
+      if (lane == found) mine = x;
+      ++found;
+      open = open && lab[i] != x;
+    }
+  }
+  if (lane <= kCodePieces) cc.picks[b * (kCodePieces + 1) + lane] = mine;
+}
+
+__device__ __forceinline__ u32 code_of(u32 label, const u32* picks) {
+  if (label == picks[0]) return 0;  // nearly all
+#pragma unroll 1
+  for (u32 p = 1; p < kCodePieces; ++p)
+    if (label == picks[p]) return p;
+  return kCodeOther;
+}
+
+// Code words: labeling k's code in bits 4 k .. 4 k + 3, four vertices per thread.
+// A vertex without edges (solo) needs none: it would only hold up its warp in
+// the search for its piece.
+__global__ void __launch_bounds__(256) k_codes(CutCodes cc, Labels4 L, int K, u32 n) {
+  __shared__ u32 picks[4 * (kCodePieces + 1)];
+  if (threadIdx.x < (u32)K * (kCodePieces + 1)) picks[threadIdx.x] = cc.picks[threadIdx.x];
+  __syncthreads();
+  const u32 stride = gridDim.x * blockDim.x;
+  for (u32 v0 = blockIdx.x * blockDim.x + threadIdx.x; v0 < n; v0 += stride * 4) {
+    u32 w[4] = {0, 0, 0, 0};
+    bool on[4];
+#pragma unroll
+    for (u32 q = 0; q < 4; ++q) {
+      const u32 v = v0 + q * stride;
+      on[q] = v < n && !(__ldg(cc.solo + (v >> 5)) >> (v & 31) & 1u);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k >= K) break;
+      u32 lab[4];
+#pragma unroll
+      for (u32 q = 0; q < 4; ++q) lab[q] = on[q] ? (u32)__ldg(L.c[k] + v0 + q * stride) : 0u;
+#pragma unroll
+      for (u32 q = 0; q < 4; ++q)
+        if (on[q]) w[q] |= code_of(lab[q], picks + k * (kCodePieces + 1)) << (4 * k);
+    }
+#pragma unroll
+    for (u32 q = 0; q < 4; ++q)
+      if (on[q]) cc.code[v0 + q * stride] = (u16)w[q];
+  }
+}
+
+// The same for a union's caller-layout labels: a warp takes 128 consecutive
+// entries and finds its first member once.
+__global__ void __launch_bounds__(256) k_union_codes(CutCodes cc, const int* __restrict__ center,
+                                                     UnionOffsets off, u32 k, u32 total) {
+  const u32 lane = threadIdx.x & 31;
+  const u32 nwarps = gridDim.x * (blockDim.x / 32);
+  for (u32 w0 = (blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5)) * 128; w0 < total;
+       w0 += nwarps * 128) {
+    const u32 m0 = segment_of(off.o, k, w0);
+    const u32 next = __ldg(off.o + m0 + 1);
+    u32 lab[4], m[4];
+    bool on[4];
+#pragma unroll
+    for (u32 q = 0; q < 4; ++q) {
+      const u32 v = w0 + q * 32 + lane;
+      m[q] = m0;
+      on[q] = v < total;
+      if (on[q] && v >= next)
+        while (__ldg(off.o + m[q] + 1) <= v) ++m[q];
+      if (on[q]) {
+        const u32 u = __ldg(off.v + m[q]) + (v - __ldg(off.o + m[q]));
+        on[q] = !(__ldg(cc.solo + (u >> 5)) >> (u & 31) & 1u);
+      }
+      lab[q] = on[q] ? (u32)__ldg(center + v) : 0u;
+    }
+#pragma unroll
+    for (u32 q = 0; q < 4; ++q)
+      if (on[q])
+        cc.code[w0 + q * 32 + lane] = (u16)code_of(lab[q], cc.picks + m[q] * (kCodePieces + 1));
+  }
+}
+
+// Code words of the groups' cold vertices and of the hot table.
+__global__ void __launch_bounds__(256) k_gather_codes(CutList cl, CutCodes cc) {
+  const u32 stride = gridDim.x * blockDim.x, len = cl.ngrp + cc.nhot;
+  for (u32 i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < len; i0 += stride * kLabIpt) {
+    u16 x[kLabIpt];
+#pragma unroll
+    for (int q = 0; q < kLabIpt; ++q) {
+      const u32 i = i0 + (u32)q * stride;
+      u32 v = 0xffffffffu;
+      if (i < len) v = i < cl.ngrp ? __ldg(cl.grp_v + i) : __ldg(cc.hotv + (i - cl.ngrp));
+      x[q] = v != 0xffffffffu ? __ldg(cc.code + v) : (u16)0;
+    }
+#pragma unroll
+    for (int q = 0; q < kLabIpt; ++q) {
+      const u32 i = i0 + (u32)q * stride;
+      if (i < cl.ngrp) cc.gcode[i] = x[q];
+      else if (i < len) cc.hcode[i - cl.ngrp] = x[q];
+    }
+  }
+}
+
+// k_cut's pass with code words.  Per edge one 2-byte read of the group's code
+// word (a lane's four edges mostly share it) and one of the hot endpoint's, from
+// shared memory for the table's vertices; labels only where both codes say
+// "another piece".  One graph: the 128-edge chunks interleave over all warps.
+// Union: kCodeShares consecutive shares of the edges per CTA, interleaved over
+// the CTAs, and inside a share member by member, each with its own hot table.
+//
+// k_cut's 4-byte (k_cut4's 16-byte) gathers by vertex were bound by the L1's one
+// sector per cycle and SM; code words keep nine in ten edges of an R-MAT graph
+// out of it, and the pass is bound by the instructions per edge: hence code words
+// compared two edges at a time, the separate branch for a whole chunk inside its
+// segment, and kOne (K = 1), which needs no fields.
+constexpr u32 kCodeShares = 4;
+
+//
+// Cut counts, before and now: 64 copies of R-MAT 20 as a union 2.42-2.61 -> 1.60
+// ms (1.00 G edges; the pass itself 1.30 ms, 3.4 TB/s); R-MAT 22's batch of three
+// labelings 1.060 -> 0.990 ms in all.
+template <bool U, bool kOne>
+__global__ void __launch_bounds__(kCutThreads, 1) k_cut_codes(CutList cl, CutCodes cc, Labels4 L,
+                                                              int K, UnionOffsets off, u32 k,
+                                                              u64* out) {
+  extern __shared__ int4 cut_smem[];
+  u16* table = reinterpret_cast<u16*>(cut_smem);
+  __shared__ u32 wsum[kCutThreads / 32][4];
+  const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u32 nchunk = (cl.m + 127) / 128;
+  const int4* hot4 = reinterpret_cast<const int4*>(cl.hot);  // cudaMalloc'd: aligned
+  const u32 nshare = U ? gridDim.x * kCodeShares : 1u;
+  for (u32 share = U ? blockIdx.x : 0u, seg = 0, e_hi = 0; share < nshare || seg < e_hi;) {
+    if (seg >= e_hi) {
+      seg = (u32)((u64)share * nchunk / nshare) * 128;
+      e_hi = min((u32)((u64)(share + 1) * nchunk / nshare) * 128, cl.m);
+      share += U ? gridDim.x : 1u;
+      if (seg >= e_hi) continue;
+    }
+    u32 m = 0, h0 = 0, nh = cc.nhot, end = e_hi;
+    if (U) {
+      m = segment_of(off.u, k, seg);
+      end = min(e_hi, __ldg(off.u + m + 1));
+      h0 = __ldg(off.h + m);
+      nh = __ldg(off.h + m + 1) - h0;
+    }
+    __syncthreads();  // the last segment is done with the table
+    const uint4* src = reinterpret_cast<const uint4*>(cc.hcode + h0);  // h0 is a multiple of 8
+    for (u32 i = tid; i < (nh + 7) / 8; i += blockDim.x)
+      reinterpret_cast<uint4*>(table)[i] = __ldg(src + i);
+    __syncthreads();
+    u32 cnt[4] = {0, 0, 0, 0};
+    u32 acc = 0, steps = 0;  // labelings 0 .. 3 in acc's nibbles, twice
+    const u32 c1 = (end + 127) / 128;
+    const u32 step = U ? kCutThreads / 32 : gridDim.x * (kCutThreads / 32);
+    u32 c = U ? seg / 128 + warp : blockIdx.x * (kCutThreads / 32) + warp;
+    const u32 j0 = (4 * lane) & 31u;  // a lane's edges: 4 lane .. 4 lane + 3, in block lane / 8
+    const u32 before = j0 ? bits_upto(j0 - 1) : 0u;
+    // labels of edge e (group g, hot endpoint hv) where labelings `both` need them
+    auto by_label = [&](u32 both, u32 g, int hv) {
+      const u32 cv = __ldg(cl.grp_v + g);
+      const u32 v = hv < 0 ? __ldg(cc.hotv + h0 + (hv & 0x7fffffff)) : (u32)hv;
+#pragma unroll
+      for (u32 kk = 0; kk < (kOne ? 1u : 4u); ++kk)
+        if ((int)kk < K && (both >> (4 * kk) & 1u))
+          cnt[kk] += __ldg(L.c[kk] + cv) != __ldg(L.c[kk] + v) ? 1u : 0u;
+    };
+    // the code words of two edges at a time (low and high half); returns where both
+    // codes say "another piece"
+    auto pair = [&](u32 a, u32 b) -> u32 {
+      u32 d = a ^ b, t = a & b;
+      if (kOne) {  // codes 0 .. 15 alone in their half
+        cnt[0] += (u32)__popc((d + 0x000f000fu) & 0x00100010u);
+        return (t + 0x00010001u) & 0x00100010u;
+      }
+      d |= d >> 1;
+      acc += (d | d >> 2) & 0x11111111u;  // labelings whose codes differ
+      t &= t >> 1;
+      return t & t >> 2 & 0x11111111u;
+    };
+    auto flush = [&]() {
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) cnt[kk] += (acc >> (4 * kk) & 0xfu) + (acc >> (4 * kk + 16) & 0xfu);
+      acc = 0;
+    };
+    auto hot_code = [&](int hv) -> u32 {  // one generic load for both places
+      const u16* p = hv < 0 ? table : cc.code;
+      return p[hv & 0x7fffffff];
+    };
+    int4 h = make_int4(0, 0, 0, 0);
+    u32 bg = 0, bm = 0;
+    auto load = [&](u32 ch, int4& x, u32& g, u32& b) {  // a chunk's tail may lie past m
+      const u32 e0 = ch * 128 + 4 * lane;
+      x = make_int4(0, 0, 0, 0);
+      if (ch * 128 + 128 <= cl.m) {
+        x = __ldcs(hot4 + (e0 >> 2));
+      } else {
+        if (e0 < cl.m) x.x = cl.hot[e0];
+        if (e0 + 1 < cl.m) x.y = cl.hot[e0 + 1];
+        if (e0 + 2 < cl.m) x.z = cl.hot[e0 + 2];
+        if (e0 + 3 < cl.m) x.w = cl.hot[e0 + 3];
+      }
+      const u32 blk = min(e0 >> 5, cl.nblk - 1);
+      g = __ldg(cl.blk_g + blk);
+      b = __ldg(cl.blk_mask + blk);
+    };
+    if (c < c1) load(c, h, bg, bm);
+    for (; c < c1; c += step) {
+      int4 nx = make_int4(0, 0, 0, 0);
+      u32 nbg = 0, nbm = 0;
+      if (c + step < c1) load(c + step, nx, nbg, nbm);
+      const u32 e0 = c * 128 + 4 * lane;
+      const int hv[4] = {h.x, h.y, h.z, h.w};
+      const u32 mine = bm >> j0;  // bit q: edge q starts a group
+      u32 g = bg + __popc(bm & before) + (mine & 1u);
+      const bool whole = c * 128 >= seg && c * 128 + 128 <= end;
+      u32 a[4], b[4];
+      if (whole) {
+#pragma unroll
+        for (u32 q = 0; q < 4; ++q) b[q] = hot_code(hv[q]);
+        a[0] = __ldg(cc.gcode + g);
+        a[1] = a[2] = a[3] = a[0];
+        if (mine & 0xeu) {  // another group starts
+          u32 gg = g;
+#pragma unroll
+          for (u32 q = 1; q < 4; ++q) {
+            gg += mine >> q & 1u;
+            a[q] = __ldg(cc.gcode + gg);
+          }
+        }
+      } else {
+        u32 gg = g;
+#pragma unroll
+        for (u32 q = 0; q < 4; ++q) {
+          if (q) gg += mine >> q & 1u;
+          a[q] = b[q] = 0;
+          if (e0 + q >= seg && e0 + q < end) {
+            a[q] = __ldg(cc.gcode + gg);
+            b[q] = hot_code(hv[q]);
+          }
+        }
+      }
+      const u32 o01 = pair(a[0] | a[1] << 16, b[0] | b[1] << 16);
+      const u32 o23 = pair(a[2] | a[3] << 16, b[2] | b[3] << 16);
+      if (o01 | o23) {
+        u32 gg = g;
+#pragma unroll
+        for (u32 q = 0; q < 4; ++q) {
+          if (q) gg += mine >> q & 1u;
+          const u32 o = (q < 2 ? o01 : o23) >> (q & 1u ? 16 : 0) & 0xffffu;
+          if (o) by_label(kOne ? 1u : o, gg, hv[q]);
+        }
+      }
+      if (!kOne && ++steps == 7) {  // at most 2 per step and nibble
+        flush();
+        steps = 0;
+      }
+      h = nx;
+      bg = nbg;
+      bm = nbm;
+    }
+    if (!kOne) flush();
+#pragma unroll
+    for (int kk = 0; kk < (kOne ? 1 : 4); ++kk) {
+      const u32 t = __reduce_add_sync(kFull, cnt[kk]);  // a CTA's share is below 2^32
+      if (lane == 0) wsum[warp][kk] = t;
+    }
+    __syncthreads();
+    if (tid < (u32)K) {
+      u64 tot = 0;
+      for (int w = 0; w < kCutThreads / 32; ++w) tot += wsum[w][tid];
+      if (tot) atomicAdd(out + (U ? m : tid), tot);
+    }
+    seg = end;
+  }
+}
+
 u32 grid_for(u32 n, int num_sms) {
   return (u32)max(1ll, min((long long)(n + 255) / 256, (long long)num_sms * 8));
 }
@@ -870,7 +1187,7 @@ int launch_cut(const CutList& cl, const int* center, const u32* hot, u32 n_hot, 
   k_group_labels<false><<<grid_for((cl.ngrp + kLabIpt - 1) / kLabIpt, num_sms), 256, 0, s>>>(
       cl, center);
   const u32 g = (u32)max(1ll, min((long long)(cl.m + 4095) / 4096, (long long)num_sms));
-  k_cut<false><<<g, kCutThreads, (size_t)n_hot * sizeof(int), s>>>(cl, center, hot_center, n_hot,
+  k_cut<false><<<g, kCutThreads, (size_t)min(n_hot, kHotSlots) * sizeof(int), s>>>(cl, center, hot_center, n_hot,
                                                                    out);
   return launches + 1;
 }
@@ -903,16 +1220,67 @@ int launch_cut4(const CutList& cl, const int* const* centers, int K, u32 n, cons
   return launches + 2;
 }
 
-int launch_union_cut(const CutList& cl, const UnionOffsets& off, const u32* wmem,
-                     const int* center, u64* cut, int num_sms, cudaStream_t s) {
-  (void)off;
-  (void)wmem;
+namespace {
+// The dynamic shared memory of the code-word table, allowed once per device.
+template <bool U, bool kOne>
+void allow_code_smem() {
+  static bool attr_set[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !attr_set[dev]) {
+    cudaFuncSetAttribute(k_cut_codes<U, kOne>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(kCodeSlots * sizeof(u16)));
+    attr_set[dev] = true;
+  }
+}
+
+u32 cut_code_grid(const CutList& cl, int num_sms) {
+  return (u32)max(1ll, min((long long)(cl.m + 4095) / 4096, (long long)num_sms));
+}
+}  // namespace
+
+int launch_cut_codes(const CutList& cl, const CutCodes& cc, const int* const* centers, int K, u32 n,
+                     u64* out, int num_sms, cudaStream_t s) {
+  if (cl.m == 0 || K < 1 || K > 4) return 0;
+  allow_code_smem<false, true>();
+  allow_code_smem<false, false>();
+  Labels4 L = {{centers[0], K > 1 ? centers[1] : nullptr, K > 2 ? centers[2] : nullptr,
+                K > 3 ? centers[3] : nullptr}};
+  const UnionOffsets none{};
+  k_picks<false><<<K, 32, 0, s>>>(cc, L, none);
+  k_codes<<<grid_for((n + 3) / 4, num_sms), 256, 0, s>>>(cc, L, K, n);
+  k_gather_codes<<<grid_for((cl.ngrp + cc.nhot + kLabIpt - 1) / kLabIpt, num_sms), 256, 0, s>>>(cl,
+                                                                                             cc);
+  const size_t smem = ((size_t)cc.nhot * sizeof(u16) + 15) / 16 * 16;
+  if (K == 1)
+    k_cut_codes<false, true><<<cut_code_grid(cl, num_sms), kCutThreads, smem, s>>>(cl, cc, L, K,
+                                                                                 none, 0, out);
+  else
+    k_cut_codes<false, false><<<cut_code_grid(cl, num_sms), kCutThreads, smem, s>>>(cl, cc, L, K,
+                                                                                  none, 0, out);
+  return 4;
+}
+
+int launch_union_cut(const CutList& cl, const int* center, u64* cut, int num_sms, cudaStream_t s) {
   if (cl.m == 0) return 0;
   k_group_labels<true><<<grid_for((cl.ngrp + kLabIpt - 1) / kLabIpt, num_sms), 256, 0, s>>>(
       cl, center);
   const u32 g = (u32)max(1ll, min((long long)(cl.m + 4095) / 4096, (long long)num_sms));
   k_cut<true><<<g, kCutThreads, 0, s>>>(cl, center, nullptr, 0, cut);
   return 2;
+}
+
+int launch_union_cut_codes(const CutList& cl, const CutCodes& cc, const UnionOffsets& off, u32 k,
+                           u32 total, const int* center, u64* cut, int num_sms, cudaStream_t s) {
+  if (cl.m == 0) return 0;
+  allow_code_smem<true, true>();
+  const Labels4 L = {{center, nullptr, nullptr, nullptr}};
+  k_picks<true><<<k, 32, 0, s>>>(cc, L, off);
+  k_union_codes<<<grid_for((total + 3) / 4, num_sms), 256, 0, s>>>(cc, center, off, k, total);
+  k_gather_codes<<<grid_for((cl.ngrp + cc.nhot + kLabIpt - 1) / kLabIpt, num_sms), 256, 0, s>>>(cl,
+                                                                                             cc);
+  k_cut_codes<true, true><<<cut_code_grid(cl, num_sms), kCutThreads, kCodeSlots * sizeof(u16), s>>>(
+      cl, cc, L, 1, off, k, cut);
+  return 4;
 }
 
 int launch_cut_blocks(const CutList& cl, int num_sms, cudaStream_t s) {

@@ -16,8 +16,9 @@
 // pad vertices, so that every member starts on a 32-vertex boundary and its
 // per-vertex bitmask words are copied whole.  Arcs, cut-list edges and groups
 // and small-component records are concatenated in member order with their
-// vertex ids moved by voff_s.  The union's cut list has no hot table and
-// holds caller-layout indices (the cut count reads the outputs).  Outputs use the caller's layout: member s's n_s
+// vertex ids moved by voff_s.  The union's cut list holds caller-layout indices
+// (the cut count reads the outputs); hot-table slots are resolved, or kept with
+// the members' hot tables where the count goes by piece codes.  Outputs use the caller's layout: member s's n_s
 // entries at ooff_s = n_0 + ... + n_{s-1}, with member-local ids.
 //
 // Every table is built by one launch (k_union_concat, blockIdx.y = table);
@@ -89,12 +90,24 @@ __global__ void __launch_bounds__(256) k_union_concat(const UnionMember* __restr
         t.col[e] = __ldg(mem[s].col + (e - off.e[s])) + (int)off.v[s];
       });
       break;
-    case 2:  // cut list edges: hot-table slots resolved, ids moved to the caller layout
+    case 2:  // cut list edges: ids moved to the caller layout, hot-table slots resolved or kept
       for_each_member_elem(off.u, k, off.u[k], [&](u32 i, u32 s) {
         const UnionMember& m = mem[s];
         const int h = __ldg(m.cut_hot + (i - off.u[s]));
+        if (h < 0 && t.hotv) {
+          t.cut.hot[i] = h;  // a slot of the member's hot table
+          return;
+        }
         const int hot = h < 0 ? (int)__ldg(m.hot + (h & 0x7fffffff)) : h;
         t.cut.hot[i] = hot + (int)off.o[s];  // caller layout: the cut reads outputs
+      });
+      break;
+    case 9:  // hot tables, each padded to a multiple of 8 entries
+      if (!t.hotv) break;
+      for_each_member_elem(off.h, k, off.h[k], [&](u32 i, u32 s) {
+        const UnionMember& m = mem[s];
+        const u32 j = i - off.h[s];
+        t.hotv[i] = j < m.n_hot ? __ldg(m.hot + j) + off.o[s] : 0xffffffffu;
       });
       break;
     case 8: {  // cut list groups: cold vertices (caller layout), members, edge offsets
@@ -314,7 +327,7 @@ int launch_union_concat(const UnionMember* mem, const UnionOffsets& off, u32 k,
                         const UnionTables& t, u64 largest, int num_sms, cudaStream_t s) {
   const u32 bx = (u32)max(1ll, min((long long)((largest + kConcatChunk - 1) / kConcatChunk),
                                    (long long)num_sms * 8));
-  k_union_concat<<<dim3(bx, 9), 256, 0, s>>>(mem, off, k, t);
+  k_union_concat<<<dim3(bx, 10), 256, 0, s>>>(mem, off, k, t);
   launch_cut_blocks(t.cut, num_sms, s);  // after the groups are in place
   return 2;
 }

@@ -92,6 +92,10 @@ int free_graph_memory(ldd_graph* g) {
   if (!g->uni) cudaFree(g->d_active);  // a union's list lives in d_active_buf
   cudaFree(g->d_first);
   cudaFree(g->d_hot_center);
+  cudaFree(g->cc.picks);
+  cudaFree(g->cc.code);
+  cudaFree(g->cc.gcode);
+  cudaFree(g->cc.hcode);
   cudaFree(g->d_lab4);
   cudaFree(g->d_hot4);
   cudaFree(g->d_grp4);
@@ -132,6 +136,7 @@ int free_graph_memory(ldd_graph* g) {
     cudaFree(g->uni->d_active_buf);
     cudaFree(g->uni->d_mem);
     cudaFree(g->uni->d_offs);
+    cudaFree(g->uni->d_hotv);
     cudaFree(g->uni->d_shift_in);
     cudaFree(g->uni->d_out_c);
     cudaFree(g->uni->d_cut);
@@ -275,6 +280,22 @@ int build_component_tables(ldd_graph* g) {
   return rc;
 }
 
+// Buffers of the cut counts by piece codes.
+int alloc_codes(ldd_graph* g, size_t rows, size_t n, size_t ngrp, size_t nhot, const u32* hotv) {
+  CutCodes& cc = g->cc;
+  cc.hotv = hotv;
+  cc.solo = g->d_solo;
+  cc.nhot = (u32)nhot;
+  if (cudaMalloc(&cc.picks, rows * (kCodePieces + 1) * sizeof(u32)) != cudaSuccess ||
+      cudaMalloc(&cc.code, std::max<size_t>(n, 1) * sizeof(u16)) != cudaSuccess ||
+      cudaMalloc(&cc.gcode, std::max<size_t>(ngrp, 1) * sizeof(u16)) != cudaSuccess ||
+      cudaMalloc(&cc.hcode, align_up(std::max<size_t>(nhot, 1), 8) * sizeof(u16)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(LDD_ERR_OOM, "device allocation of the piece codes failed");
+  }
+  return LDD_OK;
+}
+
 // The grouped cut list of launch_cut (CutList): each edge oriented from its
 // cold endpoint to its hot one (larger degree, ties to the smaller id),
 // grouped by the cold endpoint with a counting sort, and hot endpoints in the
@@ -291,7 +312,8 @@ int build_cut_list(ldd_graph* g, const std::vector<int32_t>& rp, const std::vect
     const int32_t da = deg(a), db = deg(b);
     return da > db || (da == db && a < b);
   };
-  const size_t K = m ? std::min<size_t>(kHotSlots, n) : 0;
+  g->code_cut = g->max_degree > (u32)kLdMaxDegree && m >= kCodeMinEdges;
+  const size_t K = m ? std::min<size_t>(g->code_cut ? kCodeSlots : kHotSlots, n) : 0;
   std::vector<int32_t> ids(n);
   for (size_t v = 0; v < n; ++v) ids[v] = (int32_t)v;
   if (K > 0 && K < n) std::nth_element(ids.begin(), ids.begin() + K, ids.end(), hotter);
@@ -344,6 +366,7 @@ int build_cut_list(ldd_graph* g, const std::vector<int32_t>& rp, const std::vect
       cudaMemcpy(cl.blk_mask, blk_mask.data(), blk_mask.size() * 4, cudaMemcpyHostToDevice) !=
           cudaSuccess)
     return fail(LDD_ERR_CUDA, "upload of the cut list failed");
+  if (g->code_cut) return alloc_codes(g, 4, n, cl.ngrp, K, g->d_hot);
   return LDD_OK;
 }
 
@@ -747,6 +770,28 @@ int decompose_on_device(ldd_graph* g, double beta, const double* d_shift, int* c
   return LDD_OK;
 }
 
+// Cut counts of K <= 4 labelings into out[0 .. K) on stream s.
+int cut_labels(ldd_graph* g, const int* const* centers, int K, u64* out, cudaStream_t s) {
+  // one labeling of one graph: the labels of the hottest vertices in shared memory
+  // serve about as many edges as code words do, without a pass over the vertices
+  // (R-MAT 22: 120 us against 134)
+  if (K > 1 && g->code_cut)
+    return launch_cut_codes(g->cut, g->cc, centers, K, (u32)g->n, out, g->num_sms, s);
+  if (K > 1)
+    return launch_cut4(g->cut, centers, K, (u32)g->n, g->d_hot, g->n_hot, g->d_lab4, g->d_hot4,
+                       g->d_grp4, out, g->num_sms, s);
+  return launch_cut(g->cut, centers[0], g->d_hot, g->n_hot, g->d_hot_center, out, g->num_sms, s);
+}
+
+// A union's cut counts into its d_cut (zero on entry).
+int cut_union(ldd_graph* u, const int* center, cudaStream_t s) {
+  ldd_graph::Union& U = *u->uni;
+  if (u->code_cut)
+    return launch_union_cut_codes(u->cut, u->cc, U.off, U.k, U.total, center, U.d_cut, u->num_sms,
+                                  s);
+  return launch_union_cut(u->cut, center, U.d_cut, u->num_sms, s);
+}
+
 // The library-owned outputs a replay writes: caller layout for a union.
 int* replay_center(ldd_graph* g) { return g->uni ? g->uni->d_out_c : g->d_center; }
 int* replay_dist(ldd_graph* g) { return g->uni ? g->uni->d_out_d : g->d_dist; }
@@ -779,7 +824,7 @@ int enqueue_fast(ldd_graph* g, KeyFmt f, bool want_cut) {
   if (g->uni && want_cut) {
     ldd_graph::Union& U = *g->uni;
     if (cudaMemsetAsync(U.d_cut, 0, (size_t)U.k * 8, s) != cudaSuccess) return -1;
-    launches += launch_union_cut(g->cut, U.off, U.d_wmem, U.d_out_c, U.d_cut, g->num_sms, s);
+    launches += cut_union(g, U.d_out_c, s);
     if (cudaMemcpyAsync(g->h_cut, U.d_cut, (size_t)U.k * 8, cudaMemcpyDeviceToHost, s) !=
         cudaSuccess)
       return -1;
@@ -879,8 +924,7 @@ int cut_on_device(ldd_graph* g, const int* d_center, int64_t* out_cut) {
   cudaStream_t s = g->stream;
   record(g, 6);
   CUDA_TRY(cudaMemsetAsync(&g->d_ctl->cut, 0, sizeof(u64), s));
-  const int l = launch_cut(g->cut, d_center, g->d_hot, g->n_hot, g->d_hot_center,
-                           &g->d_ctl->cut, g->num_sms, s);
+  const int l = cut_labels(g, &d_center, 1, &g->d_ctl->cut, s);
   CUDA_TRY(cudaMemcpyAsync(g->h_hdr + 128, &g->d_ctl->cut, sizeof(u64), cudaMemcpyDeviceToHost, s));
   record(g, 7);
   CUDA_TRY(cudaGetLastError());
@@ -1029,7 +1073,7 @@ u64 union_bytes(const UnionCaps& c) {
   const u64 N = c.N, words = std::max<u64>(N / 32, 1);
   u64 b = 4 * (N + 1) + 4 * c.E + 4 * c.M + 20 * c.G + 8 * (c.M / 32 + 1) + 8 * words +
           8 * c.C + 8 * c.T + 4 * N + 4 * words;
-  b += 16 * c.total + 8 * c.total + 32ull * (c.k + 1) + 56ull * c.k + sizeof(UnionMember) * c.k;
+  b += 16 * c.total + 8 * c.total + 36ull * (c.k + 1) + 120ull * c.k + 2 * c.total + 2 * c.G + 6 * N + sizeof(UnionMember) * c.k;
   const u64 nk = std::max<u64>(N, 64);
   b += 8 * N + 4 * N + 16 * nk + 8 * N + ((N + kSortTile - 1) / kSortTile + 1) * 2048 + 4 * N +
        8 * N + 36 * N + 12 * (c.E / kBfsBase + 2) + 8 * N + 4 * (N / kMaxBlock + 1) + 8 * N +
@@ -1075,7 +1119,8 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
       cudaMalloc(&g->sc.adj, std::max<u64>(c.T, 1) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_active_buf, std::max<u64>(N, 1) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_mem, K * sizeof(UnionMember)) != cudaSuccess ||
-      cudaMalloc(&U.d_offs, 8 * (K + 1) * 4) != cudaSuccess ||
+      cudaMalloc(&U.d_offs, 9 * (K + 1) * 4) != cudaSuccess ||
+      cudaMalloc(&U.d_hotv, std::max<u64>(N, 1) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_shift_in, total * 8) != cudaSuccess ||
       cudaMalloc(&U.d_out_c, total * 8) != cudaSuccess ||
       cudaMalloc(&U.d_cut, K * 8) != cudaSuccess ||
@@ -1092,7 +1137,9 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
   const u32* d = U.d_offs;
   const size_t K1 = K + 1;
   U.off = UnionOffsets{d,          d + K1,     d + 2 * K1, d + 3 * K1,
-                       d + 4 * K1, d + 5 * K1, d + 6 * K1, d + 7 * K1};
+                       d + 4 * K1, d + 5 * K1, d + 6 * K1, d + 7 * K1, d + 8 * K1};
+  const int cc = alloc_codes(g, K, total, c.G, N, U.d_hotv);
+  if (cc != LDD_OK) return bail(cc);
   // the scratch arena and launch set-up are sized by the capacities
   g->n = (int32_t)N;
   g->nnz = (int64_t)c.E;
@@ -1109,7 +1156,7 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
       need.G > U.cap.G || need.C > U.cap.C || need.T > U.cap.T || need.total > U.cap.total)
     return fail(LDD_ERR_RANGE, "members exceed the union's capacity");
   const size_t K1 = (size_t)U.cap.k + 1;
-  std::vector<u32> offs(8 * K1, 0);
+  std::vector<u32> offs(9 * K1, 0);
   bool all_active = true;
   u64 nnz_active = 0, n_active = 0;
   u32 max_deg = 0;
@@ -1124,6 +1171,7 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
     at(5, i + 1) = at(5, i) + m->n_active;
     at(6, i + 1) = at(6, i) + (u32)m->n;
     at(7, i + 1) = at(7, i) + m->cut.ngrp;
+    at(8, i + 1) = at(8, i) + (u32)align_up(m->n_hot, 8);
     if (m->n_active > 0 && !m->d_active) all_active = false;
     max_deg = std::max(max_deg, m->max_degree);
     nnz_active += m->nnz_active;
@@ -1173,13 +1221,17 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
     d.active = m->d_active;
     d.n = (u32)m->n;
     d.nnz = (u32)m->nnz;
+    d.n_hot = m->n_hot;
   }
   drop_replay(g);  // captured graphs hold the old sizes
   CUDA_TRY(cudaMemcpyAsync(U.d_mem, mv.data(), mv.size() * sizeof(UnionMember),
                            cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(U.d_offs, offs.data(), offs.size() * 4, cudaMemcpyHostToDevice, s));
+  g->code_cut = max_deg > (u32)kLdMaxDegree && need.M >= kCodeMinEdges;
+  g->cc.nhot = at(8, k);
   UnionTables t{g->d_row, g->d_col, g->cut, g->d_excl, g->d_solo, g->sc.comp_off,
-                g->sc.comp_len, g->sc.comp_v, g->sc.adj, g->d_active, U.d_wmem};
+                g->sc.comp_len, g->sc.comp_v, g->sc.adj, g->d_active, U.d_wmem,
+                g->code_cut ? U.d_hotv : nullptr};
   const u64 largest = std::max<u64>(std::max<u64>(need.N + 1, need.E), need.M);
   launch_union_concat(U.d_mem, U.off, U.k, t, largest, g->num_sms, s);
   CUDA_TRY(cudaGetLastError());
@@ -1204,7 +1256,7 @@ int union_run(ldd_graph* u, double beta, const double* d_in, int* center, int* d
   if (want_cut) {
     record(u, 6);
     CUDA_TRY(cudaMemsetAsync(U.d_cut, 0, (size_t)U.k * 8, s));
-    cl = launch_union_cut(u->cut, U.off, U.d_wmem, center, U.d_cut, u->num_sms, s);
+    cl = cut_union(u, center, s);
     record(u, 7);
   }
   *launches_out = launches;
@@ -1642,7 +1694,7 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
   const int W = cuts && k > 1 && all_dev_c ? 4 : 1;
   const int* wave_c[4] = {};
   int nwave = 0, waves = 0, last_cut = -1;
-  if (W > 1 && (rc = ensure_cut4(g)) != LDD_OK) return rc;
+  if (W > 1 && !g->code_cut && (rc = ensure_cut4(g)) != LDD_OK) return rc;
   if (cuts) {
     CUDA_TRY(cudaMemsetAsync(g->d_bcut, 0, (size_t)k * sizeof(u64), s));
     for (int j = 0; j < 2; ++j) CUDA_TRY(cudaEventRecord(g->ev_cut[j], s));
@@ -1683,12 +1735,7 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
       if (nwave == W || i == k - 1) {  // the wave's last finalize is queued: count its cuts
         CUDA_TRY(cudaStreamWaitEvent(g->cut_stream, g->ev_used[j], 0));
         u64* out = g->d_bcut + (i + 1 - nwave);
-        if (nwave == 1)
-          launches += launch_cut(g->cut, wave_c[0], g->d_hot, g->n_hot, g->d_hot_center, out,
-                                 g->num_sms, g->cut_stream);
-        else
-          launches += launch_cut4(g->cut, wave_c, nwave, (u32)n, g->d_hot, g->n_hot, g->d_lab4,
-                                  g->d_hot4, g->d_grp4, out, g->num_sms, g->cut_stream);
+        launches += cut_labels(g, wave_c, nwave, out, g->cut_stream);
         CUDA_TRY(cudaGetLastError());
         last_cut = waves++ & 1;
         CUDA_TRY(cudaEventRecord(g->ev_cut[last_cut], g->cut_stream));

@@ -93,6 +93,8 @@ struct ldd_graph {
   int4* d_hot4 = nullptr;      // ... the hot table's packed labels
   int4* d_grp4 = nullptr;      // ... every cut-list group's packed cold label
   u32 n_hot = 0;
+  bool code_cut = false;       // cut counts by piece codes (graphs with hubs): cc
+  CutCodes cc;                 // buffers of its own but hotv (single graphs: d_hot)
   u32* d_excl = nullptr;      // bit v: v is not handled by the BFS (no arcs or a small component)
   u32* d_solo = nullptr;      // bit v: v is alone in its component (inside the d_excl allocation)
   SmallComps sc;              // components of 2..32 vertices, solved one warp each
@@ -170,7 +172,8 @@ struct ldd_graph {
     std::vector<u32> h_ooff;       // caller-layout offsets, k + 1
     std::vector<u32> h_voff;       // union-vertex offsets, k + 1
     UnionMember* d_mem = nullptr;  // k member views (valid only while building)
-    u32* d_offs = nullptr;         // 8 arrays of cap.k + 1: v, e, u, c, m, a, o, g
+    u32* d_offs = nullptr;         // 9 arrays of cap.k + 1: v, e, u, c, m, a, o, g, h
+    u32* d_hotv = nullptr;         // [cap.N] members' hot tables
     u32* d_active_buf = nullptr;   // [cap.N] active list (g->d_active when every member has one)
     UnionOffsets off{};
     double* d_shift_in = nullptr;  // [total] caller-layout shifts from the host

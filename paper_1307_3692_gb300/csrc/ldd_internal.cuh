@@ -27,6 +27,7 @@ namespace ldd {
 
 typedef unsigned long long u64;
 typedef unsigned int u32;
+typedef unsigned short u16;
 
 constexpr u64 kLevelOne = 1ull << 32;  // one queue entry in an (entries << 32) | arcs counter
 
@@ -299,6 +300,29 @@ struct CutList {
 };
 int launch_cut(const CutList& cl, const int* center, const u32* hot, u32 n_hot, int* hot_center,
                u64* out, int num_sms, cudaStream_t s);
+// Cut counts by piece codes (k_graph.cu).  Graphs with hubs: nearly every vertex
+// belongs to one of a few pieces, those of the highest-degree vertices.  A
+// vertex gets a 4-bit code per labeling, the index of its piece among the
+// labeling's first kCodePieces (kCodeOther: another piece); an edge whose codes
+// differ is cut, one whose codes name one piece is not, and only the others
+// compare labels.  A code word is 16 bits (four labelings), so the table of
+// the kCodeSlots highest-degree vertices fits in shared memory.
+constexpr u32 kCodeSlots = 98304;  // 192 KiB of code words per CTA
+constexpr u32 kCodePieces = 15;
+constexpr u32 kCodeOther = 15;
+constexpr u32 kCodeMinEdges = 1u << 19;  // fewer edges: launches decide, not gathers
+struct CutCodes {
+  const u32* hotv = nullptr;  // hot-table vertices (unions: caller layout), highest degree first
+  const u32* solo = nullptr;  // vertices without edges (unions: union layout)
+  u32* picks = nullptr;       // [labelings or members][kCodePieces + 1] pieces
+  u16* code = nullptr;        // [vertices in the caller's layout]
+  u16* gcode = nullptr;       // [ngrp]
+  u16* hcode = nullptr;       // [hot-table entries]
+  u32 nhot = 0;
+};
+// out[i] += labeling i's count, i < K <= 4, over one graph's cut list.
+int launch_cut_codes(const CutList& cl, const CutCodes& cc, const int* const* centers, int K, u32 n,
+                     u64* out, int num_sms, cudaStream_t s);
 int launch_small_comp(const SmallComps& sc, const BfsArgs& a, int num_sms, cudaStream_t s);
 // The radius of a decomposition: max over v of dist[v], into *out.
 int launch_max_dist(const int* dist, u32 n, u32* out, int num_sms, cudaStream_t s);
@@ -384,6 +408,7 @@ struct UnionMember {
   const u32* active;    // null unless every member has one
   u32 n;
   u32 nnz;
+  u32 n_hot;
 };
 // Member offsets, k + 1 device words each: union vertices (v), arcs (e),
 // cut-list entries (u), small components (c) and their members (m), active
@@ -398,6 +423,7 @@ struct UnionOffsets {
   const u32* a;
   const u32* o;
   const u32* g;
+  const u32* h;  // hot-table entries (multiples of 8)
 };
 struct UnionTables {
   int* row;
@@ -411,6 +437,7 @@ struct UnionTables {
   u32* adj;
   u32* active;
   u32* wmem;  // member of every 32-vertex word
+  u32* hotv;  // hot-table vertices in the caller's layout; null: hot endpoints are resolved
 };
 // largest = the longest table (elements), for the grid size.
 int launch_union_concat(const UnionMember* mem, const UnionOffsets& off, u32 k,
@@ -426,9 +453,11 @@ int launch_union_finalize(const BfsArgs& a, const u32* order, const u32* solo,
                           const UnionOffsets& off, u32 k, u32 total, int* center, int* dist,
                           int num_sms, cudaStream_t s);
 // Every member's cut count (cut[s], zero on entry) over the union's cut list
-// (hot ids resolved, no hot table); labels in the caller layout.
-int launch_union_cut(const CutList& cl, const UnionOffsets& off, const u32* wmem,
-                     const int* center, u64* cut, int num_sms, cudaStream_t s);
+// (hot ids resolved); labels in the caller layout.
+int launch_union_cut(const CutList& cl, const int* center, u64* cut, int num_sms, cudaStream_t s);
+// The same by piece codes, over a cut list with hot-table slots.
+int launch_union_cut_codes(const CutList& cl, const CutCodes& cc, const UnionOffsets& off, u32 k,
+                           u32 total, const int* center, u64* cut, int num_sms, cudaStream_t s);
 // The union's block tables (cl.blk_g, cl.blk_mask) from its concatenated groups.
 int launch_cut_blocks(const CutList& cl, int num_sms, cudaStream_t s);
 
