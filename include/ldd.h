@@ -259,8 +259,9 @@ int ldd_block_decompose(ldd_graph* g, int k, const double* betas, const double* 
  * A server owns `slots` workspaces (union graphs of fixed capacity, bought
  * with the HBM budget) and one worker thread per workspace.  Requests --
  * (graph, beta, shifts, output buffers), any mix of graphs -- queue in arrival
- * order.  A free worker takes every waiting request that still fits its
- * workspace (the admission test: the requests' device footprint -- vertices,
+ * order.  A free worker takes the first waiting request and every other one
+ * of its kind (graphs whose rows have at most 32 arcs, or the others) that still
+ * fits its workspace (the admission test: the requests' device footprint -- vertices,
  * arcs, cut-list entries, small components -- against the workspace's
  * capacities) and decomposes them as one disjoint union (see
  * ldd_create_union): exactly the per-request results, computed together.
@@ -432,8 +433,10 @@ int ldd_set_timing(ldd_graph* g, int enable);
  * result; each changes only speed.
  */
 typedef struct {
-  int32_t bfs_blocks_per_sm; /* CTAs of the persistent round loop per SM (1 or 2) */
-  int32_t pull_alpha;        /* go bottom-up when frontier arcs x alpha > unsettled arcs */
+  int32_t bfs_blocks_per_sm; /* CTAs of the persistent round loop per SM (1 or 2); by default
+                                1, and 2 in a union with rows of more than 32 arcs */
+  int32_t pull_alpha;        /* go bottom-up when frontier arcs x alpha > unsettled arcs;
+                                until it is changed, low-degree rounds stay top-down */
   int32_t pull_beta;         /* back to top-down when frontier vertices x beta < BFS vertices */
   int32_t pull_gamma;        /* ... and bottom-up only when frontier arcs x gamma > BFS vertices */
   int32_t probe_min_arcs;    /* top-down rounds with at least this many arcs read a key
@@ -445,7 +448,7 @@ typedef struct {
   int32_t window_levels;     /* low-degree rounds: levels relaxed between two grid barriers
                                 (each CTA going on with the vertices it reaches; exact, but a
                                 vertex may be expanded twice); 0 or 1: one level per barrier;
-                                8 by default */
+                                8 by default, 1 in a union (four until it is changed) */
   int32_t window_max_frontier; /* ... a window only while the frontier has at most this many
                                 vertices (>= 0; 2^18 by default) */
   int32_t window_queue;      /* ... entries of a CTA's local queue per level: 0 for as many

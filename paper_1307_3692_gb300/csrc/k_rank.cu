@@ -77,49 +77,6 @@ __device__ __forceinline__ void finish_split(u32 err, int amax, Control* ctl) {
 }
 
 // ---------------------------------------------------------------- direct keys
-// Adds one to the count of floor value a for every lane with take set, one
-// atomic per distinct a in the warp; floors below kRBins go to the CTA's
-// shared histogram.  A floor beyond the table (a + 2 > cap) sets kErrBucketCap.
-__device__ __forceinline__ void count_floor(int a, bool take, u32* sh, u32* acnt, u32 cap,
-                                            u32& err) {
-  const u32 act = __ballot_sync(kFull, take);
-  if (!act) return;
-  const u32 peers = __match_any_sync(kFull, take ? (u32)a : 0xffffffffu) & act;
-  if (take && (peers & lanemask_lt()) == 0) {
-    const u32 c = (u32)__popc(peers);
-    if ((u32)a < kRBins) atomicAdd(&sh[a], c);
-    else if ((u64)(u32)a + 2 <= cap) atomicAdd(acnt + a, c);
-    else err |= kErrBucketCap;
-  }
-}
-
-// floor(d), and the complement of the leading cb bits of the fraction
-// (floor(f * 2^cb), cb <= kMaxCodeBits, so larger fractions get smaller codes),
-// from the bits of d.  A bad shift gets floor 0 and an error bit (split_bits).
-__device__ __forceinline__ u64 split_code(double d, u32 cb, u32& err, int& a) {
-  constexpr u64 kMan = (1ull << 52) - 1;
-  const u64 b = (u64)__double_as_longlong(d);
-  const u32 ex = (u32)(b >> 52);  // with the sign bit
-  const u64 M = (b & kMan) | (1ull << 52);
-  u64 top = 0;  // floor(f * 2^cb)
-  a = 0;
-  if (ex - 1023u < 31u) {  // 1 <= d < 2^31: d = M * 2^(E - 52)
-    const u32 E = ex - 1023u;
-    a = (int)(M >> (52 - E));
-    top = (M << (12 + E)) >> (64 - cb);  // the 52 - E fraction bits, left-aligned
-  } else if (ex < 1023u) {  // d < 1: f = d (a subnormal's code is 0)
-    const u32 sh = 1023u + 52u - cb - ex;
-    top = sh >= 64 ? 0ull : M >> sh;
-  } else if (ex == 0x7ffu && (b & kMan)) {
-    err |= kErrShiftArg;  // NaN
-  } else if (ex >= 0x800u) {
-    if (b << 1) err |= kErrShiftArg;  // negative or NaN; -0 is +0
-  } else {
-    err |= kErrShiftRange;  // >= 2^31 or +inf
-  }
-  return ~top & ((1ull << cb) - 1);
-}
-
 // The only pass over the shifts (vertices u0 .. n-1 per launch; one launch per
 // chunk while the shifts are still arriving, u0 a multiple of kMaxBlock): every
 // vertex's direct key, the counts of the floors among the vertices the BFS
@@ -136,6 +93,12 @@ __device__ __forceinline__ u64 split_code(double d, u32 cb, u32& err, int& a) {
 // sectors.  Keys and buckets, before and now: 256^3 grid 1236 -> 149 us, R-MAT
 // 22 145-168 -> 32-42 us, 64 copies of R-MAT 20 as a union 3700 -> 410 us (and
 // its lifts 1300 -> 200), 1000^2 grid 81 -> 32 us.
+//
+// Then bound by instruction issue (119 per 32 vertices of a union, issue slots 55
+// % busy at 2.5 TB/s): the split works on one fixed-point word, the floors are
+// counted without grouping equal ones, and a warp whose vertices belong to one
+// member (nearly all) reads the member's offsets once: 64 copies of R-MAT 20 408 -> 237 us (and the
+// lifts' pass alike), 256^3 grid 149 -> 73 us, R-MAT 22 32-42 -> 28-36 us.
 constexpr int kDirectIpt = kMaxBlock / 32;
 
 template <bool U>
@@ -153,59 +116,90 @@ __global__ void __launch_bounds__(256) k_direct(const double* __restrict__ delta
   for (u32 i = tid; i < kRBins; i += blockDim.x) sh[i] = 0;
   if (tid == 0) s_ab = 0;
   __syncthreads();
-  int amax = 0;
-  u32 err = 0, ab = 0;  // ab: largest handled floor of this warp's blocks, plus one
+  u32 amax = 0, err = 0, ab = 0;  // ab: largest handled floor of this warp's blocks, plus one
+  const u32 code_shift = 32 - f.cb;
   const u32 stride = gridDim.x * (blockDim.x / 32) * kMaxBlock;
   for (u32 wb = u0 + (blockIdx.x * (blockDim.x / 32) + (tid >> 5)) * kMaxBlock; wb < n;
        wb += stride) {
     double d[kDirectIpt];
-    u32 id[kDirectIpt], ex[kDirectIpt];
-    int lf[kDirectIpt];
+    u32 id[kDirectIpt], ex[kDirectIpt], lf[kDirectIpt];
     bool live[kDirectIpt];
+    u32 m0 = 0, m1 = 0;  // the members of the first and last word
+    if (U) {
+      m0 = __ldg(wmem + (wb >> 5));
+      m1 = __ldg(wmem + (min(wb + kMaxBlock, n) - 1) / 32);
+    }
+    if (!U || m0 == m1) {
+      u32 base = 0, at = 0, size = n, lift0 = 0;
+      if (U) {
+        base = __ldg(voff + m0);
+        at = __ldg(ooff + m0);
+        size = __ldg(ooff + m0 + 1) - at;
+        lift0 = (u32)__ldg(lift + m0);
+      }
+#pragma unroll
+      for (int k = 0; k < kDirectIpt; ++k) {
+        id[k] = wb + (u32)k * 32 + lane - base;
+        live[k] = id[k] < size;  // else a pad, or past the end
+        if (!U) live[k] = live[k] && id[k] < n;
+        lf[k] = lift0;
+        d[k] = live[k] ? __ldcs(delta + at + id[k]) : 0.0;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < kDirectIpt; ++k) {
+        const u32 u = wb + (u32)k * 32 + lane;
+        live[k] = u < n;
+        id[k] = lf[k] = 0;
+        d[k] = 0.0;
+        if (live[k]) {
+          const u32 m = __ldg(wmem + (u >> 5)), o = __ldg(ooff + m);
+          id[k] = u - __ldg(voff + m);
+          live[k] = o + id[k] < __ldg(ooff + m + 1);
+          lf[k] = (u32)__ldg(lift + m);
+          if (live[k]) d[k] = __ldcs(delta + o + id[k]);
+        }
+      }
+    }
 #pragma unroll
     for (int k = 0; k < kDirectIpt; ++k) {
-      const u32 u = wb + (u32)k * 32 + lane;
-      live[k] = u < n;
-      ex[k] = live[k] ? __ldg(excl + (u >> 5)) : 0xffffffffu;
-      id[k] = u;
-      lf[k] = 0;
-      u32 at = u;
-      if (U && live[k]) {
-        const u32 m = __ldg(wmem + (u >> 5)), o = __ldg(ooff + m);
-        id[k] = u - __ldg(voff + m);
-        at = o + id[k];
-        live[k] = at < __ldg(ooff + m + 1);  // else a pad
-        lf[k] = __ldg(lift + m);
-      }
-      d[k] = live[k] ? __ldcs(delta + at) : 0.0;
+      const u32 word = (wb >> 5) + (u32)k;
+      ex[k] = word * 32 < n ? __ldg(excl + word) : 0xffffffffu;
     }
     u32 top = 0;
 #pragma unroll
     for (int k = 0; k < kDirectIpt; ++k) {
-      int a;
-      const u64 code = split_code(d[k], f.cb, err, a);
-      a += lf[k];
-      const bool own = live[k] && !((ex[k] >> lane) & 1u);
-      if (live[k]) {
-        amax = max(amax, a);
-        if ((u32)a > f.cap) err |= kErrLevelCap;
-        key[wb + (u32)k * 32 + lane] =
-            level_key(f, f.cap - (u32)a) | (code << f.ib) | id[k];
+      bool ok;
+      const u64 x = fixed_shift(d[k], &ok);
+      if (!ok) {
+        int a;
+        u64 fb;
+        split_bits(d[k], err, a, fb);
+        continue;
       }
-      if (own) top = max(top, (u32)a + 1u);
-      count_floor(a, own, sh, acnt, cap, err);
+      if (!live[k]) continue;
+      const u32 a = (u32)(x >> 32) + lf[k];
+      amax = max(amax, a);
+      key[wb + (u32)k * 32 + lane] =
+          level_key(f, f.cap - a) | ((u64)(~(u32)x >> code_shift) << f.ib) | id[k];
+      if ((ex[k] >> lane) & 1u) continue;
+      top = max(top, a + 1u);
+      if (a < kRBins) atomicAdd(&sh[a], 1u);
+      else if ((u64)a + 2 <= cap) atomicAdd(acnt + a, 1u);
+      else err |= kErrBucketCap;
     }
     top = __reduce_max_sync(kFull, top);
     ab = max(ab, top);
     if (lane == 0) bmax[wb / kMaxBlock] = top;
   }
+  if (amax > f.cap) err |= kErrLevelCap;
   if (lane == 0 && ab) atomicMax(&s_ab, (int)ab - 1);
   __syncthreads();
   for (u32 i = tid; i < kRBins; i += blockDim.x)
     if (sh[i] && (u64)i + 2 <= cap) atomicAdd(acnt + i, sh[i]);
     else if (sh[i]) err |= kErrBucketCap;
   if (tid == 0 && s_ab) atomicMax(&ctl->Ab, s_ab);
-  finish_split(err, amax, ctl);
+  finish_split(err, (int)min(amax, 0x7fffffffu), ctl);
 }
 
 // ---------------------------------------------------------------- exact path

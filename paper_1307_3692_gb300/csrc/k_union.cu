@@ -162,16 +162,6 @@ __global__ void __launch_bounds__(256) k_union_concat(const UnionMember* __restr
   }
 }
 
-// floor(d) of a valid shift (finite, 0 <= d < 2^31), from the bits of d; 0
-// for anything else (the rank's split rejects those shifts).
-__device__ __forceinline__ int floor_of(double d) {
-  const u64 b = (u64)__double_as_longlong(d);
-  const u32 ex = (u32)(b >> 52) & 0x7ffu;
-  if ((b >> 63) || ex < 1023u || ex >= 1023u + 31u) return 0;
-  const u64 M = (b & ((1ull << 52) - 1)) | (1ull << 52);
-  return (int)(M >> (52 - (ex - 1023u)));
-}
-
 // Into amax[s] (zero on entry) the largest floor among member s's vertices that
 // the round loop handles (excl bit clear): isolated vertices and small
 // components never enter the rounds, so they must not set the alignment.
@@ -183,34 +173,49 @@ constexpr int kSpreadIpt = 8;
 
 __global__ void __launch_bounds__(256) k_union_amax(const double* __restrict__ in,
                                                     UnionOffsets off, u32 k,
-                                                    const u32* __restrict__ excl, int* amax) {
+                                                    const u32* __restrict__ excl,
+                                                    const u32* __restrict__ wmem, int* amax) {
   const u32 N = off.v[k];
   const u32 lane = threadIdx.x & 31;
   const u32 span = 32u * kSpreadIpt;
   const u32 nwarps = gridDim.x * (blockDim.x / 32);
   for (u32 wb0 = (blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5)) * span; wb0 < N;
        wb0 += nwarps * span) {
-    u32 sm[kSpreadIpt];
     double d[kSpreadIpt];
-    u32 m = member_of(off.v, k, wb0);
+    u32 sm[kSpreadIpt];
+    const u32 m0 = __ldg(wmem + (wb0 >> 5)), m1 = __ldg(wmem + (min(wb0 + span, N) - 1) / 32);
+    if (m0 == m1) {
+      const u32 v0 = wb0 - __ldg(off.v + m0), o = __ldg(off.o + m0);
+      const u32 n = __ldg(off.o + m0 + 1) - o;
 #pragma unroll
-    for (int q = 0; q < kSpreadIpt; ++q) {
-      const u32 wb = wb0 + (u32)q * 32;
-      if (wb < N)
-        while (__ldg(off.v + m + 1) <= wb) ++m;
-      sm[q] = m;
-      const u32 v = wb + lane - off.v[m];
-      const u32 n = off.o[m + 1] - off.o[m];
-      d[q] = (wb < N && v < n && !((__ldg(excl + (wb >> 5)) >> lane) & 1u))
-                 ? __ldcg(in + off.o[m] + v) : 0.0;
+      for (int q = 0; q < kSpreadIpt; ++q) {
+        const u32 v = v0 + (u32)q * 32 + lane;
+        d[q] = v < n ? __ldcg(in + o + v) : 0.0;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < kSpreadIpt; ++q) {
+        const u32 wb = wb0 + (u32)q * 32;
+        d[q] = 0.0;
+        sm[q] = 0xffffffffu;
+        if (wb >= N) continue;
+        sm[q] = __ldg(wmem + (wb >> 5));
+        const u32 v = wb + lane - __ldg(off.v + sm[q]), o = __ldg(off.o + sm[q]);
+        if (v < __ldg(off.o + sm[q] + 1) - o) d[q] = __ldcg(in + o + v);
+      }
     }
     u32 best = 0;
 #pragma unroll
     for (int q = 0; q < kSpreadIpt; ++q) {
-      best = max(best, (u32)floor_of(d[q]));
-      if (q + 1 == kSpreadIpt || sm[q + 1] != sm[q]) {  // warp-uniform
+      const u32 word = (wb0 >> 5) + (u32)q;
+      const u32 ex = word * 32 < N ? __ldg(excl + word) : 0xffffffffu;
+      bool ok;
+      const u64 x = fixed_shift(d[q], &ok);  // a bad shift counts as 0: k_direct rejects it
+      if (ok && !((ex >> lane) & 1u)) best = max(best, (u32)(x >> 32));
+      const bool last = q + 1 == kSpreadIpt || (m0 != m1 && sm[q + 1] != sm[q]);  // warp-uniform
+      if (last) {
         best = __reduce_max_sync(0xffffffffu, best);
-        if (lane == 0 && best > 0) atomicMax(amax + sm[q], (int)best);
+        if (lane == 0 && best > 0) atomicMax(amax + (m0 == m1 ? m0 : sm[q]), (int)best);
         best = 0;
       }
     }
@@ -333,10 +338,10 @@ int launch_union_concat(const UnionMember* mem, const UnionOffsets& off, u32 k,
 }
 
 int launch_union_lift(const double* in, const UnionOffsets& off, u32 k, u32 N, const u32* excl,
-                      int* amax, int* lift, u64* mlow, u64* mpivot, int num_sms, cudaStream_t s) {
+                      const u32* wmem, int* amax, int* lift, u64* mlow, u64* mpivot, int num_sms, cudaStream_t s) {
   cudaMemsetAsync(amax, 0, (size_t)k * sizeof(int), s);
-  k_union_amax<<<blocks_for((N + kSpreadIpt - 1) / kSpreadIpt, num_sms), 256, 0, s>>>(in, off, k,
-                                                                                    excl, amax);
+  k_union_amax<<<blocks_for((N + kSpreadIpt - 1) / kSpreadIpt, num_sms), 256, 0, s>>>(
+      in, off, k, excl, wmem, amax);
   k_union_lift<<<1, 1024, 0, s>>>(amax, k, lift, mlow, mpivot);
   return 2;
 }

@@ -408,6 +408,17 @@ float elapsed(ldd_graph* g, int a, int b) {
   return ms;
 }
 
+// Low-degree rounds of a single graph relax eight levels between grid barriers
+// (deeper windows help where pieces grow slowly -- 1000^2 grid at beta 0.01, depth
+// 8 2.00 ms, 32 1.79 -- and hurt elsewhere: random geometric graph of 150,001
+// vertices, 8 0.59 ms, 16 0.79, 32 1.26).
+constexpr u32 kDefaultWindowLevels = 8;
+// Unions: one, and four where the tuning has not been touched and low-degree
+// rounds run (64 random geometric graphs: 1 level 4.37, 2 3.40, 3 3.22, 4 3.12,
+// 6 3.12, 8 3.21 ms).
+constexpr u32 kDefaultUnionWindowLevels = 1;
+constexpr u32 kLdUnionWindowLevels = 4;
+
 BfsArgs bfs_args(ldd_graph* g, KeyFmt f, const double* shift) {
   BfsArgs a;
   a.row_ptr = g->d_row;
@@ -442,7 +453,7 @@ BfsArgs bfs_args(ldd_graph* g, KeyFmt f, const double* shift) {
   a.pull_gamma = g->pull_gamma;
   a.probe_min_arcs = g->probe_min_arcs;
   a.low_degree = g->low_degree() ? 1u : 0u;
-  a.window_levels = g->window_levels;
+  a.window_levels = g->uni && !g->window_set ? kLdUnionWindowLevels : g->window_levels;
   a.window_max_q = g->window_max_q;
   a.window_queue = g->window_queue;
   a.span = g->bfs_span;
@@ -508,13 +519,6 @@ int run_bfs_finalize(ldd_graph* g, KeyFmt f, const double* shift, int* center, i
 
 constexpr u32 kDefaultBarrierPolls = 1u << 22;   // grid barrier: each poll >= 20 ns after 64
 constexpr u32 kDefaultLookbackPolls = 1u << 24;  // look-back: each poll >= 64 ns after 16
-// Low-degree rounds of a single graph relax eight levels between grid
-// barriers by default, those of a union one (ldd_autotune tries both).
-// Measured: 256^3 grid 4.0 -> 3.4 ms, 256^2 0.49 -> 0.35 ms with windows;
-// unions of random geometric graphs were as fast or faster level by level.
-constexpr u32 kDefaultWindowLevels = 8;
-constexpr u32 kDefaultUnionWindowLevels = 1;
-
 // Scratch arena, pinned header, events and launch parameters: the part of
 // graph creation that only depends on the sizes and the tables being built.
 int finish_setup(ldd_graph* g) {
@@ -549,6 +553,7 @@ int finish_setup(ldd_graph* g) {
   g->low_degree_rounds = !(ldr && ldr[0] == '0' && ldr[1] == 0);
   g->window_levels =
       env_u32("LDD_WINDOW_LEVELS", g->uni ? kDefaultUnionWindowLevels : kDefaultWindowLevels);
+  g->window_set = getenv("LDD_WINDOW_LEVELS") != nullptr;
   g->window_max_q = env_u32("LDD_WINDOW_MAX_FRONTIER", 1u << 18);
   g->stats.n = g->n;
   g->stats.nnz = g->nnz;
@@ -808,7 +813,7 @@ int enqueue_fast(ldd_graph* g, KeyFmt f, bool want_cut) {
   if (cudaMemsetAsync(g->d_status, 0, words * sizeof(u64), s) != cudaSuccess) return -1;
   if (g->uni) {
     ldd_graph::Union& U = *g->uni;
-    launches += launch_union_lift(U.d_shift_in, U.off, U.k, (u32)g->n, g->d_excl, U.d_amax,
+    launches += launch_union_lift(U.d_shift_in, U.off, U.k, (u32)g->n, g->d_excl, U.d_wmem, U.d_amax,
                                   U.d_amax + U.k, U.d_mlow, U.d_mpivot, g->num_sms, s);
   }
   u32 epoch = 0;  // the scan runs with epoch 1 on cleared status words
@@ -1247,7 +1252,7 @@ int union_run(ldd_graph* u, double beta, const double* d_in, int* center, int* d
               int* launches_out, int* cut_launches_out) {
   ldd_graph::Union& U = *u->uni;
   cudaStream_t s = u->stream;
-  int launches = launch_union_lift(d_in, U.off, U.k, (u32)u->n, u->d_excl, U.d_amax,
+  int launches = launch_union_lift(d_in, U.off, U.k, (u32)u->n, u->d_excl, U.d_wmem, U.d_amax,
                                    U.d_amax + U.k, U.d_mlow, U.d_mpivot, u->num_sms, s);
   int l = 0, rc;
   if ((rc = decompose_on_device(u, beta, d_in, center, dist, &l)) != LDD_OK) return rc;
@@ -1939,6 +1944,7 @@ int ldd_set_tuning(ldd_graph* g, const ldd_tuning* t) {
     return fail(LDD_ERR_ARG, "tuning out of range (blocks per SM 1 .. %d)", max_per_sm);
   g->per_sm_set = g->per_sm_set || g->bfs_per_sm != t->bfs_blocks_per_sm;
   g->pull_set = g->pull_set || g->pull_alpha != (u32)t->pull_alpha;
+  g->window_set = g->window_set || g->window_levels != (u32)t->window_levels;
   g->bfs_per_sm = t->bfs_blocks_per_sm;
   g->bfs_grid = g->bfs_per_sm * g->num_sms;
   g->pull_alpha = (u32)t->pull_alpha;
@@ -1998,6 +2004,16 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out) 
   };
   ldd_tuning cur;
   ldd_get_tuning(g, &cur);
+  // a field at its first value keeps following the graph if it did
+  const ldd_tuning t0 = cur;
+  const bool per0 = g->per_sm_set, pull0 = g->pull_set, window0 = g->window_set;
+  auto apply = [&](const ldd_tuning& t) {
+    const int status = ldd_set_tuning(g, &t);
+    g->per_sm_set = per0 || t.bfs_blocks_per_sm != t0.bfs_blocks_per_sm;
+    g->pull_set = pull0 || t.pull_alpha != t0.pull_alpha;
+    g->window_set = window0 || t.window_levels != t0.window_levels;
+    return status;
+  };
   float best_ms;
   int rc = measure(&best_ms);
   int max_per_sm = 1;
@@ -2039,7 +2055,7 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out) 
                      : param == 6 ? &t.low_degree_rounds : &t.bfs_span;
       if (*field == vals[i]) continue;
       *field = vals[i];
-      if ((rc = ldd_set_tuning(g, &t)) != LDD_OK) break;
+      if ((rc = apply(t)) != LDD_OK) break;
       float ms;
       if ((rc = measure(&ms)) != LDD_OK) break;
       if (ms < best_ms * 0.98f) {  // keep only a clear gain
@@ -2051,7 +2067,7 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out) 
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   g->replay = saved_replay;
-  const int rc2 = ldd_set_tuning(g, &cur);
+  const int rc2 = apply(cur);
   if (rc != LDD_OK) return rc;
   if (rc2 != LDD_OK) return rc2;
   *out = cur;

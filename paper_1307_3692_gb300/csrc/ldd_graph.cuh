@@ -140,8 +140,8 @@ struct ldd_graph {
   u32 max_degree = 0;          // largest row of the CSR (unions: of any member)
   bool low_degree_rounds = true;  // tuning: low-degree rounds when max_degree allows
   bool low_degree() const { return low_degree_rounds && max_degree <= (u32)kLdMaxDegree; }
-  // Set by the user (else bfs_per_sm and pull_alpha follow the graph).
-  bool per_sm_set = false, pull_set = false;
+  // Set by the user (else bfs_per_sm, pull_alpha and window_levels follow the graph).
+  bool per_sm_set = false, pull_set = false, window_set = false;
   // Low-degree rounds stay top-down unless the tuning says otherwise: a scan of
   // a few arcs has next to none to save, and it reads every unsettled vertex (64
   // random geometric graphs: 5.09 -> 4.60 ms).

@@ -445,7 +445,7 @@ int launch_union_concat(const UnionMember* mem, const UnionOffsets& off, u32 k,
 // Every member's floor lift (amax, lift: k ints) from the caller-layout shifts;
 // also sets the round loop's per-member tables (BfsArgs) to their start values.
 int launch_union_lift(const double* in, const UnionOffsets& off, u32 k, u32 N, const u32* excl,
-                      int* amax, int* lift, u64* mlow, u64* mpivot, int num_sms, cudaStream_t s);
+                      const u32* wmem, int* amax, int* lift, u64* mlow, u64* mpivot, int num_sms, cudaStream_t s);
 // Caller-layout shifts to the union layout (ranked keys).
 int launch_union_spread(const double* in, const UnionOffsets& off, u32 k, u32 N, double* out,
                         int num_sms, cudaStream_t s);
@@ -484,6 +484,16 @@ __device__ __forceinline__ u32 key_id(const KeyFmt& f, u64 k) { return (u32)k & 
 __device__ __forceinline__ bool key_tie(const KeyFmt& f, u64 x, u64 y) {
   const u64 d = x ^ y;
   return ((u32)(d >> 32) | ((u32)d >> f.ib)) == 0u && (u32)d != 0u;
+}
+
+// floor(d * 2^32) of a shift 0 <= d < 2^31 (*ok; -0 counts as 0): the integer part
+// in the high word, the leading 32 bits of the fraction in the low one.
+__device__ __forceinline__ u64 fixed_shift(double d, bool* ok) {
+  const u64 b = (u64)__double_as_longlong(d);
+  *ok = b < (u64)(1023 + 31) << 52 || (b << 1) == 0;
+  const u64 M = (b & ((1ull << 52) - 1)) | (1ull << 52);  // d = M * 2^(ex - 1075)
+  const int sh = 1023 + 20 - (int)((u32)(b >> 52) & 0x7ffu);
+  return sh >= 0 ? (sh < 64 ? M >> sh : 0ull) : M << -sh;  // (a subnormal: sh is large)
 }
 
 // Splits a shift d into a = floor(d) and the IEEE-754 bits of its fraction
