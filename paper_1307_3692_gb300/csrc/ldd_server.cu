@@ -5,7 +5,7 @@
 // in one FIFO queue.  Each of the server's slots is a worker thread that owns
 // a union workspace (a disjoint-union graph object with fixed capacities,
 // ldd_graph.cuh) and a CUDA stream.  A free worker takes, in arrival order,
-// every waiting request that still fits its workspace -- the admission test is
+// every waiting request of the first one's kind that still fits its workspace -- the admission test is
 // the requests' device footprint: vertices, arcs, cut-list entries and small
 // components against the capacities the HBM budget bought -- and runs them as
 // one decomposition of their disjoint union (Algorithm 2 never crosses from
@@ -221,11 +221,22 @@ void worker_batched(ldd_server* S, int slot) {
       std::unique_lock<std::mutex> lk(S->mu);
       S->cv_work.wait(lk, [&] { return S->stop || !S->queue.empty(); });
       if (S->queue.empty()) return;  // stop, and nothing left
+      // Requests of one kind: a union with one graph of hubs runs edge-balanced
+      // rounds, level by level, for the hundreds of levels that its low-degree
+      // members have; apart, they run windows of levels and top-down rounds, and
+      // the others a handful of rounds.  The other kind waits for the next worker.
+      // A burst of 24 over four R-MAT graphs and four grids: 7.1-7.6 -> 4.0 ms.
       UnionCaps sum;
-      while (!S->queue.empty() && fits(sum, S->queue.front()->need, S->cap)) {
-        add_to(sum, S->queue.front()->need);
-        batch.push_back(S->queue.front());
-        S->queue.pop_front();
+      const bool kind = S->queue.front()->g->low_degree();
+      for (auto it = S->queue.begin(); it != S->queue.end();) {
+        if ((*it)->g->low_degree() != kind) {
+          ++it;
+          continue;
+        }
+        if (!fits(sum, (*it)->need, S->cap)) break;
+        add_to(sum, (*it)->need);
+        batch.push_back(*it);
+        it = S->queue.erase(it);
       }
       bid = S->next_batch++;
     }
