@@ -104,8 +104,16 @@ constexpr int kPullCoop = 4;   // neighbours per lane per step of a warp-wide sc
 // in shared memory (after Smem: 24 bytes per member, 30 KB, so that two CTAs
 // per SM still fit); larger unions use the global tables directly.
 constexpr u32 kSmemMembers = 1280;
-constexpr int kLdBatch = 8;    // low-degree rounds: arcs per frontier vertex and step
-constexpr int kLdItems = 1;    // low-degree rounds: items per thread in flight
+// Low-degree expansions give an item a thread, or eight lanes when the items then
+// still take at most this many passes of the threads (the CTA's for a local
+// queue, the grid's for the frontier).  A thread per item issues up to eight
+// atomics and pushes one after the other with few warps active, eight lanes one:
+// a level of a window with 11 items per CTA (1000 x 1000 grid) went from 3.0 to
+// 1.9 us.  With many items the divergent atomics' number is what counts, and a
+// thread per item keeps more of them in flight (256^3 grid: 2.76 ms with a thread
+// always, 2.67 with up to 2 passes, 2.79 with up to 4; 150 k geometric graph .60,
+// .46, .46 ms; two, four lanes per item in between gained nothing).
+constexpr u32 kLdGroupPasses = 2;
 
 __device__ __forceinline__ void note_tie(const BfsArgs& a, u32 w, u64 x, u64 y) {
   note_tie(a.ctl, a.f, w, x, y);
@@ -151,8 +159,8 @@ struct Smem {
   u64 pivot;             // the round's pivot
   int built;             // build_buckets: the last level filled
 };
-// Windows of levels keep two local queues whose entries carry a vertex, the
-// key it was pushed with and its adjacency range (20 bytes, as four arrays).
+// Windows of levels keep two local queues whose entries carry a vertex and the
+// key it was pushed with (12 bytes, as two arrays).
 // The first queue sits in the memory the edge-balanced rounds use for their
 // span windows.  With two CTAs per SM the second shares it; with one, which
 // has the room, it gets as much again after Smem.
@@ -160,7 +168,7 @@ constexpr size_t kSpanBytes = sizeof(int) * kBfsMaxSpan * 2 + sizeof(u64) * kBfs
 static_assert(offsetof(Smem, owner) == 0 && offsetof(Smem, rowd) < offsetof(Smem, cand) &&
                   offsetof(Smem, cand) + sizeof(u64) * (kBfsMaxSpan + 1) >= kSpanBytes,
               "the span-window arrays lead Smem and cover its first kSpanBytes bytes");
-constexpr size_t kLqEntry = sizeof(u64) + 3 * sizeof(u32);
+constexpr size_t kLqEntry = sizeof(u64) + sizeof(u32);
 constexpr int lq_cap(int per_sm) {
   return (int)((per_sm >= 2 ? kSpanBytes / 2 : kSpanBytes) / kLqEntry) / 32 * 32;
 }
@@ -172,8 +180,6 @@ __device__ __forceinline__ u32 lq_limit(const BfsArgs& a) {
 }
 struct LocalQueue {
   u64* key;
-  u32* rs;
-  u32* re;
   u32* v;
 };
 template <int kCap>
@@ -184,9 +190,7 @@ __device__ __forceinline__ LocalQueue lq_buf(Smem& s, int b) {
   else base = b == 0 ? span : reinterpret_cast<unsigned char*>(&s) + sizeof(Smem);
   LocalQueue q;
   q.key = reinterpret_cast<u64*>(base);
-  q.rs = reinterpret_cast<u32*>(q.key + kCap);
-  q.re = q.rs + kCap;
-  q.v = q.re + kCap;
+  q.v = reinterpret_cast<u32*>(q.key + kCap);
   return q;
 }
 
@@ -664,103 +668,103 @@ __device__ __forceinline__ void expand(const BfsArgs& a, Smem& s, int cur, u32 Q
   }
 }
 
+// Low-degree rounds read neighbours from the padded rows (BfsArgs::ell), a chunk
+// of eight at a time by a group of 8 / P lanes, P words (one load, two for P = 8)
+// per lane: words P * q .. of v's chunk ch, q the lane's place in its group; ~0
+// past the row's end, and all ~0 unless `on`.  Returns whether the row may go on
+// (the chunk's last word is a neighbour), the same for the group.  Every lane of
+// the warp calls this.
+template <int P>
+__device__ __forceinline__ bool ell_load(const BfsArgs& a, u32 v, u32 ch, bool on, u32 (&w)[P]) {
+  constexpr u32 G = 8 / P;
+  const u32 lane = threadIdx.x & 31;
+  if (on) {
+    const u32* p = a.ell + ((size_t)v * a.ell_s + 8 * ch + P * (lane & (G - 1)));
+    if constexpr (P == 1) {
+      w[0] = __ldg(p);
+    } else if constexpr (P == 2) {
+      const uint2 x = __ldg(reinterpret_cast<const uint2*>(p));
+      w[0] = x.x;
+      w[1] = x.y;
+    } else {
+#pragma unroll
+      for (int h = 0; h < P; h += 4) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4*>(p + h));
+        w[h] = x.x;
+        w[h + 1] = x.y;
+        w[h + 2] = x.z;
+        w[h + 3] = x.w;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < P; ++h) w[h] = ~0u;
+  }
+  if (8 * (ch + 1) >= a.ell_s) return false;  // the same for the whole grid
+  const u32 b = __ballot_sync(kFull, on && w[P - 1] != ~0u);
+  return b >> (lane | (G - 1)) & 1u;
+}
+
 // Low-degree round (every vertex of the graph has at most kLdMaxDegree
 // arcs): one pass over Q frontier vertices (the list qv_cur) and the cnt
-// entries of start bucket rb (from lo in rv), a thread per item.
-//   * A frontier vertex v offers key[v] + 2^32 to each of its neighbours
-//     (64-bit atomicMin, after a probe of the key when `probe`), kLdBatch arcs
-//     per step, and appends the neighbours whose level it lowered to lvl + 1.
+// entries of start bucket rb (from lo in rv), 8 / P lanes per item.
+//   * A frontier vertex v offers key[v], one level further out, to each of its
+//     neighbours (64-bit atomicMin, after a probe of the key when `probe`), P
+//     arcs per lane and step, and appends the neighbours whose level it lowered to lvl + 1.
 //   * A start-bucket entry u joins the next frontier if its key still has its
 //     start level rb (Section 4's delayed start; stable during the round, see
 //     the file comment).
-// v's key and adjacency range, and the bucket entries' keys, load in one round
+// v's key and first neighbours, and the bucket entries' keys, load in one round
 // trip, and the bucket test runs beside the expansion instead of after it: a
-// thin round is a short chain of dependent loads.  A thread takes kLdItems
-// items at a time (a warp 32 kLdItems consecutive ones) and interleaves their
-// loads, so that a round with more items than threads still costs about one
-// such chain.  `pushed` adds the arcs offered.
-template <bool U>
+// thin round is a short chain of dependent loads.  `pushed` adds the arcs
+// offered.
+template <bool U, int P>
 __device__ __forceinline__ void expand_ld(const BfsArgs& a, const u32* qv_cur, u32 Q, u32 lvl_next,
                                           int lo, u32 cnt, u32 rb, bool probe, int qi, int qb,
                                           u64& pushed) {
-  constexpr u32 kNone = 0xffffffffu;
-  constexpr int KI = kLdItems;
-  constexpr int KA = kLdItems * kLdBatch;
+  constexpr u32 G = 8 / P;  // lanes per item
   const u32 lane = threadIdx.x & 31;
   const u32 total = Q + cnt;
-  const u32 stride = gridDim.x * blockDim.x * KI;
-  for (u32 base = warp_first_item(KI); base < total; base += stride) {
-    u32 v[KI];
-    bool front[KI], buck[KI];
+  const u32 stride = gridDim.x * blockDim.x / G;
+  for (u32 base = warp_first_item(1) / G; base < total; base += stride) {
+    const u32 i = base + lane / G;
+    const bool front = i < Q, buck = !front && i < total && (lane & (G - 1)) == 0;
+    u32 v[1] = {0};
+    if (front) v[0] = ld_cg_u32(qv_cur + i);
+    else if (buck) v[0] = ld_cg_u32(a.rv + lo + (int)(i - Q));
+    u64 kv = 0;
+    if (front || buck) kv = ld_cg_u64(a.key + v[0]);
+    warp_append<1, true>(buck && key_level(a.f, kv) == rb ? 1u : 0u, v, a, qi, qb);
+    const u64 cand = key_up(a.f, kv);
+    bool more = front;
+    for (u32 ch = 0; __any_sync(kFull, more); ++ch) {
+      u32 w[P];
+      more = ell_load<P>(a, v[0], ch, more, w);
+      u64 cur[P];
 #pragma unroll
-    for (int t = 0; t < KI; ++t) {
-      const u32 i = base + (u32)t * 32 + lane;
-      front[t] = i < Q;
-      buck[t] = !front[t] && i < total;
-      v[t] = 0;
-      if (front[t]) v[t] = ld_cg_u32(qv_cur + i);
-      else if (buck[t]) v[t] = ld_cg_u32(a.rv + lo + (int)(i - Q));
-    }
-    u64 kv[KI];
-    int rs[KI], re[KI];
-#pragma unroll
-    for (int t = 0; t < KI; ++t) {
-      kv[t] = 0;
-      rs[t] = 0;
-      re[t] = 0;
-      if (front[t] || buck[t]) kv[t] = ld_cg_u64(a.key + v[t]);
-      if (front[t]) {
-        rs[t] = __ldg(a.row_ptr + v[t]);
-        re[t] = __ldg(a.row_ptr + v[t] + 1);
-      }
-    }
-    u32 smask = 0;
-#pragma unroll
-    for (int t = 0; t < KI; ++t) {
-      if (buck[t] && key_level(a.f, kv[t]) == rb) smask |= 1u << t;
-    }
-    warp_append<KI, true>(smask, v, a, qi, qb);
-    int nch = 0;
-#pragma unroll
-    for (int t = 0; t < KI; ++t) {
-      pushed += (u64)(re[t] - rs[t]);
-      nch = max(nch, (re[t] - rs[t] + kLdBatch - 1) / kLdBatch);
-    }
-    nch = (int)__reduce_max_sync(kFull, (u32)nch);
-    for (int ch = 0; ch < nch; ++ch) {
-      u32 w[KA];
-#pragma unroll
-      for (int t = 0; t < KI; ++t)
-#pragma unroll
-        for (int q = 0; q < kLdBatch; ++q) {
-          const int e = rs[t] + ch * kLdBatch + q;
-          w[t * kLdBatch + q] = e < re[t] ? (u32)__ldg(a.col + e) : kNone;
-        }
-      u64 cur[KA];
-#pragma unroll
-      for (int x = 0; x < KA; ++x)
+      for (int x = 0; x < P; ++x) {
+        pushed += w[x] < a.n ? 1u : 0u;
         cur[x] = (w[x] < a.n) ? (probe ? ld_cg_u64(a.key + w[x]) : ~0ull) : 0ull;
+      }
       u32 mask = 0;
 #pragma unroll
-      for (int x = 0; x < KA; ++x) {
-        const u64 cand = key_up(a.f, kv[x / kLdBatch]);
+      for (int x = 0; x < P; ++x) {
         const bool on = cand < cur[x];
         if (on) mask |= 1u << x;
         cur[x] = offer_min(a.key + (on ? w[x] : 0u), cand, on, cur[x]);
       }
 #pragma unroll
-      for (int x = 0; x < KA; ++x)
+      for (int x = 0; x < P; ++x)
         if (key_level(a.f, cur[x]) <= lvl_next) mask &= ~(1u << x);
       bool tie = false;  // one branch for the batch: meetings are rare
 #pragma unroll
-      for (int x = 0; x < KA; ++x)
-        tie |= w[x] < a.n && key_near(key_up(a.f, kv[x / kLdBatch]), cur[x]);
+      for (int x = 0; x < P; ++x) tie |= w[x] < a.n && key_near(cand, cur[x]);
       if (tie) {
 #pragma unroll
-        for (int x = 0; x < KA; ++x)
-          if (w[x] < a.n) note_tie(a, w[x], key_up(a.f, kv[x / kLdBatch]), cur[x]);
+        for (int x = 0; x < P; ++x)
+          if (w[x] < a.n) note_tie(a, w[x], cand, cur[x]);
       }
-      warp_append<KA, true>(mask, w, a, qi, qb);
+      warp_append<P, true>(mask, w, a, qi, qb);
     }
   }
 }
@@ -798,14 +802,12 @@ __device__ __forceinline__ void expand_ld(const BfsArgs& a, const u32* qv_cur, u
 // level for the next one that still holds an unclaimed vertex (one pass and
 // one grid barrier) instead of stopping when every vertex is settled.
 
-// Pushes vertex w[i] with key k[i] and adjacency range [rs[i], re[i]) for
-// every bit i of mask: to the CTA's local queue nb while it has room, the rest
-// (as vertex and level) to the overflow list of the next round.
+// Pushes vertex w[i] with the lane's key k for every bit i of mask: to the CTA's
+// local queue nb while it has room, the rest (as vertex and level) to the
+// overflow list of the next round.
 template <int K, int kCap>
-__device__ __forceinline__ void window_push(u32 mask, const u32 (&w)[K], const u64 (&k)[K],
-                                            const int (&rs)[K], const int (&re)[K],
-                                            const BfsArgs& a, Smem& s, int nb, int nc, int qi,
-                                            int qb) {
+__device__ __forceinline__ void window_push(u32 mask, const u32 (&w)[K], u64 k, const BfsArgs& a,
+                                            Smem& s, int nb, int nc, int qi, int qb) {
   const u32 lane = threadIdx.x & 31;
   u32 tot;
   const u32 excl = warp_excl_small<bits_for<K>()>(__popc(mask), &tot);
@@ -820,9 +822,7 @@ __device__ __forceinline__ void window_push(u32 mask, const u32 (&w)[K], const u
   for (int i = 0; i < K; ++i)
     if (mask >> i & 1u) {
       if (base < cap) {
-        lq.key[base] = k[i];
-        lq.rs[base] = (u32)rs[i];
-        lq.re[base] = (u32)re[i];
+        lq.key[base] = k;
         lq.v[base] = w[i];
       } else {
         spill |= 1u << i;
@@ -841,7 +841,7 @@ __device__ __forceinline__ void window_push(u32 mask, const u32 (&w)[K], const u
     if (spill >> i & 1u) {
       if (sbase < a.n) {
         reinterpret_cast<u32*>(a.qrow[qb])[sbase] = w[i];
-        a.qoff[qb][sbase] = key_level(a.f, k[i]);
+        a.qoff[qb][sbase] = key_level(a.f, k);
       } else {
         atomicOr(&a.ctl->err, kErrInternal);  // more pushes than vertices: cannot happen
       }
@@ -849,51 +849,34 @@ __device__ __forceinline__ void window_push(u32 mask, const u32 (&w)[K], const u
     }
 }
 
-// Expands one item per lane -- valid: key kv, adjacency range [rs, re) -- in a
-// window whose end is H: kv + 2^32 is offered to the neighbours.  Winners
-// below H go to the local queue nb with the key they got and their adjacency
-// range (loaded beside the atomicMin, not after it), winners at H that reach
-// it for the first time to the global queue qb.  A kv that is no longer the
-// vertex's key (it was lowered again, and its lowerer pushed it again) only
+// Expands one item per lane -- valid: vertex v with key kv -- in a window whose
+// end is H: kv, one level further out, is offered to the neighbours.  Winners
+// below H go to the local queue nb with the key they got, winners at H that
+// reach it for the first time to the global queue qb.  A kv that is no longer
+// the vertex's key (it was lowered again, and its lowerer pushed it again) only
 // makes offers that the better key dominates.  Every lane of the warp calls
 // this.
-template <bool U, int kCap>
-__device__ __forceinline__ void window_expand(const BfsArgs& a, Smem& s, bool valid, u64 kv,
-                                              int rs, int re, u32 H, int nb, int nc, int qi,
-                                              int qb, u64& pushed, u64& expanded) {
-  constexpr u32 kNone = 0xffffffffu;
-  if (!valid) re = rs;
-  else ++expanded;
-  pushed += (u64)(re - rs);
+template <bool U, int kCap, int P>
+__device__ __forceinline__ void window_expand(const BfsArgs& a, Smem& s, bool valid, u64 kv, u32 v,
+                                              u32 H, int nb, int nc, int qi, int qb, u64& pushed,
+                                              u64& expanded) {
+  if (valid && (threadIdx.x & (8 / P - 1)) == 0) ++expanded;
   const u64 cand = key_up(a.f, kv);
   const u32 cl = key_level(a.f, cand);
-  const int nch = (int)__reduce_max_sync(kFull, (u32)((re - rs + kLdBatch - 1) / kLdBatch));
-  for (int ch = 0; ch < nch; ++ch) {
-    const int e0 = rs + ch * kLdBatch;
-    u32 w[kLdBatch];
-#pragma unroll
-    for (int q = 0; q < kLdBatch; ++q) w[q] = (e0 + q < re) ? (u32)__ldg(a.col + e0 + q) : kNone;
-    u64 kk[kLdBatch];
-    int wrs[kLdBatch], wre[kLdBatch];
-    u64 met[kLdBatch];
+  bool more = valid;
+  for (u32 ch = 0; __any_sync(kFull, more); ++ch) {
+    u32 w[P];
+    more = ell_load<P>(a, v, ch, more, w);
+    u64 met[P];
     u32 local = 0, glob = 0;
 #pragma unroll
-    for (int q = 0; q < kLdBatch; ++q) {
-      kk[q] = cand;
-      wrs[q] = 0;
-      wre[q] = 0;
-      if (w[q] < a.n && cl < H) {  // the range of a vertex that may be pushed locally, beside the offer
-        wrs[q] = __ldg(a.row_ptr + w[q]);
-        wre[q] = __ldg(a.row_ptr + w[q] + 1);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < kLdBatch; ++q) {
+    for (int q = 0; q < P; ++q) {
       const bool on = w[q] < a.n;
       met[q] = offer_min(a.key + (on ? w[q] : 0u), cand, on, cand);
     }
 #pragma unroll
-    for (int q = 0; q < kLdBatch; ++q) {
+    for (int q = 0; q < P; ++q) {
+      pushed += w[q] < a.n ? 1u : 0u;
       if (met[q] > cand) {
         if (cl < H) local |= 1u << q;
         else if (key_level(a.f, met[q]) > H) glob |= 1u << q;
@@ -901,13 +884,56 @@ __device__ __forceinline__ void window_expand(const BfsArgs& a, Smem& s, bool va
     }
     bool tie = false;  // one branch for the batch: meetings are rare
 #pragma unroll
-    for (int q = 0; q < kLdBatch; ++q) tie |= key_near(cand, met[q]);
+    for (int q = 0; q < P; ++q) tie |= key_near(cand, met[q]);
     if (tie) {
 #pragma unroll
-      for (int q = 0; q < kLdBatch; ++q) note_tie(a, w[q], cand, met[q]);
+      for (int q = 0; q < P; ++q) note_tie(a, w[q], cand, met[q]);
     }
-    window_push<kLdBatch, kCap>(local, w, kk, wrs, wre, a, s, nb, nc, qi, qb);
-    warp_append<kLdBatch, true>(glob, w, a, qi, qb);
+    window_push<P, kCap>(local, w, cand, a, s, nb, nc, qi, qb);
+    warp_append<P, true>(glob, w, a, qi, qb);
+  }
+}
+
+// A window's first level: the global frontier (Q entries of side qcur) and the
+// overflow list up to item `total`, whose keys are loaded here.
+template <bool U, int kCap, int P>
+__device__ __forceinline__ void window_first(const BfsArgs& a, Smem& s, u32 Q, u32 total, int qcur,
+                                             u32 L, u32 H, int nb, int nc, int qi, int qb,
+                                             u64& pushed, u64& expanded) {
+  constexpr u32 G = 8 / P;
+  const u32 sub = (threadIdx.x & 31) / G;
+  for (u32 base = warp_first_item(1) / G; base < total; base += gridDim.x * blockDim.x / G) {
+    const u32 i = base + sub;
+    u32 v = 0, lev = L;
+    if (i < Q) {
+      v = ld_cg_u32(a.qv[qcur] + i);
+    } else if (i < total) {
+      v = ld_cg_u32(reinterpret_cast<const u32*>(a.qrow[qcur]) + (i - Q));
+      lev = ld_cg_u32(a.qoff[qcur] + (i - Q));
+    }
+    u64 kv = 0;
+    bool ok = i < total;
+    if (ok) {
+      kv = ld_cg_u64(a.key + v);
+      ok = key_level(a.f, kv) >= lev;  // lowered since: its lowerer pushed it again
+    }
+    window_expand<U, kCap, P>(a, s, ok, kv, v, H, nb, nc, qi, qb, pushed, expanded);
+  }
+}
+
+// The CTA's local queue lb: nloc entries.
+template <bool U, int kCap, int P>
+__device__ __forceinline__ void window_local(const BfsArgs& a, Smem& s, u32 nloc, int lb, u32 H,
+                                             int nb, int nc, int qi, int qb, u64& pushed,
+                                             u64& expanded) {
+  constexpr u32 G = 8 / P;
+  const LocalQueue lq = lq_buf<kCap>(s, lb);
+  const u32 sub = (threadIdx.x & 31) / G;
+  for (u32 base = (threadIdx.x & ~31u) / G; base < nloc; base += blockDim.x / G) {
+    const u32 i = base + sub;
+    const bool ok = i < nloc;
+    window_expand<U, kCap, P>(a, s, ok, ok ? lq.key[i] : 0ull, ok ? lq.v[i] : 0u, H, nb, nc, qi,
+                              qb, pushed, expanded);
   }
 }
 
@@ -965,13 +991,8 @@ __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, int lv0, in
     // it is empty: entries of overflow from an earlier window run behind the
     // frontier, and their chains end here instead of one hop per round.
     if (lv >= H && nloc == 0) break;
-    u64 pk = 0;  // its key and adjacency range
-    int pr0 = 0, pr1 = 0;
-    if (pu != kNoItem) {
-      pk = ld_cg_u64(a.key + pu);
-      pr0 = __ldg(a.row_ptr + pu);
-      pr1 = __ldg(a.row_ptr + pu + 1);
-    }
+    u64 pk = 0;  // its key
+    if (pu != kNoItem) pk = ld_cg_u64(a.key + pu);
     u32 pu2 = kNoItem;
     if (i0 < (u32)(b2hi - b2lo)) pu2 = ld_cg_u32(rv + b2lo + (int)i0);
     int b3lo = 0, b3hi = 0;
@@ -980,65 +1001,39 @@ __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, int lv0, in
       b3hi = (int)ld_cg_u32(rc + lv + 3);
     }
     // (1) the window's first level: the global frontier and the overflow list,
-    // whose keys and ranges are loaded here
+    // whose keys are loaded here
     if (lv == L) {
       const u32 total = Q + nov;
-      for (u32 base = warp_first_item(1); base < total; base += gridDim.x * blockDim.x) {
-        const u32 i = base + lane;
-        u32 v = 0, lev = L;
-        if (i < Q) {
-          v = ld_cg_u32(a.qv[qcur] + i);
-        } else if (i < total) {
-          v = ld_cg_u32(reinterpret_cast<const u32*>(a.qrow[qcur]) + (i - Q));
-          lev = ld_cg_u32(a.qoff[qcur] + (i - Q));
-        }
-        u64 kv = 0;
-        int rs = 0, re = 0;
-        bool ok = i < total;
-        if (ok) {
-          kv = ld_cg_u64(a.key + v);
-          rs = __ldg(a.row_ptr + v);
-          re = __ldg(a.row_ptr + v + 1);
-          ok = key_level(a.f, kv) >= lev;  // lowered since: its lowerer pushed it again
-        }
-        window_expand<U, kCap>(a, s, ok, kv, rs, re, H, nb, nc, qi, qb, pushed, expanded);
-      }
+      if (total <= gstride / 8 * kLdGroupPasses)
+        window_first<U, kCap, 1>(a, s, Q, total, qcur, L, H, nb, nc, qi, qb, pushed, expanded);
+      else
+        window_first<U, kCap, 8>(a, s, Q, total, qcur, L, H, nb, nc, qi, qb, pushed, expanded);
     }
-    // (2) this CTA's local queue of level lv: keys and ranges come with the entries
-    {
-      const LocalQueue lq = lq_buf<kCap>(s, lb);
-      for (u32 base = threadIdx.x & ~31u; base < nloc; base += blockDim.x) {
-        const u32 i = base + lane;
-        const bool ok = i < nloc;
-        window_expand<U, kCap>(a, s, ok, ok ? lq.key[i] : 0ull, ok ? (int)lq.rs[i] : 0,
-                               ok ? (int)lq.re[i] : 0, H, nb, nc, qi, qb, pushed, expanded);
-      }
-    }
+    // (2) this CTA's local queue of level lv: keys come with the entries
+    if (nloc <= blockDim.x / 8 * kLdGroupPasses)
+      window_local<U, kCap, 1>(a, s, nloc, lb, H, nb, nc, qi, qb, pushed, expanded);
+    else
+      window_local<U, kCap, 8>(a, s, nloc, lb, H, nb, nc, qi, qb, pushed, expanded);
     // (3) start bucket lv + 1: a vertex whose key still has its start level joins level lv + 1
     if (bucket_ok(lv + 1)) {
       const u32 cnt = (u32)(b1hi - b1lo);
       for (u32 base = i0 - lane; base < cnt; base += gstride) {  // warp-uniform
         const u32 i = base + lane;
         u32 u[1] = {0};
-        u64 k[1] = {0};
-        int urs[1] = {0}, ure[1] = {0};
+        u64 k = 0;
         bool start = false;
         if (i < cnt) {
           if (i == i0) {  // the entry read ahead
             u[0] = pu;
-            k[0] = pk;
-            urs[0] = pr0;
-            ure[0] = pr1;
+            k = pk;
           } else {
             u[0] = ld_cg_u32(rv + b1lo + (int)i);
-            k[0] = ld_cg_u64(a.key + u[0]);
-            urs[0] = __ldg(a.row_ptr + u[0]);
-            ure[0] = __ldg(a.row_ptr + u[0] + 1);
+            k = ld_cg_u64(a.key + u[0]);
           }
-          start = key_level(a.f, k[0]) == lv + 1;
+          start = key_level(a.f, k) == lv + 1;
         }
         if (lv + 1 < H) {
-          window_push<1, kCap>(start ? 1u : 0u, u, k, urs, ure, a, s, nb, nc, qi, qb);
+          window_push<1, kCap>(start ? 1u : 0u, u, k, a, s, nb, nc, qi, qb);
         } else {
           warp_append<1, true>(start ? 1u : 0u, u, a, qi, qb);
         }
@@ -1712,7 +1707,7 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
   } else {
     const int lo = __ldg(a.bptr), hi = (int)ld_cg_u32(a.rcur);
     if (LD)
-      expand_ld<U>(a, nullptr, 0, 0, lo, (u32)(hi - lo), (u32)lv0, false, 0, 0, pushed);
+      expand_ld<U, 8>(a, nullptr, 0, 0, lo, (u32)(hi - lo), (u32)lv0, false, 0, 0, pushed);
     else
       append_bucket<U>(a, lv0, lo, hi, 0, 0, mylow);
   }
@@ -1865,15 +1860,21 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
         if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
         if (lvl + 1 <= A) {
           if (LD) {
-            expand_ld<U>(a, nullptr, 0, 0, nb_lo, (u32)(nb_hi - nb_lo), (u32)lvl + 1, false, qi, qb,
-                         pushed);
+            expand_ld<U, 8>(a, nullptr, 0, 0, nb_lo, (u32)(nb_hi - nb_lo), (u32)lvl + 1, false, qi,
+                            qb, pushed);
           } else {
             append_bucket<U>(a, lvl + 1, nb_lo, nb_hi, qi, qb, mylow);
           }
         }
       } else if (LD) {  // expansion and start bucket lvl + 1 in one pass
-        expand_ld<U>(a, a.qv[phase & 1], Q, (u32)lvl + 1, nb_lo, (u32)(nb_hi - nb_lo),
-                     (u32)lvl + 1, E >= a.probe_min_arcs, qi, qb, pushed);
+        const bool probe = E >= a.probe_min_arcs;
+        const u32* qv = a.qv[phase & 1];
+        if (Q + (u32)(nb_hi - nb_lo) <= gridDim.x * blockDim.x / 8 * kLdGroupPasses)
+          expand_ld<U, 1>(a, qv, Q, (u32)lvl + 1, nb_lo, (u32)(nb_hi - nb_lo), (u32)lvl + 1, probe,
+                          qi, qb, pushed);
+        else
+          expand_ld<U, 8>(a, qv, Q, (u32)lvl + 1, nb_lo, (u32)(nb_hi - nb_lo), (u32)lvl + 1, probe,
+                          qi, qb, pushed);
         if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
       } else {
         expand<U>(a, s, (int)(phase & 1), Q, E, lvl, qi, qb, mylow);
@@ -1899,7 +1900,7 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
       if (profiler && phase + 1 < (u32)kRoundProfile) ctl->round_clk[phase + 1][0] = clock64();
       const int lo = __ldg(a.bptr + (rr - lv0)), hi = (int)ld_cg_u32(a.rcur + (rr - lv0));
       if (LD)
-        expand_ld<U>(a, nullptr, 0, 0, lo, (u32)(hi - lo), (u32)rr, false, qi, qb, pushed);
+        expand_ld<U, 8>(a, nullptr, 0, 0, lo, (u32)(hi - lo), (u32)rr, false, qi, qb, pushed);
       else
         append_bucket<U>(a, rr, lo, hi, qi, qb, mylow);
       // this round left no unsettled list: a bottom-up round after it starts

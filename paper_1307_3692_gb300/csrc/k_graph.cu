@@ -636,6 +636,24 @@ __global__ void __launch_bounds__(256) k_first_neighbours(const int* __restrict_
   }
 }
 
+// A thread writes four neighbours of a padded row.
+__global__ void __launch_bounds__(256) k_padded_rows(const int* __restrict__ row_ptr,
+                                                     const int* __restrict__ col, u32 n, u32 S4,
+                                                     uint4* __restrict__ ell) {
+  const u64 total = (u64)n * S4;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+       i += (u64)gridDim.x * blockDim.x) {
+    const u32 v = (u32)(i / S4), j = (u32)(i % S4) * 4;
+    const int e = __ldg(row_ptr + v) + (int)j, end = __ldg(row_ptr + v + 1);
+    uint4 x;
+    x.x = e < end ? (u32)__ldg(col + e) : ~0u;
+    x.y = e + 1 < end ? (u32)__ldg(col + e + 1) : ~0u;
+    x.z = e + 2 < end ? (u32)__ldg(col + e + 2) : ~0u;
+    x.w = e + 3 < end ? (u32)__ldg(col + e + 3) : ~0u;
+    ell[i] = x;
+  }
+}
+
 // Compaction of G_{i+1} to the vertices that kept an arc.  off: the kept arcs'
 // row offsets over G_i's n vertices (off[n] = all of them).
 __global__ void __launch_bounds__(256) k_kept_flags(const int* __restrict__ off, u32 n,
@@ -1418,6 +1436,15 @@ int launch_first_neighbours(const int* row_ptr, const int* col, u32 n, u32* firs
                             cudaStream_t s) {
   if (n == 0) return 0;
   k_first_neighbours<<<grid_for(n, num_sms), 256, 0, s>>>(row_ptr, col, n, first);
+  return 1;
+}
+
+int launch_padded_rows(const int* row_ptr, const int* col, u32 n, u32 S, u32* ell, int num_sms,
+                       cudaStream_t s) {
+  if (n == 0) return 0;
+  const u64 total = (u64)n * (S / 4);
+  const u32 g = (u32)min((long long)((total + 255) / 256), (long long)num_sms * 8);
+  k_padded_rows<<<g, 256, 0, s>>>(row_ptr, col, n, S / 4, reinterpret_cast<uint4*>(ell));
   return 1;
 }
 

@@ -91,6 +91,7 @@ int free_graph_memory(ldd_graph* g) {
   cudaFree(g->d_hot);
   if (!g->uni) cudaFree(g->d_active);  // a union's list lives in d_active_buf
   cudaFree(g->d_first);
+  if (!g->uni) cudaFree(g->d_ell);
   cudaFree(g->d_hot_center);
   cudaFree(g->cc.picks);
   cudaFree(g->cc.code);
@@ -137,6 +138,7 @@ int free_graph_memory(ldd_graph* g) {
     cudaFree(g->uni->d_mem);
     cudaFree(g->uni->d_offs);
     cudaFree(g->uni->d_hotv);
+    cudaFree(g->uni->d_ell_buf);
     cudaFree(g->uni->d_shift_in);
     cudaFree(g->uni->d_out_c);
     cudaFree(g->uni->d_cut);
@@ -453,6 +455,8 @@ BfsArgs bfs_args(ldd_graph* g, KeyFmt f, const double* shift) {
   a.pull_gamma = g->pull_gamma;
   a.probe_min_arcs = g->probe_min_arcs;
   a.low_degree = g->low_degree() ? 1u : 0u;
+  a.ell = g->d_ell;
+  a.ell_s = g->ell_s;
   a.window_levels = g->uni && !g->window_set ? kLdUnionWindowLevels : g->window_levels;
   a.window_max_q = g->window_max_q;
   a.window_queue = g->window_queue;
@@ -1058,6 +1062,7 @@ int setup_batch(ldd_graph* g) {
 UnionCaps union_needs(int k, ldd_graph* const* members) {
   UnionCaps c;
   c.k = (u32)k;
+  bool rows = true;  // every member has padded rows
   for (int i = 0; i < k; ++i) {
     const ldd_graph* m = members[i];
     c.N += ((u64)m->n + 31) / 32 * 32;
@@ -1067,7 +1072,11 @@ UnionCaps union_needs(int k, ldd_graph* const* members) {
     c.C += m->sc.ncomp;
     c.T += m->sc.total;
     c.total += (u64)m->n;
+    c.S = std::max(c.S, m->ell_s);
+    rows = rows && m->ell_s > 0;
   }
+  if (!rows) c.S = 0;
+  c.L = c.N * c.S;
   return c;
 }
 
@@ -1078,7 +1087,8 @@ u64 union_bytes(const UnionCaps& c) {
   const u64 N = c.N, words = std::max<u64>(N / 32, 1);
   u64 b = 4 * (N + 1) + 4 * c.E + 4 * c.M + 20 * c.G + 8 * (c.M / 32 + 1) + 8 * words +
           8 * c.C + 8 * c.T + 4 * N + 4 * words;
-  b += 16 * c.total + 8 * c.total + 36ull * (c.k + 1) + 120ull * c.k + 2 * c.total + 2 * c.G + 6 * N + sizeof(UnionMember) * c.k;
+  b += 16 * c.total + 8 * c.total + 36ull * (c.k + 1) + 120ull * c.k + 2 * c.total + 2 * c.G +
+       6 * N + 4 * c.L + sizeof(UnionMember) * c.k;
   const u64 nk = std::max<u64>(N, 64);
   b += 8 * N + 4 * N + 16 * nk + 8 * N + ((N + kSortTile - 1) / kSortTile + 1) * 2048 + 4 * N +
        8 * N + 36 * N + 12 * (c.E / kBfsBase + 2) + 8 * N + 4 * (N / kMaxBlock + 1) + 8 * N +
@@ -1126,6 +1136,7 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
       cudaMalloc(&U.d_mem, K * sizeof(UnionMember)) != cudaSuccess ||
       cudaMalloc(&U.d_offs, 9 * (K + 1) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_hotv, std::max<u64>(N, 1) * 4) != cudaSuccess ||
+      cudaMalloc(&U.d_ell_buf, std::max<u64>(c.L, 8) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_shift_in, total * 8) != cudaSuccess ||
       cudaMalloc(&U.d_out_c, total * 8) != cudaSuccess ||
       cudaMalloc(&U.d_cut, K * 8) != cudaSuccess ||
@@ -1190,6 +1201,9 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
   g->n_active = (u32)n_active;
   g->nnz_active = nnz_active;
   g->max_degree = max_deg;
+  const bool rows = need.S > 0 && need.L <= U.cap.L;
+  g->ell_s = rows ? need.S : 0;
+  g->d_ell = rows ? U.d_ell_buf : nullptr;
   if (!g->per_sm_set) {  // two CTAs per SM are for wide bottom-up rounds (see finish_setup)
     int most = 1;
     bfs_grid_size(g->num_sms, &most);
@@ -1239,6 +1253,8 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
                 g->code_cut ? U.d_hotv : nullptr};
   const u64 largest = std::max<u64>(std::max<u64>(need.N + 1, need.E), need.M);
   launch_union_concat(U.d_mem, U.off, U.k, t, largest, g->num_sms, s);
+  if (rows)
+    launch_padded_rows(g->d_row, g->d_col, (u32)g->n, g->ell_s, g->d_ell, g->num_sms, s);
   CUDA_TRY(cudaGetLastError());
   if (sync) CUDA_TRY(cudaStreamSynchronize(s));
   g->stats.n = g->n;
@@ -1399,6 +1415,16 @@ int ldd_create_graph(int32_t n, int64_t nnz, const int32_t* row_ptr, const int32
     launch_first_neighbours(g->d_row, g->d_col, (u32)n, g->d_first, g->num_sms, nullptr);
     if (cudaStreamSynchronize(nullptr) != cudaSuccess)
       return bail(fail(LDD_ERR_CUDA, "first-neighbour table"));
+  }
+  if (g->max_degree <= (u32)kLdMaxDegree) {  // padded rows for the low-degree rounds
+    g->ell_s = (u32)align_up(std::max(g->max_degree, 1u), 8);
+    if (cudaMalloc(&g->d_ell, (size_t)std::max<int64_t>(n, 1) * g->ell_s * 4) != cudaSuccess) {
+      cudaGetLastError();
+      return bail(fail(LDD_ERR_OOM, "device allocation of the padded rows failed"));
+    }
+    launch_padded_rows(g->d_row, g->d_col, (u32)n, g->ell_s, g->d_ell, g->num_sms, nullptr);
+    if (cudaStreamSynchronize(nullptr) != cudaSuccess)
+      return bail(fail(LDD_ERR_CUDA, "padded rows"));
   }
   if ((rc = finish_setup(g)) != LDD_OK) return bail(rc);
   // low-degree rounds are latency-bound: a key probe before every atomicMin

@@ -40,6 +40,7 @@ struct Blocks {
   int* src[2] = {};            // [nnz] source vertex of every arc of G_i, i >= 1
   u32* map[2] = {};            // [n] input id of every vertex of G_i, i >= 1
   int* off = nullptr;          // [n + 1] kept arcs per vertex of G_i, then their offsets
+  u32* ell = nullptr;          // [n * g->ell_s] padded rows of G_i, i >= 1 (low-degree graphs)
   u32* cid = nullptr;          // [n + 1] vertices with kept arcs, then their ids in G_{i+1}
   int* src0 = nullptr;         // [nnz] source vertex of every arc of G_0
   u32* klist = nullptr;        // [nnz] the count pass's kept arcs
@@ -60,6 +61,7 @@ void free_blocks(ldd_graph* g) {
     // the CSR and the small-component lists belong to b, not to r
     b->r->d_row = nullptr;
     b->r->d_col = nullptr;
+    b->r->d_ell = nullptr;
     b->r->sc.comp_off = b->r->sc.comp_len = b->r->sc.comp_v = nullptr;
     free_graph_memory(b->r);
     delete b->r;
@@ -73,6 +75,7 @@ void free_blocks(ldd_graph* g) {
   }
   cudaFree(b->off);
   cudaFree(b->cid);
+  cudaFree(b->ell);
   cudaFree(b->src0);
   cudaFree(b->klist);
   cudaFree(b->cursor);
@@ -104,7 +107,8 @@ int setup_blocks(ldd_graph* g) {
          cudaMalloc(&b->src[j], nnz * 4) == cudaSuccess &&
          cudaMalloc(&b->map[j], std::max<size_t>(n, 1) * 4) == cudaSuccess;
   ok = ok && cudaMalloc(&b->off, (n + 1) * 4) == cudaSuccess &&
-       cudaMalloc(&b->cid, (n + 1) * 4) == cudaSuccess;
+       cudaMalloc(&b->cid, (n + 1) * 4) == cudaSuccess &&
+       (g->ell_s == 0 || cudaMalloc(&b->ell, n * g->ell_s * 4) == cudaSuccess);
   ok = ok && cudaMalloc(&b->src0, nnz * 4) == cudaSuccess &&
        cudaMalloc(&b->klist, nnz * 4) == cudaSuccess &&
        cudaMalloc(&b->cursor, (n + 1) * 4) == cudaSuccess &&
@@ -177,6 +181,7 @@ void sync_params(ldd_graph* g, ldd_graph* r) {
   r->probe_min_arcs = g->probe_min_arcs;
   r->low_degree_rounds = g->low_degree_rounds;
   r->max_degree = g->max_degree;  // residual rows are never longer
+  r->ell_s = g->ell_s;
 }
 
 }  // namespace
@@ -330,6 +335,8 @@ extern "C" int ldd_block_decompose(ldd_graph* g, int k, const double* betas,
     r->m_up = (u32)edges_left;
     r->d_row = B.row[j];
     r->d_col = B.col[j];
+    r->d_ell = B.ell;
+    if (B.ell) launch_padded_rows(r->d_row, r->d_col, n_next, r->ell_s, B.ell, g->num_sms, s);
     if ((e = components_phase2(r->d_row, r->d_col, B.t, r->sc, g->num_sms, s)) != cudaSuccess)
       return fail(LDD_ERR_CUDA, "component adjacency: %s", cudaGetErrorString(e));
     CUDA_TRY(cudaEventRecord(B.ev[3], s));

@@ -54,6 +54,8 @@ struct UnionCaps {
   u64 C = 0;      // small components
   u64 T = 0;      // their members
   u64 total = 0;  // caller-layout entries (sum of member sizes)
+  u64 L = 0;      // entries of the padded rows (all members low-degree)
+  u32 S = 0;      // ... per row, or 0
   u32 k = 0;      // members
 };
 struct Blocks;  // state of ldd_block_decompose (ldd_blocks.cu)
@@ -139,7 +141,11 @@ struct ldd_graph {
   u32 probe_min_arcs = 1u << 16;
   u32 max_degree = 0;          // largest row of the CSR (unions: of any member)
   bool low_degree_rounds = true;  // tuning: low-degree rounds when max_degree allows
-  bool low_degree() const { return low_degree_rounds && max_degree <= (u32)kLdMaxDegree; }
+  u32* d_ell = nullptr;           // rows padded to ell_s neighbours (low-degree rounds), if any
+  u32 ell_s = 0;
+  bool low_degree() const {
+    return low_degree_rounds && max_degree <= (u32)kLdMaxDegree && ell_s > 0;
+  }
   // Set by the user (else bfs_per_sm, pull_alpha and window_levels follow the graph).
   bool per_sm_set = false, pull_set = false, window_set = false;
   // Low-degree rounds stay top-down unless the tuning says otherwise: a scan of
@@ -174,6 +180,7 @@ struct ldd_graph {
     UnionMember* d_mem = nullptr;  // k member views (valid only while building)
     u32* d_offs = nullptr;         // 9 arrays of cap.k + 1: v, e, u, c, m, a, o, g, h
     u32* d_hotv = nullptr;         // [cap.N] members' hot tables
+    u32* d_ell_buf = nullptr;      // [cap.L] padded rows (g->d_ell when the members have them)
     u32* d_active_buf = nullptr;   // [cap.N] active list (g->d_active when every member has one)
     UnionOffsets off{};
     double* d_shift_in = nullptr;  // [total] caller-layout shifts from the host

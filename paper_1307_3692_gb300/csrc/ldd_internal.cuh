@@ -173,6 +173,8 @@ struct BfsArgs {
   u32 probe_min_arcs;  // top-down rounds with at least this many arcs read a key before its atomicMin
   u32 low_degree;    // 1: every vertex has at most kLdMaxDegree arcs and the low-degree rounds
                      // run (the frontier a plain vertex list, a thread per vertex)
+  const u32* ell;    // low-degree rounds: rows padded to ell_s neighbours (a multiple of 8) with ~0
+  u32 ell_s;
   u32 window_levels; // low-degree rounds: levels per window (0 or 1: one level per grid barrier)
   u32 window_max_q;  // ... a window only while the frontier has at most this many vertices
   u32 window_queue;  // ... local-queue entries per CTA and level at most (0: as many as fit)
@@ -378,6 +380,9 @@ int launch_blocks_output(const int* cc, const int* dc, const u32* map, u32 nc, u
 // first[v] = col[row_ptr[v]], or ~0 for a vertex without arcs.
 int launch_first_neighbours(const int* row_ptr, const int* col, u32 n, u32* first, int num_sms,
                             cudaStream_t s);
+// Rows padded to S neighbours (a multiple of 8, at least the longest row) with ~0.
+int launch_padded_rows(const int* row_ptr, const int* col, u32 n, u32 S, u32* ell, int num_sms,
+                       cudaStream_t s);
 // src[e] = v for every arc e of row v of the CSR (row_ptr, n).
 int launch_fill_src(const int* row, u32 n, int* src, int num_sms, cudaStream_t s);
 // Exclusive scan of data[0 .. len) in place (k_rank.cu; decoupled look-back

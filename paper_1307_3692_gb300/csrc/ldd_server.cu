@@ -75,6 +75,13 @@ bool fits(const UnionCaps& a, const UnionCaps& b, const UnionCaps& cap) {
          a.k + b.k <= cap.k;
 }
 
+// Whether a batch that already holds a request can take b too and keep padded
+// rows.  (A batch of one runs on its own graph object.)  A workspace with room
+// for few rows does not split its batches for them.
+bool rows_fit(const UnionCaps& a, const UnionCaps& b, const UnionCaps& cap) {
+  return a.k == 0 || cap.L < cap.N || (a.N + b.N) * std::max(a.S, b.S) <= cap.L;
+}
+
 void add_to(UnionCaps& a, const UnionCaps& b) {
   a.N += b.N;
   a.E += b.E;
@@ -84,6 +91,7 @@ void add_to(UnionCaps& a, const UnionCaps& b) {
   a.T += b.T;
   a.total += b.total;
   a.k += b.k;
+  a.S = std::max(a.S, b.S);
 }
 
 // Workspace capacities that fit a per-slot budget: arcs up to half of it (at
@@ -104,6 +112,10 @@ UnionCaps caps_for(u64 budget, int max_batch, u64 max_vertices, u64 max_arcs) {
     if (max_vertices || N <= 32 || union_bytes(c) <= budget) break;
     N = std::max<u64>(32, N / 10 * 9 / 32 * 32);
   }
+  // padded rows take what is left, up to 8 entries per vertex: they never cost a
+  // request its place.  A batch without room for them runs the general rounds.
+  const u64 used = union_bytes(c);
+  c.L = used < budget ? std::min<u64>(8 * c.N, (budget - used) / 4 / 8 * 8) : 0;
   return c;
 }
 
@@ -233,7 +245,7 @@ void worker_batched(ldd_server* S, int slot) {
           ++it;
           continue;
         }
-        if (!fits(sum, (*it)->need, S->cap)) break;
+        if (!fits(sum, (*it)->need, S->cap) || !rows_fit(sum, (*it)->need, S->cap)) break;
         add_to(sum, (*it)->need);
         batch.push_back(*it);
         it = S->queue.erase(it);
