@@ -250,6 +250,55 @@ __global__ void __launch_bounds__(kCutThreads, 1) k_cut(CutList cl, const int* _
   }
 }
 
+// One labeling of a small graph in one launch: an edge's two labels come straight
+// from center (a group's through its vertex, a hot endpoint's through the hot
+// list), and the count needs no clearing and no copy -- blocks add to *acc, zero
+// on entry, with their arrival in the upper bits, and the last one writes *out
+// (pinned host memory) and leaves *acc at zero.
+__global__ void __launch_bounds__(256) k_cut_one(CutList cl, const int* __restrict__ center,
+                                                 const u32* __restrict__ hot, u64* acc, u64* out) {
+  __shared__ u32 wsum[8];
+  const u32 lane = threadIdx.x & 31;
+  const int4* hot4 = reinterpret_cast<const int4*>(cl.hot);
+  u32 cnt = 0;  // a thread's share of at most kCutOneEdges edges
+  for (u32 e0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x); e0 < cl.m;
+       e0 += 4 * gridDim.x * blockDim.x) {
+    int hv[4] = {0, 0, 0, 0};
+    if (e0 + 3 < cl.m) {
+      const int4 h = __ldg(hot4 + (e0 >> 2));
+      hv[0] = h.x;
+      hv[1] = h.y;
+      hv[2] = h.z;
+      hv[3] = h.w;
+    } else {
+      for (u32 q = 0; q < cl.m - e0; ++q) hv[q] = cl.hot[e0 + q];
+    }
+    const u32 bg = __ldg(cl.blk_g + (e0 >> 5)), bm = __ldg(cl.blk_mask + (e0 >> 5));
+    u32 x[4], y[4];
+#pragma unroll
+    for (u32 q = 0; q < 4; ++q) {
+      const bool valid = e0 + q < cl.m;
+      x[q] = valid ? __ldg(cl.grp_v + bg + __popc(bm & bits_upto((e0 & 31u) + q))) : 0u;
+      y[q] = hv[q] >= 0 ? (u32)hv[q] : __ldg(hot + (hv[q] & 0x7fffffff));
+    }
+#pragma unroll
+    for (u32 q = 0; q < 4; ++q) cnt += e0 + q < cl.m && center[x[q]] != center[y[q]];
+  }
+  cnt = __reduce_add_sync(kFull, cnt);
+  if (lane == 0) wsum[threadIdx.x >> 5] = cnt;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    u64 mine = 1ull << 40;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) mine += wsum[w];
+    const u64 sum = atomicAdd(reinterpret_cast<unsigned long long*>(acc), mine) + mine;
+    if (sum >> 40 == gridDim.x) {
+      *out = sum & ((1ull << 40) - 1);
+      *acc = 0;
+    }
+  }
+}
+
 // blk_g and blk_mask of a union's concatenated groups (blk_mask zero on entry).
 __global__ void k_cut_blocks(CutList cl) {
   for (u32 g = blockIdx.x * blockDim.x + threadIdx.x; g < cl.ngrp; g += gridDim.x * blockDim.x) {
@@ -1208,6 +1257,13 @@ int launch_cut(const CutList& cl, const int* center, const u32* hot, u32 n_hot, 
   k_cut<false><<<g, kCutThreads, (size_t)min(n_hot, kHotSlots) * sizeof(int), s>>>(cl, center, hot_center, n_hot,
                                                                    out);
   return launches + 1;
+}
+
+int launch_cut_one(const CutList& cl, const int* center, const u32* hot, u64* acc, u64* out,
+                   int num_sms, cudaStream_t s) {
+  const u32 g = (u32)max(1ll, min((long long)(cl.m + 1023) / 1024, (long long)num_sms * 8));
+  k_cut_one<<<g, 256, 0, s>>>(cl, center, hot, acc, out);
+  return 1;
 }
 
 int launch_cut4(const CutList& cl, const int* const* centers, int K, u32 n, const u32* hot,

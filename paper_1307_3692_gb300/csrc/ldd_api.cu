@@ -91,6 +91,7 @@ int free_graph_memory(ldd_graph* g) {
   cudaFree(g->d_hot);
   if (!g->uni) cudaFree(g->d_active);  // a union's list lives in d_active_buf
   cudaFree(g->d_first);
+  cudaFree(g->d_cut_acc);
   if (!g->uni) cudaFree(g->d_ell);
   cudaFree(g->d_hot_center);
   cudaFree(g->cc.picks);
@@ -353,7 +354,9 @@ int build_cut_list(ldd_graph* g, const std::vector<int32_t>& rp, const std::vect
       cudaMalloc(&cl.blk_g, blk_g.size() * 4) != cudaSuccess ||
       cudaMalloc(&cl.blk_mask, blk_mask.size() * 4) != cudaSuccess ||
       cudaMalloc(&g->d_hot, std::max<size_t>(K, 1) * 4) != cudaSuccess ||
-      cudaMalloc(&g->d_hot_center, std::max<size_t>(K, 1) * 4) != cudaSuccess) {
+      cudaMalloc(&g->d_hot_center, std::max<size_t>(K, 1) * 4) != cudaSuccess ||
+      cudaMalloc(&g->d_cut_acc, sizeof(u64)) != cudaSuccess ||
+      cudaMemset(g->d_cut_acc, 0, sizeof(u64)) != cudaSuccess) {
     cudaGetLastError();
     return fail(LDD_ERR_OOM, "device allocation of the cut list failed");
   }
@@ -932,9 +935,16 @@ int replay_fast(ldd_graph* g, double beta, bool want_cut, int* launches_out) {
 int cut_on_device(ldd_graph* g, const int* d_center, int64_t* out_cut) {
   cudaStream_t s = g->stream;
   record(g, 6);
-  CUDA_TRY(cudaMemsetAsync(&g->d_ctl->cut, 0, sizeof(u64), s));
-  const int l = cut_labels(g, &d_center, 1, &g->d_ctl->cut, s);
-  CUDA_TRY(cudaMemcpyAsync(g->h_hdr + 128, &g->d_ctl->cut, sizeof(u64), cudaMemcpyDeviceToHost, s));
+  int l;
+  if (g->cut.m <= kCutOneEdges) {
+    l = launch_cut_one(g->cut, d_center, g->d_hot, g->d_cut_acc,
+                       reinterpret_cast<u64*>(g->h_hdr + 128), g->num_sms, s);
+  } else {
+    CUDA_TRY(cudaMemsetAsync(&g->d_ctl->cut, 0, sizeof(u64), s));
+    l = cut_labels(g, &d_center, 1, &g->d_ctl->cut, s);
+    CUDA_TRY(
+        cudaMemcpyAsync(g->h_hdr + 128, &g->d_ctl->cut, sizeof(u64), cudaMemcpyDeviceToHost, s));
+  }
   record(g, 7);
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(s));

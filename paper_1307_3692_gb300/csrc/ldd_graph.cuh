@@ -141,6 +141,7 @@ struct ldd_graph {
   u32 probe_min_arcs = 1u << 16;
   u32 max_degree = 0;          // largest row of the CSR (unions: of any member)
   bool low_degree_rounds = true;  // tuning: low-degree rounds when max_degree allows
+  u64* d_cut_acc = nullptr;       // launch_cut_one's sum, zero between calls
   u32* d_ell = nullptr;           // rows padded to ell_s neighbours (low-degree rounds), if any
   u32 ell_s = 0;
   bool low_degree() const {

@@ -302,6 +302,16 @@ struct CutList {
 };
 int launch_cut(const CutList& cl, const int* center, const u32* hot, u32 n_hot, int* hot_center,
                u64* out, int num_sms, cudaStream_t s);
+// One labeling of a graph of at most kCutOneEdges edges in one launch: the count into
+// *out (pinned host memory); *acc is zero on entry and left at zero.
+// Clearing, group labels, (hot labels,) count and copy were up to five stream
+// operations: 30 us however small the graph, against 13 (a call, host to host; 64 x 64
+// and 256 x 256 grids 30 -> 13, 1000 x 1000 30 -> 16, 2000 x 2000 with 8 M edges 43 ->
+// 26, R-MAT 14 30 -> 14, R-MAT 18 with 3.8 M edges 32 -> 25).  Beyond, two random reads
+// per edge cost more than the tables save (R-MAT 20, 15.7 M edges: 55 against 66).
+constexpr u32 kCutOneEdges = 1u << 23;
+int launch_cut_one(const CutList& cl, const int* center, const u32* hot, u64* acc, u64* out,
+                   int num_sms, cudaStream_t s);
 // Cut counts by piece codes (k_graph.cu).  Graphs with hubs: nearly every vertex
 // belongs to one of a few pieces, those of the highest-degree vertices.  A
 // vertex gets a 4-bit code per labeling, the index of its piece among the
