@@ -1736,8 +1736,9 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
   const int* wave_c[4] = {};
   int nwave = 0, waves = 0, last_cut = -1;
   if (W > 1 && !g->code_cut && (rc = ensure_cut4(g)) != LDD_OK) return rc;
+  const bool cut_one = W == 1 && g->cut.m <= kCutOneEdges;  // counts go straight to h_bcut
   if (cuts) {
-    CUDA_TRY(cudaMemsetAsync(g->d_bcut, 0, (size_t)k * sizeof(u64), s));
+    if (!cut_one) CUDA_TRY(cudaMemsetAsync(g->d_bcut, 0, (size_t)k * sizeof(u64), s));
     for (int j = 0; j < 2; ++j) CUDA_TRY(cudaEventRecord(g->ev_cut[j], s));
   }
   record(g, 0);
@@ -1776,7 +1777,9 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
       if (nwave == W || i == k - 1) {  // the wave's last finalize is queued: count its cuts
         CUDA_TRY(cudaStreamWaitEvent(g->cut_stream, g->ev_used[j], 0));
         u64* out = g->d_bcut + (i + 1 - nwave);
-        launches += cut_labels(g, wave_c, nwave, out, g->cut_stream);
+        launches += cut_one ? launch_cut_one(g->cut, center, g->d_hot, g->d_cut_acc,
+                                             g->h_bcut + i, g->num_sms, g->cut_stream)
+                            : cut_labels(g, wave_c, nwave, out, g->cut_stream);
         CUDA_TRY(cudaGetLastError());
         last_cut = waves++ & 1;
         CUDA_TRY(cudaEventRecord(g->ev_cut[last_cut], g->cut_stream));
@@ -1784,7 +1787,7 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
       }
     }
   }
-  if (cuts)
+  if (cuts && !cut_one)
     CUDA_TRY(cudaMemcpyAsync(g->h_bcut, g->d_bcut, (size_t)k * sizeof(u64), cudaMemcpyDeviceToHost,
                              g->cut_stream));
   CUDA_TRY(cudaStreamSynchronize(g->cut_stream));

@@ -39,3 +39,17 @@ def test_full_grids(ldd, cuda, make):
     want = _cut(G, c)
     assert [g.cut_edges(c) for _ in range(3)] == [want] * 3
     g.close()
+
+
+@pytest.mark.parametrize("host", [True, False])
+def test_batches(ldd, cuda, host):
+    """Every count of a batch with host outputs, and of a batch of one, is its own."""
+    G = gen.rgg(3000, 7)
+    g = ldd.LddGraph(G.row_ptr, G.col)
+    for betas in ((0.3,), (0.05, 0.8, 0.3)):
+        S = [gen.shifts(G.n, b, 5) for b in betas]
+        new = lambda: torch.empty(G.n, dtype=torch.int32, device="cpu" if host else "cuda")
+        c, d = [new() for _ in betas], [new() for _ in betas]
+        cut = g.decompose_batch(list(betas), S, c, d)
+        assert [int(x) for x in cut] == [_cut(G, x.cpu().numpy()) for x in c]
+    g.close()
