@@ -399,7 +399,7 @@ typedef struct {
   int64_t launches;       /* kernels launched by the last ldd_decompose */
   int64_t cut_launches;   /* kernels launched by the last ldd_cut_edges */
   int64_t exact_rank;     /* 1 if the fraction rank needed the exact radix-sort
-                             path (a fraction bucket overflowed), else 0 */
+                             path (equal direct keys met in the wrong order, or too many of them), else 0 */
   int32_t bfs_grid;       /* CTAs of the persistent BFS kernel */
   int32_t bfs_block;      /* threads per CTA */
   float ms_h2d;           /* shifts host -> device (0 if already on device) */
@@ -479,7 +479,7 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out);
  * ldd_set_graph_replay -- enable (1) or disable (0) CUDA-graph replay of the
  * decomposition on g (a plain graph or a union).  Once enabled, the first
  * call runs as usual and the next one captures the fast path -- every kernel
- * from the control-block reset (a union's shift spread included) through
+ * from the control-block reset (a union's lifts included) through
  * finalize, a union's cut counts when asked for, and the status copy to the
  * host -- into a CUDA graph on an internal stream; later calls copy their
  * shifts into the library's input buffer, replay that graph on g's stream
@@ -511,7 +511,7 @@ int ldd_set_graph_replay(ldd_graph* g, int enable);
  *                   polls -- for tests of the timeout path; 0 normally.
  *   stall_lookback  1: the first tile of each scan waits on a predecessor that
  *                   does not exist, so every look-back runs out of polls (when
- *                   the call takes the fraction-bucket rank) -- for tests; 0
+ *                   the call scans its start buckets on the device) -- for tests; 0
  *                   normally.
  * ldd_set_wait_limits drops a captured replay (ldd_set_graph_replay), since it
  * holds the old values.  LDD_ERR_ARG if a stall field is not 0 or 1.

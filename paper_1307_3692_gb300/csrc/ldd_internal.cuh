@@ -279,7 +279,8 @@ int launch_finalize(const BfsArgs& a, const u32* order, const u32* solo, int* ce
 // group g (one per cold vertex that has edges, ascending) is hot[grp_off[g] ..
 // grp_off[g + 1]) with cold vertex grp_v[g].  hot[e] < 0 stands for slot
 // hot[e] & 0x7fffffff of the hot table (the at most kHotSlots highest-degree
-// vertices, whose labels the cut kernel keeps in shared memory).  The edges
+// vertices, whose labels the cut kernel keeps in shared memory; kCodeSlots where
+// counts go by piece codes).  The edges
 // come in blocks of 32: blk_g[b] is the group of edge 32 b, and bit j of
 // blk_mask[b] is set when edge 32 b + j (j > 0) starts a group, so edge
 // 32 b + j is in group blk_g[b] + popc(blk_mask[b] & bits 0 .. j).  About 4.3

@@ -5,15 +5,15 @@
 // in one FIFO queue.  Each of the server's slots is a worker thread that owns
 // a union workspace (a disjoint-union graph object with fixed capacities,
 // ldd_graph.cuh) and a CUDA stream.  A free worker takes, in arrival order,
-// every waiting request of the first one's kind that still fits its workspace -- the admission test is
-// the requests' device footprint: vertices, arcs, cut-list entries and small
+// every waiting request of the first one's kind (low-degree or not) that still
+// fits its workspace -- the admission test is the requests' device footprint: vertices, arcs, cut-list entries and small
 // components against the capacities the HBM budget bought -- and runs them as
 // one decomposition of their disjoint union (Algorithm 2 never crosses from
 // one member to another, so every member's result is exactly its result
 // alone):
 //   1. union tables from the members' resident tables (one kernel launch) and
 //      the members' shifts copied in (host -> device);
-//   2. spread, rank, round loop, finalize and the members' cut counts on the
+//   2. lifts, direct keys, round loop, finalize and the members' cut counts on the
 //      worker's stream;
 //   3. results copied out (device -> host), requests completed.
 // The workers' streams run side by side on the device except for the round

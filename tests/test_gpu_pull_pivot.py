@@ -97,3 +97,33 @@ def test_pivot_rounds_exact_in_unions(ldd, cuda, extra):
     u.close()
     for g in gs:
         g.close()
+
+
+@pytest.mark.parametrize("beta", [0.05, 0.6])
+def test_scan_steps(ldd, cuda, beta):
+    """Bottom-up rows of every length around the scan's steps, the only settled neighbour last."""
+    lengths = [1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 15, 16, 17, 30, 31, 32, 33, 34, 40] * 3
+    pool = 40
+    c = pool + len(lengths)  # the center: the largest id, so the last of every row
+    edges = [(d, pool + i) for i, n in enumerate(lengths) for d in range(n - 1)]
+    edges += [(pool + i, c) for i in range(len(lengths))]
+    G = gen.from_edges(c + 1, edges)
+    g = ldd.LddGraph(G.row_ptr, G.col)
+    u = ldd.LddUnion([g, g])
+    for x in (g, u):
+        x.set_tuning(pull_alpha=1000, pull_gamma=1000)
+    parts = []
+    for seed in range(2):
+        s = gen.shifts(G.n, beta, seed)
+        s[c] = s.max() + 1.25
+        oc, od = oracle.oracle_ldd(G.row_ptr, G.col, s)
+        cc, dd = np.empty(G.n, np.int32), np.empty(G.n, np.int32)
+        g.decompose(beta, s, cc, dd)
+        assert np.array_equal(cc, oc) and np.array_equal(dd, od)
+        parts.append((s, oc, od))
+    cc, dd = np.empty(2 * G.n, np.int32), np.empty(2 * G.n, np.int32)
+    u.decompose([beta, beta], np.concatenate([p[0] for p in parts]), cc, dd)
+    assert np.array_equal(cc, np.concatenate([p[1] for p in parts]))
+    assert np.array_equal(dd, np.concatenate([p[2] for p in parts]))
+    u.close()
+    g.close()
