@@ -415,12 +415,12 @@ float elapsed(ldd_graph* g, int a, int b) {
 
 // Low-degree rounds of a single graph relax eight levels between grid barriers
 // (deeper windows help where pieces grow slowly -- 1000^2 grid at beta 0.01, depth
-// 8 2.00 ms, 32 1.79 -- and hurt elsewhere: random geometric graph of 150,001
-// vertices, 8 0.59 ms, 16 0.79, 32 1.26).
+// 8 1.19 ms, 12 1.11, 24 1.08; 256^3 grid 2.56, 2.47, 2.62 -- and hurt elsewhere:
+// random geometric graph of 150,001 vertices 0.43, 0.52, 0.85).
 constexpr u32 kDefaultWindowLevels = 8;
 // Unions: one, and four where the tuning has not been touched and low-degree
-// rounds run (64 random geometric graphs: 1 level 4.37, 2 3.40, 3 3.22, 4 3.12,
-// 6 3.12, 8 3.21 ms).
+// rounds run (64 random geometric graphs: 1 level 3.55, 3 2.70, 4 2.63, 6 2.65,
+// 8 2.74 ms).
 constexpr u32 kDefaultUnionWindowLevels = 1;
 constexpr u32 kLdUnionWindowLevels = 4;
 
