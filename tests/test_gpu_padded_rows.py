@@ -4,6 +4,8 @@ ones (a thread per vertex), in unions of members with different row widths and o
 residual graphs."""
 from __future__ import annotations
 
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -71,5 +73,31 @@ def test_union_of_row_widths(ldd, cuda, side):
             assert np.array_equal(c[at:at + G.n], oc) and np.array_equal(d[at:at + G.n], od)
             at += G.n
     u.close()
+    for g in gs:
+        g.close()
+
+
+@pytest.mark.parametrize("extra", [0, 1 << 14, 1 << 16, 1 << 20])
+def test_server_budget_without_room_for_rows(ldd, cuda, extra):
+    """A workspace whose budget leaves no room, little and enough for padded rows takes the same
+    requests and gives the same results."""
+    caps = dict(max_batch=8, slots=1, max_vertices=8192, max_arcs=1 << 18)
+    with pytest.raises(ldd.LddError) as e:
+        ldd.LddServer(1 << 12, **caps)
+    need = int(re.search(r"need (\d+) bytes", str(e.value)).group(1))
+    Gs = [gen.grid2d(60, 60), gen.grid2d(32, 32), _graph(300, (32, 8, 1), 1), gen.rgg(900, 3)]
+    gs = [ldd.LddGraph(G.row_ptr, G.col) for G in Gs]
+    srv = ldd.LddServer(need + extra, **caps)
+    jobs = []
+    for i in range(16):
+        G = Gs[i % 4]
+        jobs.append((i % 4, gen.shifts(G.n, 0.1, i), np.empty(G.n, np.int32),
+                     np.empty(G.n, np.int32)))
+    tickets = [srv.submit(gs[i], 0.1, s, c, d) for i, s, c, d in jobs]
+    for t, (i, s, c, d) in zip(tickets, jobs):
+        srv.wait(t)
+        oc, od = oracle.oracle_ldd(Gs[i].row_ptr, Gs[i].col, s)
+        assert np.array_equal(c, oc) and np.array_equal(d, od)
+    srv.close()
     for g in gs:
         g.close()
