@@ -1,7 +1,7 @@
 """Padded neighbour rows of the low-degree rounds: exact at every row length
 around the chunk of eight, for thin frontiers (eight lanes per vertex) and thick
-ones (a thread per vertex), in unions of members with different row widths and on
-residual graphs."""
+ones (a thread per vertex), in unions of members with different row widths and where a
+server has no room for them."""
 from __future__ import annotations
 
 import re
