@@ -58,8 +58,9 @@
 // Graphs whose vertices have at most kLdMaxDegree arcs run low-degree rounds
 // (a plain vertex list and padded neighbour rows; a thread per frontier vertex,
 // or eight lanes while the frontier is thin) and relax several levels between two
-// grid barriers (windows of levels, below).  All device-side waits are bounded: a barrier that does not complete
-// within the spin limit sets kErrTimeout and the kernel returns.
+// grid barriers (windows of levels, below).  All device-side waits are bounded:
+// a barrier that does not complete within the spin limit sets kErrTimeout and
+// the kernel returns.
 #include <cstddef>
 
 #include "ldd_internal.cuh"
@@ -212,7 +213,8 @@ __device__ __forceinline__ u64 warp_max64(u64 x) { return ~warp_min64(~x); }
 // kErrTimeout, or once any CTA has recorded an error.  Thread 0 then reads,
 // in one round trip, the error word and the next round's state (slot `post`
 // of the frontier counter, bottom-up floor and unsettled-list length, and the
-// bounds of start bucket blevel, of levels from lv0 on, unless it is negative) into shared memory, so that every thread of the CTA sees the same values and
+// bounds of start bucket blevel, of levels from lv0 on, unless it is negative)
+// into shared memory, so that every thread of the CTA sees the same values and
 // takes the same branch after the barrier (a thread that left the loop alone
 // would leave the others at a CTA barrier).  a.bar_phantom > 0 waits for CTAs that
 // do not exist: the barrier can then only end by running out of polls, which
@@ -979,8 +981,8 @@ struct BucketsAhead {
 
 template <bool U, int kCap>
 __device__ __forceinline__ void window_ld(const BfsArgs& a, Smem& s, int lv0, int A, int built,
-                                          BucketsAhead& ahead, u32 Q, u32 nov, int qcur, u32 L, u32 H, int qi, int qb,
-                                          u64& pushed, u64& expanded) {
+                                          BucketsAhead& ahead, u32 Q, u32 nov, int qcur, u32 L, u32 H,
+                                          int qi, int qb, u64& pushed, u64& expanded) {
   const int* bp = a.bptr - lv0;    // start buckets by level
   const u32* rc = a.rcur - lv0;
   const u32* rv = a.rv;

@@ -1254,8 +1254,8 @@ int launch_cut(const CutList& cl, const int* center, const u32* hot, u32 n_hot, 
   k_group_labels<false><<<grid_for((cl.ngrp + kLabIpt - 1) / kLabIpt, num_sms), 256, 0, s>>>(
       cl, center);
   const u32 g = (u32)max(1ll, min((long long)(cl.m + 4095) / 4096, (long long)num_sms));
-  k_cut<false><<<g, kCutThreads, (size_t)min(n_hot, kHotSlots) * sizeof(int), s>>>(cl, center, hot_center, n_hot,
-                                                                   out);
+  const size_t smem = (size_t)min(n_hot, kHotSlots) * sizeof(int);
+  k_cut<false><<<g, kCutThreads, smem, s>>>(cl, center, hot_center, n_hot, out);
   return launches + 1;
 }
 
