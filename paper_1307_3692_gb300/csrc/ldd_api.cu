@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <chrono>
 #include <new>
+#include <string>
 #include <vector>
 
 #include "../../include/ldd.h"
@@ -110,6 +111,7 @@ int free_graph_memory(ldd_graph* g) {
   cudaFree(g->d_bptr);
   cudaFree(g->d_rcur);
   cudaFree(g->d_acnt);
+  cudaFree(g->d_status);
   cudaFree(g->batch_arena);
   if (g->h_hdr) cudaFreeHost(g->h_hdr);
   if (g->h_bhdr) cudaFreeHost(g->h_bhdr);
@@ -175,12 +177,43 @@ int validate_csr(int32_t n, int64_t nnz, const int32_t* rp, const int32_t* col) 
   return LDD_OK;
 }
 
+// The start-bucket tables of `cap` entries, and the look-back status words: the
+// radix sort takes 256 per tile of vertices, the scan of the tables one per tile of
+// entries, and there may be far more entries than vertices (floors beyond n).
+// Frees the ones there were; nothing on the device may still use them.
+int alloc_start_buckets(ldd_graph* g, size_t cap) {
+  const size_t tiles = ((size_t)g->n + kSortTile - 1) / kSortTile + 1;
+  cudaFree(g->d_bptr);
+  cudaFree(g->d_rcur);
+  cudaFree(g->d_acnt);
+  cudaFree(g->d_status);
+  g->d_bptr = nullptr;
+  g->d_rcur = nullptr;
+  g->d_acnt = nullptr;
+  g->d_status = nullptr;
+  g->bptr_cap = 0;
+  // (a workspace's n may be below the one it was made for: never fewer than before)
+  g->status_bytes = std::max(g->status_bytes,
+                             std::max(tiles * 256, scan_status_words((u32)cap)) * sizeof(u64));
+  if (cudaMalloc(&g->d_bptr, cap * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&g->d_rcur, cap * sizeof(u32)) != cudaSuccess ||
+      cudaMalloc(&g->d_acnt, cap * sizeof(u32)) != cudaSuccess ||
+      cudaMalloc(&g->d_status, g->status_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(LDD_ERR_OOM, "start-bucket table of %zu entries", cap);
+  }
+  CUDA_TRY(cudaMemsetAsync(g->d_status, 0, g->status_bytes, g->stream));
+  CUDA_TRY(cudaStreamSynchronize(g->stream));
+  g->epoch = 0;
+  g->bptr_cap = (u32)cap;
+  g->acnt_dirty = true;  // cleared by the next attempt with direct keys
+  return LDD_OK;
+}
+
 int alloc_scratch(ldd_graph* g) {
   const size_t n = (size_t)g->n;
   const size_t nk = std::max<size_t>(n, 64);  // 64-bit words per key buffer
-  const size_t ntiles = (n + kSortTile - 1) / kSortTile + 1;
   const size_t ncf = (size_t)g->nnz / kBfsBase + 2;
-  g->status_bytes = ntiles * 256 * sizeof(u64);
   struct Part {
     void** p;
     size_t bytes;
@@ -188,7 +221,6 @@ int alloc_scratch(ldd_graph* g) {
       {(void**)&g->d_shift, 8 * n},       {(void**)&g->d_a, 4 * n},
       {(void**)&g->d_k[0], 8 * nk},       {(void**)&g->d_k[1], 8 * nk},
       {(void**)&g->d_v[0], 4 * n},        {(void**)&g->d_v[1], 4 * n},
-      {(void**)&g->d_status, g->status_bytes},
       {(void**)&g->d_order, 4 * n},       {(void**)&g->d_key, 8 * n},
       {(void**)&g->d_qv[0], 4 * n},       {(void**)&g->d_qv[1], 4 * n},
       {(void**)&g->d_qrow[0], 4 * n},     {(void**)&g->d_qrow[1], 4 * n},
@@ -212,16 +244,7 @@ int alloc_scratch(ldd_graph* g) {
     *p.p = (char*)g->arena + off;
     off += align_up(p.bytes ? p.bytes : 1, 256);
   }
-  CUDA_TRY(cudaMemset(g->d_status, 0, g->status_bytes));
-  g->bptr_cap = (u32)std::min<size_t>(n + 2, 0xffffffffu);
-  g->acnt_dirty = true;  // cleared by the first fast-path attempt
-  if (cudaMalloc(&g->d_bptr, (size_t)g->bptr_cap * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&g->d_rcur, (size_t)g->bptr_cap * sizeof(u32)) != cudaSuccess ||
-      cudaMalloc(&g->d_acnt, (size_t)g->bptr_cap * sizeof(u32)) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(LDD_ERR_OOM, "cudaMalloc of the start-bucket table failed");
-  }
-  return LDD_OK;
+  return alloc_start_buckets(g, n + 2);
 }
 
 // Component labels and the small-component tables (two device phases, the
@@ -751,23 +774,14 @@ int decompose_on_device(ldd_graph* g, double beta, const double* d_shift, int* c
     }
     if (h.err & kErrBucketCap) {
       // floor(delta_max) + 2 exceeds the start-bucket table: grow it, redo.
-      const size_t need = (size_t)h.A + 2;
-      cudaFree(g->d_bptr);
-      cudaFree(g->d_rcur);
-      cudaFree(g->d_acnt);
-      g->d_bptr = nullptr;
-      g->d_rcur = nullptr;
-      g->d_acnt = nullptr;
-      g->bptr_cap = 0;
-      if (cudaMalloc(&g->d_bptr, need * sizeof(int)) != cudaSuccess ||
-          cudaMalloc(&g->d_rcur, need * sizeof(u32)) != cudaSuccess ||
-          cudaMalloc(&g->d_acnt, need * sizeof(u32)) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(LDD_ERR_OOM, "start-bucket table of %zu entries", need);
+      drop_replay(g);  // a captured replay holds the old tables
+      const size_t had = g->bptr_cap;
+      const int grown = alloc_start_buckets(g, (size_t)h.A + 2);
+      if (grown != LDD_OK) {  // later calls find the tables they had
+        const std::string why = g_last_error;
+        alloc_start_buckets(g, had);
+        return fail(grown, "%s", why.c_str());
       }
-      g->bptr_cap = (u32)need;
-      g->acnt_dirty = true;  // cleared by the next attempt with direct keys
-      drop_replay(g);        // a captured replay holds the old table
     }
   }
   if (h.err) return header_error(h.err);
