@@ -941,7 +941,10 @@ __global__ void __launch_bounds__(32) k_picks(CutCodes cc, Labels4 L, UnionOffse
 #pragma unroll
   for (u32 i = 0; i < kPickFrom / 32; ++i) {
     bool open = lab[i] != 0xffffffffu;
-    for (u32 p = 0; p < found; ++p) open = open && lab[i] != __shfl_sync(kFull, mine, p);
+    for (u32 p = 0; p < found; ++p) {
+      const u32 named = __shfl_sync(kFull, mine, p);  // every lane, closed ones too
+      open = open && lab[i] != named;
+    }
     u32 m;
     while (found < kCodePieces && (m = __ballot_sync(kFull, open)) != 0u) {
       const u32 x = __shfl_sync(kFull, lab[i], __ffs(m) - 1);
