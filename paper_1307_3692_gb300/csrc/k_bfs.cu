@@ -9,8 +9,9 @@
 // offer made in round r carries level r + 1, the minimum over all offers is the
 // exact label the paper's super-source shortest path assigns (Section 4),
 // including the fraction tie-break.  Wherever two direct keys that differ only
-// in their ids meet -- at a vertex, or in the minimum that a bottom-up round
-// stops at -- the meeting is listed (note_tie) and finalize compares the exact
+// in their ids meet -- at a vertex, in the minimum that a bottom-up round stops
+// at, or between that minimum and what a candidate holds when its scan stops or
+// is left out -- the meeting is listed (note_tie) and finalize compares the exact
 // fractions, so a decomposition that ends without an error bit is exact.
 //
 // Start buckets.  With direct keys the loop itself fills the buckets, some
@@ -1371,7 +1372,10 @@ __device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lv
         best = ~0ull;
       }
       const u32 stop = min(end, p1);
-      if (!push && p < stop && min(kw, best) <= fl) p = stop;  // nothing can beat it
+      if (!push && p < stop && min(kw, best) <= fl) {  // nothing can beat it
+        note_tie(a, w, min(kw, best), fl);             // (as in pull_round)
+        p = stop;
+      }
       u32 vv[kRestBatch];
 #pragma unroll
       for (int q = 0; q < kRestBatch; ++q)
@@ -1674,6 +1678,16 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u64 stop_l
           scanned += (u32)(min(pos, ee) - eb);
         }
       }
+    }
+    // what the scan stopped at, or was not begun for, against what w holds: the offers
+    // left unread are no better than (L + 1, fr), and may only tie with it
+    bool tie = false;
+#pragma unroll
+    for (int j = 0; j < kPullV; ++j) tie |= key_tie(a.f, best[j], lvl_key | fr[j]);
+    if (tie) {
+#pragma unroll
+      for (int j = 0; j < kPullV; ++j)
+        if (w[j] != kNone) note_tie(a, w[j], best[j], lvl_key | fr[j]);
     }
     u64 kwn[kPullV];  // the next pass's keys and ranges, beside this pass's appends
     int en[kPullV], ren[kPullV];
