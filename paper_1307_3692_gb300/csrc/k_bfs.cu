@@ -1993,10 +1993,14 @@ __global__ void __launch_bounds__(kBfsThreads, kPerSm) k_bfs(BfsArgs a) {
     post_cta_min<kTrack>(a, s, mylow);
     grid_barrier<kTrack>(a, gen, (u32)qi, lv0, nlvl + 1 <= A ? nlvl + 1 : -1, s);
     if (!LD && defer && !s.stop && (u32)s.next_rest) {  // pushes and put-off scans are listed
+      const u64 first_low = s.next_minlow;
       pull_rest<U>(a, (u32)(s.next_rest >> 32), (u32)s.next_rest, lvl, stop_low, phase % 3, qi, qb,
                    mylow, s_floor);
       post_cta_min<kTrack>(a, s, mylow);
       grid_barrier<kTrack>(a, gen, (u32)qi, lv0, nlvl + 1 <= A ? nlvl + 1 : -1, s);
+      // the CTAs compared what they posted before with the minimum of the first pass: it
+      // stands for them all
+      if (kTrack && profiler) note_tie(a, 0, first_low, s.next_minlow);
     }
     ++phase;
     lvl = nlvl;

@@ -1,6 +1,7 @@
 """Direct keys whose codes tie across the steps of a bottom-up round: a vertex that
-starts one level later than the center that reaches it, and a scan that stops at
-the pivot's code before it has seen the pivot's own piece.  The ids agree with the
+starts one level later than the center that reaches it, a scan that stops at the
+pivot's code before it has seen the pivot's own piece, and a center whose push
+comes after a start of the same code was counted.  The ids agree with the
 fractions, or not; a third center with a better code hides the pair, or not."""
 from __future__ import annotations
 
@@ -94,4 +95,24 @@ def test_scan_that_stops_before_the_pivot(ldd, cuda, larger_wins, wide, third):
     st = _single(ldd, G, s)
     assert st["pull_rounds"] > 0
     assert st["exact_rank"] == 1 or not larger_wins
+    _union(ldd, G, [s])
+
+
+@pytest.mark.parametrize("start_wins", [False, True])
+def test_push_after_a_counted_start(ldd, cuda, start_wins):
+    """The first pass of a round appends vertex t (level L + 1).  Vertex a's long row is put off, so
+    that the small hub's push reaches it in the second pass: same code as t, smaller id.  In the
+    next round w's scan meets a first and stops."""
+    n = 80000
+    a, hub, t, w, big = 2, 5000, 6000, 7000, 9000
+    edges = [(big, v) for v in range(9001, n)] + [(a, v) for v in range(100, 3100)]
+    edges += [(hub, a), (a, w), (t, w)]
+    G = gen.from_edges(n, edges)
+    s = np.full(n, 0.125)
+    s[hub] = 5.5 + (0.0 if start_wins else EPS)
+    s[big] = 5.25
+    s[t] = 4.5 + (EPS if start_wins else 0.0)
+    st = _single(ldd, G, s)
+    assert st["pull_rounds"] > 1
+    assert st["exact_rank"] == 1 or not start_wins
     _union(ldd, G, [s])
