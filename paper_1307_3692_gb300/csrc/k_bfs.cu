@@ -1423,7 +1423,10 @@ __device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lv
       p += got;
       // the end of a scan, or of this lane's share of it: offer what was found
       const bool offer = !push && w != kNone && p == stop && best < kw;
-      if (!push && w != kNone && p == stop && best > kw) note_tie(a, w, best, kw);
+      if (!push && w != kNone && p == stop && best > kw) {
+        note_tie(a, w, best, kw);
+        best = ~0ull;  // once
+      }
       const u32 om = __ballot_sync(kFull, offer);
       if (om) {
         const int first = __ffs(om) - 1;

@@ -551,26 +551,29 @@ __device__ __forceinline__ bool key_near(u64 x, u64 y) {
 }
 
 // Two keys of vertex w's member met, x and y.  If only their ids differ, the
-// meeting is listed for finalize (tie_check).
+// meeting is listed for finalize (tie_check).  The first one that finds the list
+// full fails the attempt, so that the round loop ends at its next barrier, and
+// from then on the counter is only read: shifts with few distinct fractions make
+// almost every meeting a tie.
 __device__ __forceinline__ void note_tie(Control* ctl, const KeyFmt& f, u32 w, u64 x, u64 y) {
-  if (key_tie(f, x, y)) {
+  if (key_tie(f, x, y) && *(volatile u32*)&ctl->ties <= kMaxTies) {
     const u32 at = atomicAdd(&ctl->ties, 1u);
     if (at < kMaxTies) {
       ctl->tie[at][0] = w;
       ctl->tie[at][1] = key_id(f, x);
       ctl->tie[at][2] = key_id(f, y);
+    } else if (at == kMaxTies) {
+      atomicOr(&ctl->err, kErrRankRetry);
     }
   }
 }
 
 // Thread t of one CTA checks listed meeting t: the ids are ordered as the exact
-// fractions are (larger first), or the attempt fails, as it does when meetings
-// were too many.
+// fractions are (larger first), or the attempt fails.  (With too many meetings it
+// has failed before.)
 __device__ __forceinline__ void tie_check(const double* shift, const u32* wmem, const u32* ooff,
                                           Control* ctl, u32 t) {
-  const u32 ties = ctl->ties;
-  if (t == 0 && ties > kMaxTies) atomicOr(&ctl->err, kErrRankRetry);
-  if (t >= min(ties, kMaxTies)) return;
+  if (t >= min(ctl->ties, kMaxTies)) return;
   const double* own = shift + (wmem ? ooff[wmem[ctl->tie[t][0] >> 5]] : 0u);
   const u32 x = ctl->tie[t][1], y = ctl->tie[t][2];
   u32 err = 0;

@@ -116,3 +116,37 @@ def test_push_after_a_counted_start(ldd, cuda, start_wins):
     assert st["pull_rounds"] > 1
     assert st["exact_rank"] == 1 or not start_wins
     _union(ldd, G, [s])
+
+
+@pytest.mark.parametrize("how", ["single", "batch", "replay", "union", "blocks"])
+@pytest.mark.parametrize("name", ["rmat", "grid"])
+def test_fractions_that_all_tie(ldd, cuda, name, how):
+    """Integer shifts and halves: every meeting ties, the ranked keys answer."""
+    G = gen.rmat(14, seed=5) if name == "rmat" else gen.grid2d(150, 131)
+    g = ldd.LddGraph(G.row_ptr, G.col)
+    S = [np.floor(gen.shifts(G.n, 0.1, 1)), np.floor(gen.shifts(G.n, 0.3, 2) * 2.0) / 2.0]
+    out = [np.empty(G.n, np.int32) for _ in range(4)]
+    if how == "single" or how == "replay":
+        g.set_graph_replay(how == "replay")
+        for _ in range(3):
+            for s in S:
+                g.decompose(0.1, s, out[0], out[1])
+                _check(G, s, out[0], out[1])
+                assert g.stats()["exact_rank"] == 1 or name == "rmat"
+    elif how == "batch":
+        g.decompose_batch([0.1, 0.3], S, out[:2], out[2:])
+        _check(G, S[0], out[0], out[2])
+        _check(G, S[1], out[1], out[3])
+    elif how == "union":
+        u = ldd.LddUnion([g, g])
+        c, d = np.empty(2 * G.n, np.int32), np.empty(2 * G.n, np.int32)
+        u.decompose([0.1, 0.3], np.concatenate(S), c, d)
+        for i, s in enumerate(S):
+            _check(G, s, c[i * G.n:(i + 1) * G.n], d[i * G.n:(i + 1) * G.n])
+        u.close()
+    else:
+        c = [np.empty(G.n, np.int32) for _ in S]
+        d = [np.empty(G.n, np.int32) for _ in S]
+        g.block_decompose([0.1, 0.3], S, c, d)
+        _check(G, S[0], c[0], d[0])
+    g.close()
