@@ -435,8 +435,9 @@ int ldd_set_timing(ldd_graph* g, int enable);
 typedef struct {
   int32_t bfs_blocks_per_sm; /* CTAs of the persistent round loop per SM (1 or 2); by default
                                 1, and 2 in a union with rows of more than 32 arcs */
-  int32_t pull_alpha;        /* go bottom-up when frontier arcs x alpha > unsettled arcs;
-                                until it is changed, low-degree rounds stay top-down */
+  int32_t pull_alpha;        /* go bottom-up when frontier arcs x alpha > unsettled arcs
+                                (0: never); 14 by default, 0 for graphs that run
+                                low-degree rounds */
   int32_t pull_beta;         /* back to top-down when frontier vertices x beta < BFS vertices */
   int32_t pull_gamma;        /* ... and bottom-up only when frontier arcs x gamma > BFS vertices */
   int32_t probe_min_arcs;    /* top-down rounds with at least this many arcs read a key
@@ -448,7 +449,8 @@ typedef struct {
   int32_t window_levels;     /* low-degree rounds: levels relaxed between two grid barriers
                                 (each CTA going on with the vertices it reaches; exact, but a
                                 vertex may be expanded twice); 0 or 1: one level per barrier;
-                                8 by default, 1 in a union (four until it is changed) */
+                                8 by default, 1 in a union; while no tuning has been set on
+                                it, a union that runs low-degree rounds relaxes four */
   int32_t window_max_frontier; /* ... a window only while the frontier has at most this many
                                 vertices (>= 0; 2^18 by default) */
   int32_t window_queue;      /* ... entries of a CTA's local queue per level: 0 for as many

@@ -441,8 +441,8 @@ float elapsed(ldd_graph* g, int a, int b) {
 // 8 1.19 ms, 12 1.11, 24 1.08; 256^3 grid 2.56, 2.47, 2.62 -- and hurt elsewhere:
 // random geometric graph of 150,001 vertices 0.43, 0.52, 0.85).
 constexpr u32 kDefaultWindowLevels = 8;
-// Unions: one, and four where the tuning has not been touched and low-degree
-// rounds run (64 random geometric graphs: 1 level 3.55, 3 2.70, 4 2.63, 6 2.65,
+// Unions: one is what a fresh union reports, and what ldd_set_tuning(1) gives; while
+// its tuning has not been set, one of low-degree graphs relaxes four (64 random geometric graphs: 1 level 3.55, 3 2.70, 4 2.63, 6 2.65,
 // 8 2.74 ms).
 constexpr u32 kDefaultUnionWindowLevels = 1;
 constexpr u32 kLdUnionWindowLevels = 4;
@@ -476,7 +476,7 @@ BfsArgs bfs_args(ldd_graph* g, KeyFmt f, const double* shift) {
   a.nnz_active = g->nnz_active;
   a.spin_limit = g->spin_limit;
   a.bar_phantom = g->stall_barrier ? 1u : 0u;
-  a.pull_alpha = g->low_pull() ? 0 : g->pull_alpha;
+  a.pull_alpha = g->pull_alpha;
   a.pull_beta = g->pull_beta;
   a.pull_gamma = g->pull_gamma;
   a.probe_min_arcs = g->probe_min_arcs;
@@ -547,8 +547,16 @@ int run_bfs_finalize(ldd_graph* g, KeyFmt f, const double* shift, int* center, i
   return launches;
 }
 
+constexpr u32 kDefaultPullAlpha = 14;
 constexpr u32 kDefaultBarrierPolls = 1u << 22;   // grid barrier: each poll >= 20 ns after 64
 constexpr u32 kDefaultLookbackPolls = 1u << 24;  // look-back: each poll >= 64 ns after 16
+// Low-degree rounds stay top-down unless the tuning says otherwise: a scan of
+// a few arcs has next to none to save, and it reads every unsettled vertex (64
+// random geometric graphs: 5.09 -> 4.60 ms).
+void follow_degrees(ldd_graph* g) {
+  if (!g->pull_set) g->pull_alpha = g->low_degree() ? 0 : kDefaultPullAlpha;
+}
+
 // Scratch arena, pinned header, events and launch parameters: the part of
 // graph creation that only depends on the sizes and the tables being built.
 int finish_setup(ldd_graph* g) {
@@ -574,8 +582,8 @@ int finish_setup(ldd_graph* g) {
   g->bfs_grid = g->bfs_per_sm * g->num_sms;
   g->spin_limit = env_u32("LDD_SPIN_LIMIT", kDefaultBarrierPolls);
   g->lookback_limit = kDefaultLookbackPolls;
-  g->pull_alpha = env_u32("LDD_PULL_ALPHA", 14);
   g->pull_set = getenv("LDD_PULL_ALPHA") != nullptr;
+  g->pull_alpha = env_u32("LDD_PULL_ALPHA", kDefaultPullAlpha);
   g->pull_beta = env_u32("LDD_PULL_BETA", 24);
   g->pull_gamma = env_u32("LDD_PULL_GAMMA", 8);
   g->probe_min_arcs = env_u32("LDD_PROBE_MIN_ARCS", 1u << 16);
@@ -585,6 +593,7 @@ int finish_setup(ldd_graph* g) {
       env_u32("LDD_WINDOW_LEVELS", g->uni ? kDefaultUnionWindowLevels : kDefaultWindowLevels);
   g->window_set = getenv("LDD_WINDOW_LEVELS") != nullptr;
   g->window_max_q = env_u32("LDD_WINDOW_MAX_FRONTIER", 1u << 18);
+  follow_degrees(g);
   g->stats.n = g->n;
   g->stats.nnz = g->nnz;
   g->stats.n_active = g->n_active;
@@ -1235,6 +1244,7 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
     g->bfs_grid = g->bfs_per_sm * g->num_sms;
     g->stats.bfs_grid = g->bfs_grid;
   }
+  follow_degrees(g);
   g->d_active = (all_active && n_active > 0) ? U.d_active_buf : nullptr;
   U.k = (u32)k;
   U.max_n = 0;
@@ -1995,9 +2005,7 @@ int ldd_set_tuning(ldd_graph* g, const ldd_tuning* t) {
       t->window_levels > 4096 || t->window_max_frontier < 0 || t->window_queue < 0 ||
       t->bfs_span < kBfsBase || t->bfs_span > kBfsMaxSpan || t->bfs_span % kBfsBase != 0)
     return fail(LDD_ERR_ARG, "tuning out of range (blocks per SM 1 .. %d)", max_per_sm);
-  g->per_sm_set = g->per_sm_set || g->bfs_per_sm != t->bfs_blocks_per_sm;
-  g->pull_set = g->pull_set || g->pull_alpha != (u32)t->pull_alpha;
-  g->window_set = g->window_set || g->window_levels != (u32)t->window_levels;
+  g->per_sm_set = g->pull_set = g->window_set = true;  // every value as it is given
   g->bfs_per_sm = t->bfs_blocks_per_sm;
   g->bfs_grid = g->bfs_per_sm * g->num_sms;
   g->pull_alpha = (u32)t->pull_alpha;
@@ -2057,18 +2065,12 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out) 
   };
   ldd_tuning cur;
   ldd_get_tuning(g, &cur);
-  // a field at its first value keeps following the graph if it did
-  const ldd_tuning t0 = cur;
-  const bool per0 = g->per_sm_set, pull0 = g->pull_set, window0 = g->window_set;
-  auto apply = [&](const ldd_tuning& t) {
-    const int status = ldd_set_tuning(g, &t);
-    g->per_sm_set = per0 || t.bfs_blocks_per_sm != t0.bfs_blocks_per_sm;
-    g->pull_set = pull0 || t.pull_alpha != t0.pull_alpha;
-    g->window_set = window0 || t.window_levels != t0.window_levels;
-    return status;
-  };
+  // from here on every value as it is given; first what has run so far
+  const bool ld_possible = g->max_degree <= (u32)kLdMaxDegree;
+  if (g->uni && !g->window_set && g->low_degree()) cur.window_levels = (int)kLdUnionWindowLevels;
+  const int given = ldd_set_tuning(g, &cur);
   float best_ms;
-  int rc = measure(&best_ms);
+  int rc = given == LDD_OK ? measure(&best_ms) : given;
   int max_per_sm = 1;
   bfs_grid_size(g->num_sms, &max_per_sm);
   // coordinate descent, one parameter at a time over a few candidates
@@ -2079,7 +2081,6 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out) 
   const int32_t ld_vals[2] = {0, 1};
   const int32_t window_vals[3] = {1, 8, 16};
   const int32_t span_vals[3] = {1024, 2048, 4096};
-  const bool ld_possible = g->max_degree <= (u32)kLdMaxDegree;
   for (int param = 0; param < 8 && rc == LDD_OK; ++param) {
     const int32_t* vals = param == 0 ? alphas : param == 1 ? betas : param == 2 ? gammas : probes;
     int nv = param == 3 ? 4 : 5;
@@ -2108,7 +2109,10 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out) 
                      : param == 6 ? &t.low_degree_rounds : &t.bfs_span;
       if (*field == vals[i]) continue;
       *field = vals[i];
-      if ((rc = apply(t)) != LDD_OK) break;
+      // edge-balanced rounds are worth trying with bottom-up ones only
+      if (param == 6 && t.low_degree_rounds == 0 && t.pull_alpha == 0)
+        t.pull_alpha = (int)kDefaultPullAlpha;
+      if ((rc = ldd_set_tuning(g, &t)) != LDD_OK) break;
       float ms;
       if ((rc = measure(&ms)) != LDD_OK) break;
       if (ms < best_ms * 0.98f) {  // keep only a clear gain
@@ -2120,7 +2124,7 @@ int ldd_autotune(ldd_graph* g, const double* shifts, int reps, ldd_tuning* out) 
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   g->replay = saved_replay;
-  const int rc2 = apply(cur);
+  const int rc2 = ldd_set_tuning(g, &cur);
   if (rc != LDD_OK) return rc;
   if (rc2 != LDD_OK) return rc2;
   *out = cur;

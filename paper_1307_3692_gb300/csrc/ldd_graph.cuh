@@ -147,12 +147,8 @@ struct ldd_graph {
   bool low_degree() const {
     return low_degree_rounds && max_degree <= (u32)kLdMaxDegree && ell_s > 0;
   }
-  // Set by the user (else bfs_per_sm, pull_alpha and window_levels follow the graph).
+  // Set by the user (else bfs_per_sm, pull_alpha and a union's windows follow the graph).
   bool per_sm_set = false, pull_set = false, window_set = false;
-  // Low-degree rounds stay top-down unless the tuning says otherwise: a scan of
-  // a few arcs has next to none to save, and it reads every unsettled vertex (64
-  // random geometric graphs: 5.09 -> 4.60 ms).
-  bool low_pull() const { return low_degree() && !pull_set; }
   u32 window_levels = 0;          // tuning: levels per window in low-degree rounds (0: none)
   u32 window_max_q = 1u << 18;    // tuning: windows only for frontiers up to this size
   u32 window_queue = 0;           // tuning: local-queue entries per CTA and level (0: all that fit)
