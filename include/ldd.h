@@ -74,8 +74,10 @@ int ldd_create_graph(int32_t n, int64_t nnz, const int32_t* row_ptr, const int32
  * as Algorithm 1 / Section 4).
  *   g          graph from ldd_create_graph.
  *   beta       the Exp(beta) parameter the shifts were drawn with; must be
- *              finite and > 0.  It is checked and recorded, not used: the
- *              assignment depends on the shifts alone.
+ *              finite and > 0.  The assignment depends on the shifts alone;
+ *              beta only suggests how large they get.  Shifts beyond 36.8 / beta
+ *              (none drawn with Exp(beta) is) are accepted; the first such call
+ *              in a row may pass over its shifts twice.
  *   shifts     double[n]: delta_u for every vertex, each finite, >= 0 and
  *              < 2^31 (a NaN or negative value gives LDD_ERR_ARG, a value
  *              >= 2^31 or infinite gives LDD_ERR_RANGE).
@@ -203,7 +205,7 @@ int ldd_union_size(const ldd_graph* u, int32_t* out_k, int64_t* out_total);
  * Arrays use the caller layout: member s's n_s entries at offset
  * n_0 + ... + n_{s-1}, in member order.
  *   betas       double[k] on the host: each member's beta (finite, > 0;
- *               checked, not used, as in ldd_decompose).
+ *               used as in ldd_decompose).
  *   shifts      double[total] (host or device): member s's shifts, each as
  *               in ldd_decompose.
  *   out_center  int32[total] (host or device): member-local center ids.
@@ -227,8 +229,8 @@ int ldd_union_decompose(ldd_graph* u, const double* betas, const double* shifts,
  * block i, and the edges it cuts are E_{i+1}.  The loop stops after the first
  * iteration that leaves no edge, or after k iterations.
  *   k            number of shift vectors available (iterations at most).
- *   betas        double[k] on the host: each finite and > 0 (checked, not used;
- *                the paper's choice is beta = 1/2).
+ *   betas        double[k] on the host: each finite and > 0 (used as in
+ *                ldd_decompose; the paper's choice is beta = 1/2).
  *   shifts       k pointers to n doubles (host or device), as in
  *                ldd_decompose; shift vector i is read only if iteration i runs.
  *   out_center, out_dist  NULL, or k pointers to n int32 (host or device):

@@ -627,13 +627,26 @@ KeyFmt direct_fmt(const ldd_graph* g, u64 floors) {
 }
 
 // The largest floor to expect of shifts drawn with Exp(beta): -ln(U) / beta with
-// a 53-bit U is below 36.8 / beta.  Only a hint for the key layout: larger floors
-// make the call widen the level field and run again.  In a union a vertex that
-// the round loop does not handle may be lifted beyond it.
-u64 floors_for(const ldd_graph* g, double beta) {
+// a 53-bit U is below 36.8 / beta.  In a union a vertex that the round loop does
+// not handle may be lifted beyond it.
+u64 floors_for_beta(const ldd_graph* g, double beta) {
   if (!(beta > 0.0)) return 65534;
   const double x = std::min(36.8 / beta + 2.0, 1073741824.0);
   return (u64)x * (g->uni ? 2 : 1);
+}
+
+// The range of floors a call lays its keys out for: what beta suggests, or the one of
+// the call before if its shifts went beyond that.  Only a hint: larger floors make the call
+// widen the level field and run its key pass again.
+u64 floors_for(const ldd_graph* g, double beta) {
+  return std::max(floors_for_beta(g, beta), g->wide_floors);
+}
+
+// Floors beyond what beta suggests are expected again, up to twice as large; the first
+// call without them ends that, so a single huge shift costs the next call's codes a
+// few bits and no more.
+u64 wide_floors(const ldd_graph* g, double beta, int A) {
+  return (u64)A > floors_for_beta(g, beta) ? 2 * (u64)A : 0;
 }
 
 struct Header {  // the control block up to and including the BFS runtime state
@@ -794,6 +807,7 @@ int decompose_on_device(ldd_graph* g, double beta, const double* d_shift, int* c
     }
   }
   if (h.err) return header_error(h.err);
+  if (!d_levels) g->wide_floors = wide_floors(g, beta, h.A);
   header_stats(g, h, exact64);
   ldd_stats& st = g->stats;
   st.ms_rank = elapsed(g, 1, 2);
@@ -945,6 +959,7 @@ int replay_fast(ldd_graph* g, double beta, bool want_cut, int* launches_out) {
     return kRunRegular;
   }
   if (h.err) return header_error(h.err);
+  g->wide_floors = wide_floors(g, beta, h.A);
   header_stats(g, h, false);
   ldd_stats& st = g->stats;
   st.ms_rank = st.ms_bfs = st.ms_finalize = -1.f;
@@ -1245,6 +1260,7 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
     g->stats.bfs_grid = g->bfs_grid;
   }
   follow_degrees(g);
+  g->wide_floors = 0;
   g->d_active = (all_active && n_active > 0) ? U.d_active_buf : nullptr;
   U.k = (u32)k;
   U.max_n = 0;
@@ -1768,6 +1784,8 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
   record(g, 0);
   if ((rc = upload(0)) != LDD_OK) return drain(rc);
   int launches = 0;
+  const u64 wide = g->wide_floors;
+  u64 wide_next = 0;
   for (int i = 0; i < k; ++i) {
     const int j = i & 1;
     if (i + 1 < k && (rc = upload(i + 1)) != LDD_OK) return drain(rc);  // overlaps decomposition i
@@ -1824,6 +1842,8 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
     Header h;
     memcpy(&h, g->h_bhdr + (size_t)i * sizeof(Header), sizeof(h));
     if (h.err & ~kErrRetry) return header_error(h.err);
+    g->wide_floors = wide;  // as the items were laid out
+    wide_next = std::max(wide_next, wide_floors(g, betas[i], h.A));
     if (h.err == 0) {
       header_stats(g, h, direct_fmt(g, floors_for(g, betas[i])).cap == 0);
       if (out_cut) out_cut[i] = (int64_t)g->h_bcut[i];
@@ -1836,6 +1856,7 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
     int* center = dev_c ? out_center[i] : d_c[0];
     int* dist = dev_d ? out_dist[i] : d_d[0];
     int l = 0;
+    g->wide_floors = std::max(wide, wide_floors(g, betas[i], h.A));
     if ((rc = decompose_on_device(g, betas[i], dev_in ? shifts[i] : d_in[0], center, dist, &l)) !=
         LDD_OK)
       return drain(rc);
@@ -1846,6 +1867,7 @@ int ldd_decompose_batch(ldd_graph* g, int k, const double* betas, const double* 
     if (!dev_d) CUDA_TRY(cudaMemcpyAsync(out_dist[i], dist, n * 4, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
   }
+  g->wide_floors = wide_next;
   g->stats.launches = launches;
   g->stats.ms_h2d = -1.f;  // overlapped: not attributable
   g->stats.ms_d2h = -1.f;
