@@ -884,11 +884,9 @@ int enqueue_fast(ldd_graph* g, KeyFmt f, bool want_cut) {
   return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 
-// Captures enqueue_fast into an executable graph (slot: with union cut
-// counts).  A capture that fails marks the graph replay_broken; the regular
+// Captures enqueue_fast into executable graph `slot`.  A capture that fails marks the graph replay_broken; the regular
 // path then runs.
-void capture_fast(ldd_graph* g, KeyFmt f, bool want_cut) {
-  const int slot = want_cut ? 1 : 0;
+void capture_fast(ldd_graph* g, KeyFmt f, bool want_cut, int slot) {
   if (!g->cap_stream &&
       cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
@@ -924,6 +922,7 @@ void capture_fast(ldd_graph* g, KeyFmt f, bool want_cut) {
   g->replay_launches[slot] = launches;
 }
 
+constexpr u64 kUsualFloors = 4094;  // beta >= 0.009 (a union's: 0.018)
 constexpr int kRunRegular = 1;  // replay_fast: take the regular path instead
 
 // One decomposition by graph replay, the shifts already in the library's
@@ -932,21 +931,28 @@ constexpr int kRunRegular = 1;  // replay_fast: take the regular path instead
 // direct keys asked for a retry).
 int replay_fast(ldd_graph* g, double beta, bool want_cut, int* launches_out) {
   if (!g->replay || g->replay_broken || g->regular_runs == 0) return kRunRegular;
-  // a captured key layout serves every smaller range of floors
+  // A captured key layout serves every smaller range of floors, with fewer code bits
+  // than that range's own.  The ranges of usual betas and larger ones are captured
+  // apart, so that a call of the second kind takes no bits from the first.
   const u64 floors = floors_for(g, beta);
-  if (floors > g->replay_floors) {
-    drop_replay(g);
-    g->replay_floors = floors;
+  if (direct_fmt(g, floors).cap == 0) return kRunRegular;
+  const int kind = floors > kUsualFloors ? 1 : 0;
+  if (floors > g->replay_floors[kind]) {
+    for (int i = 2 * kind; i < 2 * kind + 2; ++i)
+      if (g->gexec[i]) {
+        cudaGraphExecDestroy(g->gexec[i]);
+        g->gexec[i] = nullptr;
+      }
+    g->replay_floors[kind] = floors;
   }
-  const KeyFmt f = direct_fmt(g, g->replay_floors);
-  if (f.cap == 0) return kRunRegular;
-  const int slot = want_cut ? 1 : 0;
+  const KeyFmt f = direct_fmt(g, g->replay_floors[kind]);
+  const int slot = 2 * kind + (want_cut ? 1 : 0);
   cudaStream_t s = g->stream;
   if (g->acnt_dirty) {
     CUDA_TRY(cudaMemsetAsync(g->d_acnt, 0, (size_t)g->bptr_cap * 4, s));
     g->acnt_dirty = false;
   }
-  if (!g->gexec[slot]) capture_fast(g, f, want_cut);
+  if (!g->gexec[slot]) capture_fast(g, f, want_cut, slot);
   if (!g->gexec[slot]) return kRunRegular;
   record(g, 1);
   CUDA_TRY(cudaGraphLaunch(g->gexec[slot], s));

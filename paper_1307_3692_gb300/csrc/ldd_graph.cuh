@@ -197,11 +197,11 @@ struct ldd_graph {
   // captured CUDA graph of one fast-path decomposition (ldd_set_graph_replay)
   bool replay = false;
   bool replay_broken = false;        // capture failed once: regular path only
-  u64 replay_floors = 0;             // range of floors the captured key layout holds
+  u64 replay_floors[2] = {};         // ranges of floors the captured key layouts hold
   int regular_runs = 0;              // regular decompositions so far (capture waits for one)
   cudaStream_t cap_stream = nullptr;
-  cudaGraphExec_t gexec[2] = {};     // [with union cut counts]
-  int replay_launches[2] = {};
+  cudaGraphExec_t gexec[4] = {};     // [2 * range + with union cut counts]
+  int replay_launches[4] = {};
   u64* h_cut = nullptr;              // pinned copy of a union's cut counts
   ldd_stats stats;
 };

@@ -1,5 +1,6 @@
 """Shifts larger than beta suggests: the wider range is remembered, so that later
-calls, batches and replays need no second key pass."""
+calls, batches and replays need no second key pass; and one call with a tiny
+beta or a huge shift does not change what others run."""
 from __future__ import annotations
 
 import numpy as np
@@ -82,4 +83,28 @@ def test_replay_with_shifts_beyond_beta(ldd, cuda):
         replayed.append(u.stats()["replayed"])
     assert replayed[2:] == [1] * 4
     u.close()
+    g.close()
+
+
+@pytest.mark.parametrize("beta", [1e-12, 1e-6, 1e-4])
+def test_a_tiny_beta_changes_nothing_for_the_others(ldd, cuda, beta):
+    """A replayed graph: after one call whose beta leaves few code bits or none, calls with an
+    ordinary beta are replayed with the keys they had."""
+    G = gen.rmat(17, edge_factor=4, seed=3)
+    g = ldd.LddGraph(G.row_ptr, G.col, validate=False)
+    g.set_graph_replay(True)
+    (c,), (d,) = _bufs(G, cuda)
+    s = gen.shifts(G.n, 0.1, 1)
+    t = torch.from_numpy(s).to(cuda)
+    for b in (0.1, 0.1, beta, beta, 0.1, 0.05, beta, 0.1):
+        g.decompose(b, t, c, d)
+        _check(G, s, c, d)
+    assert g.stats()["replayed"] == 1 and g.stats()["exact_rank"] == 0
+    # one huge shift: the next ordinary call has its own layout again
+    h = s.copy()
+    h[int(np.argmax(np.diff(G.row_ptr)))] = 2.0e6 + 0.5
+    for x in (h, s, s):
+        g.decompose(0.1, torch.from_numpy(x).to(cuda), c, d)
+        _check(G, x, c, d)
+    assert g.stats()["replayed"] == 1 and g.stats()["exact_rank"] == 0
     g.close()
