@@ -63,6 +63,10 @@ typedef enum {
  *            meaning (a repeated edge is counted with its multiplicity).
  *            With validate = 0 an asymmetric CSR gives undefined results.
  *   out      receives the graph handle.
+ * Besides its tables and scratch a graph of at most 32 arcs per vertex keeps rows
+ * of equal length (up to 128 bytes per vertex) where they take at most a quarter
+ * of the memory that is left; without them it runs the general rounds, slower but
+ * with the same results.
  * Row order inside a row is free.  The input buffers may be freed after the
  * call returns.
  */
@@ -248,7 +252,8 @@ int ldd_union_decompose(ldd_graph* u, const double* betas, const double* shifts,
  * Errors as in ldd_decompose; a failure in iteration i leaves the outputs of
  * earlier iterations complete and *out_blocks = the iterations that finished.
  * The first call allocates the residual graphs' buffers (about 36 bytes per
- * arc and 220 per vertex), which stay with g until ldd_destroy_graph.
+ * arc and 180 per vertex, and on graphs of at most 32 arcs per vertex up to 128
+ * more where there is room), which stay with g until ldd_destroy_graph.
  * LDD_ERR_ARG for a union.
  */
 int ldd_block_decompose(ldd_graph* g, int k, const double* betas, const double* const* shifts,

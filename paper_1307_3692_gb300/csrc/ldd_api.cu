@@ -550,6 +550,26 @@ int run_bfs_finalize(ldd_graph* g, KeyFmt f, const double* shift, int* center, i
 constexpr u32 kDefaultPullAlpha = 14;
 constexpr u32 kDefaultBarrierPolls = 1u << 22;   // grid barrier: each poll >= 20 ns after 64
 constexpr u32 kDefaultLookbackPolls = 1u << 24;  // look-back: each poll >= 64 ns after 16
+// Padded rows (BfsArgs::ell) are for speed only, so they never take what something
+// else may need: at most a quarter of the memory that is free, after all else has been
+// allocated, and a graph or union without them runs the general rounds.
+u32 padded_width(u32 max_degree) {
+  return max_degree <= (u32)kLdMaxDegree ? (u32)align_up(std::max(max_degree, 1u), 8) : 0;
+}
+
+bool room_for_rows(u64 entries, u64 others) {  // others: bytes to be allocated besides
+  size_t avail = 0, total = 0;
+  return cudaMemGetInfo(&avail, &total) == cudaSuccess && others <= avail &&
+         entries * 4 <= (avail - others) / 4;
+}
+
+bool alloc_rows(u32** ell, u64 entries) {
+  if (cudaMalloc(ell, entries * 4) == cudaSuccess) return true;
+  cudaGetLastError();
+  *ell = nullptr;
+  return false;
+}
+
 // Low-degree rounds stay top-down unless the tuning says otherwise: a scan of
 // a few arcs has next to none to save, and it reads every unsettled vertex (64
 // random geometric graphs: 5.09 -> 4.60 ms).
@@ -1116,7 +1136,7 @@ int setup_batch(ldd_graph* g) {
 UnionCaps union_needs(int k, ldd_graph* const* members) {
   UnionCaps c;
   c.k = (u32)k;
-  bool rows = true;  // every member has padded rows
+  u32 max_deg = 0;
   for (int i = 0; i < k; ++i) {
     const ldd_graph* m = members[i];
     c.N += ((u64)m->n + 31) / 32 * 32;
@@ -1126,10 +1146,9 @@ UnionCaps union_needs(int k, ldd_graph* const* members) {
     c.C += m->sc.ncomp;
     c.T += m->sc.total;
     c.total += (u64)m->n;
-    c.S = std::max(c.S, m->ell_s);
-    rows = rows && m->ell_s > 0;
+    max_deg = std::max(max_deg, m->max_degree);
   }
-  if (!rows) c.S = 0;
+  c.S = padded_width(max_deg);
   c.L = c.N * c.S;
   return c;
 }
@@ -1190,7 +1209,6 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
       cudaMalloc(&U.d_mem, K * sizeof(UnionMember)) != cudaSuccess ||
       cudaMalloc(&U.d_offs, 9 * (K + 1) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_hotv, std::max<u64>(N, 1) * 4) != cudaSuccess ||
-      cudaMalloc(&U.d_ell_buf, std::max<u64>(c.L, 8) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_shift_in, total * 8) != cudaSuccess ||
       cudaMalloc(&U.d_out_c, total * 8) != cudaSuccess ||
       cudaMalloc(&U.d_cut, K * 8) != cudaSuccess ||
@@ -1215,6 +1233,7 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
   g->nnz = (int64_t)c.E;
   int rc = finish_setup(g);
   if (rc != LDD_OK) return bail(rc);
+  if (c.L > 0 && !alloc_rows(&U.d_ell_buf, c.L)) U.cap.L = 0;
   *out = g;
   return LDD_OK;
 }
@@ -1472,17 +1491,17 @@ int ldd_create_graph(int32_t n, int64_t nnz, const int32_t* row_ptr, const int32
     if (cudaStreamSynchronize(nullptr) != cudaSuccess)
       return bail(fail(LDD_ERR_CUDA, "first-neighbour table"));
   }
-  if (g->max_degree <= (u32)kLdMaxDegree) {  // padded rows for the low-degree rounds
-    g->ell_s = (u32)align_up(std::max(g->max_degree, 1u), 8);
-    if (cudaMalloc(&g->d_ell, (size_t)std::max<int64_t>(n, 1) * g->ell_s * 4) != cudaSuccess) {
-      cudaGetLastError();
-      return bail(fail(LDD_ERR_OOM, "device allocation of the padded rows failed"));
-    }
+  if ((rc = finish_setup(g)) != LDD_OK) return bail(rc);
+  // padded rows for the low-degree rounds; without room for them the general ones run
+  const u32 width = padded_width(g->max_degree);
+  if (width > 0 && room_for_rows((u64)n * width, 0) &&
+      alloc_rows(&g->d_ell, (u64)std::max<int64_t>(n, 1) * width)) {
+    g->ell_s = width;
     launch_padded_rows(g->d_row, g->d_col, (u32)n, g->ell_s, g->d_ell, g->num_sms, nullptr);
     if (cudaStreamSynchronize(nullptr) != cudaSuccess)
       return bail(fail(LDD_ERR_CUDA, "padded rows"));
+    follow_degrees(g);
   }
-  if ((rc = finish_setup(g)) != LDD_OK) return bail(rc);
   // low-degree rounds are latency-bound: a key probe before every atomicMin
   // is one more dependent round trip, worth it only in wide rounds
   if (g->max_degree <= (u32)kLdMaxDegree && !getenv("LDD_PROBE_MIN_ARCS"))
@@ -1916,13 +1935,14 @@ int ldd_create_union(int k, ldd_graph* const* members, ldd_graph** out) {
   }
   DeviceGuard dg(dev);
   if (!dg.ok) return fail(LDD_ERR_CUDA, "cannot select device %d", dev);
-  const UnionCaps c = union_needs(k, members);
+  UnionCaps c = union_needs(k, members);
   if (c.N >= (1u << 30))
     return fail(LDD_ERR_RANGE, "union of %llu vertices (padded) must be < 2^30",
                 (unsigned long long)c.N);
   if (c.E >= (1ull << 31))
     return fail(LDD_ERR_RANGE, "union of %llu arcs must be < 2^31", (unsigned long long)c.E);
   ldd_graph* g = nullptr;
+  if (!room_for_rows(c.L, union_bytes(c) - 4 * c.L)) c.L = 0;
   int rc = union_alloc(&g, dev, c);
   if (rc != LDD_OK) return rc;
   if ((rc = union_fill(g, k, members, nullptr, true)) != LDD_OK) {

@@ -40,7 +40,7 @@ struct Blocks {
   int* src[2] = {};            // [nnz] source vertex of every arc of G_i, i >= 1
   u32* map[2] = {};            // [n] input id of every vertex of G_i, i >= 1
   int* off = nullptr;          // [n + 1] kept arcs per vertex of G_i, then their offsets
-  u32* ell = nullptr;          // [n * g->ell_s] padded rows of G_i, i >= 1 (low-degree graphs)
+  u32* ell = nullptr;          // [n * g->ell_s] padded rows of G_i, i >= 1 (if there is room)
   u32* cid = nullptr;          // [n + 1] vertices with kept arcs, then their ids in G_{i+1}
   int* src0 = nullptr;         // [nnz] source vertex of every arc of G_0
   u32* klist = nullptr;        // [nnz] the count pass's kept arcs
@@ -107,8 +107,7 @@ int setup_blocks(ldd_graph* g) {
          cudaMalloc(&b->src[j], nnz * 4) == cudaSuccess &&
          cudaMalloc(&b->map[j], std::max<size_t>(n, 1) * 4) == cudaSuccess;
   ok = ok && cudaMalloc(&b->off, (n + 1) * 4) == cudaSuccess &&
-       cudaMalloc(&b->cid, (n + 1) * 4) == cudaSuccess &&
-       (g->ell_s == 0 || cudaMalloc(&b->ell, n * g->ell_s * 4) == cudaSuccess);
+       cudaMalloc(&b->cid, (n + 1) * 4) == cudaSuccess;
   ok = ok && cudaMalloc(&b->src0, nnz * 4) == cudaSuccess &&
        cudaMalloc(&b->klist, nnz * 4) == cudaSuccess &&
        cudaMalloc(&b->cursor, (n + 1) * 4) == cudaSuccess &&
@@ -157,6 +156,7 @@ int setup_blocks(ldd_graph* g) {
     free_blocks(g);
     return rc;
   }
+  if (g->ell_s > 0 && room_for_rows((u64)n * g->ell_s, 0)) alloc_rows(&b->ell, (u64)n * g->ell_s);
   launch_fill_src(g->d_row, (u32)n, b->src0, g->num_sms, g->stream);
   if (cudaGetLastError() != cudaSuccess) {
     free_blocks(g);
@@ -181,7 +181,8 @@ void sync_params(ldd_graph* g, ldd_graph* r) {
   r->probe_min_arcs = g->probe_min_arcs;
   r->low_degree_rounds = g->low_degree_rounds;
   r->max_degree = g->max_degree;  // residual rows are never longer
-  r->ell_s = g->ell_s;
+  r->ell_s = g->blk->ell ? g->ell_s : 0;
+  follow_degrees(r);
 }
 
 }  // namespace

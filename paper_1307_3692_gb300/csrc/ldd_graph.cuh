@@ -54,7 +54,7 @@ struct UnionCaps {
   u64 C = 0;      // small components
   u64 T = 0;      // their members
   u64 total = 0;  // caller-layout entries (sum of member sizes)
-  u64 L = 0;      // entries of the padded rows (all members low-degree)
+  u64 L = 0;      // entries of the padded rows (all members low-degree), if there is room
   u32 S = 0;      // ... per row, or 0
   u32 k = 0;      // members
 };
@@ -213,6 +213,11 @@ int free_graph_memory(ldd_graph* g);
 // Scratch arena, pinned header, events and launch parameters of a graph whose
 // sizes (n, nnz, device, num_sms) are set (ldd_api.cu).
 int finish_setup(ldd_graph* g);
+// Launch parameters that follow the graph until the tuning is set.
+void follow_degrees(ldd_graph* g);
+// Room for padded rows beside `others` bytes, and their allocation (false: none).
+bool room_for_rows(u64 entries, u64 others);
+bool alloc_rows(u32** ell, u64 entries);
 // The block decomposition's state of g (ldd_blocks.cu); null is a no-op.
 void free_blocks(ldd_graph* g);
 void record(ldd_graph* g, int i);

@@ -355,6 +355,7 @@ int ldd_server_create(const ldd_server_config* cfg, ldd_server** out) {
       u64* h = nullptr;
       int rc = union_alloc(&u, S->device, S->cap);
       S->ws.push_back(u);
+      if (rc == LDD_OK) S->cap.L = std::min(S->cap.L, u->uni->cap.L);  // rows may have found no room
       if (rc == LDD_OK && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess)
         rc = fail(LDD_ERR_CUDA, "cudaStreamCreate failed");
       S->streams.push_back(st);
