@@ -306,20 +306,31 @@ int build_component_tables(ldd_graph* g) {
   return rc;
 }
 
-// Buffers of the cut counts by piece codes.
-int alloc_codes(ldd_graph* g, size_t rows, size_t n, size_t ngrp, size_t nhot, const u32* hotv) {
+// Buffers of the cut counts by piece codes.  False where there is no room: the counts
+// then go by labels.
+bool alloc_codes(ldd_graph* g, size_t rows, size_t n, size_t ngrp, size_t nhot, const u32* hotv) {
   CutCodes& cc = g->cc;
-  cc.hotv = hotv;
-  cc.solo = g->d_solo;
-  cc.nhot = (u32)nhot;
   if (cudaMalloc(&cc.picks, rows * (kCodePieces + 1) * sizeof(u32)) != cudaSuccess ||
       cudaMalloc(&cc.code, std::max<size_t>(n, 1) * sizeof(u16)) != cudaSuccess ||
       cudaMalloc(&cc.gcode, std::max<size_t>(ngrp, 1) * sizeof(u16)) != cudaSuccess ||
       cudaMalloc(&cc.hcode, align_up(std::max<size_t>(nhot, 1), 8) * sizeof(u16)) != cudaSuccess) {
     cudaGetLastError();
-    return fail(LDD_ERR_OOM, "device allocation of the piece codes failed");
+    cudaFree(cc.picks);
+    cudaFree(cc.code);
+    cudaFree(cc.gcode);
+    cudaFree(cc.hcode);
+    cc = CutCodes();
+    return false;
   }
-  return LDD_OK;
+  cc.hotv = hotv;
+  cc.solo = g->d_solo;
+  cc.nhot = (u32)nhot;
+  return true;
+}
+
+// Whether cut counts go by piece codes: graphs with hubs, and edges enough.
+bool wants_codes(u32 max_degree, u64 m) {
+  return max_degree > (u32)kLdMaxDegree && m >= kCodeMinEdges;
 }
 
 // The grouped cut list of launch_cut (CutList): each edge oriented from its
@@ -338,7 +349,7 @@ int build_cut_list(ldd_graph* g, const std::vector<int32_t>& rp, const std::vect
     const int32_t da = deg(a), db = deg(b);
     return da > db || (da == db && a < b);
   };
-  g->code_cut = g->max_degree > (u32)kLdMaxDegree && m >= kCodeMinEdges;
+  g->code_cut = wants_codes(g->max_degree, m);
   const size_t K = m ? std::min<size_t>(g->code_cut ? kCodeSlots : kHotSlots, n) : 0;
   std::vector<int32_t> ids(n);
   for (size_t v = 0; v < n; ++v) ids[v] = (int32_t)v;
@@ -394,7 +405,7 @@ int build_cut_list(ldd_graph* g, const std::vector<int32_t>& rp, const std::vect
       cudaMemcpy(cl.blk_mask, blk_mask.data(), blk_mask.size() * 4, cudaMemcpyHostToDevice) !=
           cudaSuccess)
     return fail(LDD_ERR_CUDA, "upload of the cut list failed");
-  if (g->code_cut) return alloc_codes(g, 4, n, cl.ngrp, K, g->d_hot);
+  g->code_cut = g->code_cut && alloc_codes(g, 4, n, cl.ngrp, K, g->d_hot);
   return LDD_OK;
 }
 
@@ -1149,6 +1160,7 @@ UnionCaps union_needs(int k, ldd_graph* const* members) {
     max_deg = std::max(max_deg, m->max_degree);
   }
   c.S = padded_width(max_deg);
+  c.codes = wants_codes(max_deg, c.M);
   c.L = c.N * c.S;
   return c;
 }
@@ -1160,8 +1172,9 @@ u64 union_bytes(const UnionCaps& c) {
   const u64 N = c.N, words = std::max<u64>(N / 32, 1);
   u64 b = 4 * (N + 1) + 4 * c.E + 4 * c.M + 20 * c.G + 8 * (c.M / 32 + 1) + 8 * words +
           8 * c.C + 8 * c.T + 4 * N + 4 * words;
-  b += 16 * c.total + 8 * c.total + 36ull * (c.k + 1) + 120ull * c.k + 2 * c.total + 2 * c.G +
-       6 * N + 4 * c.L + sizeof(UnionMember) * c.k;
+  b += 16 * c.total + 8 * c.total + 36ull * (c.k + 1) + 64ull * c.k + 4 * c.L +
+       sizeof(UnionMember) * c.k;
+  if (c.codes) b += 2 * c.total + 2 * c.G + 6 * N + 64ull * c.k;
   const u64 nk = std::max<u64>(N, 64);
   b += 8 * N + 4 * N + 16 * nk + 8 * N + ((N + kSortTile - 1) / kSortTile + 1) * 2048 + 4 * N +
        8 * N + 36 * N + 12 * (c.E / kBfsBase + 2) + 8 * N + 4 * (N / kMaxBlock + 1) + 8 * N +
@@ -1208,7 +1221,6 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
       cudaMalloc(&U.d_active_buf, std::max<u64>(N, 1) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_mem, K * sizeof(UnionMember)) != cudaSuccess ||
       cudaMalloc(&U.d_offs, 9 * (K + 1) * 4) != cudaSuccess ||
-      cudaMalloc(&U.d_hotv, std::max<u64>(N, 1) * 4) != cudaSuccess ||
       cudaMalloc(&U.d_shift_in, total * 8) != cudaSuccess ||
       cudaMalloc(&U.d_out_c, total * 8) != cudaSuccess ||
       cudaMalloc(&U.d_cut, K * 8) != cudaSuccess ||
@@ -1226,13 +1238,16 @@ int union_alloc(ldd_graph** out, int dev, const UnionCaps& c) {
   const size_t K1 = K + 1;
   U.off = UnionOffsets{d,          d + K1,     d + 2 * K1, d + 3 * K1,
                        d + 4 * K1, d + 5 * K1, d + 6 * K1, d + 7 * K1, d + 8 * K1};
-  const int cc = alloc_codes(g, K, total, c.G, N, U.d_hotv);
-  if (cc != LDD_OK) return bail(cc);
   // the scratch arena and launch set-up are sized by the capacities
   g->n = (int32_t)N;
   g->nnz = (int64_t)c.E;
   int rc = finish_setup(g);
   if (rc != LDD_OK) return bail(rc);
+  if (c.codes && cudaMalloc(&U.d_hotv, std::max<u64>(N, 1) * 4) != cudaSuccess) {
+    cudaGetLastError();
+    U.d_hotv = nullptr;
+  }
+  U.cap.codes = U.d_hotv != nullptr && alloc_codes(g, K, total, c.G, N, U.d_hotv);
   if (c.L > 0 && !alloc_rows(&U.d_ell_buf, c.L)) U.cap.L = 0;
   *out = g;
   return LDD_OK;
@@ -1321,7 +1336,7 @@ int union_fill(ldd_graph* g, int k, ldd_graph* const* members, cudaStream_t s, b
   CUDA_TRY(cudaMemcpyAsync(U.d_mem, mv.data(), mv.size() * sizeof(UnionMember),
                            cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(U.d_offs, offs.data(), offs.size() * 4, cudaMemcpyHostToDevice, s));
-  g->code_cut = max_deg > (u32)kLdMaxDegree && need.M >= kCodeMinEdges;
+  g->code_cut = need.codes && U.cap.codes;
   g->cc.nhot = at(8, k);
   UnionTables t{g->d_row, g->d_col, g->cut, g->d_excl, g->d_solo, g->sc.comp_off,
                 g->sc.comp_len, g->sc.comp_v, g->sc.adj, g->d_active, U.d_wmem,

@@ -56,6 +56,7 @@ struct UnionCaps {
   u64 total = 0;  // caller-layout entries (sum of member sizes)
   u64 L = 0;      // entries of the padded rows (all members low-degree), if there is room
   u32 S = 0;      // ... per row, or 0
+  bool codes = false;  // cut counts by piece codes: their buffers
   u32 k = 0;      // members
 };
 struct Blocks;  // state of ldd_block_decompose (ldd_blocks.cu)
@@ -177,7 +178,7 @@ struct ldd_graph {
     std::vector<u32> h_voff;       // union-vertex offsets, k + 1
     UnionMember* d_mem = nullptr;  // k member views (valid only while building)
     u32* d_offs = nullptr;         // 9 arrays of cap.k + 1: v, e, u, c, m, a, o, g, h
-    u32* d_hotv = nullptr;         // [cap.N] members' hot tables
+    u32* d_hotv = nullptr;         // [cap.N] members' hot tables (cap.codes)
     u32* d_ell_buf = nullptr;      // [cap.L] padded rows (g->d_ell when the members have them)
     u32* d_active_buf = nullptr;   // [cap.N] active list (g->d_active when every member has one)
     UnionOffsets off{};

@@ -101,6 +101,7 @@ UnionCaps caps_for(u64 budget, int max_batch, u64 max_vertices, u64 max_arcs) {
   c.k = (u32)max_batch;
   c.E = max_arcs ? max_arcs : std::min<u64>((1ull << 31) - 64, budget / 2 / 12);
   c.M = c.E / 2 + 1;
+  c.codes = c.M >= kCodeMinEdges;
   u64 N = max_vertices ? max_vertices : (1u << 30) - 64;
   N = N / 32 * 32;
   for (;;) {

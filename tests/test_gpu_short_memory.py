@@ -1,5 +1,6 @@
-"""Padded neighbour rows are for speed only: where device memory is too short for
-them, graphs, unions and block decompositions run without."""
+"""Padded neighbour rows and piece codes are for speed only: where device memory is
+too short for rows, graphs, unions and block decompositions run without, and
+unions without hubs have no buffers for codes."""
 from __future__ import annotations
 
 import gc
@@ -32,9 +33,9 @@ class _Hold:
         torch.cuda.empty_cache()
 
 
-def _wide_path(n):
+def _wide_path(n, chords=30):
     """A path with chords at vertex 0, whose row of 31 makes every padded row 32 wide."""
-    e = [(i, i + 1) for i in range(n - 1)] + [(0, (i + 1) * (n // 40)) for i in range(30)]
+    e = [(i, i + 1) for i in range(n - 1)] + [(0, (i + 1) * (n // 90)) for i in range(chords)]
     a = np.array(e, dtype=np.int64)
     src = np.concatenate([a[:, 0], a[:, 1]])
     dst = np.concatenate([a[:, 1], a[:, 0]])
@@ -116,3 +117,16 @@ def test_graph_union_and_blocks_without_rows(ldd, cuda):
         for x, y in zip(want, h.out):
             assert np.array_equal(x, y)
         h.close()
+
+
+def test_union_without_hubs_has_no_code_buffers(ldd, cuda):
+    n = 1 << 21
+    took = []
+    for chords in (30, 60):
+        row, col = _wide_path(n, chords)
+        g = ldd.LddGraph(row, col, validate=False)
+        took.append(_used(lambda: ldd.LddUnion([g, g])))
+        g.close()
+    rows = 2 * n * 32 * 4
+    codes = 2 * n * (2 + 2 + 6)  # code words of vertices, groups and hot table, and that table
+    assert abs(took[1] - (took[0] - rows) - codes) < codes // 4, (took, rows, codes)
