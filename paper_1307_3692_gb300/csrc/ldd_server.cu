@@ -76,10 +76,19 @@ bool fits(const UnionCaps& a, const UnionCaps& b, const UnionCaps& cap) {
 }
 
 // Whether a batch that already holds a request can take b too and keep padded
-// rows.  (A batch of one runs on its own graph object.)  A workspace with room
-// for few rows does not split its batches for them.
+// rows.  (A batch of one runs on its own graph object.)
 bool rows_fit(const UnionCaps& a, const UnionCaps& b, const UnionCaps& cap) {
-  return a.k == 0 || cap.L < cap.N || (a.N + b.N) * std::max(a.S, b.S) <= cap.L;
+  return a.k == 0 || (a.N + b.N) * std::max(a.S, b.S) <= cap.L;
+}
+
+// Whether a batch of `all` vertices is split for one of `rows` vertices that keeps
+// padded rows: if that is a quarter of it at least, and the workspace has room for
+// rows worth the name.  A burst of 48 geometric graphs of 150,000 vertices (rows of
+// 24), split against not split: 3 of 26 graphs per batch 10.8 and 6.3 ms, 3 of 26 on
+// two workspaces 9.7 and 5.6, 12 of 45 5.1 and 5.6; 64 grids of 400 x 400 (rows of 8):
+// 8 of 25 6.1 and 6.7, 34 of 61 3.2 and 4.5.
+bool split_for_rows(u64 rows, u64 all, const UnionCaps& cap) {
+  return cap.L >= cap.N && 4 * rows >= all;
 }
 
 void add_to(UnionCaps& a, const UnionCaps& b) {
@@ -113,10 +122,10 @@ UnionCaps caps_for(u64 budget, int max_batch, u64 max_vertices, u64 max_arcs) {
     if (max_vertices || N <= 32 || union_bytes(c) <= budget) break;
     N = std::max<u64>(32, N / 10 * 9 / 32 * 32);
   }
-  // padded rows take what is left, up to 8 entries per vertex: they never cost a
-  // request its place.  A batch without room for them runs the general rounds.
+  // padded rows take what is left, up to the longest for every vertex: they never cost
+  // a request its place.  A batch without room for them runs the general rounds.
   const u64 used = union_bytes(c);
-  c.L = used < budget ? std::min<u64>(8 * c.N, (budget - used) / 4 / 8 * 8) : 0;
+  c.L = used < budget ? std::min<u64>((u64)kLdMaxDegree * c.N, (budget - used) / 4 / 8 * 8) : 0;
   return c;
 }
 
@@ -241,15 +250,29 @@ void worker_batched(ldd_server* S, int slot) {
       // A burst of 24 over four R-MAT graphs and four grids: 7.1-7.6 -> 4.0 ms.
       UnionCaps sum;
       const bool kind = S->queue.front()->g->low_degree();
-      for (auto it = S->queue.begin(); it != S->queue.end();) {
-        if ((*it)->g->low_degree() != kind) {
-          ++it;
-          continue;
+      size_t with_rows = 0;  // the first requests of the batch, with room for their rows
+      u64 with_rows_n = 0;
+      for (Request* r : S->queue) {
+        if (r->g->low_degree() != kind) continue;
+        if (!fits(sum, r->need, S->cap)) break;
+        const bool rows = with_rows == batch.size() && rows_fit(sum, r->need, S->cap);
+        add_to(sum, r->need);
+        batch.push_back(r);
+        if (rows) {
+          with_rows = batch.size();
+          with_rows_n = sum.N;
         }
-        if (!fits(sum, (*it)->need, S->cap) || !rows_fit(sum, (*it)->need, S->cap)) break;
-        add_to(sum, (*it)->need);
-        batch.push_back(*it);
-        it = S->queue.erase(it);
+      }
+      if (with_rows < batch.size() && split_for_rows(with_rows_n, sum.N, S->cap))
+        batch.resize(with_rows);
+      size_t taken = 0;  // the batch is a subsequence of the queue
+      for (auto it = S->queue.begin(); it != S->queue.end() && taken < batch.size();) {
+        if (*it == batch[taken]) {
+          it = S->queue.erase(it);
+          ++taken;
+        } else {
+          ++it;
+        }
       }
       bid = S->next_batch++;
     }
