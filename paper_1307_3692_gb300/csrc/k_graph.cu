@@ -1060,17 +1060,19 @@ __global__ void __launch_bounds__(256) k_gather_codes(CutList cl, CutCodes cc) {
 // sector per cycle and SM; code words keep nine in ten edges of an R-MAT graph
 // out of it, and the pass is bound by the instructions per edge: hence code words
 // compared two edges at a time, the separate branch for a whole chunk inside its
-// segment, and kOne (K = 1), which needs no fields.
-constexpr u32 kCodeShares = 4;
-
+// segment, and a union's one labeling without fields.  (One labeling of one graph
+// goes by labels: see cut_labels.)
 //
 // Cut counts, before and now: 64 copies of R-MAT 20 as a union 2.42-2.61 -> 1.60
 // ms (1.00 G edges; the pass itself 1.30 ms, 3.4 TB/s); R-MAT 22's batch of three
 // labelings 1.060 -> 0.990 ms in all.
-template <bool U, bool kOne>
+constexpr u32 kCodeShares = 4;
+
+template <bool U>
 __global__ void __launch_bounds__(kCutThreads, 1) k_cut_codes(CutList cl, CutCodes cc, Labels4 L,
                                                               int K, UnionOffsets off, u32 k,
                                                               u64* out) {
+  constexpr bool kOne = U;  // one labeling
   extern __shared__ int4 cut_smem[];
   u16* table = reinterpret_cast<u16*>(cut_smem);
   __shared__ u32 wsum[kCutThreads / 32][4];
@@ -1299,12 +1301,12 @@ int launch_cut4(const CutList& cl, const int* const* centers, int K, u32 n, cons
 
 namespace {
 // The dynamic shared memory of the code-word table, allowed once per device.
-template <bool U, bool kOne>
+template <bool U>
 void allow_code_smem() {
   static bool attr_set[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !attr_set[dev]) {
-    cudaFuncSetAttribute(k_cut_codes<U, kOne>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_cut_codes<U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(kCodeSlots * sizeof(u16)));
     attr_set[dev] = true;
   }
@@ -1317,10 +1319,9 @@ u32 cut_code_grid(const CutList& cl, int num_sms) {
 
 int launch_cut_codes(const CutList& cl, const CutCodes& cc, const int* const* centers, int K, u32 n,
                      u64* out, int num_sms, cudaStream_t s) {
-  if (cl.m == 0 || K < 1 || K > 4) return 0;
-  allow_code_smem<false, true>();
-  allow_code_smem<false, false>();
-  Labels4 L = {{centers[0], K > 1 ? centers[1] : nullptr, K > 2 ? centers[2] : nullptr,
+  if (cl.m == 0 || K < 2 || K > 4) return 0;
+  allow_code_smem<false>();
+  Labels4 L = {{centers[0], centers[1], K > 2 ? centers[2] : nullptr,
                 K > 3 ? centers[3] : nullptr}};
   const UnionOffsets none{};
   k_picks<false><<<K, 32, 0, s>>>(cc, L, none);
@@ -1328,12 +1329,8 @@ int launch_cut_codes(const CutList& cl, const CutCodes& cc, const int* const* ce
   k_gather_codes<<<grid_for((cl.ngrp + cc.nhot + kLabIpt - 1) / kLabIpt, num_sms), 256, 0, s>>>(cl,
                                                                                              cc);
   const size_t smem = ((size_t)cc.nhot * sizeof(u16) + 15) / 16 * 16;
-  if (K == 1)
-    k_cut_codes<false, true><<<cut_code_grid(cl, num_sms), kCutThreads, smem, s>>>(cl, cc, L, K,
-                                                                                 none, 0, out);
-  else
-    k_cut_codes<false, false><<<cut_code_grid(cl, num_sms), kCutThreads, smem, s>>>(cl, cc, L, K,
-                                                                                  none, 0, out);
+  k_cut_codes<false><<<cut_code_grid(cl, num_sms), kCutThreads, smem, s>>>(cl, cc, L, K, none, 0,
+                                                                         out);
   return 4;
 }
 
@@ -1349,13 +1346,13 @@ int launch_union_cut(const CutList& cl, const int* center, u64* cut, int num_sms
 int launch_union_cut_codes(const CutList& cl, const CutCodes& cc, const UnionOffsets& off, u32 k,
                            u32 total, const int* center, u64* cut, int num_sms, cudaStream_t s) {
   if (cl.m == 0) return 0;
-  allow_code_smem<true, true>();
+  allow_code_smem<true>();
   const Labels4 L = {{center, nullptr, nullptr, nullptr}};
   k_picks<true><<<k, 32, 0, s>>>(cc, L, off);
   k_union_codes<<<grid_for((total + 3) / 4, num_sms), 256, 0, s>>>(cc, center, off, k, total);
   k_gather_codes<<<grid_for((cl.ngrp + cc.nhot + kLabIpt - 1) / kLabIpt, num_sms), 256, 0, s>>>(cl,
                                                                                              cc);
-  k_cut_codes<true, true><<<cut_code_grid(cl, num_sms), kCutThreads, kCodeSlots * sizeof(u16), s>>>(
+  k_cut_codes<true><<<cut_code_grid(cl, num_sms), kCutThreads, kCodeSlots * sizeof(u16), s>>>(
       cl, cc, L, 1, off, k, cut);
   return 4;
 }

@@ -439,20 +439,19 @@ __global__ void __launch_bounds__(256) k_rank_scatter(const u32* __restrict__ v0
 // histogram read in reverse, data[r] = rev_src[A - r] for
 // r = 0 .. A and 0 for r = A + 1, and rev_src is cleared on the way (all zero
 // for the next decomposition); a table of fewer than A + 2 entries (cap) sets
-// kErrBucketCap.  Optionally copies the result to copy[] and records the
-// largest input value in *maxv.  Tiles take tickets in order, so every tile's
-// predecessors are running or done; every wait is bounded (spin_limit polls,
-// then kErrTimeout).  One warp looks back over 32 predecessor tiles at a time.
+// kErrBucketCap.  Optionally copies the result to copy[].  Tiles take tickets in
+// order, so every tile's predecessors are running or done; every wait is bounded
+// (spin_limit polls, then kErrTimeout).  One warp looks back over 32 predecessor
+// tiles at a time.
 // stall = 1 makes tile 0 wait, like the others, on a predecessor that does not
 // exist, so that every look-back runs out of polls (tests of the timeout path).
 __global__ void __launch_bounds__(kScanThreads) k_scan_excl(u32* data, u32* copy, u32 len_host,
                                                             int len_from_A, u64* __restrict__ status,
-                                                            u32 epoch, u32* tile_ctr, u32* maxv,
-                                                            u32* rev_src, u32 cap, Control* ctl,
+                                                            u32 epoch, u32* tile_ctr, u32* rev_src,
+                                                            u32 cap, Control* ctl,
                                                             u32 spin_limit, u32 stall) {
   __shared__ u32 s_tile, s_excl, s_bad;
   __shared__ u32 s_wsum[kScanThreads / 32];
-  __shared__ u32 s_wmax[kScanThreads / 32];
   if (failed(ctl)) {
     // an upstream error skips the scan; the floor counts are still cleared, so
     // a decomposition queued behind this one starts from zero counts
@@ -484,7 +483,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_excl(u32* data, u32* copy
   if (t0 >= len) return;  // tiles past the end: no later tile needs them
   const u32 my0 = t0 + tid * kScanIpt;
   u32 v[kScanIpt];
-  u32 tot = 0, mx = 0;
+  u32 tot = 0;
 #pragma unroll
   for (int i = 0; i < kScanIpt; ++i) {
     const u32 r = my0 + i;
@@ -498,7 +497,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_excl(u32* data, u32* copy
       v[i] = (r < len) ? data[r] : 0u;
     }
     tot += v[i];
-    mx = max(mx, v[i]);
   }
   u32 x = tot;
 #pragma unroll
@@ -506,16 +504,12 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_excl(u32* data, u32* copy
     const u32 y = __shfl_up_sync(kFull, x, o);
     if (lane >= (u32)o) x += y;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, o));
   if (lane == 31) s_wsum[warp] = x;
-  if (lane == 0) s_wmax[warp] = mx;
   __syncthreads();
-  u32 wpre = 0, tile_tot = 0, tile_max = 0;
+  u32 wpre = 0, tile_tot = 0;
   for (u32 w = 0; w < kScanThreads / 32; ++w) {
     if (w < warp) wpre += s_wsum[w];
     tile_tot += s_wsum[w];
-    tile_max = max(tile_max, s_wmax[w]);
   }
   if (warp == 0) {
     const u64 tag = (u64)epoch << 32;
@@ -567,7 +561,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_excl(u32* data, u32* copy
   }
   __syncthreads();
   if (s_bad) return;
-  if (tid == 0 && maxv && tile_max) atomicMax(maxv, tile_max);
   u32 run = s_excl + wpre + x - tot;
 #pragma unroll
   for (int i = 0; i < kScanIpt; ++i) {
@@ -796,8 +789,8 @@ int launch_rank_and_buckets(const RankBufs& r, bool exact64, cudaStream_t s,
     const u32 tiles = (u32)((std::min<u64>(r.bptr_cap, (u64)r.f.cap + 2) + kScanTile - 1) /
                             kScanTile);
     k_scan_excl<<<tiles, kScanThreads, 0, s>>>(rcnt, r.rcur, 0, 1, r.status, ++(*r.epoch),
-                                               &ctl->tile_ctr[1], nullptr, r.acnt, r.bptr_cap,
-                                               ctl, r.lookback_limit, r.stall_lookback);
+                                               &ctl->tile_ctr[1], r.acnt, r.bptr_cap, ctl,
+                                               r.lookback_limit, r.stall_lookback);
     return launches + 1;
   }
   // exact path: stable LSD radix sort of all fractions, then keys and the
@@ -822,7 +815,7 @@ int launch_rank_and_buckets(const RankBufs& r, bool exact64, cudaStream_t s,
                                                                             ctl);
   k_keys<<<gs, 256, 0, s>>>(r.a, rank, r.excl, ctl, n, r.key, rcnt);
   k_scan_excl<<<rtiles, kScanThreads, 0, s>>>(rcnt, r.rcur, 0, 1, r.status, ++(*r.epoch),
-                                               &ctl->tile_ctr[1], nullptr, nullptr, 0, ctl,
+                                               &ctl->tile_ctr[1], nullptr, 0, ctl,
                                                r.lookback_limit, r.stall_lookback);
   k_rscatter<<<(u32)min((long long)(n + 256 * kRChunk - 1) / (256 * kRChunk),
                         (long long)r.num_sms * 8),
@@ -835,7 +828,7 @@ int launch_exclusive_scan(u32* data, u32 len, u64* status, u32* epoch, u32* tile
   const u32 tiles = (len + kScanTile - 1) / kScanTile;
   if (tiles == 0) return 0;
   k_scan_excl<<<tiles, kScanThreads, 0, s>>>(data, copy, len, 0, status, ++(*epoch), tile_ctr,
-                                             nullptr, nullptr, 0, ctl, spin_limit, 0);
+                                             nullptr, 0, ctl, spin_limit, 0);
   return 1;
 }
 
@@ -853,7 +846,7 @@ int launch_ranked_and_buckets(const RankBufs& r, const int* levels, const int* p
                                                                             ctl);
   k_keys<<<gs, 256, 0, s>>>(r.a, rank, r.excl, ctl, n, r.key, rcnt);
   k_scan_excl<<<rtiles, kScanThreads, 0, s>>>(rcnt, r.rcur, 0, 1, r.status, ++(*r.epoch),
-                                               &ctl->tile_ctr[1], nullptr, nullptr, 0, ctl,
+                                               &ctl->tile_ctr[1], nullptr, 0, ctl,
                                                r.lookback_limit, r.stall_lookback);
   k_rscatter<<<(u32)min((long long)(n + 256 * kRChunk - 1) / (256 * kRChunk),
                         (long long)r.num_sms * 8),

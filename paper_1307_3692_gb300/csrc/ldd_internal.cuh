@@ -333,7 +333,7 @@ struct CutCodes {
   u16* hcode = nullptr;       // [hot-table entries]
   u32 nhot = 0;
 };
-// out[i] += labeling i's count, i < K <= 4, over one graph's cut list.
+// out[i] += labeling i's count, i < K (2 .. 4), over one graph's cut list.
 int launch_cut_codes(const CutList& cl, const CutCodes& cc, const int* const* centers, int K, u32 n,
                      u64* out, int num_sms, cudaStream_t s);
 int launch_small_comp(const SmallComps& sc, const BfsArgs& a, int num_sms, cudaStream_t s);
