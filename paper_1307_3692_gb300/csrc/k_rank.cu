@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(256) k_direct(const double* __restrict__ delta
     if (lane == 0) bmax[wb / kMaxBlock] = top;
   }
   if (amax > f.cap) err |= kErrLevelCap;
-  if (lane == 0 && ab) atomicMax(&s_ab, (int)ab - 1);
+  if (lane == 0 && ab) atomicMax(&s_ab, (int)(ab - 1));
   __syncthreads();
   for (u32 i = tid; i < kRBins; i += blockDim.x)
     if (sh[i] && (u64)i + 2 <= cap) atomicAdd(acnt + i, sh[i]);
