@@ -10,9 +10,10 @@
 // exact label the paper's super-source shortest path assigns (Section 4),
 // including the fraction tie-break.  Wherever two direct keys that differ only
 // in their ids meet -- at a vertex, in the minimum that a bottom-up round stops
-// at, or between that minimum and what a candidate holds when its scan stops or
-// is left out -- the meeting is listed (note_tie) and finalize compares the exact
-// fractions, so a decomposition that ends without an error bit is exact.
+// at, between that minimum and a start that it passes over, or between a pivot and
+// the frontier's other keys -- the meeting is listed (note_tie) and finalize
+// compares the exact fractions, so a decomposition that ends without an error bit
+// is exact.
 //
 // Start buckets.  With direct keys the loop itself fills the buckets, some
 // levels ahead at a time (build_buckets): it passes over the blocks of vertices
@@ -1285,6 +1286,7 @@ __device__ __forceinline__ void list_pushes(const BfsArgs& a, int cur, u32 Q, u6
       const u64 pv = U ? member_floor(a, v[0], mslot, s_floor, true) : pivot;
       push = r < pv || key_tie(a.f, r, pv);
       if (push) {
+        note_tie(a, v[0], r, pv);  // a scan may stop at r, the pivot's own offer unread
         rs[0] = __ldg(a.row_ptr + v[0]);
         re[0] = __ldg(a.row_ptr + v[0] + 1);
         v[0] |= kPushFlag;
@@ -1372,10 +1374,7 @@ __device__ __forceinline__ void pull_rest(const BfsArgs& a, u32 Q, u32 E, int lv
         best = ~0ull;
       }
       const u32 stop = min(end, p1);
-      if (!push && p < stop && min(kw, best) <= fl) {  // nothing can beat it
-        note_tie(a, w, min(kw, best), fl);             // (as in pull_round)
-        p = stop;
-      }
+      if (!push && p < stop && min(kw, best) <= fl) p = stop;  // nothing can beat it
       u32 vv[kRestBatch];
 #pragma unroll
       for (int q = 0; q < kRestBatch; ++q)
@@ -1571,6 +1570,15 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u64 stop_l
       if (!(key_level(a.f, kw[j]) > L && kw[j] > (lvl_key | fr[j]))) re[j] = e[j];  // settled or unbeatable
       if (U && fr[j] == ~0ull) re[j] = e[j];  // w's member has no level-L key
     }
+    // a start of level L + 1 may only tie with the floor or pivot that it is passed over for
+    bool tie = false;
+#pragma unroll
+    for (int j = 0; j < kPullV; ++j) tie |= key_near(kw[j], lvl_key | fr[j]);
+    if (tie) {
+#pragma unroll
+      for (int j = 0; j < kPullV; ++j)
+        if (w[j] != kNone) note_tie(a, w[j], kw[j], lvl_key | fr[j]);
+    }
     // the first neighbour of every candidate, then two of every one still
     // scanning per step, for about kPullLong neighbours: most scans stop at the
     // first, and the warp's slowest lane sets the pass (one per step: 64 R-MAT 20
@@ -1681,16 +1689,6 @@ __device__ __forceinline__ void pull_round(const BfsArgs& a, int lvl, u64 stop_l
           scanned += (u32)(min(pos, ee) - eb);
         }
       }
-    }
-    // what the scan stopped at, or was not begun for, against what w holds: the offers
-    // left unread are no better than (L + 1, fr), and may only tie with it
-    bool tie = false;
-#pragma unroll
-    for (int j = 0; j < kPullV; ++j) tie |= key_tie(a.f, best[j], lvl_key | fr[j]);
-    if (tie) {
-#pragma unroll
-      for (int j = 0; j < kPullV; ++j)
-        if (w[j] != kNone) note_tie(a, w[j], best[j], lvl_key | fr[j]);
     }
     u64 kwn[kPullV];  // the next pass's keys and ranges, beside this pass's appends
     int en[kPullV], ren[kPullV];
