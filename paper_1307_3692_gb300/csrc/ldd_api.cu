@@ -673,11 +673,17 @@ u64 floors_for(const ldd_graph* g, double beta) {
   return std::max(floors_for_beta(g, beta), g->wide_floors);
 }
 
-// Floors beyond what beta suggests are expected again, up to twice as large; the first
-// call without them ends that, so a single huge shift costs the next call's codes a
-// few bits and no more.
+// Floors beyond what beta suggests are expected again, up to twice as large, as long as
+// that leaves kWideCodeBits; the first call without them ends it.  So one huge shift
+// costs the call after it a few code bits at most.  (With 20 bits R-MAT 22's meetings
+// would tie for certain, with 28 they do in one call of a few hundred.)
+constexpr u32 kWideCodeBits = 28;
 u64 wide_floors(const ldd_graph* g, double beta, int A) {
-  return (u64)A > floors_for_beta(g, beta) ? 2 * (u64)A : 0;
+  if ((u64)A <= floors_for_beta(g, beta)) return 0;
+  const u64 wide[2] = {2 * (u64)A, (u64)A};
+  for (u64 w : wide)
+    if (direct_fmt(g, w).cb >= kWideCodeBits) return w;
+  return 0;
 }
 
 struct Header {  // the control block up to and including the BFS runtime state
