@@ -453,8 +453,8 @@ float elapsed(ldd_graph* g, int a, int b) {
 // random geometric graph of 150,001 vertices 0.43, 0.52, 0.85).
 constexpr u32 kDefaultWindowLevels = 8;
 // Unions: one is what a fresh union reports, and what ldd_set_tuning(1) gives; while
-// its tuning has not been set, one of low-degree graphs relaxes four (64 random geometric graphs: 1 level 3.55, 3 2.70, 4 2.63, 6 2.65,
-// 8 2.74 ms).
+// its tuning has not been set, one of low-degree graphs relaxes four (64 random
+// geometric graphs: 1 level 3.55, 3 2.70, 4 2.63, 6 2.65, 8 2.74 ms).
 constexpr u32 kDefaultUnionWindowLevels = 1;
 constexpr u32 kLdUnionWindowLevels = 4;
 
@@ -667,22 +667,21 @@ u64 floors_for_beta(const ldd_graph* g, double beta) {
 }
 
 // The range of floors a call lays its keys out for: what beta suggests, or the one of
-// the call before if its shifts went beyond that.  Only a hint: larger floors make the call
-// widen the level field and run its key pass again.
+// the call before if its shifts went beyond that.  Only a hint: larger floors make the
+// call widen the level field and run its key pass again.
 u64 floors_for(const ldd_graph* g, double beta) {
   return std::max(floors_for_beta(g, beta), g->wide_floors);
 }
 
-// Floors beyond what beta suggests are expected again, up to twice as large, as long as
-// that leaves kWideCodeBits; the first call without them ends it.  So one huge shift
-// costs the call after it a few code bits at most.  (With 20 bits R-MAT 22's meetings
-// would tie for certain, with 28 they do in one call of a few hundred.)
-constexpr u32 kWideCodeBits = 28;
+// Floors beyond what beta suggests are expected again, up to twice as large, if that
+// leaves a direct layout; the first call without them ends it.  So one huge shift costs
+// the call after it code bits and no more: at kMinCodeBits none of 16 shift seeds of R-MAT
+// 22 (beta 0.1 and 0.5), or of the 256^3 grid (0.05), needed ranks.
 u64 wide_floors(const ldd_graph* g, double beta, int A) {
   if ((u64)A <= floors_for_beta(g, beta)) return 0;
   const u64 wide[2] = {2 * (u64)A, (u64)A};
   for (u64 w : wide)
-    if (direct_fmt(g, w).cb >= kWideCodeBits) return w;
+    if (direct_fmt(g, w).cap) return w;
   return 0;
 }
 
@@ -921,8 +920,8 @@ int enqueue_fast(ldd_graph* g, KeyFmt f, bool want_cut) {
   return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 
-// Captures enqueue_fast into executable graph `slot`.  A capture that fails marks the graph replay_broken; the regular
-// path then runs.
+// Captures enqueue_fast into executable graph `slot`.  A capture that fails marks
+// the graph replay_broken; the regular path then runs.
 void capture_fast(ldd_graph* g, KeyFmt f, bool want_cut, int slot) {
   if (!g->cap_stream &&
       cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {

@@ -150,7 +150,7 @@ struct ldd_graph {
   }
   // Set by the user (else bfs_per_sm, pull_alpha and a union's windows follow the graph).
   bool per_sm_set = false, pull_set = false, window_set = false;
-  u64 wide_floors = 0;            // range of floors, if the last call's went beyond what its beta suggests
+  u64 wide_floors = 0;            // range of floors, if the last call's went beyond beta's
   u32 window_levels = 0;          // tuning: levels per window in low-degree rounds (0: none)
   u32 window_max_q = 1u << 18;    // tuning: windows only for frontiers up to this size
   u32 window_queue = 0;           // tuning: local-queue entries per CTA and level (0: all that fit)
